@@ -42,6 +42,12 @@ void set_global_error(const char* msg) noexcept {
 
 namespace {
 
+// The block form pays for an eigenproblem per k from this many frequencies on.
+constexpr int kBlkMinFreq = 16;
+// Lowest pi / beta of the block form (eV): below it an eigenvalue of the n2 block that happens
+// to lie near mu would cost more digits than the pivoted inverse loses.
+constexpr double kBlkMinW = 1e-4;
+
 gf_status ensure_einf(gf_ctx* c) {
   if (!c->einf_dirty) return GF_OK;
   GF_CU(gf::launch_einf(c->kinfo_d.as<KInfo>(), c->sinfo_d.as<SInfo>(), c->H.as<double2>(),
@@ -76,12 +82,123 @@ gf_status ensure_lr(gf_ctx* c) {
   return GF_OK;
 }
 
-// rho_k partial sums: the low-rank kernel leaves them in the eigenbasis of H_k;
-// sum the chunks and rotate back, leaving one chunk for k_rho_finalize.
+// Block form (gf_block.cuh) of the uploaded H and P, once per upload.  blk_ok is false when an
+// H_k is not Hermitian to rounding, a P_k has (nearly) dependent rows, an eigenproblem does not
+// converge or the tables do not fit: every call then takes the general kernels.
+gf_status ensure_block(gf_ctx* c) {
+  if (!c->blk_shape || !c->blk_dirty) return GF_OK;
+  c->blk_ok = false;
+  const size_t mm = (size_t)c->mmax * c->mmax, npm = (size_t)c->mmax * (c->mmax + 1) / 2;
+  const bool mixed = c->precision == GF_PREC_MIXED;
+  const size_t smem = gf::heev_smem(c->blk_n2max), limit = (size_t)c->smem_optin - 8192;
+  const int in_smem = smem <= limit ? 1 : 0;
+  const int grid = std::max(1, std::min(c->n_k, c->sm_count * (in_smem ? std::min(8, std::max(1, (int)(limit / smem))) : 2)));
+  const size_t ws = std::max(gf::block_reduce_ws_elems(c->nbmax, c->mmax, c->smem_optin, c->sm_count),
+                             in_smem ? (size_t)0 : gf::heev_ws_elems(c->blk_n2max) * grid);
+  struct {
+    DevBuf* b;
+    size_t bytes;
+  } need[] = {{&c->blk_e, 8 * (size_t)c->totNb},    {&c->blk_T, 16 * (size_t)c->blk_totT},
+              {&c->blk_Ts, mixed ? 8 * (size_t)c->blk_totT : 0}, {&c->blk_B, 16 * (size_t)c->totP},
+              {&c->blk_Bs, mixed ? 8 * (size_t)c->totP : 0},     {&c->blk_HO, 32 * npm * c->n_k},
+              {&c->blk_U, 16 * (size_t)c->totH},     {&c->blk_D22, 16 * (size_t)c->totH},
+              {&c->blk_V, 16 * (size_t)c->totP},     {&c->blk_R, 16 * mm * c->n_k},
+              {&c->blk_H11, 16 * mm * c->n_k},       {&c->blk_tau, 8 * (size_t)c->mmax * c->n_k},
+              {&c->blk_ws, 16 * ws},                 {&c->blk_info, 8 * ((size_t)c->n_k + 1)}};
+  for (auto& n : need) {
+    if (ensure(*n.b, n.bytes) == cudaSuccess) continue;
+    cudaGetLastError();
+    for (auto& r : need) release(*r.b);
+    c->blk_shape = false;  // no room for the tables: the general kernels from now on
+    c->tune_log += "block form: tables do not fit in device memory; ";
+    return GF_OK;
+  }
+  gf::BlockSetup b{};
+  b.H = c->H.as<double2>();
+  b.P = c->P.as<double2>();
+  b.kinfo = c->kinfo_d.as<KInfo>();
+  b.sinfo = c->sinfo_d.as<SInfo>();
+  b.n_k = c->n_k;
+  b.nbmax = c->nbmax;
+  b.mmax = c->mmax;
+  b.n2max = c->blk_n2max;
+  b.npmax = (int)npm;
+  b.D22 = c->blk_D22.as<double2>();
+  b.V = c->blk_V.as<double2>();
+  b.R = c->blk_R.as<double2>();
+  b.tau = c->blk_tau.as<double>();
+  b.H11 = c->blk_H11.as<double2>();
+  b.B = c->blk_B.as<double2>();
+  b.e = c->blk_e.as<double>();
+  b.offD = c->offD_d.as<int64_t>();
+  b.T = c->blk_T.as<double2>();
+  b.Ts = mixed ? c->blk_Ts.as<float2>() : nullptr;
+  b.offT = c->blk_offT.as<int64_t>();
+  b.Bs = mixed ? c->blk_Bs.as<float2>() : nullptr;
+  b.HO = c->blk_HO.as<double2>();
+  b.U = c->blk_U.as<double2>();
+  b.ws = c->blk_ws.as<double2>();
+  b.hnorm = c->blk_info.as<double>();
+  b.flags = reinterpret_cast<int*>(b.hnorm + c->n_k);
+  GF_CU(cudaMemsetAsync(b.flags, 0, sizeof(double), c->stream));
+  GF_CU(gf::launch_block_reduce(b, c->smem_optin, c->sm_count, c->stream));
+  GF_CU(gf::launch_block_eig(b, c->blk_ws.as<double2>(), grid, in_smem, c->stream));
+  GF_CU(gf::launch_block_finish(b, c->stream));
+  c->last_launches += 3;
+  std::vector<double> info((size_t)c->n_k + 1);
+  GF_CU(cudaMemcpyAsync(info.data(), c->blk_info.p, 8 * info.size(), cudaMemcpyDeviceToHost, c->stream));
+  GF_CU(cudaStreamSynchronize(c->stream));
+  c->blk_dirty = false;
+  int flags = 0;
+  std::memcpy(&flags, &info[c->n_k], sizeof(int));
+  c->blk_ok = flags == 0;
+  if (flags) {
+    c->tune_log += "block form: general kernels (" +
+                   std::string(flags & gf::kBlkNonHermitian ? "H not Hermitian" :
+                               flags & gf::kBlkRankDeficient ? "P rank deficient" : "eigensolver") + "); ";
+    return GF_OK;
+  }
+  // mixed precision: frequencies w_n below a quarter of the rms eigenvalue of H run in FP64
+  // (an eigenvalue e_b within w_n of mu loses |B|^2 / w_n in FP32)
+  double h = 0.0, bmax = 0.0;
+  for (int k = 0; k < c->n_k; ++k) h = std::max(h, info[k]);
+  for (int s = 0; s < c->n_sys; ++s) bmax = std::max(bmax, c->beta[s]);
+  const double nc = std::ceil(0.5 * (0.25 * h * bmax / M_PI - 1.0));
+  const int batch = gf::block_batch(c->mmax);
+  const int64_t up = (int64_t)std::min((double)c->n_iw, std::max(1.0, nc));
+  c->blk_nc = mixed && !c->lowrank ? (int)std::min<int64_t>(c->n_iw, (up + batch - 1) / batch * batch) : c->n_iw;
+  return GF_OK;
+}
+
+// Whether a call of this mode runs on the block form.  GF_KERNEL=direct keeps the general
+// kernels; with GF_PREC_MIXED every value of GF_KERNEL does, as it names one of them.
+bool use_block(const gf_ctx* c, int mode) {
+  if (!c->blk_shape || !c->blk_ok) return false;
+  const char* only = std::getenv("GF_KERNEL");
+  if (only && (std::strcmp(only, "direct") == 0 || (c->precision == GF_PREC_MIXED && !c->lowrank))) return false;
+  if (c->precision == GF_PREC_MIXED && !c->lowrank && mode == gf::kOcc) return false;
+  // sizes that the general kernels refuse stay refused
+  const size_t limit = (size_t)c->smem_optin - 1024;
+  const size_t general = c->lowrank ? gf::point_lr_smem(c->nbmax, c->mmax, mode, 0, c->precision != GF_PREC_FP64)
+                                    : gf::point_fp64_smem(c->nbmax, c->mmax, mode, 0);
+  if (general > limit || (c->lowrank && c->nbmax > gf::heev_max_n())) return false;
+  return gf::block_smem(c->mmax, c->blk_n2max, mode, 0) <= limit;
+}
+
+// rho_k partial sums: the low-rank and the block kernels leave them in the basis that makes
+// H_k (its n2 block) diagonal; sum the chunks and rotate back, leaving one chunk for
+// k_rho_finalize.
 gf_status rho_partials(gf_ctx* c, int* n_chunks) {
-  *n_chunks = c->n_chunks;
-  if (!c->lowrank) return GF_OK;
+  *n_chunks = c->run_chunks;
+  if (!c->lowrank && !c->run_on_block) return GF_OK;
   GF_CU(ensure(c->lr_T, sizeof(double2) * c->totH));
+  if (c->run_on_block) {
+    GF_CU(gf::launch_block_rotate(c->kinfo_d.as<KInfo>(), c->n_k, c->blk_U.as<double2>(), c->rho_part.as<double2>(),
+                                  c->totH, c->run_chunks, c->lr_T.as<double2>(), c->stream));
+    c->last_launches += 1;
+    *n_chunks = 1;
+    return GF_OK;
+  }
   GF_CU(gf::launch_lr_rotate(c->kinfo_d.as<KInfo>(), c->n_k, c->lr_U.as<double2>(),
                              c->rho_part.as<double2>(), c->totH, c->n_chunks, c->lr_T.as<double2>(),
                              c->stream));
@@ -378,6 +495,100 @@ double point_flops_lr(int N, int M, int mode) {
   return 8.0 * cmac;
 }
 
+// The point kernels on the block form, for every k (or k-group) and frequency chunk: one
+// launch in FP64, and in mixed precision a second one for the frequencies from blk_nc on,
+// whose traces and rho_k need FP32 only.
+gf_status run_block(gf_ctx* c, int mode, gf::PointParams p) {
+  const bool kred = (mode & (gf::kGloc | gf::kAdj)) != 0;
+  const bool low = c->precision == GF_PREC_MIXED && !c->lowrank && !(mode & gf::kAdj);
+  const int nc = low ? c->blk_nc : c->n_iw;
+  const int ch0 = (nc + c->blk_cw - 1) / c->blk_cw;
+  const int ch1 = (c->n_iw - nc + c->blk_cw - 1) / c->blk_cw;
+  c->run_chunks = ch0 + ch1;
+  p.n_chunks = c->run_chunks;
+  if (mode & gf::kOcc) {
+    GF_CU(ensure(c->occ_part, sizeof(double) * 2 * (size_t)c->n_k * c->run_chunks));
+    p.occ_part = c->occ_part.as<double>();
+  }
+  if (mode & gf::kRho) {
+    p.rho_chunk_stride = c->totH;
+    GF_CU(ensure(c->rho_part, sizeof(double2) * (size_t)c->totH * c->run_chunks));
+    p.rho_part = c->rho_part.as<double2>();
+  }
+  if (mode & gf::kAdj) {
+    GF_CU(ensure(c->mubar_part, sizeof(double) * (size_t)c->n_k * c->run_chunks));
+    p.mubar_part = c->mubar_part.as<double>();
+  }
+  gf::BlockForm b{};
+  b.e = c->blk_e.as<double>();
+  b.offD = c->offD_d.as<int64_t>();
+  b.T = c->blk_T.as<double2>();
+  b.Ts = c->blk_Ts.as<float2>();
+  b.offT = c->blk_offT.as<int64_t>();
+  b.B = c->blk_B.as<double2>();
+  b.Bs = c->blk_Bs.as<float2>();
+  b.HO = c->blk_HO.as<double2>();
+  b.npmax = c->mmax * (c->mmax + 1) / 2;
+  gf::BlockLaunch l{};
+  l.n2max = c->blk_n2max;
+  l.chunk_w = c->blk_cw;
+  // units: the k-groups in order, then the single k-points by decreasing window
+  l.units = c->blk_units.as<int2>() + (kred ? 0 : c->blk_groups);
+  l.kperm = c->blk_perm.as<int>() + (kred ? 0 : c->n_k);
+  const int n_units = kred ? c->blk_groups : c->n_k;
+  const size_t per_group = sizeof(double2) * (size_t)c->n_iw * c->mmax * c->mmax;
+  const int step = kred ? (int)std::max<size_t>(1, std::min<size_t>(n_units, c->gq_budget / per_group)) : n_units;
+  int max_total = 0;
+  for (const SInfo& si : c->sinfo) max_total = std::max(max_total, c->n_iw * si.m * si.m);
+  for (int u0 = 0; u0 < n_units; u0 += step) {
+    l.unit0 = u0;
+    l.n_units = std::min(step, n_units - u0);
+    if (kred) {
+      GF_CU(ensure(c->gq, per_group * l.n_units));
+      p.gq = c->gq.as<double2>();
+      p.gb0 = u0;
+    }
+    reserve_events(c, c->ev_used + 2);
+    while ((int)c->ev.size() < c->ev_used + 2) {
+      cudaEvent_t e;
+      GF_CU(cudaEventCreate(&e));
+      c->ev.push_back(e);
+    }
+    if (!c->capturing) GF_CU(cudaEventRecord(c->ev[c->ev_used], c->stream));
+    for (int part = 0; part < 2; ++part) {
+      l.n_begin = part ? nc : 0;
+      l.n_end = part ? c->n_iw : nc;
+      l.chunk0 = part ? ch0 : 0;
+      l.n_chunks = part ? ch1 : ch0;
+      if (l.n_chunks == 0) continue;
+      GF_CU(gf::launch_point_block(p, b, l, part, c->stream));
+      c->last_launches += 1;
+    }
+    if (!c->capturing) {
+      GF_CU(cudaEventRecord(c->ev[c->ev_used + 1], c->stream));
+      c->ev_used += 2;
+    }
+    if (kred) {
+      GF_CU(gf::launch_gq_reduce(c->sinfo_d.as<SInfo>(), c->n_sys, max_total, c->blk_sysg.as<int>(),
+                                 c->blk_sysg.as<int>() + c->n_sys, c->gq.as<double2>(), u0, u0 + l.n_units, c->n_iw,
+                                 c->mmax, u0 == 0, c->gacc.as<double2>(), c->stream));
+      c->last_launches += 1;
+    }
+  }
+  for (int k = 0; k < c->n_k; ++k) {
+    const int m = c->msys[c->ksys[k]];
+    c->last_flops += c->n_iw * (c->lowrank ? point_flops_lr(c->nb[k], m, mode) : point_flops(c->nb[k], m, mode));
+  }
+  c->last_points += (int64_t)c->n_k * c->n_iw;
+  const int key = -1 - mode;
+  if (c->tuned.find(key) == c->tuned.end()) {
+    c->tuned[key] = 0;
+    c->tune_log += "mode " + std::to_string(mode) + ": block form, " + std::to_string(nc) + " frequencies in FP64" +
+                   (ch1 ? ", " + std::to_string(c->n_iw - nc) + " with FP32 traces" : std::string()) + "; ";
+  }
+  return GF_OK;
+}
+
 // Run the point kernel over every (k, chunk) item with the given mode.  For
 // kGloc / kAdj the per-(k, n) m x m results are reduced over k into c->gacc,
 // k-batch by k-batch, in increasing k order.
@@ -387,8 +598,14 @@ gf_status run_points(gf_ctx* c, int mode) {
   st = ensure_einf(c);
   if (st) return st;
   GF_CU(cudaMemsetAsync(c->status.p, 0, sizeof(int), c->stream));
-  st = ensure_lr(c);
+  st = ensure_block(c);
   if (st) return st;
+  const bool block = c->run_on_block = use_block(c, mode);
+  if (!block) {
+    st = ensure_lr(c);
+    if (st) return st;
+  }
+  c->run_chunks = c->n_chunks;
   const bool df64 = (c->precision != GF_PREC_FP64);
   gf::PointParams p{};
   p.H = c->H.as<double2>();
@@ -412,6 +629,14 @@ gf_status run_points(gf_ctx* c, int mode) {
   p.mode = mode;
   p.mmax = c->mmax;
   p.nmat = 1;
+  p.n_iw = c->n_iw;
+  p.status = c->status.as<int>();
+  if (mode & gf::kAdj) {
+    p.gbar = c->have_gbar_for_call ? c->gbar.as<double2>() : nullptr;
+    p.Gbd = (df64 && c->have_gbar_for_call) ? c->Gbd.as<float4>() : nullptr;
+    p.nbar = c->nbar.as<double>();
+  }
+  if (block) return run_block(c, mode, p);
   if (mode & gf::kOcc) {
     GF_CU(ensure(c->occ_part, sizeof(double) * 2 * (size_t)c->n_k * c->n_chunks));
     p.occ_part = c->occ_part.as<double>();
@@ -424,15 +649,6 @@ gf_status run_points(gf_ctx* c, int mode) {
   if (mode & gf::kAdj) {
     GF_CU(ensure(c->mubar_part, sizeof(double) * (size_t)c->n_k * c->n_chunks));
     p.mubar_part = c->mubar_part.as<double>();
-  }
-  p.n_iw = c->n_iw;
-  p.status = c->status.as<int>();
-  p.gbar = nullptr;
-  p.nbar = nullptr;
-  if (mode & gf::kAdj) {
-    p.gbar = c->have_gbar_for_call ? c->gbar.as<double2>() : nullptr;
-    p.Gbd = (df64 && c->have_gbar_for_call) ? c->Gbd.as<float4>() : nullptr;
-    p.nbar = c->nbar.as<double>();
   }
   const bool kred = (mode & (gf::kGloc | gf::kAdj)) != 0;
   const int nb_batches = kred ? (int)c->batch_g0.size() - 1 : 1;
@@ -528,7 +744,7 @@ gf_status enqueue_occupation(gf_ctx* c) {
   gf_status st = run_points(c, gf::kOcc);
   if (st) return st;
   GF_CU(gf::launch_occ_finalize(c->kinfo_d.as<KInfo>(), c->sinfo_d.as<SInfo>(), c->trHE.as<double>(),
-                                c->mu.as<double>(), c->occ_part.as<double>(), c->n_chunks, c->n_k,
+                                c->mu.as<double>(), c->occ_part.as<double>(), c->run_chunks, c->n_k,
                                 c->kN.as<double>(), c->kdN.as<double>(), c->stream));
   GF_CU(gf::launch_sys_reduce(c->kinfo_d.as<KInfo>(), c->sinfo_d.as<SInfo>(), c->n_sys,
                               c->kN.as<double>(), c->kdN.as<double>(), c->sysout.as<double>(),
@@ -568,6 +784,19 @@ gf_status occupation_impl(gf_ctx* c, const double* mu, double* n_out, double* dn
     if (!std::isfinite(mu[s2])) return fail(c, GF_EINVAL, "mu is not finite");
   gf_status st = check_ready(c);
   if (st) return st;
+  if (c->use_graph) {
+    // a new H or P can change the path (or the FP64 frequencies of mixed precision): the
+    // captured graph then goes, and the next call runs normally (scratch, autotuner)
+    st = ensure_block(c);
+    if (st) return st;
+    const int path = use_block(c, gf::kOcc) ? 1 + c->blk_nc : 0;
+    if (c->occ_path != path) {
+      if (c->occ_exec) GF_CU(cudaGraphExecDestroy(c->occ_exec));
+      c->occ_exec = nullptr;
+      c->occ_calls = 0;
+      c->occ_path = path;
+    }
+  }
   if (!c->use_graph || c->occ_calls == 0) {
     // ordinary enqueue (also the warm-up of graph mode: scratch, autotuner)
     ++c->occ_calls;
@@ -582,7 +811,7 @@ gf_status occupation_impl(gf_ctx* c, const double* mu, double* n_out, double* dn
   GF_CU(cudaStreamSynchronize(c->stream));
   st = ensure_einf(c);
   if (st) return st;
-  if (c->lowrank && c->lr_dirty) {
+  if (c->lowrank && c->lr_dirty && !use_block(c, gf::kOcc)) {
     GF_CU(cudaMemsetAsync(c->status.p, 0, sizeof(int), c->stream));
     st = ensure_lr(c);
     if (st) return st;
@@ -859,6 +1088,47 @@ gf_status init_ctx(gf_ctx* c, const gf_desc* d) {
     c->items.insert(c->items.end(), all.begin(), all.end());
   }
 
+  // block form: every window wider than its orbitals, one lane per orbital, eigenproblems within
+  // the Jacobi kernel's size, and enough frequencies to pay for the eigenproblem per k
+  c->blk_shape = c->n_iw >= kBlkMinFreq;
+  std::vector<int64_t> offT(c->n_k);
+  for (int k = 0; k < c->n_k; ++k) {
+    const int m = c->msys[c->ksys[k]], n2 = c->nb[k] - m;
+    if (n2 < 1 || n2 > gf::heev_max_n() || m > gf::kBlkMaxM) c->blk_shape = false;
+    c->blk_n2max = std::max(c->blk_n2max, n2);
+    offT[k] = c->blk_totT;
+    if (n2 > 0) c->blk_totT += (int64_t)n2 * m * (m + 1) / 2;
+  }
+  for (int s = 0; s < c->n_sys; ++s)
+    if (M_PI / c->beta[s] < kBlkMinW) c->blk_shape = false;
+  std::vector<int2> units;
+  std::vector<int> perm(2 * (size_t)c->n_k), bsysg;
+  if (c->blk_shape) {
+    // chunks: whole batches of a CTA, about eight CTAs per resident one; k-groups: about six
+    const int batch = gf::block_batch(c->mmax);
+    const double res = 3.0 * c->sm_count, pts = (double)c->n_k * c->n_iw;
+    const double w = std::ceil(pts / (8.0 * res) / batch) * batch;
+    c->blk_cw = (int)std::min(std::max((double)batch, w), std::ceil((double)c->n_iw / batch) * batch);
+    const int nch = (c->n_iw + c->blk_cw - 1) / c->blk_cw;
+    c->blk_kg = (int)std::max(1.0, std::min((double)gf::kMaxKGroup, std::floor((double)c->n_k * nch / (6.0 * res))));
+    c->blk_sys_g0.assign(c->n_sys, 0);
+    c->blk_sys_g1.assign(c->n_sys, 0);
+    for (int s = 0; s < c->n_sys; ++s) {
+      c->blk_sys_g0[s] = (int)units.size();
+      for (int k = c->sinfo[s].k0; k < c->sinfo[s].k1; k += c->blk_kg)
+        units.push_back(make_int2(k, std::min(c->blk_kg, c->sinfo[s].k1 - k)));
+      c->blk_sys_g1[s] = (int)units.size();
+    }
+    c->blk_groups = (int)units.size();
+    for (int k = 0; k < c->n_k; ++k) {
+      perm[k] = perm[(size_t)c->n_k + k] = k;
+      units.push_back(make_int2(k, 1));
+    }
+    std::stable_sort(perm.begin() + c->n_k, perm.end(), [&](int x, int y) { return c->nb[x] > c->nb[y]; });
+    bsysg = c->blk_sys_g0;
+    bsysg.insert(bsysg.end(), c->blk_sys_g1.begin(), c->blk_sys_g1.end());
+  }
+
   auto alloc_all = [&]() -> cudaError_t {
     cudaError_t e;
     if ((e = ensure(c->H, sizeof(double2) * c->totH))) return e;
@@ -915,6 +1185,20 @@ gf_status init_ctx(gf_ctx* c, const gf_desc* d) {
     if ((e = cudaMemcpyAsync(c->offD_d.p, c->offD.data(), sizeof(int64_t) * c->n_k,
                              cudaMemcpyHostToDevice, c->stream)))
       return e;
+    if (c->blk_shape) {
+      const struct {
+        DevBuf* b;
+        const void* p;
+        size_t bytes;
+      } up[] = {{&c->blk_units, units.data(), sizeof(int2) * units.size()},
+                {&c->blk_perm, perm.data(), sizeof(int) * perm.size()},
+                {&c->blk_sysg, bsysg.data(), sizeof(int) * bsysg.size()},
+                {&c->blk_offT, offT.data(), sizeof(int64_t) * offT.size()}};
+      for (const auto& u : up) {
+        if ((e = ensure(*u.b, u.bytes))) return e;
+        if ((e = cudaMemcpyAsync(u.b->p, u.p, u.bytes, cudaMemcpyHostToDevice, c->stream))) return e;
+      }
+    }
     if ((e = cudaMemsetAsync(c->status.p, 0, sizeof(int), c->stream))) return e;
     if (c->use_graph) {
       if ((e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking))) return e;
@@ -1006,7 +1290,10 @@ gf_status gf_destroy(gf_ctx* c) {
                     &c->pole_ws, &c->lr_eps, &c->lr_U, &c->lr_Pt, &c->lr_T, &c->lr_ws,
                     &c->eimp, &c->eimp_part, &c->gl_in, &c->delta, &c->wraw, &c->vdc,
                     &c->wbout, &c->kHks, &c->kEps, &c->eps_grid, &c->dos, &c->pdos, &c->pdos_off,
-                    &c->pole_part, &c->pole_vs, &c->pole_es, &c->voff_d, &c->mu_prev};
+                    &c->pole_part, &c->pole_vs, &c->pole_es, &c->voff_d, &c->mu_prev,
+                    &c->blk_units, &c->blk_perm, &c->blk_sysg, &c->blk_offT, &c->blk_e, &c->blk_T, &c->blk_Ts,
+                    &c->blk_B, &c->blk_Bs, &c->blk_HO, &c->blk_U, &c->blk_D22, &c->blk_V, &c->blk_R, &c->blk_H11,
+                    &c->blk_tau, &c->blk_ws, &c->blk_info};
   for (DevBuf* b : bufs) release(*b);
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
   if (c->occ_exec) cudaGraphExecDestroy(c->occ_exec);
@@ -1049,6 +1336,7 @@ gf_status gf_set_hamiltonian(gf_ctx* c, const void* h, int32_t is_diagonal) try 
   }
   c->have_H = true;
   c->lr_dirty = true;
+  c->blk_dirty = true;
   c->einf_dirty = true;
   return GF_OK;
 } catch (...) {
@@ -1067,6 +1355,7 @@ gf_status gf_set_projectors(gf_ctx* c, const void* p) try {
   GF_CU(cudaStreamSynchronize(c->stream));
   c->have_P = true;
   c->lr_dirty = true;
+  c->blk_dirty = true;
   c->einf_dirty = true;
   return GF_OK;
 } catch (...) {
@@ -1186,7 +1475,7 @@ gf_status gf_evaluate(gf_ctx* c, const double* mu, void* gloc_out, void* rho_out
   if (mode & gf::kOcc) {
     GF_CU(gf::launch_occ_finalize(c->kinfo_d.as<KInfo>(), c->sinfo_d.as<SInfo>(),
                                   c->trHE.as<double>(), c->mu.as<double>(), c->occ_part.as<double>(),
-                                  c->n_chunks, c->n_k, c->kN.as<double>(), c->kdN.as<double>(),
+                                  c->run_chunks, c->n_k, c->kN.as<double>(), c->kdN.as<double>(),
                                   c->stream));
     GF_CU(gf::launch_sys_reduce(c->kinfo_d.as<KInfo>(), c->sinfo_d.as<SInfo>(), c->n_sys,
                                 c->kN.as<double>(), c->kdN.as<double>(), c->sysout.as<double>(),
@@ -1262,13 +1551,13 @@ gf_status gf_backward(gf_ctx* c, const double* mu, const void* gbar, const doubl
   st = run_points(c, mode);
   if (st) return st;
   GF_CU(gf::launch_mubar_reduce(c->kinfo_d.as<KInfo>(), c->sinfo_d.as<SInfo>(), c->n_sys,
-                                c->n_chunks, c->mubar_part.as<double>(), c->mubar_sys.as<double>(),
+                                c->run_chunks, c->mubar_part.as<double>(), c->mubar_sys.as<double>(),
                                 c->stream));
   c->last_launches += 1;
   if (any_nbar) {
     GF_CU(gf::launch_occ_finalize(c->kinfo_d.as<KInfo>(), c->sinfo_d.as<SInfo>(),
                                   c->trHE.as<double>(), c->mu.as<double>(), c->occ_part.as<double>(),
-                                  c->n_chunks, c->n_k, c->kN.as<double>(), c->kdN.as<double>(),
+                                  c->run_chunks, c->n_k, c->kN.as<double>(), c->kdN.as<double>(),
                                   c->stream));
     GF_CU(gf::launch_sys_reduce(c->kinfo_d.as<KInfo>(), c->sinfo_d.as<SInfo>(), c->n_sys,
                                 c->kN.as<double>(), c->kdN.as<double>(), c->sysout.as<double>(),

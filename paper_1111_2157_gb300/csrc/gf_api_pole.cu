@@ -305,6 +305,7 @@ gf_status gf_set_projectors_lowdin(gf_ctx* c, const void* w, void* p_out) try {
   if (st) return st;
   c->have_P = true;
   c->lr_dirty = true;
+  c->blk_dirty = true;
   c->einf_dirty = true;
   return GF_OK;
 } catch (...) {

@@ -1,0 +1,900 @@
+// Block form of the lattice points (gf_block.cuh): setup kernels and the FP64 point kernel.
+//
+// FP64 on GB300 issues two DFMAs per clock and SM, so a warp-wide FP64 instruction occupies
+// its SM sub-partition for 64 clocks and everything else (shared-memory and L2 loads, index
+// arithmetic, FP32) runs in its shadow.  The point kernel is therefore laid out for the
+// fewest FP64 warp instructions with full lanes: a warp takes 32 / LW frequencies of one
+// k-point (LW = 8, 16 or 32 lanes per m x m matrix), the band sums run over the flattened
+// (frequency, pair) list, the elimination over the flattened entries, and the pair table
+// B_a conj(B_c) of the k-point is formed once per uploaded H_k instead of per frequency.
+//
+// Bound: the FP64 pipe.  Per point of a 40-band window with 14 orbitals: 56 k FP64 FMAs for
+// N(mu) and dN/dmu (band sums 33 k, S^{-1} 11 k, S^{-1} F 11 k) where the inverse of the window
+// takes 281 k; 135 k with G_loc and rho_k.  Measured (GB300, 216 k-points x 1024 frequencies):
+// every output in 62 ms, 210 ms by the inverse; mu search and G_loc of 64 k-points 57 ms, 340 ms.
+#include <math.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#include "gf_block.cuh"
+#include "gf_complex.cuh"
+
+namespace gf {
+
+namespace {
+
+using namespace cx;
+
+constexpr int kSetupThreads = 256;
+
+__device__ __forceinline__ double setup_sum(double v, double* red) {
+  for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __syncthreads();
+  if (lane == 0) red[warp] = v;
+  __syncthreads();
+  double r = 0.0;
+  for (int w = 0; w < kSetupThreads / 32; ++w) r += red[w];
+  return r;  // the same value in every thread
+}
+
+__device__ __forceinline__ double warp_sum(double v) {
+  for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+
+// P_k^+ = Q [R; 0] by Householder reflections H_j = I - tau v v^+ (real tau, so H_j is
+// Hermitian and unitary; the phases stay in R), then Q^+ H_k Q by one rank-2 update per
+// reflection.  One CTA per k-point (grid-stride).
+__global__ void __launch_bounds__(kSetupThreads) k_block_reduce(const BlockSetup b, int in_smem) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ double red[kSetupThreads / 32];
+  double2* X = reinterpret_cast<double2*>(smraw);      // [m][N]: columns of P^+, then the vectors v_j
+  double2* R = X + (size_t)b.mmax * b.nbmax;           // [m][m]
+  double2* pv = R + (size_t)b.mmax * b.mmax;           // [N]
+  double2* A = in_smem ? pv + b.nbmax : b.ws + (size_t)blockIdx.x * b.nbmax * b.nbmax;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kWarps = kSetupThreads / 32;
+  for (int k = blockIdx.x; k < b.n_k; k += gridDim.x) {
+    const KInfo ki = b.kinfo[k];
+    const int N = ki.nb, M = b.sinfo[ki.sys].m, n2 = N - M;
+    const double2* H = b.H + ki.offH;
+    const double2* P = b.P + ki.offP;
+    __syncthreads();
+    // H_k, its norm and its distance from a Hermitian matrix
+    double nrm = 0.0, anti = 0.0, big = 0.0;
+    for (int e = tid; e < N * N; e += kSetupThreads) {
+      const int i = e / N, j = e - i * N;
+      const double2 h = H[e], t = H[j * N + i];
+      A[e] = h;
+      nrm += h.x * h.x + h.y * h.y;
+      anti = fmax(anti, fmax(fabs(h.x - t.x), fabs(h.y + t.y)));
+      big = fmax(big, fmax(fabs(h.x), fabs(h.y)));
+    }
+    nrm = setup_sum(nrm, red);
+    for (int off = 16; off; off >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, off));
+    __syncthreads();
+    if (lane == 0) red[warp] = big;
+    __syncthreads();
+    big = red[0];
+    for (int w = 1; w < kWarps; ++w) big = fmax(big, red[w]);
+    // (NaN and infinity fail the comparison and take the general path)
+    if (!(anti <= 8.9e-16 * big) || !isfinite(nrm)) atomicOr(b.flags, kBlkNonHermitian);
+    if (tid == 0) b.hnorm[k] = sqrt(nrm / N);
+    for (int e = tid; e < M * N; e += kSetupThreads) {
+      const double2 p = P[e];
+      X[e] = make_double2(p.x, -p.y);
+    }
+    __syncthreads();
+    for (int j = 0; j < M; ++j) {
+      double2* x = X + j * N;
+      double s = 0.0;
+      for (int i = j + tid; i < N; i += kSetupThreads) s += x[i].x * x[i].x + x[i].y * x[i].y;
+      s = setup_sum(s, red);
+      const double nx = sqrt(s);
+      const double2 x0 = x[j];
+      const double ax = sqrt(x0.x * x0.x + x0.y * x0.y);
+      const double2 ph = ax > 0.0 ? make_double2(x0.x / ax, x0.y / ax) : make_double2(1.0, 0.0);
+      const double tau = nx > 0.0 ? 1.0 / (nx * (nx + ax)) : 0.0;
+      __syncthreads();
+      if (tid == 0) {
+        x[j] = make_double2(x0.x + ph.x * nx, x0.y + ph.y * nx);
+        R[j * M + j] = make_double2(-ph.x * nx, -ph.y * nx);
+        b.tau[(size_t)k * b.mmax + j] = tau;
+      }
+      __syncthreads();
+      // the later columns: x_c -= tau v (v^+ x_c)
+      for (int c = j + 1 + warp; c < M; c += kWarps) {
+        double2* y = X + c * N;
+        double2 d = make_double2(0.0, 0.0);
+        for (int i = j + lane; i < N; i += 32) cmac_ca(d, x[i], y[i]);
+        d.x = tau * warp_sum(d.x);
+        d.y = tau * warp_sum(d.y);
+        for (int i = j + lane; i < N; i += 32) {
+          const double2 v = x[i];
+          y[i].x -= fma(v.x, d.x, -v.y * d.y);
+          y[i].y -= fma(v.x, d.y, v.y * d.x);
+        }
+        __syncwarp();
+        if (lane == 0) R[j * M + c] = y[j];
+      }
+      // A <- H_j A H_j: p = tau A v, w = p - (tau / 2) (v^+ p) v, A -= v w^+ + w v^+
+      for (int i = warp; i < N; i += kWarps) {
+        double2 d = make_double2(0.0, 0.0);
+        for (int c = j + lane; c < N; c += 32) cmac(d, A[i * N + c], x[c]);
+        d.x = warp_sum(d.x);
+        d.y = warp_sum(d.y);
+        if (lane == 0) pv[i] = make_double2(tau * d.x, tau * d.y);
+      }
+      __syncthreads();
+      double vp = 0.0;
+      for (int i = j + tid; i < N; i += kSetupThreads) vp += x[i].x * pv[i].x + x[i].y * pv[i].y;
+      vp = 0.5 * tau * setup_sum(vp, red);
+      __syncthreads();
+      for (int i = j + tid; i < N; i += kSetupThreads) {
+        pv[i].x = fma(-vp, x[i].x, pv[i].x);
+        pv[i].y = fma(-vp, x[i].y, pv[i].y);
+      }
+      __syncthreads();
+      for (int e = tid; e < N * N; e += kSetupThreads) {
+        const int i = e / N, c = e - i * N;
+        double2 a = A[e];
+        if (i >= j) {
+          const double2 v = x[i], w = pv[c];  // v_i conj(w_c)
+          a.x -= fma(v.x, w.x, v.y * w.y);
+          a.y -= fma(v.y, w.x, -v.x * w.y);
+        }
+        if (c >= j) {
+          const double2 w = pv[i], v = x[c];
+          a.x -= fma(w.x, v.x, w.y * v.y);
+          a.y -= fma(w.y, v.x, -w.x * v.y);
+        }
+        A[e] = a;
+      }
+      __syncthreads();
+    }
+    // rank of P: the triangular factor must be safely invertible
+    if (tid == 0) {
+      double lo = INFINITY, hi = 0.0;
+      for (int j = 0; j < M; ++j) {
+        const double d = fmax(fabs(R[j * M + j].x), fabs(R[j * M + j].y));
+        lo = fmin(lo, d);
+        for (int c = j; c < M; ++c) hi = fmax(hi, fmax(fabs(R[j * M + c].x), fabs(R[j * M + c].y)));
+        if (!(d > 0.0)) lo = 0.0;
+      }
+      if (!(lo > 1e-3 * hi) || !isfinite(hi)) atomicOr(b.flags, kBlkRankDeficient);
+    }
+    for (int e = tid; e < M * N; e += kSetupThreads) {
+      const int j = e / N, i = e - j * N;
+      b.V[ki.offP + e] = i < j ? make_double2(0.0, 0.0) : X[e];
+    }
+    for (int e = tid; e < M * M; e += kSetupThreads) {
+      const int i = e / M, c = e - i * M;
+      b.R[(size_t)k * b.mmax * b.mmax + e] = c >= i ? R[e] : make_double2(0.0, 0.0);
+      b.H11[(size_t)k * b.mmax * b.mmax + e] = A[i * N + c];
+    }
+    for (int e = tid; e < M * n2; e += kSetupThreads) {
+      const int i = e / n2, c = e - i * n2;
+      b.B[ki.offP + e] = A[i * N + M + c];
+    }
+    for (int e = tid; e < n2 * n2; e += kSetupThreads) {
+      const int i = e / n2, c = e - i * n2;
+      b.D22[ki.offH + e] = A[(M + i) * N + M + c];
+    }
+  }
+}
+
+// B, H11, O, the pair table and U of one k-point per CTA (gf_block.cuh).
+__global__ void __launch_bounds__(kSetupThreads) k_block_finish(const BlockSetup b) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int k = blockIdx.x;
+  const KInfo ki = b.kinfo[k];
+  const int N = ki.nb, M = b.sinfo[ki.sys].m, n2 = N - M, np = M * (M + 1) / 2;
+  const int tid = threadIdx.x;
+  double2* Ri = reinterpret_cast<double2*>(smraw);        // R^{-1}
+  double2* W = Ri + (size_t)b.mmax * b.mmax;              // m x m
+  double2* Bs = W + (size_t)b.mmax * b.mmax;              // m x n2: H12 V, then B
+  const double2* R = b.R + (size_t)k * b.mmax * b.mmax;
+  const double2* V2 = b.D22 + ki.offH;
+  // column c of R^{-1} by back substitution
+  for (int c = tid; c < M; c += kSetupThreads) {
+    for (int i = M - 1; i >= 0; --i) {
+      if (i > c) {
+        Ri[i * M + c] = make_double2(0.0, 0.0);
+        continue;
+      }
+      double2 s = make_double2(i == c ? 1.0 : 0.0, 0.0);
+      for (int j = i + 1; j <= c; ++j) {
+        const double2 r = R[i * M + j], x = Ri[j * M + c];
+        s.x -= fma(r.x, x.x, -r.y * x.y);
+        s.y -= fma(r.x, x.y, r.y * x.x);
+      }
+      Ri[i * M + c] = cmul(s, crcp(R[i * M + i]));
+    }
+  }
+  for (int e = tid; e < M * n2; e += kSetupThreads) {
+    const int a = e / n2, c = e - a * n2;
+    double2 s = make_double2(0.0, 0.0);
+    for (int x = 0; x < n2; ++x) cmac(s, b.B[ki.offP + a * n2 + x], V2[x * n2 + c]);
+    Bs[e] = s;
+  }
+  __syncthreads();
+  // B = R^{-1} (H12 V), column by column in place (row a takes the rows from a on)
+  for (int c = tid; c < n2; c += kSetupThreads) {
+    for (int a = 0; a < M; ++a) {
+      double2 s = make_double2(0.0, 0.0);
+      for (int x = a; x < M; ++x) cmac(s, Ri[a * M + x], Bs[x * n2 + c]);
+      Bs[a * n2 + c] = s;
+    }
+  }
+  // W = R^{-1} H11
+  for (int e = tid; e < M * M; e += kSetupThreads) {
+    const int a = e / M, c = e - a * M;
+    double2 s = make_double2(0.0, 0.0);
+    for (int x = a; x < M; ++x) cmac(s, Ri[a * M + x], b.H11[(size_t)k * b.mmax * b.mmax + x * M + c]);
+    W[e] = s;
+  }
+  __syncthreads();
+  for (int e = tid; e < M * n2; e += kSetupThreads) {
+    b.B[ki.offP + e] = Bs[e];
+    if (b.Bs) b.Bs[ki.offP + e] = make_float2((float)Bs[e].x, (float)Bs[e].y);
+  }
+  double2* HO = b.HO + (size_t)k * 2 * b.npmax;
+  for (int pr = tid; pr < np; pr += kSetupThreads) {
+    int a = 0, rem = pr;
+    while (rem >= M - a) { rem -= M - a; ++a; }
+    const int c = a + rem;
+    double2 h = make_double2(0.0, 0.0), o = make_double2(0.0, 0.0);
+    for (int x = c; x < M; ++x) {
+      cmac_cb(h, W[a * M + x], Ri[c * M + x]);
+      cmac_cb(o, Ri[a * M + x], Ri[c * M + x]);
+    }
+    if (a == c) h.y = o.y = 0.0;
+    HO[pr] = h;
+    HO[b.npmax + pr] = o;
+  }
+  for (int e = tid; e < np * n2; e += kSetupThreads) {
+    const int l = e / np, pr = e - l * np;
+    int a = 0, rem = pr;
+    while (rem >= M - a) { rem -= M - a; ++a; }
+    const int c = a + rem;
+    double2 t = make_double2(0.0, 0.0);
+    cmac_cb(t, Bs[a * n2 + l], Bs[c * n2 + l]);
+    if (a == c) t.y = 0.0;
+    b.T[b.offT[k] + e] = t;
+    if (b.Ts) b.Ts[b.offT[k] + e] = make_float2((float)t.x, (float)t.y);
+  }
+  // U = Q diag(R^{-+}, V2): one column per thread, the reflections in reverse order
+  double2* U = b.U + ki.offH;
+  const double2* Vh = b.V + ki.offP;
+  const double* tau = b.tau + (size_t)k * b.mmax;
+  for (int c = tid; c < N; c += kSetupThreads) {
+    for (int i = 0; i < N; ++i) {
+      double2 v = make_double2(0.0, 0.0);
+      if (c < M) {
+        if (i < M) v = make_double2(Ri[c * M + i].x, -Ri[c * M + i].y);
+      } else if (i >= M) {
+        v = V2[(i - M) * n2 + c - M];
+      }
+      U[i * N + c] = v;
+    }
+    for (int j = M - 1; j >= 0; --j) {
+      const double2* v = Vh + j * N;
+      double2 s0 = make_double2(0.0, 0.0), s1 = s0;
+      int i = j;
+      for (; i + 1 < N; i += 2) {
+        cmac_ca(s0, v[i], U[i * N + c]);
+        cmac_ca(s1, v[i + 1], U[(i + 1) * N + c]);
+      }
+      if (i < N) cmac_ca(s0, v[i], U[i * N + c]);
+      const double2 s = make_double2(tau[j] * (s0.x + s1.x), tau[j] * (s0.y + s1.y));
+      for (i = j; i < N; ++i) {
+        double2 u = U[i * N + c];
+        u.x -= fma(v[i].x, s.x, -v[i].y * s.y);
+        u.y -= fma(v[i].x, s.y, v[i].y * s.x);
+        U[i * N + c] = u;
+      }
+    }
+  }
+}
+
+// ------------------------------------------------------------------ point kernel
+
+template <bool LOW>
+struct Rest {  // type of the parts that mixed precision takes from an FP32 inverse
+  using c = double2;
+  using r = double;
+};
+template <>
+struct Rest<true> {
+  using c = float2;
+  using r = float;
+};
+__device__ __forceinline__ double2 to_rest(double2 v, double2) { return v; }
+__device__ __forceinline__ float2 to_rest(double2 v, float2) { return make_float2((float)v.x, (float)v.y); }
+__device__ __forceinline__ void rmac(double2& a, double2 x, double2 y) { cmac(a, x, y); }
+__device__ __forceinline__ void rmac(float2& a, float2 x, float2 y) { fmac(a, x, y); }
+__device__ __forceinline__ void rmac_ca(double2& a, double2 x, double2 y) { cmac_ca(a, x, y); }
+__device__ __forceinline__ void rmac_ca(float2& a, float2 x, float2 y) { fmac_ca(a, x, y); }
+__device__ __forceinline__ double2 rzero(double2) { return make_double2(0.0, 0.0); }
+__device__ __forceinline__ float2 rzero(float2) { return make_float2(0.f, 0.f); }
+__device__ __forceinline__ double rfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double2 rmul(double2 a, double2 b) { return cmul(a, b); }
+__device__ __forceinline__ float2 rmul(float2 a, float2 b) { return fmul(a, b); }
+
+// 1 / a with one division: scaled by a power of two near 1 / max(|Re|, |Im|) (bit arithmetic),
+// so that the squared modulus neither overflows nor underflows.
+__device__ __forceinline__ double2 crcp_scaled(double2 a, unsigned long long key) {
+  int ex = 2046 - (int)(key >> 52);
+  ex = ex < 1 ? 1 : ex;
+  const double s = __longlong_as_double((long long)ex << 52);
+  const double x = a.x * s, y = a.y * s;
+  const double q = s / fma(x, x, y * y);
+  return make_double2(x * q, -y * q);
+}
+
+// Shared memory of the point kernel in bytes: per warp S (then S^{-1}), F, d / d^2 / d^3, the
+// pivot row and column, Gbar A^+ (adjoint) and the pivot tables, for F frequencies; per CTA
+// the pair list and the columns S^{-1} B D of rho_k.
+struct LayoutB {
+  size_t wS, wF, wd, wd2, wrc, wM, wp, wstride, oPair, oY, bytes;
+  int nf;   // frequencies per warp
+  int yf;   // frequencies of the rho_k columns staged at once
+};
+
+__host__ __device__ inline int block_lanes(int m) { return m <= 8 ? 8 : (m <= 16 ? 16 : 32); }
+
+__host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, int low) {
+  LayoutB L;
+  L.nf = 32 / block_lanes(mmax);
+  const size_t f = L.nf, mm = (size_t)mmax * mmax, r = low ? 8 : 16;
+  const bool needF = (mode & (kOcc | kAdj)) != 0;
+  auto al = [](size_t x) { return (x + 15) & ~(size_t)15; };
+  size_t o = 0;
+  L.wS = o; o += 16 * f * mm;
+  L.wF = o; o = al(o + (needF ? r * f * mm : 0));
+  L.wd = o; o += 16 * f * n2max;
+  L.wd2 = o; o = al(o + (needF ? 2 * r * f * n2max : 0));
+  L.wrc = o; o += 16 * f * 2 * mmax;
+  L.wM = o; o += (mode & kAdj) ? 16 * f * mm : 0;
+  L.wp = o; o = al(o + 4 * f * 2 * mmax);
+  L.wstride = o;
+  o *= kBlkWarps;
+  L.oPair = o; o = al(o + 2 * (size_t)mmax * (mmax + 1) / 2);
+  L.oY = o;
+  L.yf = 0;
+  if (mode & kRho) {
+    const size_t one = r * (size_t)mmax * n2max;
+    const size_t fit = (48u << 10) / one;
+    L.yf = fit < 1 ? 1 : (fit > f * kBlkWarps ? (int)(f * kBlkWarps) : (int)fit);
+    o = al(o + one * L.yf);
+  }
+  L.bytes = o;
+  return L;
+}
+
+__device__ __forceinline__ double2 ld_cg(const double2* p) { return __ldg(p); }
+__device__ __forceinline__ float2 ld_cg(const float2* p) { return __ldg(p); }
+
+// S^{-1} in place for the warp's matrices: LW lanes each, Gauss-Jordan in exchange form with
+// partial pivoting and no row interchanges (X[i][c] = A[p_i][q_c], q = p^{-1}).  Every lane
+// group holds a valid matrix, so no lane diverges.
+template <int LW>
+__device__ __forceinline__ void block_invert(double2* A, int M, double2* rc, int* sp, int sl, int* status) {
+  double2* su = rc;
+  double2* sc = rc + M;
+  int* sq = sp + M;
+  bool used = sl >= M;
+  for (int j = 0; j < M; ++j) {
+    unsigned long long best = used ? 0ULL : pivot_key(A[sl * M + j]);
+    int bi = used ? 0x7fffffff : sl;
+    for (int off = LW / 2; off; off >>= 1) {
+      const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, off);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
+      if (ob > best || (ob == best && oi < bi)) {
+        best = ob;
+        bi = oi;
+      }
+    }
+    if (sl == 0 && (best == 0ULL || best >= 0x7ff0000000000000ULL)) atomicOr(status, kFlagSingular);
+    const double2 r = crcp_scaled(A[bi * M + j], best);
+    if (sl < M) {
+      const double2 u = A[bi * M + sl], l = A[sl * M + j];
+      su[sl] = (sl == j) ? r : cmul(u, r);
+      sc[sl] = (sl == bi) ? make_double2(-1.0, 0.0) : l;
+    }
+    if (sl == bi) used = true;
+    if (sl == 0) {
+      sp[j] = bi;
+      sq[bi] = j;
+    }
+    __syncwarp();
+    int i = sl / M, c = sl - (sl / M) * M;
+    const int di = LW / M, dc = LW - (LW / M) * M;
+    for (int e = sl; e < M * M; e += LW) {
+      const double2 l = sc[i], u = su[c];
+      double2 v = (i == bi || c == j) ? make_double2(0.0, 0.0) : A[e];
+      v.x = fma(-l.x, u.x, fma(l.y, u.y, v.x));
+      v.y = fma(-l.x, u.y, fma(-l.y, u.x, v.y));
+      A[e] = v;
+      i += di;
+      c += dc;
+      if (c >= M) {
+        c -= M;
+        ++i;
+      }
+    }
+    __syncwarp();
+  }
+}
+
+template <int LW, bool LOW>
+__global__ void __launch_bounds__(32 * kBlkWarps, 4)
+    k_point_block(const PointParams p, const BlockForm bf, const BlockLaunch bl) {
+  using rc_t = typename Rest<LOW>::c;
+  using rr_t = typename Rest<LOW>::r;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ double s_part[kBlkWarps][3];
+  constexpr int F = 32 / LW;
+  constexpr int W = kBlkWarps;
+  const LayoutB L = make_layout_b(p.mmax, bl.n2max, p.mode, LOW ? 1 : 0);
+  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5, sl = lane % LW, mf = lane / LW;
+  unsigned char* wb = smraw + (size_t)wp * L.wstride;
+  double2* sS = reinterpret_cast<double2*>(wb + L.wS);
+  rc_t* sF = reinterpret_cast<rc_t*>(wb + L.wF);
+  double2* sd = reinterpret_cast<double2*>(wb + L.wd);
+  rc_t* sd2 = reinterpret_cast<rc_t*>(wb + L.wd2);
+  double2* sM = reinterpret_cast<double2*>(wb + L.wM);
+  uchar2* pair = reinterpret_cast<uchar2*>(smraw + L.oPair);
+  rc_t* sY = reinterpret_cast<rc_t*>(smraw + L.oY);
+  const int unit = bl.unit0 + blockIdx.x / bl.n_chunks, ch = blockIdx.x % bl.n_chunks;
+  const int2 un = bl.units[unit];
+  const int n0 = bl.n_begin + ch * bl.chunk_w, n1 = min(bl.n_end, n0 + bl.chunk_w);
+  const int chunk = bl.chunk0 + ch;
+  const bool occ = (p.mode & kOcc) != 0, adj = (p.mode & kAdj) != 0, rho = (p.mode & kRho) != 0;
+
+  for (int q = 0; q < un.y; ++q) {
+    const int kk = bl.kperm[un.x + q];
+    const KInfo ki = p.kinfo[kk];
+    const SInfo si = p.sinfo[ki.sys];
+    const int M = si.m, n2 = ki.nb - M, NP = M * (M + 1) / 2, MM = M * M;
+    const double mu = p.mu[ki.sys], pib = M_PI / si.beta, wk = ki.w;
+    const double* e_k = bf.e + bf.offD[kk];
+    const double2* T = bf.T + bf.offT[kk];
+    const double2* HO = bf.HO + (size_t)kk * 2 * bf.npmax;
+    const double cb = (adj && p.nbar) ? p.nbar[ki.sys] * 2.0 / si.beta : 0.0;
+    const bool have_gbar = adj && p.gbar != nullptr;
+    double2* A = sS + mf * MM;  // this lane group's matrix
+    double2* rcb = reinterpret_cast<double2*>(wb + L.wrc) + mf * 2 * M;
+    int* sp = reinterpret_cast<int*>(wb + L.wp) + mf * 2 * M;
+    __syncthreads();
+    for (int pr = tid; pr < NP; pr += 32 * W) {
+      int a = 0, rem = pr;
+      while (rem >= M - a) { rem -= M - a; ++a; }
+      pair[pr] = make_uchar2((unsigned char)a, (unsigned char)(a + rem));
+    }
+    __syncthreads();
+    double acc_tr = 0.0, acc_g2 = 0.0, acc_mu = 0.0;
+    for (int base = n0; base < n1; base += W * F) {
+      const int n = base + wp * F;
+      const int nv = min(F, n1 - n);  // frequencies of this warp (<= 0: none)
+      if (nv > 0) {
+        __syncwarp();
+        for (int i = lane; i < F * n2; i += 32) {
+          const int f = i / n2, bb = i - f * n2;
+          const double wn = (2.0 * min(n + f, n1 - 1) + 1.0) * pib;
+          const double x = mu - e_k[bb];
+          const double s = 1.0 / fma(x, x, wn * wn);
+          const double2 d = make_double2(x * s, -wn * s);
+          sd[i] = d;
+          if (occ || adj) {
+            const double2 d2 = cmul(d, d);
+            sd2[i] = to_rest(d2, rc_t{});
+            if (occ) {
+              sd2[F * n2 + i] = to_rest(cmul(d2, d), rc_t{});
+              if (f < nv) {
+                acc_tr += d.x;
+                acc_g2 += d2.x;
+              }
+            }
+          }
+        }
+        __syncwarp();
+        // S and F, pair by pair: with t = B_a conj(B_c), sum t Re d and sum t Im d give both
+        // (a, c) and (c, a)
+        for (int i = lane; i < F * NP; i += 32) {
+          const int f = i / NP, pr = i - f * NP;
+          const int a = pair[pr].x, c = pair[pr].y;
+          const int nn = min(n + f, n1 - 1);
+          const double2* t = T + pr;
+          const double2* df = sd + f * n2;
+          double2 xr = make_double2(0.0, 0.0), xi = xr;
+          rc_t yr = rzero(rc_t{}), yi = yr;
+          if (occ || adj) {
+            const rc_t* d2f = sd2 + f * n2;
+            if constexpr (LOW) {
+              const float2* ts = bf.Ts + bf.offT[kk] + pr;
+#pragma unroll 4
+              for (int bb = 0; bb < n2; ++bb) {
+                const double2 tv = ld_cg(t + (size_t)bb * NP), d = df[bb];
+                const float2 tf = ld_cg(ts + (size_t)bb * NP), d2 = d2f[bb];
+                xr.x = fma(tv.x, d.x, xr.x); xr.y = fma(tv.y, d.x, xr.y);
+                xi.x = fma(tv.x, d.y, xi.x); xi.y = fma(tv.y, d.y, xi.y);
+                yr.x = rfma(tf.x, d2.x, yr.x); yr.y = rfma(tf.y, d2.x, yr.y);
+                yi.x = rfma(tf.x, d2.y, yi.x); yi.y = rfma(tf.y, d2.y, yi.y);
+              }
+            } else {
+#pragma unroll 4
+              for (int bb = 0; bb < n2; ++bb) {
+                const double2 tv = ld_cg(t + (size_t)bb * NP), d = df[bb];
+                const rc_t d2 = d2f[bb];
+                xr.x = fma(tv.x, d.x, xr.x); xr.y = fma(tv.y, d.x, xr.y);
+                xi.x = fma(tv.x, d.y, xi.x); xi.y = fma(tv.y, d.y, xi.y);
+                yr.x = rfma(tv.x, d2.x, yr.x); yr.y = rfma(tv.y, d2.x, yr.y);
+                yi.x = rfma(tv.x, d2.y, yi.x); yi.y = rfma(tv.y, d2.y, yi.y);
+              }
+            }
+            const rc_t o = to_rest(HO[bf.npmax + pr], rc_t{});
+            rc_t* Fm = sF + f * MM;
+            rc_t v;
+            v.x = o.x + (yr.x - yi.y);
+            v.y = o.y + (yr.y + yi.x);
+            Fm[a * M + c] = v;
+            v.x = o.x + (yr.x + yi.y);
+            v.y = (yi.x - yr.y) - o.y;
+            if (a != c) Fm[c * M + a] = v;
+          } else {
+#pragma unroll 4
+            for (int bb = 0; bb < n2; ++bb) {
+              const double2 tv = ld_cg(t + (size_t)bb * NP), d = df[bb];
+              xr.x = fma(tv.x, d.x, xr.x); xr.y = fma(tv.y, d.x, xr.y);
+              xi.x = fma(tv.x, d.y, xi.x); xi.y = fma(tv.y, d.y, xi.y);
+            }
+          }
+          const double2 h = HO[pr], o = HO[bf.npmax + pr];
+          const double wn = (2.0 * nn + 1.0) * pib;
+          const double2* Sg = p.Sig + si.offSig + (int64_t)nn * MM;
+          // z o_ac - h_ac - Sigma_ac - g_ac, and (c, a) with conj(o), conj(h)
+          const double2 s1 = Sg[a * M + c], s2 = Sg[c * M + a];
+          double2 v;
+          v.x = fma(mu, o.x, -wn * o.y) - h.x - s1.x - (xr.x - xi.y);
+          v.y = fma(mu, o.y, wn * o.x) - h.y - s1.y - (xr.y + xi.x);
+          double2* Sm = sS + f * MM;
+          Sm[a * M + c] = v;
+          v.x = fma(mu, o.x, wn * o.y) - h.x - s2.x - (xr.x + xi.y);
+          v.y = fma(-mu, o.y, wn * o.x) + h.y - s2.y - (xi.x - xr.y);
+          if (a != c) Sm[c * M + a] = v;
+        }
+        __syncwarp();
+        block_invert<LW>(A, M, rcb, sp, sl, p.status);
+        if (occ) {
+          for (int i = lane; i < F * NP; i += 32) {
+            const int f = i / NP, pr = i - f * NP;
+            const int a = pair[pr].x, c = pair[pr].y;
+            const int* pf = reinterpret_cast<const int*>(wb + L.wp) + f * 2 * M;
+            const int* qf = pf + M;
+            const double2* Af = sS + f * MM;
+            const rc_t* Fm = sF + f * MM;
+            const int pa = pf[a] * M, pc = pf[c] * M;
+            rc_t x1 = rzero(rc_t{}), x2 = x1;
+            for (int j = 0; j < M; ++j) {
+              const int fj = pf[j] * M;
+              rmac(x1, to_rest(Af[pa + j], rc_t{}), Fm[fj + c]);
+              if (a != c) rmac(x2, to_rest(Af[pc + j], rc_t{}), Fm[fj + a]);
+            }
+            rc_t zr = rzero(rc_t{}), zi = zr;
+            const rc_t* d3f = sd2 + F * n2 + f * n2;
+            if constexpr (LOW) {
+              const float2* ts = bf.Ts + bf.offT[kk] + pr;
+#pragma unroll 4
+              for (int bb = 0; bb < n2; ++bb) {
+                const float2 tv = ld_cg(ts + (size_t)bb * NP), d = d3f[bb];
+                zr.x = rfma(tv.x, d.x, zr.x); zr.y = rfma(tv.y, d.x, zr.y);
+                zi.x = rfma(tv.x, d.y, zi.x); zi.y = rfma(tv.y, d.y, zi.y);
+              }
+            } else {
+              const double2* t = T + pr;
+#pragma unroll 4
+              for (int bb = 0; bb < n2; ++bb) {
+                const double2 tv = ld_cg(t + (size_t)bb * NP);
+                const rc_t d = d3f[bb];
+                zr.x = rfma(tv.x, d.x, zr.x); zr.y = rfma(tv.y, d.x, zr.y);
+                zi.x = rfma(tv.x, d.y, zi.x); zi.y = rfma(tv.y, d.y, zi.y);
+              }
+            }
+            if (f < nv) {
+              // Tr X^2 and 2 Tr(S^{-1} B D^3 B^+): the pair's (a, c) and (c, a) terms
+              const rc_t g1 = to_rest(Af[pa + qf[c]], rc_t{}), g2 = to_rest(Af[pc + qf[a]], rc_t{});
+              const rr_t z1x = zr.x - zi.y, z1y = zr.y + zi.x;  // (a, c)
+              const rr_t z2x = zr.x + zi.y, z2y = zi.x - zr.y;  // (c, a)
+              rr_t s = rfma(g1.x, z2x, -g1.y * z2y);
+              if (a == c) {
+                acc_tr += (double)x1.x;
+                s = rfma(rr_t(2), s, rfma(x1.x, x1.x, -x1.y * x1.y));
+              } else {
+                s = rfma(g2.x, z1x, rfma(-g2.y, z1y, s));
+                s = rr_t(2) * (s + rfma(x1.x, x2.x, -x1.y * x2.y));
+              }
+              acc_g2 += (double)s;
+              if (have_gbar) acc_mu += cb * wk * (double)((a == c ? rr_t(1) : rr_t(2)) *
+                                                          (a == c ? rfma(x1.x, x1.x, -x1.y * x1.y)
+                                                                  : rfma(x1.x, x2.x, -x1.y * x2.y)));
+            }
+          }
+          __syncwarp();
+        }
+        const int* sq = sp + M;
+        const bool mine = mf < nv;
+        double2* out = (p.mode & (kGloc | kAdj))
+                           ? p.gq + ((int64_t)(unit - p.gb0) * p.n_iw + min(n + mf, n1 - 1)) * p.mmax * p.mmax
+                           : nullptr;
+        if ((p.mode & kGloc) && mine) {
+          for (int i = sl; i < MM; i += LW) {
+            const int a = i / M, c = i - a * M;
+            const double2 g = A[sp[a] * M + sq[c]];
+            gq_put(&out[i], q, make_double2(wk * g.x, wk * g.y));
+          }
+        }
+        if constexpr (!LOW) {
+          if (adj) {
+            // Sigma_bar = A^+ Ghat A^+ with Ghat = Gbar + c F^+ (c = n_bar 2 / beta), A = S^{-1}:
+            // Mt = Ghat A^+, then A^+ Mt; Re<Gbar, A F A> = Re Tr(F^+ Sigma_bar) - c Re Tr (A F)^2
+            double2* Mt = sM + mf * MM;
+            double2* Fm = reinterpret_cast<double2*>(sF) + mf * MM;
+            const double2* Gb = have_gbar ? p.gbar + si.offSig + (int64_t)min(n + mf, n1 - 1) * MM : nullptr;
+            for (int i = sl; i < MM; i += LW) {
+              const int a = i / M, c = i - a * M;
+              double2 acc = make_double2(0.0, 0.0);
+              const int pc = sp[c] * M;
+              for (int x = 0; x < M; ++x) {
+                // Ghat[a][x'] conj(A[c][x']) with x' = p_x, A[c][p_x] at column q_{p_x} = x
+                const int xx = sp[x];
+                const double2 fv = Fm[xx * M + a];
+                double2 g = make_double2(cb * fv.x, -cb * fv.y);
+                if (have_gbar) {
+                  const double2 gb = Gb[a * M + xx];
+                  g.x += gb.x;
+                  g.y += gb.y;
+                }
+                cmac_cb(acc, g, A[pc + x]);
+              }
+              Mt[i] = acc;
+            }
+            __syncwarp();
+            for (int i = sl; i < MM; i += LW) {
+              const int a = i / M, c = i - a * M;
+              double2 acc = make_double2(0.0, 0.0);
+              const int qa = sq[a];
+              // conj(A[x][a]) Mt[x][c], A[x][a] at row p_x, column q_a
+              for (int x = 0; x < M; ++x) cmac_ca(acc, A[sp[x] * M + qa], Mt[x * M + c]);
+              if (mine) {
+                gq_put(&out[i], q, make_double2(wk * acc.x, wk * acc.y));
+                if (have_gbar) {
+                  const double2 fv = Fm[i];
+                  acc_mu -= wk * fma(fv.x, acc.x, fv.y * acc.y);
+                }
+              }
+            }
+          }
+        }
+      }
+      if (rho) {
+        // S_k of the whole CTA's frequencies: columns S^{-1} B D staged in sY for yf
+        // frequencies at a time, then the blocks of G are added to the chunk's sum
+        const int nb = ki.nb, tot = min(W * F, n1 - base);
+        double2* Sk = p.rho_part + (int64_t)chunk * p.rho_chunk_stride + ki.offH;
+        const rc_t* Bk;
+        if constexpr (LOW) Bk = bf.Bs + ki.offP;
+        else Bk = bf.B + ki.offP;
+        auto mat = [&](int f) { return reinterpret_cast<const double2*>(smraw + (size_t)(f / F) * L.wstride + L.wS) + (f % F) * MM; };
+        auto piv = [&](int f) { return reinterpret_cast<const int*>(smraw + (size_t)(f / F) * L.wstride + L.wp) + (f % F) * 2 * M; };
+        auto dof = [&](int f) { return reinterpret_cast<const double2*>(smraw + (size_t)(f / F) * L.wstride + L.wd) + (f % F) * n2; };
+        const bool first = (base == n0);
+        __syncthreads();
+        for (int f0 = 0; f0 < tot; f0 += L.yf) {
+          const int nf = min(L.yf, tot - f0);
+          const bool put = first && f0 == 0;
+          auto add = [&](int at, double2 v) {
+            if (!put) {
+              const double2 o = Sk[at];
+              v.x += o.x;
+              v.y += o.y;
+            }
+            Sk[at] = v;
+          };
+          // (1,1) block
+          for (int i = tid; i < MM; i += 32 * W) {
+            const int a = i / M, c = i - a * M;
+            double2 v = make_double2(0.0, 0.0);
+            for (int f = f0; f < f0 + nf; ++f) {
+              const int* pf = piv(f);
+              const double2 g = mat(f)[pf[a] * M + pf[M + c]];
+              v.x += g.x;
+              v.y += g.y;
+            }
+            add(a * nb + c, v);
+          }
+          // (1,2) and (2,1): Y = S^{-1} B D, Z = D B^+ S^{-1}
+          for (int i = tid; i < M * n2; i += 32 * W) {
+            const int a = i / n2, bb = i - a * n2;
+            double2 v12 = make_double2(0.0, 0.0), v21 = v12;
+            for (int f = f0; f < f0 + nf; ++f) {
+              const int* pf = piv(f);
+              const int* qf = pf + M;
+              const double2* Af = mat(f);
+              rc_t y = rzero(rc_t{}), z = y;
+              const int pa = pf[a] * M, qa = qf[a];
+              for (int x = 0; x < M; ++x) {
+                const int xx = pf[x];  // orbital of column x; also the row of orbital x
+                rmac(y, to_rest(Af[pa + x], rc_t{}), ld_cg(Bk + xx * n2 + bb));
+                rmac_ca(z, ld_cg(Bk + x * n2 + bb), to_rest(Af[xx * M + qa], rc_t{}));
+              }
+              const rc_t d = to_rest(dof(f)[bb], rc_t{});
+              y = rmul(y, d);
+              z = rmul(z, d);
+              sY[(size_t)(f - f0) * M * n2 + i] = y;
+              v12.x += (double)y.x; v12.y += (double)y.y;
+              v21.x += (double)z.x; v21.y += (double)z.y;
+            }
+            add(a * nb + M + bb, v12);
+            add((M + bb) * nb + a, v21);
+          }
+          __syncthreads();
+          // (2,2): d_b (delta_bc + sum_a conj(B_ab) Y_ac)
+          for (int i = tid; i < n2 * n2; i += 32 * W) {
+            const int bb = i / n2, c = i - bb * n2;
+            double2 v = make_double2(0.0, 0.0);
+            for (int f = f0; f < f0 + nf; ++f) {
+              rc_t w = rzero(rc_t{});
+              const rc_t* Y = sY + (size_t)(f - f0) * M * n2 + c;
+              for (int a = 0; a < M; ++a) rmac_ca(w, ld_cg(Bk + a * n2 + bb), Y[a * n2]);
+              const double2 d = dof(f)[bb];
+              w = rmul(w, to_rest(d, rc_t{}));
+              v.x += (double)w.x;
+              v.y += (double)w.y;
+              if (bb == c) {
+                v.x += d.x;
+                v.y += d.y;
+              }
+            }
+            add((M + bb) * nb + M + c, v);
+          }
+          __syncthreads();
+        }
+      }
+    }
+    // deterministic: xor tree in each warp, then the warps in order
+    if (p.mode & (kOcc | kAdj)) {
+      acc_tr = warp_sum(acc_tr);
+      acc_g2 = warp_sum(acc_g2);
+      acc_mu = warp_sum(acc_mu);
+      if (lane == 0) {
+        s_part[wp][0] = acc_tr;
+        s_part[wp][1] = acc_g2;
+        s_part[wp][2] = acc_mu;
+      }
+      __syncthreads();
+      if (tid == 0) {
+        double v[3] = {0.0, 0.0, 0.0};
+        for (int w = 0; w < W; ++w)
+          for (int x = 0; x < 3; ++x) v[x] += s_part[w][x];
+        if (occ) {
+          double* o = p.occ_part + ((int64_t)kk * p.n_chunks + chunk) * 2;
+          o[0] = v[0];
+          o[1] = v[1];
+        }
+        if (adj) p.mubar_part[(int64_t)kk * p.n_chunks + chunk] = v[2];
+      }
+    }
+  }
+}
+
+// rho_part chunk 0 <- U (sum_c S_c) U^+ (one CTA per k): the chunks are summed once, then two
+// products.
+__global__ void __launch_bounds__(kSetupThreads)
+    k_block_rotate(const KInfo* __restrict__ kinfo, const double2* __restrict__ U, double2* rho_part,
+                   int64_t stride, int n_chunks, double2* T) {
+  const KInfo ki = kinfo[blockIdx.x];
+  const int N = ki.nb;
+  const double2* Uk = U + ki.offH;
+  double2* S0 = rho_part + ki.offH;
+  double2* Tk = T + ki.offH;
+  for (int e = threadIdx.x; e < N * N; e += kSetupThreads) {
+    double2 s = S0[e];
+    for (int c = 1; c < n_chunks; ++c) {
+      const double2 v = rho_part[(int64_t)c * stride + ki.offH + e];
+      s.x += v.x;
+      s.y += v.y;
+    }
+    S0[e] = s;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < N * N; e += kSetupThreads) {
+    const int i = e / N, j = e - i * N;
+    double2 acc = make_double2(0.0, 0.0);
+    for (int l = 0; l < N; ++l) cmac_cb(acc, S0[i * N + l], Uk[j * N + l]);
+    Tk[e] = acc;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < N * N; e += kSetupThreads) {
+    const int i = e / N, j = e - i * N;
+    double2 acc = make_double2(0.0, 0.0);
+    for (int l = 0; l < N; ++l) cmac(acc, Uk[i * N + l], Tk[l * N + j]);
+    S0[e] = acc;
+  }
+}
+
+size_t reduce_smem(int nbmax, int mmax, bool matrix) {
+  return sizeof(double2) * ((size_t)mmax * nbmax + (size_t)mmax * mmax + nbmax +
+                            (matrix ? (size_t)nbmax * nbmax : 0));
+}
+bool reduce_in_smem(int nbmax, int mmax, int smem_optin) {
+  return reduce_smem(nbmax, mmax, true) <= (size_t)smem_optin - 1024;
+}
+int reduce_grid(int nbmax, int mmax, int n_k, int smem_optin, int sm_count) {
+  const bool in = reduce_in_smem(nbmax, mmax, smem_optin);
+  const int per_sm = in ? std::max(1, (int)((size_t)smem_optin / reduce_smem(nbmax, mmax, true))) : 2;
+  return std::max(1, std::min(n_k, sm_count * std::min(per_sm, 8)));
+}
+
+template <int LW, bool LOW>
+cudaError_t launch_lw(const PointParams& p, const BlockForm& b, const BlockLaunch& l, size_t smem, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(k_point_block<LW, LOW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_point_block<LW, LOW>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                           (int)cudaSharedmemCarveoutMaxShared);
+  if (e != cudaSuccess) return e;
+  k_point_block<LW, LOW><<<l.n_units * l.n_chunks, 32 * kBlkWarps, smem, s>>>(p, b, l);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t block_reduce_ws_elems(int nbmax, int mmax, int smem_optin, int sm_count) {
+  if (reduce_in_smem(nbmax, mmax, smem_optin)) return 0;
+  return (size_t)nbmax * nbmax * 2 * sm_count;
+}
+
+cudaError_t launch_block_reduce(const BlockSetup& b, int smem_optin, int sm_count, cudaStream_t s) {
+  const bool in = reduce_in_smem(b.nbmax, b.mmax, smem_optin);
+  const size_t smem = reduce_smem(b.nbmax, b.mmax, in);
+  cudaError_t e = cudaFuncSetAttribute(k_block_reduce, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_block_reduce<<<reduce_grid(b.nbmax, b.mmax, b.n_k, smem_optin, sm_count), kSetupThreads, smem, s>>>(b, in ? 1 : 0);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_block_finish(const BlockSetup& b, cudaStream_t s) {
+  const size_t smem = sizeof(double2) * (2 * (size_t)b.mmax * b.mmax + (size_t)b.mmax * b.n2max);
+  cudaError_t e = cudaFuncSetAttribute(k_block_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_block_finish<<<b.n_k, kSetupThreads, smem, s>>>(b);
+  return cudaGetLastError();
+}
+
+int block_batch(int mmax) { return kBlkWarps * (32 / block_lanes(mmax)); }
+
+size_t block_smem(int mmax, int n2max, int mode, int low) { return make_layout_b(mmax, n2max, mode, low).bytes; }
+
+cudaError_t launch_point_block(const PointParams& p, const BlockForm& b, const BlockLaunch& l, int low,
+                               cudaStream_t s) {
+  const size_t smem = block_smem(p.mmax, l.n2max, p.mode, low);
+  switch (block_lanes(p.mmax) + (low ? 1 : 0)) {
+    case 8: return launch_lw<8, false>(p, b, l, smem, s);
+    case 9: return launch_lw<8, true>(p, b, l, smem, s);
+    case 16: return launch_lw<16, false>(p, b, l, smem, s);
+    case 17: return launch_lw<16, true>(p, b, l, smem, s);
+    case 32: return launch_lw<32, false>(p, b, l, smem, s);
+    default: return launch_lw<32, true>(p, b, l, smem, s);
+  }
+}
+
+cudaError_t launch_block_rotate(const KInfo* kinfo, int n_k, const double2* U, double2* rho_part,
+                                int64_t stride, int n_chunks, double2* T, cudaStream_t s) {
+  k_block_rotate<<<n_k, kSetupThreads, 0, s>>>(kinfo, U, rho_part, stride, n_chunks, T);
+  return cudaGetLastError();
+}
+
+}  // namespace gf

@@ -1,0 +1,94 @@
+// Block form of the lattice points: declarations shared by gf_block.cu (the kernels) and the
+// C-ABI translation units.
+//
+// With P_k^+ = Q [R; 0] (Householder QR, Q unitary N_b x N_b, R upper triangular m x m) the
+// frequency-dependent part of A = (i w_n + mu) - H_k - P_k^+ Sigma P_k lives in the first m
+// rows and columns of Q^+ A Q.  The other n2 = N_b - m rows hold H_k alone, so one Hermitian
+// eigenproblem of that n2 x n2 block per uploaded H_k makes them diagonal for every frequency:
+//   z = i w_n + mu,   D = diag(d_b),  d_b = 1 / (z - e_b),
+//   S(z) = z O - H11 - Sigma(i w_n) - B D B^+                        (m x m)
+//   P G P^+ = S^{-1},  F = dS/dz = O + B D^2 B^+,  P G^2 P^+ = S^{-1} F S^{-1},
+//   Tr G   = sum_b d_b + Tr(S^{-1} F),
+//   Tr G^2 = sum_b d_b^2 + Tr((S^{-1} F)^2) + 2 Tr(S^{-1} B D^3 B^+),
+//   G = U [[S^{-1}, S^{-1} B D], [D B^+ S^{-1}, D + D B^+ S^{-1} B D]] U^+,
+// exactly, with O = (P P^+)^{-1}, H11 = R^{-1} Q1^+ H Q1 R^{-+}, B = R^{-1} Q1^+ H Q2 V and
+// U = [Q1 R^{-+} | Q2 V] (V: eigenvectors of the n2 x n2 block).  A point costs
+// (N_b - m) m^2 + O(m^3) complex multiply-adds instead of N_b^3.
+#pragma once
+
+#include "gf_internal.cuh"
+
+namespace gf {
+
+constexpr int kBlkMaxM = 32;    // orbitals: one lane per row of S
+constexpr int kBlkWarps = 4;    // warps per CTA of the point kernels
+
+// Device arrays of the block form of every k-point.
+struct BlockForm {
+  const double* e;        // [n2] at offD[k]
+  const int64_t* offD;
+  const double2* T;       // [n2][np] at offT[k]: B_ab conj(B_cb) over the pairs a <= c, np = m(m+1)/2
+  const float2* Ts;       // its FP32 rounding (GF_PREC_MIXED) or null
+  const int64_t* offT;
+  const double2* B;       // [m][n2] at KInfo::offP
+  const float2* Bs;
+  const double2* HO;      // [2][np] per k at k * 2 * npmax: H11 pairs, then O pairs
+  int npmax;
+};
+
+// One launch over units (k-points, or k-groups for the k-reductions) x frequency chunks.
+struct BlockLaunch {
+  int n_units, unit0;     // units [unit0, unit0 + n_units)
+  const int2* units;      // {first entry of kperm, count} per unit
+  const int* kperm;
+  int n_begin, n_end;     // frequencies [n_begin, n_end)
+  int chunk_w, n_chunks;  // chunks of this launch
+  int chunk0;             // index of the first one in the per-chunk partial sums
+  int n2max;
+};
+
+// Setup, three launches over the k-points: reduction (QR, Q^+ H Q), eigenpairs of the n2
+// block, and the tables above.  flags (device int): kBlkNonHermitian, kBlkRankDeficient,
+// kBlkNoConvergence; hnorm (device, n_k): ||H_k||_F / sqrt(N_b).
+constexpr int kBlkNonHermitian = 1, kBlkRankDeficient = 2, kBlkNoConvergence = 4;
+struct BlockSetup {
+  const double2* H;
+  const double2* P;
+  const KInfo* kinfo;
+  const SInfo* sinfo;
+  int n_k, nbmax, mmax, n2max, npmax;
+  double2* D22;           // [n2][n2] at offH: the n2 block, then its eigenvectors
+  double2* V;             // [m][N_b] at offP: Householder vectors (row j: vector j)
+  double2* R;             // [m][m] at k * mmax^2
+  double* tau;            // [m] at k * mmax
+  double2* H11;           // [m][m] at k * mmax^2
+  double2* B;             // [m][n2] at offP: Q1^+ H Q2, then B
+  double* e;              // [n2] at offD
+  const int64_t* offD;
+  double2* T;
+  float2* Ts;
+  const int64_t* offT;
+  float2* Bs;
+  double2* HO;
+  double2* U;             // [N_b][N_b] at offH
+  double2* ws;            // per-CTA slices of nbmax^2 elements when the matrix exceeds shared memory
+  int* flags;
+  double* hnorm;
+};
+cudaError_t launch_block_reduce(const BlockSetup& b, int smem_optin, int sm_count, cudaStream_t s);
+cudaError_t launch_block_eig(const BlockSetup& b, double2* ws, int grid, int in_smem, cudaStream_t s);
+cudaError_t launch_block_finish(const BlockSetup& b, cudaStream_t s);
+size_t block_reduce_ws_elems(int nbmax, int mmax, int smem_optin, int sm_count);
+
+// Frequencies a CTA takes at once.
+int block_batch(int mmax);
+// low = 1: the parts of the result that mixed precision takes from an FP32 inverse (F, the
+// traces, rho_k) in FP32; S, its inverse and G_loc stay FP64.
+size_t block_smem(int mmax, int n2max, int mode, int low);
+cudaError_t launch_point_block(const PointParams& p, const BlockForm& b, const BlockLaunch& l, int low,
+                               cudaStream_t s);
+// rho_part chunk 0 <- U (sum_c S_c) U^+ for every k; T: scratch of the size of H.
+cudaError_t launch_block_rotate(const KInfo* kinfo, int n_k, const double2* U, double2* rho_part,
+                                int64_t stride, int n_chunks, double2* T, cudaStream_t s);
+
+}  // namespace gf

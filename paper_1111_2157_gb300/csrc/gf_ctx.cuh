@@ -16,6 +16,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "gf.h"
+#include "gf_block.cuh"
 #include "gf_internal.cuh"
 
 using gf::Item;
@@ -166,6 +167,20 @@ struct gf_ctx {
   // creation is undone by gf_destroy, before that by a plain delete (no CUDA call)
   bool device_checked = false;
   DevBuf lr_eps, lr_U, lr_Pt, lr_T, lr_ws;
+  // block form (gf_block.cuh): chosen per call by use_block; blk_shape: the sizes allow it,
+  // blk_ok: the uploaded H and P do (ensure_block)
+  bool blk_shape = false, blk_ok = false, blk_dirty = true;
+  int blk_n2max = 0, blk_kg = 1, blk_cw = 1;  // largest N_b - m, k-points per group, chunk width
+  int blk_nc = 0;                             // mixed precision: frequencies below it run in FP64
+  std::vector<int> blk_sys_g0, blk_sys_g1;    // groups of each system
+  int blk_groups = 0;
+  int64_t blk_totT = 0;
+  int run_chunks = 1;                         // the current call: chunks of its partial sums,
+  bool run_on_block = false;                  // and whether it runs on the block form
+  int occ_path = 0;                           // path that the captured N(mu) graph holds
+  DevBuf blk_units, blk_perm, blk_sysg, blk_offT;
+  DevBuf blk_e, blk_T, blk_Ts, blk_B, blk_Bs, blk_HO, blk_U, blk_D22, blk_V, blk_R, blk_H11, blk_tau,
+      blk_ws, blk_info;
   // DMFT step and projector construction
   DevBuf eimp, eimp_part, gl_in, delta, wraw, vdc;
   // pole form of Sigma (gf_set_sigma_poles) and the pseudo-Hamiltonian path

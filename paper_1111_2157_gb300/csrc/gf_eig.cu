@@ -22,6 +22,7 @@
 
 #include <algorithm>
 
+#include "gf_block.cuh"
 #include "gf_complex.cuh"
 #include "gf_internal.cuh"
 
@@ -582,6 +583,36 @@ __global__ void __launch_bounds__(kEigThreads)
   }
 }
 
+// Block form: eigenpairs of the n2 x n2 block of every k (D22, replaced by its eigenvectors).
+__global__ void __launch_bounds__(kEigThreads)
+    k_block_eig(const BlockSetup b, double2* gws, int in_smem) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double rot[4 * 128];
+  __shared__ double2 ph[128];
+  __shared__ double red[kEigThreads / 32];
+  double2* A = in_smem ? reinterpret_cast<double2*>(smem_raw) : gws + blockIdx.x * eig_ws_elems(b.n2max);
+  for (int k = blockIdx.x; k < b.n_k; k += gridDim.x) {
+    const KInfo ki = b.kinfo[k];
+    const int n = ki.nb - b.sinfo[ki.sys].m, ld = n | 1;
+    double2* V = A + (size_t)n * ld;
+    double2* D = b.D22 + ki.offH;
+    for (int e = threadIdx.x; e < n * n; e += kEigThreads) {
+      const int i = e / n, j = e - i * n;
+      const double2 x = D[i * n + j], y = D[j * n + i];
+      A[i * ld + j] = make_double2(0.5 * (x.x + y.x), 0.5 * (x.y - y.y));
+    }
+    __syncthreads();
+    const int sw = jacobi_heev(A, V, n, ld, 40, rot, ph, red);
+    if (sw < 0 && threadIdx.x == 0) atomicOr(b.flags, kBlkNoConvergence);
+    for (int l = threadIdx.x; l < n; l += kEigThreads) b.e[b.offD[k] + l] = A[l * ld + l].x;
+    for (int e = threadIdx.x; e < n * n; e += kEigThreads) {
+      const int i = e / n, l = e - i * n;
+      D[e] = V[i * ld + l];
+    }
+    __syncthreads();
+  }
+}
+
 // DOS and PDOS on the real axis from the pseudo-Hamiltonian eigenpairs
 // (Eqs. DOS and PDOS) with a Lorentzian of half width eta:
 //   D(e)       = sum_k w_k sum_l |Psi_b,l|^2 L(e + mu - E_l),
@@ -696,6 +727,14 @@ cudaError_t launch_lr_setup(const double2* H, const double2* P, const KInfo* kin
   if (e != cudaSuccess) return e;
   k_lr_setup<<<grid, kEigThreads, smem, s>>>(H, P, kinfo, sinfo, offD, n_k, nbmax, eps, U, Pt, ws,
                                              in_smem, status);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_block_eig(const BlockSetup& b, double2* ws, int grid, int in_smem, cudaStream_t s) {
+  const size_t smem = in_smem ? heev_smem(b.n2max) : 0;
+  cudaError_t e = cudaFuncSetAttribute(k_block_eig, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_block_eig<<<grid, kEigThreads, smem, s>>>(b, ws, in_smem);
   return cudaGetLastError();
 }
 
