@@ -158,12 +158,12 @@ gf_status ensure_block(gf_ctx* c) {
                                flags & gf::kBlkRankDeficient ? "P rank deficient" : "eigensolver") + "); ";
     return GF_OK;
   }
-  // mixed precision: frequencies w_n below a quarter of the rms eigenvalue of H run in FP64
+  // mixed precision: frequencies w_n below a fifth of the rms eigenvalue of H run in FP64
   // (an eigenvalue e_b within w_n of mu loses |B|^2 / w_n in FP32)
   double h = 0.0, bmax = 0.0;
   for (int k = 0; k < c->n_k; ++k) h = std::max(h, info[k]);
   for (int s = 0; s < c->n_sys; ++s) bmax = std::max(bmax, c->beta[s]);
-  const double nc = std::ceil(0.5 * (0.25 * h * bmax / M_PI - 1.0));
+  const double nc = std::ceil(0.5 * (0.2 * h * bmax / M_PI - 1.0));
   const int batch = gf::block_batch(c->mmax);
   const int64_t up = (int64_t)std::min((double)c->n_iw, std::max(1.0, nc));
   c->blk_nc = mixed && !c->lowrank ? (int)std::min<int64_t>(c->n_iw, (up + batch - 1) / batch * batch) : c->n_iw;
@@ -176,13 +176,13 @@ bool use_block(const gf_ctx* c, int mode) {
   if (!c->blk_shape || !c->blk_ok) return false;
   const char* only = std::getenv("GF_KERNEL");
   if (only && (std::strcmp(only, "direct") == 0 || (c->precision == GF_PREC_MIXED && !c->lowrank))) return false;
-  if (c->precision == GF_PREC_MIXED && !c->lowrank && mode == gf::kOcc) return false;
   // sizes that the general kernels refuse stay refused
   const size_t limit = (size_t)c->smem_optin - 1024;
   const size_t general = c->lowrank ? gf::point_lr_smem(c->nbmax, c->mmax, mode, 0, c->precision != GF_PREC_FP64)
                                     : gf::point_fp64_smem(c->nbmax, c->mmax, mode, 0);
   if (general > limit || (c->lowrank && c->nbmax > gf::heev_max_n())) return false;
-  return gf::block_smem(c->mmax, c->blk_n2max, mode, 0) <= limit;
+  return gf::block_smem(c->mmax, c->blk_n2max, mode, 0) <= limit &&
+         (c->precision != GF_PREC_MIXED || gf::block32_smem(c->mmax, c->blk_n2max) <= limit);
 }
 
 // rho_k partial sums: the low-rank and the block kernels leave them in the basis that makes
@@ -561,7 +561,8 @@ gf_status run_block(gf_ctx* c, int mode, gf::PointParams p) {
       l.chunk0 = part ? ch0 : 0;
       l.n_chunks = part ? ch1 : ch0;
       if (l.n_chunks == 0) continue;
-      GF_CU(gf::launch_point_block(p, b, l, part, c->stream));
+      if (part && mode == gf::kOcc) GF_CU(gf::launch_occ_block32(p, b, l, c->stream));
+      else GF_CU(gf::launch_point_block(p, b, l, part, c->stream));
       c->last_launches += 1;
     }
     if (!c->capturing) {
@@ -584,7 +585,7 @@ gf_status run_block(gf_ctx* c, int mode, gf::PointParams p) {
   if (c->tuned.find(key) == c->tuned.end()) {
     c->tuned[key] = 0;
     c->tune_log += "mode " + std::to_string(mode) + ": block form, " + std::to_string(nc) + " frequencies in FP64" +
-                   (ch1 ? ", " + std::to_string(c->n_iw - nc) + " with FP32 traces" : std::string()) + "; ";
+                   (ch1 ? ", " + std::to_string(c->n_iw - nc) + " in FP32 (traces, rho)" : std::string()) + "; ";
   }
   return GF_OK;
 }
@@ -1104,11 +1105,15 @@ gf_status init_ctx(gf_ctx* c, const gf_desc* d) {
   std::vector<int2> units;
   std::vector<int> perm(2 * (size_t)c->n_k), bsysg;
   if (c->blk_shape) {
-    // chunks: whole batches of a CTA, about eight CTAs per resident one; k-groups: about six
-    const int batch = gf::block_batch(c->mmax);
+    // chunks: whole batches of a CTA, about eight CTAs per resident one; k-groups: about six.
+    // (the FP32 N(mu) kernel's batch is a multiple of the FP64 one's)
     const double res = 3.0 * c->sm_count, pts = (double)c->n_k * c->n_iw;
-    const double w = std::ceil(pts / (8.0 * res) / batch) * batch;
-    c->blk_cw = (int)std::min(std::max((double)batch, w), std::ceil((double)c->n_iw / batch) * batch);
+    double batch = gf::block_batch(c->mmax), w = std::ceil(pts / (8.0 * res) / batch) * batch;
+    if (c->precision == GF_PREC_MIXED && w > batch) {
+      batch = gf::block32_batch(c->mmax);
+      w = std::ceil(w / batch) * batch;
+    }
+    c->blk_cw = (int)std::min(std::max(batch, w), std::ceil((double)c->n_iw / batch) * batch);
     const int nch = (c->n_iw + c->blk_cw - 1) / c->blk_cw;
     c->blk_kg = (int)std::max(1.0, std::min((double)gf::kMaxKGroup, std::floor((double)c->n_k * nch / (6.0 * res))));
     c->blk_sys_g0.assign(c->n_sys, 0);

@@ -87,6 +87,11 @@ int block_batch(int mmax);
 size_t block_smem(int mmax, int n2max, int mode, int low);
 cudaError_t launch_point_block(const PointParams& p, const BlockForm& b, const BlockLaunch& l, int low,
                                cudaStream_t s);
+// Mixed-precision N(mu) passes: the FP32 kernel (gf_block32.cu), frequencies of a CTA batch and
+// shared memory.
+int block32_batch(int mmax);
+size_t block32_smem(int mmax, int n2max);
+cudaError_t launch_occ_block32(const PointParams& p, const BlockForm& b, const BlockLaunch& l, cudaStream_t s);
 // rho_part chunk 0 <- U (sum_c S_c) U^+ for every k; T: scratch of the size of H.
 cudaError_t launch_block_rotate(const KInfo* kinfo, int n_k, const double2* U, double2* rho_part,
                                 int64_t stride, int n_chunks, double2* T, cudaStream_t s);

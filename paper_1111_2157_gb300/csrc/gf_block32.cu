@@ -1,0 +1,380 @@
+// Block form of the lattice points (gf_block.cuh): the FP32 kernel of mixed-precision N(mu)
+// passes, for the frequencies whose FP32 rounding stays below that of an FP32 inverse of the
+// window (w_n above a fraction of H's scale; k_point_block takes the others in FP64).
+//
+// A warp takes FW frequencies of one k-point and runs without block barriers:
+//   1. d_b = 1 / (z - e_b) and its powers, one (band, frequency) per lane;
+//   2. band sums of S and F = dS/dz, one orbital pair a <= c per lane and FW frequencies in
+//      registers, so that one load of the pair table feeds 8 FW FMAs;
+//   3. S^{-1} with LW lanes per matrix, one row per lane in registers (Gauss-Jordan in exchange
+//      form, rows rotated one column per pivot, lazy row scales, as warp_invert of
+//      gf_warp_gj.cuh), then X = S^{-1} F row by row from the same registers;
+//   4. Tr X, Tr X^2, and 2 Tr(S^{-1} B D^3 B^+) from a second sweep over the pair table.
+// The sums over frequencies are FP64.
+#include <math.h>
+#include <stdint.h>
+
+#include "gf_block.cuh"
+#include "gf_complex.cuh"
+
+namespace gf {
+
+namespace {
+
+using namespace cx;
+
+__device__ __forceinline__ float2 z2() { return make_float2(0.f, 0.f); }
+
+// Shared memory (bytes): per CTA x_b = mu - e_b, mu O - H11 and O by pairs and the pair list;
+// per warp d, d^2, d^3 as [band][FW], S and F with rows of NMAX entries, the pivot rows and tables.
+struct Layout32 {
+  size_t oX, oHz, oO, oPair, warp0, wd, wS, wF, wbuf, wp, wstride, bytes;
+};
+
+__host__ __device__ inline Layout32 make_layout32(int mmax, int n2max, int nmax, int lw, int fw) {
+  Layout32 L;
+  auto al = [](size_t x) { return (x + 15) & ~(size_t)15; };
+  const size_t np = (size_t)mmax * (mmax + 1) / 2;
+  size_t o = 0;
+  L.oX = o; o = al(o + 4 * (size_t)n2max);
+  L.oHz = o; o = al(o + 8 * np);
+  L.oO = o; o = al(o + 8 * np);
+  L.oPair = o; o = al(o + 2 * np);
+  L.warp0 = o;
+  size_t g = 0;
+  L.wd = g; g = al(g + 24 * (size_t)fw * n2max);
+  L.wS = g; g = al(g + 8 * (size_t)fw * mmax * nmax);
+  L.wF = g; g = al(g + 8 * (size_t)fw * mmax * nmax);
+  L.wbuf = g; g = al(g + 8 * (size_t)(32 / lw) * nmax);
+  L.wp = g; g = al(g + 8 * (size_t)(32 / lw) * nmax);
+  L.wstride = g;
+  L.bytes = o + kBlkWarps * g;
+  return L;
+}
+
+template <int NMAX, int LW, int FW>
+__global__ void __launch_bounds__(32 * kBlkWarps, NMAX > 24 ? 2 : 3)
+    k_occ_block32(const PointParams p, const BlockForm bf, const BlockLaunch bl) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ double s_part[kBlkWarps][2];
+  constexpr int G = 32 / LW;  // matrices inverted together
+  static_assert(FW % G == 0 && FW % 2 == 0 && NMAX % 2 == 0, "batch shape");
+  const Layout32 L = make_layout32(p.mmax, bl.n2max, NMAX, LW, FW);
+  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5, sl = lane % LW, mf = lane / LW;
+  float* xs = reinterpret_cast<float*>(smraw + L.oX);
+  float2* hz = reinterpret_cast<float2*>(smraw + L.oHz);
+  float2* oo = reinterpret_cast<float2*>(smraw + L.oO);
+  uchar2* pair = reinterpret_cast<uchar2*>(smraw + L.oPair);
+  unsigned char* wb = smraw + L.warp0 + (size_t)wp * L.wstride;
+  const int unit = bl.unit0 + blockIdx.x / bl.n_chunks, ch = blockIdx.x % bl.n_chunks;
+  const int kk = bl.kperm[bl.units[unit].x];  // N(mu) units hold one k-point
+  const int n0 = bl.n_begin + ch * bl.chunk_w, n1 = min(bl.n_end, n0 + bl.chunk_w);
+  const KInfo ki = p.kinfo[kk];
+  const SInfo si = p.sinfo[ki.sys];
+  const int M = si.m, n2 = ki.nb - M, NP = M * (M + 1) / 2;
+  const double mu = p.mu[ki.sys], pib = M_PI / si.beta;
+  const float2* Ts = bf.Ts + bf.offT[kk];
+  float2* sd = reinterpret_cast<float2*>(wb + L.wd);
+  float2* sd2 = sd + FW * n2;
+  float2* sd3 = sd2 + FW * n2;
+  float2* sS = reinterpret_cast<float2*>(wb + L.wS);
+  float2* sF = reinterpret_cast<float2*>(wb + L.wF);
+  float2* sBuf = reinterpret_cast<float2*>(wb + L.wbuf) + mf * NMAX;
+  int* sp = reinterpret_cast<int*>(wb + L.wp) + mf * 2 * NMAX;
+  int* sq = sp + NMAX;
+  for (int b = tid; b < n2; b += 32 * kBlkWarps) xs[b] = __double2float_rn(mu - bf.e[bf.offD[kk] + b]);
+  const double2* HO = bf.HO + (size_t)kk * 2 * bf.npmax;
+  for (int pr = tid; pr < NP; pr += 32 * kBlkWarps) {
+    int a = 0, rem = pr;
+    while (rem >= M - a) { rem -= M - a; ++a; }
+    pair[pr] = make_uchar2((unsigned char)a, (unsigned char)(a + rem));
+    const double2 h = HO[pr], o = HO[bf.npmax + pr];
+    hz[pr] = make_float2(__double2float_rn(fma(mu, o.x, -h.x)), __double2float_rn(fma(mu, o.y, -h.y)));
+    oo[pr] = make_float2(__double2float_rn(o.x), __double2float_rn(o.y));
+  }
+  // the padding columns of F (and of X, which takes its place) stay zero
+  for (int i = lane; i < FW * M * NMAX; i += 32) sF[i] = z2();
+  __syncthreads();
+  double acc_tr = 0.0, acc_g2 = 0.0;
+
+  for (int n = n0 + wp * FW; n < n1; n += kBlkWarps * FW) {
+    float tr = 0.f, g2 = 0.f;
+    for (int i = lane; i < FW * n2; i += 32) {
+      const int b = i / FW, f = i - b * FW;
+      const float w = __double2float_rn((2.0 * min(n + f, n1 - 1) + 1.0) * pib), x = xs[b];
+      const float q = __frcp_rn(__fmaf_rn(x, x, __fmul_rn(w, w)));
+      const float2 d = make_float2(__fmul_rn(x, q), -__fmul_rn(w, q)), d2 = fmul(d, d);
+      sd[i] = d;
+      sd2[i] = d2;
+      sd3[i] = fmul(d2, d);
+      if (n + f < n1) {
+        tr += d.x;
+        g2 += d2.x;
+      }
+    }
+    __syncwarp();
+    for (int pr = lane; pr < NP; pr += 32) {
+      const int a = pair[pr].x, c = pair[pr].y;
+      float2 xr[FW], xi[FW], yr[FW], yi[FW];
+#pragma unroll
+      for (int f = 0; f < FW; ++f) xr[f] = xi[f] = yr[f] = yi[f] = z2();
+      const float2* t = Ts + pr;
+#pragma unroll 4
+      for (int b = 0; b < n2; ++b) {
+        const float2 tv = __ldg(t + (size_t)b * NP);
+        const float4* d4 = reinterpret_cast<const float4*>(sd + b * FW);
+        const float4* e4 = reinterpret_cast<const float4*>(sd2 + b * FW);
+#pragma unroll
+        for (int f = 0; f < FW; f += 2) {
+          const float4 d = d4[f / 2], e = e4[f / 2];
+          xr[f].x = __fmaf_rn(tv.x, d.x, xr[f].x);
+          xr[f].y = __fmaf_rn(tv.y, d.x, xr[f].y);
+          xi[f].x = __fmaf_rn(tv.x, d.y, xi[f].x);
+          xi[f].y = __fmaf_rn(tv.y, d.y, xi[f].y);
+          xr[f + 1].x = __fmaf_rn(tv.x, d.z, xr[f + 1].x);
+          xr[f + 1].y = __fmaf_rn(tv.y, d.z, xr[f + 1].y);
+          xi[f + 1].x = __fmaf_rn(tv.x, d.w, xi[f + 1].x);
+          xi[f + 1].y = __fmaf_rn(tv.y, d.w, xi[f + 1].y);
+          yr[f].x = __fmaf_rn(tv.x, e.x, yr[f].x);
+          yr[f].y = __fmaf_rn(tv.y, e.x, yr[f].y);
+          yi[f].x = __fmaf_rn(tv.x, e.y, yi[f].x);
+          yi[f].y = __fmaf_rn(tv.y, e.y, yi[f].y);
+          yr[f + 1].x = __fmaf_rn(tv.x, e.z, yr[f + 1].x);
+          yr[f + 1].y = __fmaf_rn(tv.y, e.z, yr[f + 1].y);
+          yi[f + 1].x = __fmaf_rn(tv.x, e.w, yi[f + 1].x);
+          yi[f + 1].y = __fmaf_rn(tv.y, e.w, yi[f + 1].y);
+        }
+      }
+      const float2 h = hz[pr], o = oo[pr];
+#pragma unroll
+      for (int f = 0; f < FW; ++f) {
+        const int nn = min(n + f, n1 - 1);
+        const float w = __double2float_rn((2.0 * nn + 1.0) * pib);
+        const float2* Sg = p.Ss + si.offSig + (int64_t)nn * M * M;
+        const float2 s1 = __ldg(Sg + a * M + c), s2 = __ldg(Sg + c * M + a);
+        float2* Sm = sS + f * M * NMAX;
+        float2* Fm = sF + f * M * NMAX;
+        // z o_ac - h_ac - Sigma_ac - g_ac and, with conj(o) and conj(h), (c, a)
+        Sm[a * NMAX + c] = make_float2(__fmaf_rn(-w, o.y, h.x) - s1.x - (xr[f].x - xi[f].y),
+                                       __fmaf_rn(w, o.x, h.y) - s1.y - (xr[f].y + xi[f].x));
+        Fm[a * NMAX + c] = make_float2(o.x + (yr[f].x - yi[f].y), o.y + (yr[f].y + yi[f].x));
+        if (a != c) {
+          Sm[c * NMAX + a] = make_float2(__fmaf_rn(w, o.y, h.x) - s2.x - (xr[f].x + xi[f].y),
+                                         __fmaf_rn(w, o.x, -h.y) - s2.y - (xi[f].x - xr[f].y));
+          Fm[c * NMAX + a] = make_float2(o.x + (yr[f].x + yi[f].y), (yi[f].x - yr[f].y) - o.y);
+        }
+      }
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int f0 = 0; f0 < FW; f0 += G) {
+      const int f = f0 + mf;
+      const bool valid = n + f < n1;
+      float2* Sm = sS + f * M * NMAX;
+      float2* Fm = sF + f * M * NMAX;
+      float2 a[NMAX];
+#pragma unroll
+      for (int c = 0; c < NMAX; c += 2) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (sl < M) {
+          const float2 v0 = (c < M) ? Sm[sl * NMAX + c] : z2(), v1 = (c + 1 < M) ? Sm[sl * NMAX + c + 1] : z2();
+          v = make_float4(v0.x, v0.y, v1.x, v1.y);
+        }
+        a[c] = make_float2(v.x, v.y);
+        a[c + 1] = make_float2(v.z, v.w);
+      }
+      bool used = sl >= M;
+      float2 sc = make_float2(1.f, 0.f);
+#pragma unroll 1
+      for (int j = 0; j < M; ++j) {
+        unsigned best = used ? 0u : ((pivot_key_s(a[0]) & ~31u) | (unsigned)(31 - sl));
+        if constexpr (LW == 32) {
+          best = __reduce_max_sync(0xffffffffu, best);
+        } else {
+#pragma unroll
+          for (int off = LW / 2; off; off >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, off));
+        }
+        const int prow = min(31 - (int)(best & 31u), M - 1);
+        if (sl == 0 && valid && ((best >> 5) == 0u || (best & ~31u) >= 0x7f800000u)) atomicOr(p.status, kFlagSingular);
+        if (sl == prow) {
+#pragma unroll
+          for (int c = 0; c < NMAX; c += 2)
+            *reinterpret_cast<float4*>(sBuf + c) = make_float4(a[c].x, a[c].y, a[c + 1].x, a[c + 1].y);
+          sp[j] = sl;
+          sq[sl] = j;
+        }
+        __syncwarp();
+        const float4* b4 = reinterpret_cast<const float4*>(sBuf);
+        const float4 u0 = b4[0];
+        const float2 r = frcp(make_float2(u0.x, u0.y));
+        const bool isp = sl == prow;
+        const float2 lq = isp ? z2() : fmul(a[0], r);
+        // a_c -= l u_c, each entry moving one register down
+        a[0] = a[1];
+        fsub_prod(a[0], lq, make_float2(u0.z, u0.w));
+#pragma unroll
+        for (int c = 2; c < NMAX; c += 2) {
+          const float4 u = b4[c / 2];
+          a[c - 1] = a[c];
+          fsub_prod(a[c - 1], lq, make_float2(u.x, u.y));
+          a[c] = a[c + 1];
+          fsub_prod(a[c], lq, make_float2(u.z, u.w));
+        }
+        a[NMAX - 1] = isp ? make_float2(1.f, 0.f) : make_float2(-lq.x, -lq.y);
+        if (isp) {
+          used = true;
+          sc = r;
+        }
+        __syncwarp();  // the buffer is rewritten by the next pivot
+      }
+      // this lane: row i = q_sl of S^{-1}; register x holds the stored column (x + M) mod NMAX,
+      // which is column p_c of the inverse.  X = S^{-1} F, row i.
+      const int row = sl < M ? sq[sl] : 0;
+      float2 x[NMAX];
+#pragma unroll
+      for (int c = 0; c < NMAX; ++c) x[c] = z2();
+#pragma unroll
+      for (int y = 0; y < NMAX; ++y) {
+        int c = y + M;
+        if (c >= NMAX) c -= NMAX;
+        if (c < M) {
+          const float2 g = fmul(sc, a[y]);
+          const int pc = sp[c];
+          if (sl < M) Sm[row * NMAX + pc] = g;
+          const float4* f4 = reinterpret_cast<const float4*>(Fm + pc * NMAX);
+#pragma unroll
+          for (int z = 0; z < NMAX; z += 2) {
+            const float4 v = f4[z / 2];
+            fmac(x[z], g, make_float2(v.x, v.y));
+            fmac(x[z + 1], g, make_float2(v.z, v.w));
+          }
+        }
+      }
+      __syncwarp();  // every lane is done with F
+      if (sl < M) {
+#pragma unroll
+        for (int z = 0; z < NMAX; z += 2)
+          *reinterpret_cast<float4*>(Fm + row * NMAX + z) = make_float4(x[z].x, x[z].y, x[z + 1].x, x[z + 1].y);
+      }
+      __syncwarp();
+      if (valid && sl < M) {
+        tr += Fm[row * NMAX + row].x;
+#pragma unroll
+        for (int z = 0; z < NMAX; ++z)
+          if (z < M) {
+            const float2 y = Fm[z * NMAX + row];
+            g2 = __fmaf_rn(x[z].x, y.x, __fmaf_rn(-x[z].y, y.y, g2));
+          }
+      }
+      __syncwarp();
+    }
+    // 2 Tr(S^{-1} B D^3 B^+)
+    for (int pr = lane; pr < NP; pr += 32) {
+      const int a = pair[pr].x, c = pair[pr].y;
+      float2 xr[FW], xi[FW];
+#pragma unroll
+      for (int f = 0; f < FW; ++f) xr[f] = xi[f] = z2();
+      const float2* t = Ts + pr;
+#pragma unroll 4
+      for (int b = 0; b < n2; ++b) {
+        const float2 tv = __ldg(t + (size_t)b * NP);
+        const float4* d4 = reinterpret_cast<const float4*>(sd3 + b * FW);
+#pragma unroll
+        for (int f = 0; f < FW; f += 2) {
+          const float4 d = d4[f / 2];
+          xr[f].x = __fmaf_rn(tv.x, d.x, xr[f].x);
+          xr[f].y = __fmaf_rn(tv.y, d.x, xr[f].y);
+          xi[f].x = __fmaf_rn(tv.x, d.y, xi[f].x);
+          xi[f].y = __fmaf_rn(tv.y, d.y, xi[f].y);
+          xr[f + 1].x = __fmaf_rn(tv.x, d.z, xr[f + 1].x);
+          xr[f + 1].y = __fmaf_rn(tv.y, d.z, xr[f + 1].y);
+          xi[f + 1].x = __fmaf_rn(tv.x, d.w, xi[f + 1].x);
+          xi[f + 1].y = __fmaf_rn(tv.y, d.w, xi[f + 1].y);
+        }
+      }
+#pragma unroll
+      for (int f = 0; f < FW; ++f) {
+        if (n + f >= n1) continue;
+        const float2* Sm = sS + f * M * NMAX;
+        const float2 g1 = Sm[a * NMAX + c];
+        const float z2x = xr[f].x + xi[f].y, z2y = xi[f].x - xr[f].y;  // (c, a)
+        float s = __fmaf_rn(g1.x, z2x, -__fmul_rn(g1.y, z2y));
+        if (a != c) {
+          const float2 gt = Sm[c * NMAX + a];
+          const float z1x = xr[f].x - xi[f].y, z1y = xr[f].y + xi[f].x;  // (a, c)
+          s = __fmaf_rn(gt.x, z1x, __fmaf_rn(-gt.y, z1y, s));
+        }
+        g2 = __fmaf_rn(2.f, s, g2);
+      }
+    }
+    __syncwarp();  // d, S and F are rewritten by the next batch
+    acc_tr += (double)tr;
+    acc_g2 += (double)g2;
+  }
+  // deterministic: xor tree in each warp, then the warps in order
+  for (int off = 16; off; off >>= 1) {
+    acc_tr += __shfl_xor_sync(0xffffffffu, acc_tr, off);
+    acc_g2 += __shfl_xor_sync(0xffffffffu, acc_g2, off);
+  }
+  if (lane == 0) {
+    s_part[wp][0] = acc_tr;
+    s_part[wp][1] = acc_g2;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    double t = 0.0, u = 0.0;
+    for (int w = 0; w < kBlkWarps; ++w) {
+      t += s_part[w][0];
+      u += s_part[w][1];
+    }
+    double* o = p.occ_part + ((int64_t)kk * p.n_chunks + bl.chunk0 + ch) * 2;
+    o[0] = t;
+    o[1] = u;
+  }
+}
+
+// Shapes by the number of orbitals: columns (registers) per row, lanes per matrix, frequencies
+// per warp.
+struct Shape32 {
+  int nmax, lw, fw;
+};
+__host__ Shape32 shape32(int m) {
+  if (m <= 8) return {8, 8, 4};
+  if (m <= 12) return {12, 16, 4};
+  if (m <= 16) return {16, 16, 4};
+  if (m <= 20) return {20, 32, 2};
+  if (m <= 24) return {24, 32, 2};
+  return {32, 32, 2};
+}
+
+template <int NMAX, int LW, int FW>
+cudaError_t launch32(const PointParams& p, const BlockForm& b, const BlockLaunch& l, size_t smem, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(k_occ_block32<NMAX, LW, FW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
+  if (e != cudaSuccess) return e;
+  k_occ_block32<NMAX, LW, FW><<<l.n_units * l.n_chunks, 32 * kBlkWarps, smem, s>>>(p, b, l);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+int block32_batch(int mmax) { return kBlkWarps * shape32(mmax).fw; }
+
+size_t block32_smem(int mmax, int n2max) {
+  const Shape32 sh = shape32(mmax);
+  return make_layout32(mmax, n2max, sh.nmax, sh.lw, sh.fw).bytes;
+}
+
+cudaError_t launch_occ_block32(const PointParams& p, const BlockForm& b, const BlockLaunch& l, cudaStream_t s) {
+  const size_t smem = block32_smem(p.mmax, l.n2max);
+  switch (shape32(p.mmax).nmax) {
+    case 8: return launch32<8, 8, 4>(p, b, l, smem, s);
+    case 12: return launch32<12, 16, 4>(p, b, l, smem, s);
+    case 16: return launch32<16, 16, 4>(p, b, l, smem, s);
+    case 20: return launch32<20, 32, 2>(p, b, l, smem, s);
+    case 24: return launch32<24, 32, 2>(p, b, l, smem, s);
+    default: return launch32<32, 32, 2>(p, b, l, smem, s);
+  }
+}
+
+}  // namespace gf

@@ -133,7 +133,7 @@ def test_mixed_block_kernels_against_fp64(nk, nb, m, n_iw):
     s = _inputs(nk, nb, m, n_iw, 100.0, nb)
     a, log = _run(s, None, precision="mixed")
     b, _ = _run(s, "direct")
-    assert "with FP32 traces" in log
+    assert "in FP32 (traces, rho)" in log
     tol = {"N": 1e-7, "occ": 1e-7, "gloc": 1e-8, "loc": 1e-8, "rho": 1e-5, "dm": 1e-5, "dN_dmu": 1e-5, "docc": 1e-5,
            "n_corr": 1e-6, "dm_nc": 1e-6}
     for key in b:
