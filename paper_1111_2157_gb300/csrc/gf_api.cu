@@ -193,9 +193,9 @@ gf_status rho_partials(gf_ctx* c, int* n_chunks) {
   if (!c->lowrank && !c->run_on_block) return GF_OK;
   GF_CU(ensure(c->lr_T, sizeof(double2) * c->totH));
   if (c->run_on_block) {
-    GF_CU(gf::launch_block_rotate(c->kinfo_d.as<KInfo>(), c->n_k, c->blk_U.as<double2>(), c->rho_part.as<double2>(),
+    GF_CU(gf::launch_block_rotate(c->kinfo_d.as<KInfo>(), c->n_k, c->nbmax, c->blk_U.as<double2>(), c->rho_part.as<double2>(),
                                   c->totH, c->run_chunks, c->lr_T.as<double2>(), c->stream));
-    c->last_launches += 1;
+    c->last_launches += 2;
     *n_chunks = 1;
     return GF_OK;
   }

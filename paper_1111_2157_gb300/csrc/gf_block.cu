@@ -315,14 +315,10 @@ __device__ __forceinline__ double2 to_rest(double2 v, double2) { return v; }
 __device__ __forceinline__ float2 to_rest(double2 v, float2) { return make_float2((float)v.x, (float)v.y); }
 __device__ __forceinline__ void rmac(double2& a, double2 x, double2 y) { cmac(a, x, y); }
 __device__ __forceinline__ void rmac(float2& a, float2 x, float2 y) { fmac(a, x, y); }
-__device__ __forceinline__ void rmac_ca(double2& a, double2 x, double2 y) { cmac_ca(a, x, y); }
-__device__ __forceinline__ void rmac_ca(float2& a, float2 x, float2 y) { fmac_ca(a, x, y); }
 __device__ __forceinline__ double2 rzero(double2) { return make_double2(0.0, 0.0); }
 __device__ __forceinline__ float2 rzero(float2) { return make_float2(0.f, 0.f); }
 __device__ __forceinline__ double rfma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double2 rmul(double2 a, double2 b) { return cmul(a, b); }
-__device__ __forceinline__ float2 rmul(float2 a, float2 b) { return fmul(a, b); }
 
 // 1 / a with one division: scaled by a power of two near 1 / max(|Re|, |Im|) (bit arithmetic),
 // so that the squared modulus neither overflows nor underflows.
@@ -336,10 +332,10 @@ __device__ __forceinline__ double2 crcp_scaled(double2 a, unsigned long long key
 }
 
 // Shared memory of the point kernel in bytes: per warp S (then S^{-1}), F, d / d^2 / d^3, the
-// pivot row and column, Gbar A^+ (adjoint) and the pivot tables, for F frequencies; per CTA
-// the pair list and the columns S^{-1} B D of rho_k.
+// pivot row and column, Gbar A^+ (adjoint), S^{-1} in FP32 (LOW) and the pivot tables, for F
+// frequencies; per CTA the pair list and the columns S^{-1} B D of rho_k.
 struct LayoutB {
-  size_t wS, wF, wd, wd2, wrc, wM, wp, wstride, oPair, oY, bytes;
+  size_t wS, wF, wd, wd2, wrc, wM, wG, wp, wstride, oPair, oY, bytes;
   int nf;   // frequencies per warp
   int yf;   // frequencies of the rho_k columns staged at once
 };
@@ -359,6 +355,7 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   L.wd2 = o; o = al(o + (needF ? 2 * r * f * n2max : 0));
   L.wrc = o; o += 16 * f * 2 * mmax;
   L.wM = o; o += (mode & kAdj) ? 16 * f * mm : 0;
+  L.wG = o; o = al(o + (low ? 8 * f * mm : 0));
   L.wp = o; o = al(o + 4 * f * 2 * mmax);
   L.wstride = o;
   o *= kBlkWarps;
@@ -366,9 +363,13 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   L.oY = o;
   L.yf = 0;
   if (mode & kRho) {
+    // as many frequencies as leave three CTAs on an SM, else two: the chunk's sum is read and
+    // written once per stage (40.9 -> 33 ms on the NiO-like mixed pass against a stage of 64 KB)
     const size_t one = r * (size_t)mmax * n2max;
-    const size_t fit = (48u << 10) / one;
-    L.yf = fit < 1 ? 1 : (fit > f * kBlkWarps ? (int)(f * kBlkWarps) : (int)fit);
+    const size_t lim = o + one <= (74u << 10) ? (74u << 10) : (112u << 10);
+    const size_t fit = o + one <= lim ? (lim - o) / one : 1;
+    const size_t all = f * kBlkWarps, stages = fit < all ? (all + fit - 1) / fit : 1;
+    L.yf = (int)((all + stages - 1) / stages);
     o = al(o + one * L.yf);
   }
   L.bytes = o;
@@ -447,6 +448,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4)
   double2* sd = reinterpret_cast<double2*>(wb + L.wd);
   rc_t* sd2 = reinterpret_cast<rc_t*>(wb + L.wd2);
   double2* sM = reinterpret_cast<double2*>(wb + L.wM);
+  float2* sG = reinterpret_cast<float2*>(wb + L.wG);
   uchar2* pair = reinterpret_cast<uchar2*>(smraw + L.oPair);
   rc_t* sY = reinterpret_cast<rc_t*>(smraw + L.oY);
   const int unit = bl.unit0 + blockIdx.x / bl.n_chunks, ch = blockIdx.x % bl.n_chunks;
@@ -569,20 +571,54 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4)
         }
         __syncwarp();
         block_invert<LW>(A, M, rcb, sp, sl, p.status);
+        const int* sq = sp + M;
+        const bool mine = mf < nv;
+        double2* out = (p.mode & (kGloc | kAdj))
+                           ? p.gq + ((int64_t)(unit - p.gb0) * p.n_iw + min(n + mf, n1 - 1)) * p.mmax * p.mmax
+                           : nullptr;
+        if constexpr (LOW) {
+          // FP32 copy in the orbitals' order: one conversion per entry (it runs on the FP64 pipe)
+          for (int i = sl; i < MM; i += LW) {
+            const int a = i / M, c = i - a * M;
+            const double2 g = A[sp[a] * M + sq[c]];
+            sG[mf * MM + i] = make_float2((float)g.x, (float)g.y);
+            if ((p.mode & kGloc) && mine) gq_put(&out[i], q, make_double2(wk * g.x, wk * g.y));
+          }
+          __syncwarp();
+        } else if ((p.mode & kGloc) && mine) {
+          for (int i = sl; i < MM; i += LW) {
+            const int a = i / M, c = i - a * M;
+            const double2 g = A[sp[a] * M + sq[c]];
+            gq_put(&out[i], q, make_double2(wk * g.x, wk * g.y));
+          }
+        }
         if (occ) {
+          float low_tr = 0.f, low_g2 = 0.f;  // LOW: this lane's sums over the warp's frequencies
           for (int i = lane; i < F * NP; i += 32) {
             const int f = i / NP, pr = i - f * NP;
             const int a = pair[pr].x, c = pair[pr].y;
-            const int* pf = reinterpret_cast<const int*>(wb + L.wp) + f * 2 * M;
-            const int* qf = pf + M;
-            const double2* Af = sS + f * MM;
             const rc_t* Fm = sF + f * MM;
-            const int pa = pf[a] * M, pc = pf[c] * M;
-            rc_t x1 = rzero(rc_t{}), x2 = x1;
-            for (int j = 0; j < M; ++j) {
-              const int fj = pf[j] * M;
-              rmac(x1, to_rest(Af[pa + j], rc_t{}), Fm[fj + c]);
-              if (a != c) rmac(x2, to_rest(Af[pc + j], rc_t{}), Fm[fj + a]);
+            rc_t x1 = rzero(rc_t{}), x2 = x1, g1, g2;
+            if constexpr (LOW) {
+              const float2* Gf = sG + f * MM;
+              for (int j = 0; j < M; ++j) {
+                rmac(x1, Gf[a * M + j], Fm[j * M + c]);
+                rmac(x2, Gf[c * M + j], Fm[j * M + a]);
+              }
+              g1 = Gf[a * M + c];
+              g2 = Gf[c * M + a];
+            } else {
+              const int* pf = reinterpret_cast<const int*>(wb + L.wp) + f * 2 * M;
+              const int* qf = pf + M;
+              const double2* Af = sS + f * MM;
+              const int pa = pf[a] * M, pc = pf[c] * M;
+              for (int j = 0; j < M; ++j) {
+                const int fj = pf[j] * M;
+                rmac(x1, Af[pa + j], Fm[fj + c]);
+                if (a != c) rmac(x2, Af[pc + j], Fm[fj + a]);
+              }
+              g1 = Af[pa + qf[c]];
+              g2 = Af[pc + qf[a]];
             }
             rc_t zr = rzero(rc_t{}), zi = zr;
             const rc_t* d3f = sd2 + F * n2 + f * n2;
@@ -606,36 +642,28 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4)
             }
             if (f < nv) {
               // Tr X^2 and 2 Tr(S^{-1} B D^3 B^+): the pair's (a, c) and (c, a) terms
-              const rc_t g1 = to_rest(Af[pa + qf[c]], rc_t{}), g2 = to_rest(Af[pc + qf[a]], rc_t{});
               const rr_t z1x = zr.x - zi.y, z1y = zr.y + zi.x;  // (a, c)
               const rr_t z2x = zr.x + zi.y, z2y = zi.x - zr.y;  // (c, a)
+              const rr_t xx = a == c ? rfma(x1.x, x1.x, -x1.y * x1.y)
+                                     : rr_t(2) * rfma(x1.x, x2.x, -x1.y * x2.y);
               rr_t s = rfma(g1.x, z2x, -g1.y * z2y);
-              if (a == c) {
-                acc_tr += (double)x1.x;
-                s = rfma(rr_t(2), s, rfma(x1.x, x1.x, -x1.y * x1.y));
+              if (a != c) s = rfma(g2.x, z1x, rfma(-g2.y, z1y, s));
+              s = rfma(rr_t(2), s, xx);
+              if constexpr (LOW) {
+                if (a == c) low_tr += x1.x;
+                low_g2 += s;
               } else {
-                s = rfma(g2.x, z1x, rfma(-g2.y, z1y, s));
-                s = rr_t(2) * (s + rfma(x1.x, x2.x, -x1.y * x2.y));
+                if (a == c) acc_tr += x1.x;
+                acc_g2 += s;
+                if (have_gbar) acc_mu += cb * wk * xx;
               }
-              acc_g2 += (double)s;
-              if (have_gbar) acc_mu += cb * wk * (double)((a == c ? rr_t(1) : rr_t(2)) *
-                                                          (a == c ? rfma(x1.x, x1.x, -x1.y * x1.y)
-                                                                  : rfma(x1.x, x2.x, -x1.y * x2.y)));
             }
           }
-          __syncwarp();
-        }
-        const int* sq = sp + M;
-        const bool mine = mf < nv;
-        double2* out = (p.mode & (kGloc | kAdj))
-                           ? p.gq + ((int64_t)(unit - p.gb0) * p.n_iw + min(n + mf, n1 - 1)) * p.mmax * p.mmax
-                           : nullptr;
-        if ((p.mode & kGloc) && mine) {
-          for (int i = sl; i < MM; i += LW) {
-            const int a = i / M, c = i - a * M;
-            const double2 g = A[sp[a] * M + sq[c]];
-            gq_put(&out[i], q, make_double2(wk * g.x, wk * g.y));
+          if constexpr (LOW) {
+            acc_tr += (double)low_tr;
+            acc_g2 += (double)low_g2;
           }
+          __syncwarp();
         }
         if constexpr (!LOW) {
           if (adj) {
@@ -685,28 +713,23 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4)
         // frequencies at a time, then the blocks of G are added to the chunk's sum
         const int nb = ki.nb, tot = min(W * F, n1 - base);
         double2* Sk = p.rho_part + (int64_t)chunk * p.rho_chunk_stride + ki.offH;
-        const rc_t* Bk;
-        if constexpr (LOW) Bk = bf.Bs + ki.offP;
-        else Bk = bf.B + ki.offP;
-        auto mat = [&](int f) { return reinterpret_cast<const double2*>(smraw + (size_t)(f / F) * L.wstride + L.wS) + (f % F) * MM; };
-        auto piv = [&](int f) { return reinterpret_cast<const int*>(smraw + (size_t)(f / F) * L.wstride + L.wp) + (f % F) * 2 * M; };
-        auto dof = [&](int f) { return reinterpret_cast<const double2*>(smraw + (size_t)(f / F) * L.wstride + L.wd) + (f % F) * n2; };
+        auto region = [&](int f) { return smraw + (size_t)(f / F) * L.wstride; };
+        auto mat = [&](int f) { return reinterpret_cast<const double2*>(region(f) + L.wS) + (f % F) * MM; };
+        auto piv = [&](int f) { return reinterpret_cast<const int*>(region(f) + L.wp) + (f % F) * 2 * M; };
+        auto dof = [&](int f) { return reinterpret_cast<const double2*>(region(f) + L.wd) + (f % F) * n2; };
         const bool first = (base == n0);
         __syncthreads();
         for (int f0 = 0; f0 < tot; f0 += L.yf) {
           const int nf = min(L.yf, tot - f0);
           const bool put = first && f0 == 0;
-          auto add = [&](int at, double2 v) {
-            if (!put) {
-              const double2 o = Sk[at];
-              v.x += o.x;
-              v.y += o.y;
-            }
-            Sk[at] = v;
-          };
+          // the chunk's sum: the old values are loaded before a thread's products and added after
+          // them, so that the L2 latency passes under the arithmetic
+          auto old = [&](int at) { return put ? make_double2(0.0, 0.0) : Sk[at]; };
+          auto add = [&](int at, double2 o, double2 v) { Sk[at] = make_double2(o.x + v.x, o.y + v.y); };
           // (1,1) block
           for (int i = tid; i < MM; i += 32 * W) {
             const int a = i / M, c = i - a * M;
+            const double2 o = old(a * nb + c);
             double2 v = make_double2(0.0, 0.0);
             for (int f = f0; f < f0 + nf; ++f) {
               const int* pf = piv(f);
@@ -714,54 +737,156 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4)
               v.x += g.x;
               v.y += g.y;
             }
-            add(a * nb + c, v);
+            add(a * nb + c, o, v);
           }
-          // (1,2) and (2,1): Y = S^{-1} B D, Z = D B^+ S^{-1}
-          for (int i = tid; i < M * n2; i += 32 * W) {
-            const int a = i / n2, bb = i - a * n2;
-            double2 v12 = make_double2(0.0, 0.0), v21 = v12;
-            for (int f = f0; f < f0 + nf; ++f) {
-              const int* pf = piv(f);
-              const int* qf = pf + M;
-              const double2* Af = mat(f);
-              rc_t y = rzero(rc_t{}), z = y;
-              const int pa = pf[a] * M, qa = qf[a];
-              for (int x = 0; x < M; ++x) {
-                const int xx = pf[x];  // orbital of column x; also the row of orbital x
-                rmac(y, to_rest(Af[pa + x], rc_t{}), ld_cg(Bk + xx * n2 + bb));
-                rmac_ca(z, ld_cg(Bk + x * n2 + bb), to_rest(Af[xx * M + qa], rc_t{}));
+          if constexpr (LOW) {
+            // FP32 products in register tiles, summed over the nf frequencies in FP32 and added
+            // to the chunk's FP64 sum once
+            auto matf = [&](int f) { return reinterpret_cast<const float2*>(region(f) + L.wG) + (f % F) * MM; };
+            const float2* Bk = bf.Bs + ki.offP;
+            // (1,2) and (2,1): Y = S^{-1} B D, Z = D B^+ S^{-1}; four orbitals per thread
+            const int at4 = (M + 3) / 4;
+            for (int i = tid; i < at4 * n2; i += 32 * W) {
+              const int a0 = (i / n2) * 4, bb = i - (i / n2) * n2;
+              float2 v12[4], v21[4];
+              double2 o12[4], o21[4];
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const int a = min(a0 + u, M - 1);
+                v12[u] = v21[u] = make_float2(0.f, 0.f);
+                o12[u] = old(a * nb + M + bb);
+                o21[u] = old((M + bb) * nb + a);
               }
-              const rc_t d = to_rest(dof(f)[bb], rc_t{});
-              y = rmul(y, d);
-              z = rmul(z, d);
-              sY[(size_t)(f - f0) * M * n2 + i] = y;
-              v12.x += (double)y.x; v12.y += (double)y.y;
-              v21.x += (double)z.x; v21.y += (double)z.y;
+              for (int f = f0; f < f0 + nf; ++f) {
+                const float2* Gf = matf(f);
+                float2 y[4], z[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) y[u] = z[u] = make_float2(0.f, 0.f);
+                for (int x = 0; x < M; ++x) {
+                  const float2 b = ld_cg(Bk + x * n2 + bb);
+#pragma unroll
+                  for (int u = 0; u < 4; ++u) {
+                    const int a = min(a0 + u, M - 1);
+                    fmac(y[u], Gf[a * M + x], b);
+                    fmac_ca(z[u], b, Gf[x * M + a]);
+                  }
+                }
+                const double2 dd = dof(f)[bb];
+                const float2 d = make_float2((float)dd.x, (float)dd.y);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  const float2 yd = fmul(y[u], d), zd = fmul(z[u], d);
+                  if (a0 + u < M) sY[(size_t)((f - f0) * M + a0 + u) * n2 + bb] = yd;
+                  v12[u].x += yd.x; v12[u].y += yd.y;
+                  v21[u].x += zd.x; v21[u].y += zd.y;
+                }
+              }
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+                if (a0 + u < M) {
+                  add((a0 + u) * nb + M + bb, o12[u], make_double2(v12[u].x, v12[u].y));
+                  add((M + bb) * nb + a0 + u, o21[u], make_double2(v21[u].x, v21[u].y));
+                }
             }
-            add(a * nb + M + bb, v12);
-            add((M + bb) * nb + a, v21);
-          }
-          __syncthreads();
-          // (2,2): d_b (delta_bc + sum_a conj(B_ab) Y_ac)
-          for (int i = tid; i < n2 * n2; i += 32 * W) {
-            const int bb = i / n2, c = i - bb * n2;
-            double2 v = make_double2(0.0, 0.0);
-            for (int f = f0; f < f0 + nf; ++f) {
-              rc_t w = rzero(rc_t{});
-              const rc_t* Y = sY + (size_t)(f - f0) * M * n2 + c;
-              for (int a = 0; a < M; ++a) rmac_ca(w, ld_cg(Bk + a * n2 + bb), Y[a * n2]);
-              const double2 d = dof(f)[bb];
-              w = rmul(w, to_rest(d, rc_t{}));
-              v.x += (double)w.x;
-              v.y += (double)w.y;
-              if (bb == c) {
-                v.x += d.x;
-                v.y += d.y;
+            __syncthreads();
+            // (2,2): d_b (delta_bc + sum_a conj(B_ab) Y_ac); four rows and two columns per thread
+            const int bt = (n2 + 3) / 4, ct = (n2 + 1) / 2;
+            for (int i = tid; i < bt * ct; i += 32 * W) {
+              const int b0 = (i / ct) * 4, c0 = i - (i / ct) * ct, c1 = min(c0 + ct, n2 - 1);
+              float2 v[4][2];
+              double2 o[4][2];
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const int at = (M + min(b0 + u, n2 - 1)) * nb + M;
+                v[u][0] = v[u][1] = make_float2(0.f, 0.f);
+                o[u][0] = old(at + c0);
+                o[u][1] = old(at + c1);
+              }
+              for (int f = f0; f < f0 + nf; ++f) {
+                float2 w[4][2];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) w[u][0] = w[u][1] = make_float2(0.f, 0.f);
+                const float2* Y = sY + (size_t)(f - f0) * M * n2;
+                for (int a = 0; a < M; ++a) {
+                  const float2 y0 = Y[a * n2 + c0], y1 = Y[a * n2 + c1];
+#pragma unroll
+                  for (int u = 0; u < 4; ++u) {
+                    const float2 b = ld_cg(Bk + a * n2 + min(b0 + u, n2 - 1));
+                    fmac_ca(w[u][0], b, y0);
+                    fmac_ca(w[u][1], b, y1);
+                  }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  const double2 dd = dof(f)[min(b0 + u, n2 - 1)];
+                  const float2 d = make_float2((float)dd.x, (float)dd.y);
+                  fmac(v[u][0], d, w[u][0]);
+                  fmac(v[u][1], d, w[u][1]);
+                }
+              }
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const int bb = b0 + u;
+                if (bb >= n2) break;
+                double2 s0 = make_double2(v[u][0].x, v[u][0].y), s1 = make_double2(v[u][1].x, v[u][1].y);
+                if (bb == c0 || bb == c1)
+                  for (int f = f0; f < f0 + nf; ++f) {
+                    const double2 d = dof(f)[bb];
+                    double2& s = bb == c0 ? s0 : s1;
+                    s.x += d.x;
+                    s.y += d.y;
+                  }
+                add((M + bb) * nb + M + c0, o[u][0], s0);
+                if (c0 + ct < n2) add((M + bb) * nb + M + c1, o[u][1], s1);
               }
             }
-            add((M + bb) * nb + M + c, v);
+            __syncthreads();
+          } else {
+            const double2* Bk = bf.B + ki.offP;
+            // (1,2) and (2,1): Y = S^{-1} B D, Z = D B^+ S^{-1}
+            for (int i = tid; i < M * n2; i += 32 * W) {
+              const int a = i / n2, bb = i - a * n2;
+              const double2 o12 = old(a * nb + M + bb), o21 = old((M + bb) * nb + a);
+              double2 v12 = make_double2(0.0, 0.0), v21 = v12;
+              for (int f = f0; f < f0 + nf; ++f) {
+                const int* pf = piv(f);
+                const int* qf = pf + M;
+                const double2* Af = mat(f);
+                double2 y = make_double2(0.0, 0.0), z = y;
+                const int pa = pf[a] * M, qa = qf[a];
+                for (int x = 0; x < M; ++x) {
+                  const int xx = pf[x];  // orbital of column x; also the row of orbital x
+                  cmac(y, Af[pa + x], ld_cg(Bk + xx * n2 + bb));
+                  cmac_ca(z, ld_cg(Bk + x * n2 + bb), Af[xx * M + qa]);
+                }
+                const double2 d = dof(f)[bb];
+                y = cmul(y, d);
+                z = cmul(z, d);
+                sY[(size_t)(f - f0) * M * n2 + i] = y;
+                v12.x += y.x; v12.y += y.y;
+                v21.x += z.x; v21.y += z.y;
+              }
+              add(a * nb + M + bb, o12, v12);
+              add((M + bb) * nb + a, o21, v21);
+            }
+            __syncthreads();
+            // (2,2): d_b (delta_bc + sum_a conj(B_ab) Y_ac)
+            for (int i = tid; i < n2 * n2; i += 32 * W) {
+              const int bb = i / n2, c = i - bb * n2;
+              const double2 o = old((M + bb) * nb + M + c);
+              double2 v = make_double2(0.0, 0.0);
+              for (int f = f0; f < f0 + nf; ++f) {
+                double2 w = make_double2(0.0, 0.0);
+                const double2* Y = sY + (size_t)(f - f0) * M * n2 + c;
+                for (int a = 0; a < M; ++a) cmac_ca(w, ld_cg(Bk + a * n2 + bb), Y[a * n2]);
+                const double2 d = dof(f)[bb];
+                if (bb == c) w.x += 1.0;
+                cmac(v, d, w);
+              }
+              add((M + bb) * nb + M + c, o, v);
+            }
+            __syncthreads();
           }
-          __syncthreads();
         }
       }
     }
@@ -791,38 +916,49 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4)
   }
 }
 
-// rho_part chunk 0 <- U (sum_c S_c) U^+ (one CTA per k): the chunks are summed once, then two
-// products.
+// rho_part chunk 0 <- U (sum_c S_c) U^+ in two launches over (k, block of rows), so that a few
+// k-points fill the chip: T = (sum_c S_c) U^+ (a row of T needs its row of S alone), then U T.
+constexpr int kRotRows = 16;
 __global__ void __launch_bounds__(kSetupThreads)
-    k_block_rotate(const KInfo* __restrict__ kinfo, const double2* __restrict__ U, double2* rho_part,
-                   int64_t stride, int n_chunks, double2* T) {
+    k_block_rotate1(const KInfo* __restrict__ kinfo, const double2* __restrict__ U,
+                    const double2* __restrict__ rho_part, int64_t stride, int n_chunks, double2* __restrict__ T) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  double2* sS = reinterpret_cast<double2*>(smraw);  // kRotRows x N
   const KInfo ki = kinfo[blockIdx.x];
-  const int N = ki.nb;
+  const int N = ki.nb, r0 = blockIdx.y * kRotRows, nr = min(kRotRows, N - r0);
+  if (nr <= 0) return;
   const double2* Uk = U + ki.offH;
-  double2* S0 = rho_part + ki.offH;
-  double2* Tk = T + ki.offH;
-  for (int e = threadIdx.x; e < N * N; e += kSetupThreads) {
-    double2 s = S0[e];
+  for (int e = threadIdx.x; e < nr * N; e += kSetupThreads) {
+    const int64_t at = ki.offH + (int64_t)r0 * N + e;
+    double2 s = rho_part[at];
     for (int c = 1; c < n_chunks; ++c) {
-      const double2 v = rho_part[(int64_t)c * stride + ki.offH + e];
+      const double2 v = rho_part[(int64_t)c * stride + at];
       s.x += v.x;
       s.y += v.y;
     }
-    S0[e] = s;
+    sS[e] = s;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < N * N; e += kSetupThreads) {
+  for (int e = threadIdx.x; e < nr * N; e += kSetupThreads) {
     const int i = e / N, j = e - i * N;
     double2 acc = make_double2(0.0, 0.0);
-    for (int l = 0; l < N; ++l) cmac_cb(acc, S0[i * N + l], Uk[j * N + l]);
-    Tk[e] = acc;
+    for (int l = 0; l < N; ++l) cmac_cb(acc, sS[i * N + l], Uk[j * N + l]);
+    T[ki.offH + (int64_t)r0 * N + e] = acc;
   }
-  __syncthreads();
-  for (int e = threadIdx.x; e < N * N; e += kSetupThreads) {
-    const int i = e / N, j = e - i * N;
+}
+
+__global__ void __launch_bounds__(kSetupThreads)
+    k_block_rotate2(const KInfo* __restrict__ kinfo, const double2* __restrict__ U,
+                    const double2* __restrict__ T, double2* __restrict__ out) {
+  const KInfo ki = kinfo[blockIdx.x];
+  const int N = ki.nb, r0 = blockIdx.y * kRotRows, nr = min(kRotRows, N - r0);
+  const double2* Uk = U + ki.offH;
+  const double2* Tk = T + ki.offH;
+  for (int e = threadIdx.x; e < nr * N; e += kSetupThreads) {
+    const int i = r0 + e / N, j = e % N;
     double2 acc = make_double2(0.0, 0.0);
     for (int l = 0; l < N; ++l) cmac(acc, Uk[i * N + l], Tk[l * N + j]);
-    S0[e] = acc;
+    out[ki.offH + i * N + j] = acc;
   }
 }
 
@@ -891,9 +1027,15 @@ cudaError_t launch_point_block(const PointParams& p, const BlockForm& b, const B
   }
 }
 
-cudaError_t launch_block_rotate(const KInfo* kinfo, int n_k, const double2* U, double2* rho_part,
+cudaError_t launch_block_rotate(const KInfo* kinfo, int n_k, int nbmax, const double2* U, double2* rho_part,
                                 int64_t stride, int n_chunks, double2* T, cudaStream_t s) {
-  k_block_rotate<<<n_k, kSetupThreads, 0, s>>>(kinfo, U, rho_part, stride, n_chunks, T);
+  const dim3 grid(n_k, (nbmax + kRotRows - 1) / kRotRows);
+  const size_t smem = sizeof(double2) * kRotRows * nbmax;
+  cudaError_t e = cudaFuncSetAttribute(k_block_rotate1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_block_rotate1<<<grid, kSetupThreads, smem, s>>>(kinfo, U, rho_part, stride, n_chunks, T);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  k_block_rotate2<<<grid, kSetupThreads, 0, s>>>(kinfo, U, T, rho_part);
   return cudaGetLastError();
 }
 

@@ -93,7 +93,7 @@ int block32_batch(int mmax);
 size_t block32_smem(int mmax, int n2max);
 cudaError_t launch_occ_block32(const PointParams& p, const BlockForm& b, const BlockLaunch& l, cudaStream_t s);
 // rho_part chunk 0 <- U (sum_c S_c) U^+ for every k; T: scratch of the size of H.
-cudaError_t launch_block_rotate(const KInfo* kinfo, int n_k, const double2* U, double2* rho_part,
+cudaError_t launch_block_rotate(const KInfo* kinfo, int n_k, int nbmax, const double2* U, double2* rho_part,
                                 int64_t stride, int n_chunks, double2* T, cudaStream_t s);
 
 }  // namespace gf
