@@ -104,6 +104,8 @@ gf_status ensure_block(gf_ctx* c) {
               {&c->blk_U, 16 * (size_t)c->totH},     {&c->blk_D22, 16 * (size_t)c->totH},
               {&c->blk_V, 16 * (size_t)c->totP},     {&c->blk_R, 16 * mm * c->n_k},
               {&c->blk_H11, 16 * mm * c->n_k},       {&c->blk_tau, 8 * (size_t)c->mmax * c->n_k},
+              {&c->blk_C, 16 * (size_t)c->blk_totC}, {&c->blk_Cs, mixed ? 8 * (size_t)c->blk_totC : 0},
+              {&c->blk_ser, 8 * ((size_t)gf::kBlkSeries + 2) * c->n_k},
               {&c->blk_ws, 16 * ws},                 {&c->blk_info, 8 * ((size_t)c->n_k + 1)}};
   for (auto& n : need) {
     if (ensure(*n.b, n.bytes) == cudaSuccess) continue;
@@ -137,6 +139,10 @@ gf_status ensure_block(gf_ctx* c) {
   b.Bs = mixed ? c->blk_Bs.as<float2>() : nullptr;
   b.HO = c->blk_HO.as<double2>();
   b.U = c->blk_U.as<double2>();
+  b.C = c->blk_C.as<double2>();
+  b.Cs = mixed ? c->blk_Cs.as<float2>() : nullptr;
+  b.offC = c->blk_offT.as<int64_t>() + c->n_k;
+  b.series = c->blk_ser.as<double>();
   b.ws = c->blk_ws.as<double2>();
   b.hnorm = c->blk_info.as<double>();
   b.flags = reinterpret_cast<int*>(b.hnorm + c->n_k);
@@ -144,7 +150,7 @@ gf_status ensure_block(gf_ctx* c) {
   GF_CU(gf::launch_block_reduce(b, c->smem_optin, c->sm_count, c->stream));
   GF_CU(gf::launch_block_eig(b, c->blk_ws.as<double2>(), grid, in_smem, c->stream));
   GF_CU(gf::launch_block_finish(b, c->stream));
-  c->last_launches += 3;
+  c->last_launches += 4;
   std::vector<double> info((size_t)c->n_k + 1);
   GF_CU(cudaMemcpyAsync(info.data(), c->blk_info.p, 8 * info.size(), cudaMemcpyDeviceToHost, c->stream));
   GF_CU(cudaStreamSynchronize(c->stream));
@@ -529,6 +535,11 @@ gf_status run_block(gf_ctx* c, int mode, gf::PointParams p) {
   b.Bs = c->blk_Bs.as<float2>();
   b.HO = c->blk_HO.as<double2>();
   b.npmax = c->mmax * (c->mmax + 1) / 2;
+  b.C = c->blk_C.as<double2>();
+  b.Cs = c->blk_Cs.as<float2>();
+  b.offC = c->blk_offT.as<int64_t>() + c->n_k;
+  b.tau = c->blk_ser.as<double>();
+  b.cr = reinterpret_cast<const double2*>(b.tau + (size_t)gf::kBlkSeries * c->n_k);
   gf::BlockLaunch l{};
   l.n2max = c->blk_n2max;
   l.chunk_w = c->blk_cw;
@@ -1092,13 +1103,17 @@ gf_status init_ctx(gf_ctx* c, const gf_desc* d) {
   // block form: every window wider than its orbitals, one lane per orbital, eigenproblems within
   // the Jacobi kernel's size, and enough frequencies to pay for the eigenproblem per k
   c->blk_shape = c->n_iw >= kBlkMinFreq;
-  std::vector<int64_t> offT(c->n_k);
+  std::vector<int64_t> offT(2 * (size_t)c->n_k);  // of T, then of C
   for (int k = 0; k < c->n_k; ++k) {
     const int m = c->msys[c->ksys[k]], n2 = c->nb[k] - m;
     if (n2 < 1 || n2 > gf::heev_max_n() || m > gf::kBlkMaxM) c->blk_shape = false;
     c->blk_n2max = std::max(c->blk_n2max, n2);
     offT[k] = c->blk_totT;
-    if (n2 > 0) c->blk_totT += (int64_t)n2 * m * (m + 1) / 2;
+    offT[(size_t)c->n_k + k] = c->blk_totC;
+    if (n2 > 0) {
+      c->blk_totT += (int64_t)n2 * m * (m + 1) / 2;
+      c->blk_totC += (int64_t)std::min(n2, gf::kBlkSeries) * m * (m + 1) / 2;
+    }
   }
   for (int s = 0; s < c->n_sys; ++s)
     if (M_PI / c->beta[s] < kBlkMinW) c->blk_shape = false;
@@ -1298,7 +1313,7 @@ gf_status gf_destroy(gf_ctx* c) {
                     &c->pole_part, &c->pole_vs, &c->pole_es, &c->voff_d, &c->mu_prev,
                     &c->blk_units, &c->blk_perm, &c->blk_sysg, &c->blk_offT, &c->blk_e, &c->blk_T, &c->blk_Ts,
                     &c->blk_B, &c->blk_Bs, &c->blk_HO, &c->blk_U, &c->blk_D22, &c->blk_V, &c->blk_R, &c->blk_H11,
-                    &c->blk_tau, &c->blk_ws, &c->blk_info};
+                    &c->blk_tau, &c->blk_ws, &c->blk_info, &c->blk_C, &c->blk_Cs, &c->blk_ser};
   for (DevBuf* b : bufs) release(*b);
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
   if (c->occ_exec) cudaGraphExecDestroy(c->occ_exec);

@@ -299,6 +299,66 @@ __global__ void __launch_bounds__(kSetupThreads) k_block_finish(const BlockSetup
   }
 }
 
+// Chebyshev moments of one k-point per CTA: C_j by pairs and tau_j.
+__global__ void __launch_bounds__(kSetupThreads) k_block_series(const BlockSetup b) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  double* Tj = reinterpret_cast<double*>(smraw);  // [jt][n2]
+  __shared__ double s_cr[2];
+  const int k = blockIdx.x;
+  const KInfo ki = b.kinfo[k];
+  const int M = b.sinfo[ki.sys].m, n2 = ki.nb - M, np = M * (M + 1) / 2, jt = min(n2, kBlkSeries);
+  const int tid = threadIdx.x;
+  const double* e = b.e + b.offD[k];
+  if (tid < 32) {
+    double lo = INFINITY, hi = -INFINITY;
+    for (int l = tid; l < n2; l += 32) {
+      lo = fmin(lo, e[l]);
+      hi = fmax(hi, e[l]);
+    }
+    for (int off = 16; off; off >>= 1) {
+      lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, off));
+      hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, off));
+    }
+    if (tid == 0) {
+      s_cr[0] = 0.5 * (lo + hi);
+      s_cr[1] = fmax(0.5 * (hi - lo), 1e-3);
+      double* cr = b.series + (size_t)kBlkSeries * b.n_k + 2 * (size_t)k;
+      cr[0] = s_cr[0];
+      cr[1] = s_cr[1];
+    }
+  }
+  __syncthreads();
+  for (int l = tid; l < n2; l += kSetupThreads) {
+    const double x = (e[l] - s_cr[0]) / s_cr[1];
+    double t0 = 1.0, t1 = x;
+    for (int j = 0; j < jt; ++j) {
+      Tj[j * n2 + l] = t0;
+      const double t2 = fma(2.0 * x, t1, -t0);
+      t0 = t1;
+      t1 = t2;
+    }
+  }
+  __syncthreads();
+  for (int j = tid; j < jt; j += kSetupThreads) {
+    double s = 0.0;
+    for (int l = 0; l < n2; ++l) s += Tj[j * n2 + l];
+    b.series[(size_t)kBlkSeries * k + j] = s;
+  }
+  const double2* T = b.T + b.offT[k];
+  for (int i = tid; i < jt * np; i += kSetupThreads) {
+    const int j = i / np, pr = i - j * np;
+    double2 v = make_double2(0.0, 0.0);
+    for (int l = 0; l < n2; ++l) {
+      const double2 t = T[(size_t)l * np + pr];
+      const double c = Tj[j * n2 + l];
+      v.x = fma(c, t.x, v.x);
+      v.y = fma(c, t.y, v.y);
+    }
+    b.C[b.offC[k] + i] = v;
+    if (b.Cs) b.Cs[b.offC[k] + i] = make_float2((float)v.x, (float)v.y);
+  }
+}
+
 // ------------------------------------------------------------------ point kernel
 
 template <bool LOW>
@@ -331,11 +391,66 @@ __device__ __forceinline__ double2 crcp_scaled(double2 a, unsigned long long key
   return make_double2(x * q, -y * q);
 }
 
+// Coefficients of the Chebyshev series at z (x = (z - c) / r, s = sqrt(x^2 - 1), xi = x - s):
+//   1/(z - e)   = sum_j eps_j xi^j / (r s) T_j,                                eps_0 = 1, eps_j = 2
+//   1/(z - e)^2 = sum_j eps_j xi^j [j/s^2 + x/s^3] / r^2 T_j                    (-d/dz)
+//   1/(z - e)^3 = sum_j eps_j xi^j [(j^2 - 1)/s^3 + 3 j x/s^4 + 3 x^2/s^5] / (2 r^3) T_j
+// The j-independent factors of one frequency:
+struct SeriesZ {
+  double2 xi, c1, c2a, c2b, c3a, c3b, c3c;  // c1; c2a j + c2b; c3a (j^2 - 1) + c3b j + c3c
+};
+__device__ __forceinline__ SeriesZ series_z(double dx, double w, double r, bool powers) {
+  SeriesZ q;
+  const double ir = 1.0 / r;
+  const double2 x = make_double2(dx * ir, w * ir);
+  // s = sqrt(x^2 - 1) with Im s > 0: from |u| and the larger component first
+  const double2 u = make_double2(fma(x.x, x.x, -fma(x.y, x.y, 1.0)), 2.0 * x.x * x.y);
+  const double au = sqrt(fma(u.x, u.x, u.y * u.y));
+  const double p = sqrt(0.5 * (au + fabs(u.x)));
+  const double h = 0.5 * u.y / p;
+  double2 s = u.x >= 0.0 ? make_double2(p, h) : make_double2(h, p);
+  if (s.y < 0.0 || (s.y == 0.0 && x.x < 0.0)) s = make_double2(-s.x, -s.y);
+  q.xi = crcp_scaled(make_double2(x.x + s.x, x.y + s.y), pivot_key(make_double2(x.x + s.x, x.y + s.y)));
+  const double2 is = crcp_scaled(s, pivot_key(s));
+  q.c1 = make_double2(is.x * ir, is.y * ir);
+  if (powers) {
+    q.c2a = cmul(q.c1, make_double2(is.x * ir, is.y * ir));                  // 1 / (s^2 r^2)
+    const double2 t = cmul(x, is);                                           // x / s
+    q.c2b = cmul(q.c2a, t);                                                  // x / (s^3 r^2)
+    const double g = 0.5 * ir;
+    const double2 is2 = make_double2(is.x * g, is.y * g);
+    q.c3a = cmul(q.c2a, is2);                                                // 1 / (2 s^3 r^3)
+    q.c3b = cmul(q.c2b, make_double2(3.0 * is2.x, 3.0 * is2.y));             // 3 x / (2 s^4 r^3)
+    q.c3c = cmul(q.c3b, t);                                                  // 3 x^2 / (2 s^5 r^3)
+  }
+  return q;
+}
+__device__ __forceinline__ double2 cpow_int(double2 b, int j) {
+  double2 v = make_double2(1.0, 0.0);
+#pragma unroll
+  for (int t = 0; t < 6; ++t) {  // j < 64
+    if ((j >> t) & 1) v = cmul(v, b);
+    b = cmul(b, b);
+  }
+  return v;
+}
+// Terms of the series that leave a remainder of 2^-56 times a margin for the j^2 of the third
+// powers, for every frequency from w on (FP32: only the count depends on it).
+__device__ __forceinline__ int series_terms(float dx, float w, float r, float bits) {
+  const float xr = dx / r, xi = w / r;
+  const float ur = xr * xr - xi * xi - 1.f, ui = 2.f * xr * xi, au = sqrtf(ur * ur + ui * ui);
+  const float p = sqrtf(0.5f * (au + fabsf(ur))), h = p > 0.f ? 0.5f * fabsf(ui) / p : 0.f;
+  const float sr = ur >= 0.f ? p : h, si = ur >= 0.f ? h : p;
+  const float R = sqrtf((fabsf(xr) + sr) * (fabsf(xr) + sr) + (fabsf(xi) + si) * (fabsf(xi) + si));
+  const float lr = logf(R);
+  return lr > 0.02f ? (int)(bits / lr) + 2 : 1 << 20;
+}
+
 // Shared memory of the point kernel in bytes: per warp S (then S^{-1}), F, d / d^2 / d^3, the
 // pivot row and column, Gbar A^+ (adjoint), S^{-1} in FP32 (LOW) and the pivot tables, for F
 // frequencies; per CTA the pair list and the columns S^{-1} B D of rho_k.
 struct LayoutB {
-  size_t wS, wF, wd, wd2, wrc, wM, wG, wp, wstride, oPair, oY, bytes;
+  size_t wS, wF, wd, wdc, wd2, wrc, wM, wG, wp, wstride, oPair, oY, bytes;
   int nf;   // frequencies per warp
   int yf;   // frequencies of the rho_k columns staged at once
 };
@@ -352,6 +467,9 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   L.wS = o; o += 16 * f * mm;
   L.wF = o; o = al(o + (needF ? r * f * mm : 0));
   L.wd = o; o += 16 * f * n2max;
+  // rho_k reads d_b also where the sums run over Chebyshev moments
+  L.wdc = (mode & kRho) ? o : L.wd;
+  o += (mode & kRho) ? 16 * f * (n2max < kBlkSeries ? n2max : kBlkSeries) : 0;
   L.wd2 = o; o = al(o + (needF ? 2 * r * f * n2max : 0));
   L.wrc = o; o += 16 * f * 2 * mmax;
   L.wM = o; o += (mode & kAdj) ? 16 * f * mm : 0;
@@ -432,7 +550,7 @@ __device__ __forceinline__ void block_invert(double2* A, int M, double2* rc, int
 }
 
 template <int LW, bool LOW>
-__global__ void __launch_bounds__(32 * kBlkWarps, 4)
+__global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
     k_point_block(const PointParams p, const BlockForm bf, const BlockLaunch bl) {
   using rc_t = typename Rest<LOW>::c;
   using rr_t = typename Rest<LOW>::r;
@@ -484,21 +602,101 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4)
       const int nv = min(F, n1 - n);  // frequencies of this warp (<= 0: none)
       if (nv > 0) {
         __syncwarp();
-        for (int i = lane; i < F * n2; i += 32) {
-          const int f = i / n2, bb = i - f * n2;
-          const double wn = (2.0 * min(n + f, n1 - 1) + 1.0) * pib;
-          const double x = mu - e_k[bb];
-          const double s = 1.0 / fma(x, x, wn * wn);
-          const double2 d = make_double2(x * s, -wn * s);
-          sd[i] = d;
-          if (occ || adj) {
-            const double2 d2 = cmul(d, d);
-            sd2[i] = to_rest(d2, rc_t{});
-            if (occ) {
-              sd2[F * n2 + i] = to_rest(cmul(d2, d), rc_t{});
-              if (f < nv) {
-                acc_tr += d.x;
-                acc_g2 += d2.x;
+        // the sums over the n2 bands, or over fewer Chebyshev moments where those converge sooner
+        // (the series' own overhead is about 150 FP64 instructions per warp)
+        int nt = n2;
+        const double2* Tt = T;
+        const float2* Tst = nullptr;
+        if constexpr (LOW) Tst = bf.Ts + bf.offT[kk];
+        double2* dv = sd;
+        {
+          const double2 cr = bf.cr[kk];
+          const int J = series_terms((float)(mu - cr.x), (float)((2.0 * n + 1.0) * pib), (float)cr.y, 44.8f);
+          const int sums = LOW ? 1 : (occ ? 3 : (adj ? 2 : 1));  // FP64 sums
+          if (J <= min(n2, kBlkSeries) && (n2 - J) * NP * F * sums > 1600) {
+            nt = J;
+            Tt = bf.C + bf.offC[kk];
+            if constexpr (LOW) Tst = bf.Cs + bf.offC[kk];
+            dv = reinterpret_cast<double2*>(wb + L.wdc);
+            const double* tau = bf.tau + (size_t)kBlkSeries * kk;
+            int fz = -1;
+            SeriesZ z;
+            float2 zf[5];
+            for (int i = lane; i < F * J; i += 32) {
+              const int f = i / J, j = i - f * J;
+              if (f != fz) {
+                z = series_z(mu - cr.x, (2.0 * min(n + f, n1 - 1) + 1.0) * pib, cr.y, occ || adj);
+                fz = f;
+                if constexpr (LOW) {
+                  zf[0] = to_rest(z.c2a, float2{});
+                  zf[1] = to_rest(z.c2b, float2{});
+                  zf[2] = to_rest(z.c3a, float2{});
+                  zf[3] = to_rest(z.c3b, float2{});
+                  zf[4] = to_rest(z.c3c, float2{});
+                }
+              }
+              double2 pw = cpow_int(z.xi, j);
+              if (j) pw = make_double2(2.0 * pw.x, 2.0 * pw.y);
+              const double2 d = cmul(pw, z.c1);
+              dv[i] = d;
+              if constexpr (LOW) {
+                if (occ) {
+                  const float2 pf = make_float2((float)pw.x, (float)pw.y);
+                  const float fj = (float)j, j2 = fj * fj - 1.f;
+                  const float2 d2 = fmul(pf, make_float2(fmaf(fj, zf[0].x, zf[1].x), fmaf(fj, zf[0].y, zf[1].y)));
+                  sd2[i] = d2;
+                  sd2[F * n2 + i] = fmul(pf, make_float2(fmaf(j2, zf[2].x, fmaf(fj, zf[3].x, zf[4].x)),
+                                                         fmaf(j2, zf[2].y, fmaf(fj, zf[3].y, zf[4].y))));
+                  if (f < nv) {
+                    acc_tr = fma(tau[j], d.x, acc_tr);
+                    acc_g2 = fma(tau[j], (double)d2.x, acc_g2);
+                  }
+                }
+              } else if (occ || adj) {
+                const double fj = j;
+                const double2 d2 = cmul(pw, make_double2(fma(fj, z.c2a.x, z.c2b.x), fma(fj, z.c2a.y, z.c2b.y)));
+                sd2[i] = d2;
+                if (occ) {
+                  const double j2 = fma(fj, fj, -1.0);
+                  sd2[F * n2 + i] = cmul(pw, make_double2(fma(j2, z.c3a.x, fma(fj, z.c3b.x, z.c3c.x)),
+                                                          fma(j2, z.c3a.y, fma(fj, z.c3b.y, z.c3c.y))));
+                  if (f < nv) {
+                    acc_tr = fma(tau[j], d.x, acc_tr);
+                    acc_g2 = fma(tau[j], d2.x, acc_g2);
+                  }
+                }
+              }
+            }
+          }
+        }
+        if (nt == n2 || rho) {
+          const bool sums = nt == n2;
+          for (int i = lane; i < F * n2; i += 32) {
+            const int f = i / n2, bb = i - f * n2;
+            const double wn = (2.0 * min(n + f, n1 - 1) + 1.0) * pib;
+            const double x = mu - e_k[bb];
+            const double s = 1.0 / fma(x, x, wn * wn);
+            const double2 d = make_double2(x * s, -wn * s);
+            sd[i] = d;
+            if constexpr (LOW) {
+              if (sums && occ) {
+                const float2 df = make_float2((float)d.x, (float)d.y), d2 = fmul(df, df);
+                sd2[i] = d2;
+                sd2[F * n2 + i] = fmul(d2, df);
+                if (f < nv) {
+                  acc_tr += d.x;
+                  acc_g2 += (double)d2.x;
+                }
+              }
+            } else if (sums && (occ || adj)) {
+              const double2 d2 = cmul(d, d);
+              sd2[i] = d2;
+              if (occ) {
+                sd2[F * n2 + i] = cmul(d2, d);
+                if (f < nv) {
+                  acc_tr += d.x;
+                  acc_g2 += d2.x;
+                }
               }
             }
           }
@@ -510,16 +708,16 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4)
           const int f = i / NP, pr = i - f * NP;
           const int a = pair[pr].x, c = pair[pr].y;
           const int nn = min(n + f, n1 - 1);
-          const double2* t = T + pr;
-          const double2* df = sd + f * n2;
+          const double2* t = Tt + pr;
+          const double2* df = dv + f * nt;
           double2 xr = make_double2(0.0, 0.0), xi = xr;
           rc_t yr = rzero(rc_t{}), yi = yr;
           if (occ || adj) {
-            const rc_t* d2f = sd2 + f * n2;
+            const rc_t* d2f = sd2 + f * nt;
             if constexpr (LOW) {
-              const float2* ts = bf.Ts + bf.offT[kk] + pr;
+              const float2* ts = Tst + pr;
 #pragma unroll 4
-              for (int bb = 0; bb < n2; ++bb) {
+              for (int bb = 0; bb < nt; ++bb) {
                 const double2 tv = ld_cg(t + (size_t)bb * NP), d = df[bb];
                 const float2 tf = ld_cg(ts + (size_t)bb * NP), d2 = d2f[bb];
                 xr.x = fma(tv.x, d.x, xr.x); xr.y = fma(tv.y, d.x, xr.y);
@@ -529,7 +727,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4)
               }
             } else {
 #pragma unroll 4
-              for (int bb = 0; bb < n2; ++bb) {
+              for (int bb = 0; bb < nt; ++bb) {
                 const double2 tv = ld_cg(t + (size_t)bb * NP), d = df[bb];
                 const rc_t d2 = d2f[bb];
                 xr.x = fma(tv.x, d.x, xr.x); xr.y = fma(tv.y, d.x, xr.y);
@@ -549,7 +747,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4)
             if (a != c) Fm[c * M + a] = v;
           } else {
 #pragma unroll 4
-            for (int bb = 0; bb < n2; ++bb) {
+            for (int bb = 0; bb < nt; ++bb) {
               const double2 tv = ld_cg(t + (size_t)bb * NP), d = df[bb];
               xr.x = fma(tv.x, d.x, xr.x); xr.y = fma(tv.y, d.x, xr.y);
               xi.x = fma(tv.x, d.y, xi.x); xi.y = fma(tv.y, d.y, xi.y);
@@ -621,19 +819,19 @@ __global__ void __launch_bounds__(32 * kBlkWarps, 4)
               g2 = Af[pc + qf[a]];
             }
             rc_t zr = rzero(rc_t{}), zi = zr;
-            const rc_t* d3f = sd2 + F * n2 + f * n2;
+            const rc_t* d3f = sd2 + F * n2 + f * nt;
             if constexpr (LOW) {
-              const float2* ts = bf.Ts + bf.offT[kk] + pr;
+              const float2* ts = Tst + pr;
 #pragma unroll 4
-              for (int bb = 0; bb < n2; ++bb) {
+              for (int bb = 0; bb < nt; ++bb) {
                 const float2 tv = ld_cg(ts + (size_t)bb * NP), d = d3f[bb];
                 zr.x = rfma(tv.x, d.x, zr.x); zr.y = rfma(tv.y, d.x, zr.y);
                 zi.x = rfma(tv.x, d.y, zi.x); zi.y = rfma(tv.y, d.y, zi.y);
               }
             } else {
-              const double2* t = T + pr;
+              const double2* t = Tt + pr;
 #pragma unroll 4
-              for (int bb = 0; bb < n2; ++bb) {
+              for (int bb = 0; bb < nt; ++bb) {
                 const double2 tv = ld_cg(t + (size_t)bb * NP);
                 const rc_t d = d3f[bb];
                 zr.x = rfma(tv.x, d.x, zr.x); zr.y = rfma(tv.y, d.x, zr.y);
@@ -1003,10 +1201,15 @@ cudaError_t launch_block_reduce(const BlockSetup& b, int smem_optin, int sm_coun
 }
 
 cudaError_t launch_block_finish(const BlockSetup& b, cudaStream_t s) {
+  const size_t ser = sizeof(double) * kBlkSeries * (size_t)b.n2max;
   const size_t smem = sizeof(double2) * (2 * (size_t)b.mmax * b.mmax + (size_t)b.mmax * b.n2max);
   cudaError_t e = cudaFuncSetAttribute(k_block_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   k_block_finish<<<b.n_k, kSetupThreads, smem, s>>>(b);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_block_series, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ser);
+  if (e != cudaSuccess) return e;
+  k_block_series<<<b.n_k, kSetupThreads, ser, s>>>(b);
   return cudaGetLastError();
 }
 

@@ -34,7 +34,16 @@ struct BlockForm {
   const float2* Bs;
   const double2* HO;      // [2][np] per k at k * 2 * npmax: H11 pairs, then O pairs
   int npmax;
+  // Chebyshev moments of the n2 block: with e_b in [c - r, c + r] and x_b = (e_b - c) / r,
+  // sum_b t_b / (z - e_b)^p = sum_j a_j^(p)(z) C_j, C_j = sum_b t_b T_j(x_b), whose terms fall
+  // off like R^-j, R the sum of the half axes of the ellipse with foci c -+ r through z.
+  const double2* C;       // [min(n2, kBlkSeries)][np] at offC[k]
+  const float2* Cs;       // its FP32 rounding (GF_PREC_MIXED) or null
+  const int64_t* offC;
+  const double* tau;      // [kBlkSeries] per k: sum_b T_j(x_b)
+  const double2* cr;      // (c, r) per k
 };
+constexpr int kBlkSeries = 40;  // moments kept
 
 // One launch over units (k-points, or k-groups for the k-reductions) x frequency chunks.
 struct BlockLaunch {
@@ -47,8 +56,8 @@ struct BlockLaunch {
   int n2max;
 };
 
-// Setup, three launches over the k-points: reduction (QR, Q^+ H Q), eigenpairs of the n2
-// block, and the tables above.  flags (device int): kBlkNonHermitian, kBlkRankDeficient,
+// Setup over the k-points: reduction (QR, Q^+ H Q), eigenpairs of the n2 block, and the
+// tables above.  flags (device int): kBlkNonHermitian, kBlkRankDeficient,
 // kBlkNoConvergence; hnorm (device, n_k): ||H_k||_F / sqrt(N_b).
 constexpr int kBlkNonHermitian = 1, kBlkRankDeficient = 2, kBlkNoConvergence = 4;
 struct BlockSetup {
@@ -71,13 +80,17 @@ struct BlockSetup {
   float2* Bs;
   double2* HO;
   double2* U;             // [N_b][N_b] at offH
+  double2* C;             // Chebyshev moments, as in BlockForm
+  float2* Cs;
+  const int64_t* offC;
+  double* series;         // tau, then (c, r) pairs
   double2* ws;            // per-CTA slices of nbmax^2 elements when the matrix exceeds shared memory
   int* flags;
   double* hnorm;
 };
 cudaError_t launch_block_reduce(const BlockSetup& b, int smem_optin, int sm_count, cudaStream_t s);
 cudaError_t launch_block_eig(const BlockSetup& b, double2* ws, int grid, int in_smem, cudaStream_t s);
-cudaError_t launch_block_finish(const BlockSetup& b, cudaStream_t s);
+cudaError_t launch_block_finish(const BlockSetup& b, cudaStream_t s);  // (two kernels)
 size_t block_reduce_ws_elems(int nbmax, int mmax, int smem_optin, int sm_count);
 
 // Frequencies a CTA takes at once.

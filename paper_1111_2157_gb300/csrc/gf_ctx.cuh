@@ -174,13 +174,13 @@ struct gf_ctx {
   int blk_nc = 0;                             // mixed precision: frequencies below it run in FP64
   std::vector<int> blk_sys_g0, blk_sys_g1;    // groups of each system
   int blk_groups = 0;
-  int64_t blk_totT = 0;
+  int64_t blk_totT = 0, blk_totC = 0;
   int run_chunks = 1;                         // the current call: chunks of its partial sums,
   bool run_on_block = false;                  // and whether it runs on the block form
   int occ_path = 0;                           // path that the captured N(mu) graph holds
-  DevBuf blk_units, blk_perm, blk_sysg, blk_offT;
+  DevBuf blk_units, blk_perm, blk_sysg, blk_offT;  // (blk_offT: offsets of T, then of C)
   DevBuf blk_e, blk_T, blk_Ts, blk_B, blk_Bs, blk_HO, blk_U, blk_D22, blk_V, blk_R, blk_H11, blk_tau,
-      blk_ws, blk_info;
+      blk_ws, blk_info, blk_C, blk_Cs, blk_ser;
   // DMFT step and projector construction
   DevBuf eimp, eimp_part, gl_in, delta, wraw, vdc;
   // pole form of Sigma (gf_set_sigma_poles) and the pseudo-Hamiltonian path
