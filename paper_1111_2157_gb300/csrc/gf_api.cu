@@ -188,7 +188,8 @@ bool use_block(const gf_ctx* c, int mode) {
                                     : gf::point_fp64_smem(c->nbmax, c->mmax, mode, 0);
   if (general > limit || (c->lowrank && c->nbmax > gf::heev_max_n())) return false;
   return gf::block_smem(c->mmax, c->blk_n2max, mode, 0) <= limit &&
-         (c->precision != GF_PREC_MIXED || gf::block32_smem(c->mmax, c->blk_n2max) <= limit);
+         (c->precision != GF_PREC_MIXED || (gf::block_smem(c->mmax, c->blk_n2max, mode, 1) <= limit &&
+                                            gf::block32_smem(c->mmax, c->blk_n2max) <= limit));
 }
 
 // rho_k partial sums: the low-rank and the block kernels leave them in the basis that makes

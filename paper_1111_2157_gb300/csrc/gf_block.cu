@@ -16,6 +16,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "gf_block.cuh"
 #include "gf_complex.cuh"
@@ -446,11 +447,14 @@ __device__ __forceinline__ int series_terms(float dx, float w, float r, float bi
   return lr > 0.02f ? (int)(bits / lr) + 2 : 1 << 20;
 }
 
-// Shared memory of the point kernel in bytes: per warp S (then S^{-1}), F, d / d^2 / d^3, the
-// pivot row and column, Gbar A^+ (adjoint), S^{-1} in FP32 (LOW) and the pivot tables, for F
-// frequencies; per CTA the pair list and the columns S^{-1} B D of rho_k.
+// Shared memory of the point kernel in bytes; every array holds the CTA's W F frequencies, warp
+// after warp.  First what is dead once the warps have S^{-1}: F, d^2 / d^3, the pivot row and
+// column, Gbar A^+ (adjoint), and with LOW also S (rho_k then reads the FP32 copy of S^{-1});
+// the columns S^{-1} B D of rho_k are staged over it, yf frequencies at a time.  Then S, the
+// copy, d (and the series coefficients), the pivot tables, the pair list and, with LOW, B.
 struct LayoutB {
-  size_t wS, wF, wd, wdc, wd2, wrc, wM, wG, wp, wstride, oPair, oY, bytes;
+  size_t oS, oF, od2, orc, oM, oY, oG, od, odc, op, oPair, oB, bytes;
+  size_t sS, sF, sd2, src, sG, sd, sdc, sp;  // bytes per warp (sS also of M)
   int nf;   // frequencies per warp
   int yf;   // frequencies of the rho_k columns staged at once
 };
@@ -460,36 +464,51 @@ __host__ __device__ inline int block_lanes(int m) { return m <= 8 ? 8 : (m <= 16
 __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, int low) {
   LayoutB L;
   L.nf = 32 / block_lanes(mmax);
-  const size_t f = L.nf, mm = (size_t)mmax * mmax, r = low ? 8 : 16;
-  const bool needF = (mode & (kOcc | kAdj)) != 0;
+  const size_t f = L.nf, mm = (size_t)mmax * mmax, r = low ? 8 : 16, W = kBlkWarps;
+  const bool needF = (mode & (kOcc | kAdj)) != 0, rho = (mode & kRho) != 0;
   auto al = [](size_t x) { return (x + 15) & ~(size_t)15; };
+  const size_t jt = n2max < kBlkSeries ? n2max : kBlkSeries;
+  L.sS = 16 * f * mm;
+  L.sF = needF ? al(r * f * mm) : 0;
+  L.sd2 = needF ? al(2 * r * f * n2max) : 0;
+  L.src = 16 * f * 2 * mmax;
+  L.sG = low ? al(8 * f * mm) : 0;
+  L.sd = 16 * f * n2max;
+  L.sdc = rho ? 16 * f * jt : 0;  // rho_k reads d_b also where the sums run over the moments
+  L.sp = al(4 * f * 2 * mmax);
   size_t o = 0;
-  L.wS = o; o += 16 * f * mm;
-  L.wF = o; o = al(o + (needF ? r * f * mm : 0));
-  L.wd = o; o += 16 * f * n2max;
-  // rho_k reads d_b also where the sums run over Chebyshev moments
-  L.wdc = (mode & kRho) ? o : L.wd;
-  o += (mode & kRho) ? 16 * f * (n2max < kBlkSeries ? n2max : kBlkSeries) : 0;
-  L.wd2 = o; o = al(o + (needF ? 2 * r * f * n2max : 0));
-  L.wrc = o; o += 16 * f * 2 * mmax;
-  L.wM = o; o += (mode & kAdj) ? 16 * f * mm : 0;
-  L.wG = o; o = al(o + (low ? 8 * f * mm : 0));
-  L.wp = o; o = al(o + 4 * f * 2 * mmax);
-  L.wstride = o;
-  o *= kBlkWarps;
-  L.oPair = o; o = al(o + 2 * (size_t)mmax * (mmax + 1) / 2);
+  if (!low) { L.oS = o; o += W * L.sS; }
   L.oY = o;
+  if (low) { L.oS = o; o += W * L.sS; }
+  L.oF = o; o += W * L.sF;
+  L.od2 = o; o += W * L.sd2;
+  L.orc = o; o += W * L.src;
+  L.oM = o; o += (mode & kAdj) ? W * L.sS : 0;
+  const size_t fixed = W * (L.sG + L.sd + L.sdc + L.sp) + al((size_t)mmax * (mmax + 1)) +
+                       (low && rho ? 8 * mmax * (((size_t)n2max + 3) & ~(size_t)3) : 0);
   L.yf = 0;
-  if (mode & kRho) {
-    // as many frequencies as leave three CTAs on an SM, else two: the chunk's sum is read and
-    // written once per stage (40.9 -> 33 ms on the NiO-like mixed pass against a stage of 64 KB)
-    const size_t one = r * (size_t)mmax * n2max;
-    const size_t lim = o + one <= (74u << 10) ? (74u << 10) : (112u << 10);
-    const size_t fit = o + one <= lim ? (lim - o) / one : 1;
-    const size_t all = f * kBlkWarps, stages = fit < all ? (all + fit - 1) / fit : 1;
+  if (rho) {
+    // as many frequencies as fit over the dead arrays, or as leave three CTAs on an SM, or two:
+    // the chunk's sum is read and written once per stage
+    const size_t one = mmax * (low ? 8 * (((size_t)n2max + 3) & ~(size_t)3) : 16 * (size_t)n2max);
+    const size_t all = f * W;
+    size_t room = o - L.oY;
+    for (size_t lim = 74u << 10; lim <= (112u << 10); lim += 38u << 10)
+      if (room < all * one && L.oY + fixed + (room > one ? room : one) <= lim) {
+        room = lim - L.oY - fixed;
+        break;
+      }
+    const size_t fit = room >= one ? room / one : 1, stages = fit < all ? (all + fit - 1) / fit : 1;
     L.yf = (int)((all + stages - 1) / stages);
-    o = al(o + one * L.yf);
+    if (L.oY + one * L.yf > o) o = al(L.oY + one * L.yf);
   }
+  L.oG = o; o += W * L.sG;
+  L.od = o; o += W * L.sd;
+  L.odc = rho ? o : L.od;
+  o += W * L.sdc;
+  L.op = o; o += W * L.sp;
+  L.oPair = o; o += al((size_t)mmax * (mmax + 1));
+  L.oB = o; o += low && rho ? 8 * mmax * (((size_t)n2max + 3) & ~(size_t)3) : 0;
   L.bytes = o;
   return L;
 }
@@ -560,15 +579,14 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
   constexpr int W = kBlkWarps;
   const LayoutB L = make_layout_b(p.mmax, bl.n2max, p.mode, LOW ? 1 : 0);
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5, sl = lane % LW, mf = lane / LW;
-  unsigned char* wb = smraw + (size_t)wp * L.wstride;
-  double2* sS = reinterpret_cast<double2*>(wb + L.wS);
-  rc_t* sF = reinterpret_cast<rc_t*>(wb + L.wF);
-  double2* sd = reinterpret_cast<double2*>(wb + L.wd);
-  rc_t* sd2 = reinterpret_cast<rc_t*>(wb + L.wd2);
-  double2* sM = reinterpret_cast<double2*>(wb + L.wM);
-  float2* sG = reinterpret_cast<float2*>(wb + L.wG);
+  double2* sS = reinterpret_cast<double2*>(smraw + L.oS + wp * L.sS);
+  rc_t* sF = reinterpret_cast<rc_t*>(smraw + L.oF + wp * L.sF);
+  double2* sd = reinterpret_cast<double2*>(smraw + L.od + wp * L.sd);
+  rc_t* sd2 = reinterpret_cast<rc_t*>(smraw + L.od2 + wp * L.sd2);
+  double2* sM = reinterpret_cast<double2*>(smraw + L.oM + wp * L.sS);
+  float2* sG = reinterpret_cast<float2*>(smraw + L.oG + wp * L.sG);
+  int* sPv = reinterpret_cast<int*>(smraw + L.op + wp * L.sp);
   uchar2* pair = reinterpret_cast<uchar2*>(smraw + L.oPair);
-  rc_t* sY = reinterpret_cast<rc_t*>(smraw + L.oY);
   const int unit = bl.unit0 + blockIdx.x / bl.n_chunks, ch = blockIdx.x % bl.n_chunks;
   const int2 un = bl.units[unit];
   const int n0 = bl.n_begin + ch * bl.chunk_w, n1 = min(bl.n_end, n0 + bl.chunk_w);
@@ -587,13 +605,20 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
     const double cb = (adj && p.nbar) ? p.nbar[ki.sys] * 2.0 / si.beta : 0.0;
     const bool have_gbar = adj && p.gbar != nullptr;
     double2* A = sS + mf * MM;  // this lane group's matrix
-    double2* rcb = reinterpret_cast<double2*>(wb + L.wrc) + mf * 2 * M;
-    int* sp = reinterpret_cast<int*>(wb + L.wp) + mf * 2 * M;
+    double2* rcb = reinterpret_cast<double2*>(smraw + L.orc + wp * L.src) + mf * 2 * M;
+    int* sp = sPv + mf * 2 * M;
     __syncthreads();
     for (int pr = tid; pr < NP; pr += 32 * W) {
       int a = 0, rem = pr;
       while (rem >= M - a) { rem -= M - a; ++a; }
       pair[pr] = make_uchar2((unsigned char)a, (unsigned char)(a + rem));
+    }
+    if constexpr (LOW) {
+      if (rho) {
+        float2* sB = reinterpret_cast<float2*>(smraw + L.oB);
+        const int pt = (n2 + 3) & ~3;
+        for (int i = tid; i < M * n2; i += 32 * W) sB[(i / n2) * pt + i % n2] = bf.Bs[ki.offP + i];
+      }
     }
     __syncthreads();
     double acc_tr = 0.0, acc_g2 = 0.0, acc_mu = 0.0;
@@ -617,7 +642,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             nt = J;
             Tt = bf.C + bf.offC[kk];
             if constexpr (LOW) Tst = bf.Cs + bf.offC[kk];
-            dv = reinterpret_cast<double2*>(wb + L.wdc);
+            dv = reinterpret_cast<double2*>(smraw + (rho ? L.odc + wp * L.sdc : L.od + wp * L.sd));
             const double* tau = bf.tau + (size_t)kBlkSeries * kk;
             int fz = -1;
             SeriesZ z;
@@ -806,7 +831,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
               g1 = Gf[a * M + c];
               g2 = Gf[c * M + a];
             } else {
-              const int* pf = reinterpret_cast<const int*>(wb + L.wp) + f * 2 * M;
+              const int* pf = sPv + f * 2 * M;
               const int* qf = pf + M;
               const double2* Af = sS + f * MM;
               const int pa = pf[a] * M, pc = pf[c] * M;
@@ -911,10 +936,9 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
         // frequencies at a time, then the blocks of G are added to the chunk's sum
         const int nb = ki.nb, tot = min(W * F, n1 - base);
         double2* Sk = p.rho_part + (int64_t)chunk * p.rho_chunk_stride + ki.offH;
-        auto region = [&](int f) { return smraw + (size_t)(f / F) * L.wstride; };
-        auto mat = [&](int f) { return reinterpret_cast<const double2*>(region(f) + L.wS) + (f % F) * MM; };
-        auto piv = [&](int f) { return reinterpret_cast<const int*>(region(f) + L.wp) + (f % F) * 2 * M; };
-        auto dof = [&](int f) { return reinterpret_cast<const double2*>(region(f) + L.wd) + (f % F) * n2; };
+        auto mat = [&](int f) { return reinterpret_cast<const double2*>(smraw + L.oS + (f / F) * L.sS) + (f % F) * MM; };
+        auto piv = [&](int f) { return reinterpret_cast<const int*>(smraw + L.op + (f / F) * L.sp) + (f % F) * 2 * M; };
+        auto dof = [&](int f) { return reinterpret_cast<const double2*>(smraw + L.od + (f / F) * L.sd) + (f % F) * n2; };
         const bool first = (base == n0);
         __syncthreads();
         for (int f0 = 0; f0 < tot; f0 += L.yf) {
@@ -930,8 +954,14 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             const double2 o = old(a * nb + c);
             double2 v = make_double2(0.0, 0.0);
             for (int f = f0; f < f0 + nf; ++f) {
-              const int* pf = piv(f);
-              const double2 g = mat(f)[pf[a] * M + pf[M + c]];
+              double2 g;
+              if constexpr (LOW) {
+                const float2 gf = reinterpret_cast<const float2*>(smraw + L.oG + (f / F) * L.sG)[(f % F) * MM + i];
+                g = make_double2((double)gf.x, (double)gf.y);
+              } else {
+                const int* pf = piv(f);
+                g = mat(f)[pf[a] * M + pf[M + c]];
+              }
               v.x += g.x;
               v.y += g.y;
             }
@@ -939,108 +969,148 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
           }
           if constexpr (LOW) {
             // FP32 products in register tiles, summed over the nf frequencies in FP32 and added
-            // to the chunk's FP64 sum once
-            auto matf = [&](int f) { return reinterpret_cast<const float2*>(region(f) + L.wG) + (f % F) * MM; };
-            const float2* Bk = bf.Bs + ki.offP;
-            // (1,2) and (2,1): Y = S^{-1} B D, Z = D B^+ S^{-1}; four orbitals per thread
-            const int at4 = (M + 3) / 4;
-            for (int i = tid; i < at4 * n2; i += 32 * W) {
-              const int a0 = (i / n2) * 4, bb = i - (i / n2) * n2;
-              float2 v12[4], v21[4];
-              double2 o12[4], o21[4];
+            // to the chunk's FP64 sum once (each FP64 add or conversion takes the SM 16 clocks)
+            auto matf = [&](int f) { return reinterpret_cast<const float2*>(smraw + L.oG + (f / F) * L.sG) + (f % F) * MM; };
+            const int pt = (n2 + 3) & ~3;
+            const float2* sB = reinterpret_cast<const float2*>(smraw + L.oB);
+            float2* sY = reinterpret_cast<float2*>(smraw + L.oY);  // [yf][M][pt]: S^{-1} B D
+            auto dlow = [&](int f, int b) {
+              const double2 d = dof(f)[b];
+              return make_float2((float)d.x, (float)d.y);
+            };
+            // (1,2) and (2,1): Y = S^{-1} B D, Z = D B^+ S^{-1}; four orbitals and two bands a thread
+            const int at4 = (M + 3) / 4, ct = (n2 + 1) / 2;
+            for (int i = tid; i < at4 * ct; i += 32 * W) {
+              const int a0 = (i / ct) * 4, c0 = i - (i / ct) * ct, c1 = min(c0 + ct, n2 - 1);
+              int ar[4];
 #pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                const int a = min(a0 + u, M - 1);
-                v12[u] = v21[u] = make_float2(0.f, 0.f);
-                o12[u] = old(a * nb + M + bb);
-                o21[u] = old((M + bb) * nb + a);
-              }
-              for (int f = f0; f < f0 + nf; ++f) {
-                const float2* Gf = matf(f);
-                float2 y[4], z[4];
+              for (int u = 0; u < 4; ++u) ar[u] = min(a0 + u, M - 1);
+              float2 v12[4][2], v21[4][2];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) y[u] = z[u] = make_float2(0.f, 0.f);
+              for (int u = 0; u < 4; ++u) v12[u][0] = v12[u][1] = v21[u][0] = v21[u][1] = make_float2(0.f, 0.f);
+              for (int f = 0; f < nf; ++f) {
+                const float2* Gf = matf(f0 + f);
+                float2 y[4][2], z[4][2];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) y[u][0] = y[u][1] = z[u][0] = z[u][1] = make_float2(0.f, 0.f);
                 for (int x = 0; x < M; ++x) {
-                  const float2 b = ld_cg(Bk + x * n2 + bb);
+                  const float2 b0 = sB[x * pt + c0], b1 = sB[x * pt + c1];
 #pragma unroll
                   for (int u = 0; u < 4; ++u) {
-                    const int a = min(a0 + u, M - 1);
-                    fmac(y[u], Gf[a * M + x], b);
-                    fmac_ca(z[u], b, Gf[x * M + a]);
+                    const float2 g = Gf[ar[u] * M + x], h = Gf[x * M + ar[u]];
+                    fmac(y[u][0], g, b0);
+                    fmac(y[u][1], g, b1);
+                    fmac_ca(z[u][0], b0, h);
+                    fmac_ca(z[u][1], b1, h);
                   }
                 }
-                const double2 dd = dof(f)[bb];
-                const float2 d = make_float2((float)dd.x, (float)dd.y);
+                const float2 d0 = dlow(f0 + f, c0), d1 = dlow(f0 + f, c1);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                  const float2 yd = fmul(y[u], d), zd = fmul(z[u], d);
-                  if (a0 + u < M) sY[(size_t)((f - f0) * M + a0 + u) * n2 + bb] = yd;
-                  v12[u].x += yd.x; v12[u].y += yd.y;
-                  v21[u].x += zd.x; v21[u].y += zd.y;
+                  y[u][0] = fmul(y[u][0], d0);
+                  y[u][1] = fmul(y[u][1], d1);
+                  fmac(v21[u][0], z[u][0], d0);
+                  fmac(v21[u][1], z[u][1], d1);
+                  v12[u][0].x += y[u][0].x; v12[u][0].y += y[u][0].y;
+                  v12[u][1].x += y[u][1].x; v12[u][1].y += y[u][1].y;
+                  if (a0 + u < M) {
+                    float2* Yr = sY + (size_t)(f * M + a0 + u) * pt;
+                    Yr[c0] = y[u][0];
+                    if (c0 + ct < n2) Yr[c1] = y[u][1];
+                  }
                 }
               }
 #pragma unroll
-              for (int u = 0; u < 4; ++u)
-                if (a0 + u < M) {
-                  add((a0 + u) * nb + M + bb, o12[u], make_double2(v12[u].x, v12[u].y));
-                  add((M + bb) * nb + a0 + u, o21[u], make_double2(v21[u].x, v21[u].y));
+              for (int v = 0; v < 2; ++v) {
+                const int c = v ? c1 : c0;
+                if (v && c0 + ct >= n2) break;
+                double2 o12[4], o21[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  o12[u] = old(ar[u] * nb + M + c);
+                  o21[u] = old((M + c) * nb + ar[u]);
                 }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                  if (a0 + u < M) {
+                    add(ar[u] * nb + M + c, o12[u], make_double2(v12[u][v].x, v12[u][v].y));
+                    add((M + c) * nb + ar[u], o21[u], make_double2(v21[u][v].x, v21[u][v].y));
+                  }
+              }
             }
             __syncthreads();
-            // (2,2): d_b (delta_bc + sum_a conj(B_ab) Y_ac); four rows and two columns per thread
-            const int bt = (n2 + 3) / 4, ct = (n2 + 1) / 2;
-            for (int i = tid; i < bt * ct; i += 32 * W) {
-              const int b0 = (i / ct) * 4, c0 = i - (i / ct) * ct, c1 = min(c0 + ct, n2 - 1);
-              float2 v[4][2];
-              double2 o[4][2];
+            // (2,2): D + D (B^+ Y) in tiles of four rows and CW columns
+            auto tiles = [&](auto cw) {
+              constexpr int CW = decltype(cw)::value;
+              const int ctl = (n2 + CW - 1) / CW, ntl = ((n2 + 3) / 4) * ctl;
+              for (int i = tid; i < ntl; i += 32 * W) {
+                const int b0 = (i / ctl) * 4, c0 = (i - (i / ctl) * ctl) * CW;
+                float2 v[4][CW];
 #pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                const int at = (M + min(b0 + u, n2 - 1)) * nb + M;
-                v[u][0] = v[u][1] = make_float2(0.f, 0.f);
-                o[u][0] = old(at + c0);
-                o[u][1] = old(at + c1);
-              }
-              for (int f = f0; f < f0 + nf; ++f) {
-                float2 w[4][2];
+                for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int u = 0; u < 4; ++u) w[u][0] = w[u][1] = make_float2(0.f, 0.f);
-                const float2* Y = sY + (size_t)(f - f0) * M * n2;
-                for (int a = 0; a < M; ++a) {
-                  const float2 y0 = Y[a * n2 + c0], y1 = Y[a * n2 + c1];
+                  for (int w = 0; w < CW; ++w) v[u][w] = make_float2(0.f, 0.f);
+                for (int f = 0; f < nf; ++f) {
+                  float2 t[4][CW];
+#pragma unroll
+                  for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int w = 0; w < CW; ++w) t[u][w] = make_float2(0.f, 0.f);
+#pragma unroll 2
+                  for (int a = 0; a < M; ++a) {
+                    const float4* bp = reinterpret_cast<const float4*>(sB + a * pt + b0);
+                    const float4* yp = reinterpret_cast<const float4*>(sY + (size_t)(f * M + a) * pt + c0);
+                    const float4 b01 = bp[0], b23 = bp[1];
+                    const float2 b[4] = {{b01.x, b01.y}, {b01.z, b01.w}, {b23.x, b23.y}, {b23.z, b23.w}};
+                    float2 y[CW];
+#pragma unroll
+                    for (int w = 0; w < CW; w += 2) {
+                      const float4 q4 = yp[w / 2];
+                      y[w] = make_float2(q4.x, q4.y);
+                      y[w + 1] = make_float2(q4.z, q4.w);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+#pragma unroll
+                      for (int w = 0; w < CW; ++w) fmac_ca(t[u][w], b[u], y[w]);
+                  }
 #pragma unroll
                   for (int u = 0; u < 4; ++u) {
-                    const float2 b = ld_cg(Bk + a * n2 + min(b0 + u, n2 - 1));
-                    fmac_ca(w[u][0], b, y0);
-                    fmac_ca(w[u][1], b, y1);
+                    const float2 d = dlow(f0 + f, min(b0 + u, n2 - 1));
+#pragma unroll
+                    for (int w = 0; w < CW; ++w) fmac(v[u][w], t[u][w], d);
                   }
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                  const double2 dd = dof(f)[min(b0 + u, n2 - 1)];
-                  const float2 d = make_float2((float)dd.x, (float)dd.y);
-                  fmac(v[u][0], d, w[u][0]);
-                  fmac(v[u][1], d, w[u][1]);
+                  const int bb = b0 + u;
+                  if (bb >= n2) break;
+                  const int at = (M + bb) * nb + M;
+                  double2 o[CW];
+#pragma unroll
+                  for (int w = 0; w < CW; ++w) o[w] = old(at + min(c0 + w, n2 - 1));
+#pragma unroll
+                  for (int w = 0; w < CW; ++w) {
+                    if (c0 + w >= n2) break;
+                    double2 s = make_double2(v[u][w].x, v[u][w].y);
+                    if (bb == c0 + w)
+                      for (int f = f0; f < f0 + nf; ++f) {
+                        const double2 d = dof(f)[bb];
+                        s.x += d.x;
+                        s.y += d.y;
+                      }
+                    add(at + c0 + w, o[w], s);
+                  }
                 }
               }
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                const int bb = b0 + u;
-                if (bb >= n2) break;
-                double2 s0 = make_double2(v[u][0].x, v[u][0].y), s1 = make_double2(v[u][1].x, v[u][1].y);
-                if (bb == c0 || bb == c1)
-                  for (int f = f0; f < f0 + nf; ++f) {
-                    const double2 d = dof(f)[bb];
-                    double2& s = bb == c0 ? s0 : s1;
-                    s.x += d.x;
-                    s.y += d.y;
-                  }
-                add((M + bb) * nb + M + c0, o[u][0], s0);
-                if (c0 + ct < n2) add((M + bb) * nb + M + c1, o[u][1], s1);
-              }
-            }
+            };
+            // the wide tile only where it still gives every thread one
+            if (n2 > 40) tiles(std::integral_constant<int, 4>{});
+            else tiles(std::integral_constant<int, 2>{});
             __syncthreads();
           } else {
             const double2* Bk = bf.B + ki.offP;
+            double2* sY = reinterpret_cast<double2*>(smraw + L.oY);
             // (1,2) and (2,1): Y = S^{-1} B D, Z = D B^+ S^{-1}
             for (int i = tid; i < M * n2; i += 32 * W) {
               const int a = i / n2, bb = i - a * n2;
