@@ -57,7 +57,7 @@ typedef enum {
     GF_ENOMEM = 2,     /* device or host allocation failed                         */
     GF_ECUDA = 3,      /* a CUDA runtime call failed (message in gf_last_error)    */
     GF_ESINGULAR = 4,  /* a zero or non-finite pivot in some (k, i w_n) inverse    */
-    GF_ENOTCONV = 5,   /* a mu search missed tol in max_iter, or Jacobi its sweep cap */
+    GF_ENOTCONV = 5,   /* a mu search missed tol in max_iter, or an eigensolver its cap  */
     GF_ETIMEOUT = 6,   /* a bounded wait of the tensor-core kernel on its MMAs gave up */
     GF_ESTATE = 7      /* inputs missing (e.g. gf_local before gf_set_sigma)        */
 } gf_status;
@@ -238,7 +238,8 @@ gf_status gf_occupation_static(const void *h_dev, const void *p_dev, const void 
  * The pole energies enter shifted by mu because Sigma is a function of i w
  * (the reading the Matsubara path uses too), so each mu diagonalises H_ps
  * again: one (N_b + n_poles)-square Hermitian eigenproblem per k, solved by
- * the library's batched Jacobi kernel (N_b + n_poles <= 256). */
+ * the library (Householder tridiagonalisation and the eigenpairs of that;
+ * N_b + n_poles <= 256). */
 
 /* Pole form of Sigma per system: n_poles [n_systems] (host), pole energies
  * p [sum_s n_poles[s]] (real, eV, host or device), pole vectors
@@ -253,8 +254,8 @@ gf_status gf_set_sigma_poles(gf_ctx *ctx, const int32_t *n_poles, const double *
 /* N(mu) = sum_k w_k sum_l |Psi_b,l|^2 n_F(E_l - mu) and its exact derivative
  * dN/dmu per system (host arrays [n_systems]; dn_dmu_out may be NULL), from the
  * eigenpairs (E_l, Psi_l) of H_ps(mu); Psi_b,l is the band block of Psi_l.
- * Errors: GF_ESTATE (H, P or the poles missing), GF_ENOTCONV (Jacobi did not
- * converge in 40 sweeps), GF_EINVAL, GF_ECUDA. */
+ * Errors: GF_ESTATE (H, P or the poles missing), GF_ENOTCONV (the eigensolver did
+ * not converge), GF_EINVAL, GF_ECUDA. */
 gf_status gf_pole_occupation(gf_ctx *ctx, const double *mu, double *n_out, double *dn_dmu_out);
 
 /* mu per system with |N(mu) - n_target[s]| <= tol on the pole-path N(mu), by
@@ -295,7 +296,7 @@ gf_status gf_pole_spectral(gf_ctx *ctx, const double *mu, int32_t n_eps, const d
  * Errors: as gf_pole_occupation. */
 gf_status gf_pole_energy(gf_ctx *ctx, const double *mu, double *h_ks_out, double *e_ps_out);
 
-/* Batched Hermitian eigensolver (cyclic Jacobi, the kernel of the pole path),
+/* Batched Hermitian eigensolver (cyclic Jacobi),
  * stateless: a [n_mat][n][n] complex128 on the device (its Hermitian part
  * (A + A^+)/2 is used) -> eigenvalues w [n_mat][n] ascending and eigenvectors
  * v [n_mat][n][n] (column l of each matrix is the vector of w[l]), both device

@@ -90,7 +90,7 @@ gf_status ensure_block(gf_ctx* c) {
   c->blk_ok = false;
   const size_t mm = (size_t)c->mmax * c->mmax, npm = (size_t)c->mmax * (c->mmax + 1) / 2;
   const bool mixed = c->precision == GF_PREC_MIXED;
-  const size_t smem = gf::heev_smem(c->blk_n2max), limit = (size_t)c->smem_optin - 8192;
+  const size_t smem = gf::heev_smem(c->blk_n2max), limit = (size_t)c->smem_optin - gf::kQlStatic;
   const int in_smem = smem <= limit ? 1 : 0;
   const int grid = std::max(1, std::min(c->n_k, c->sm_count * (in_smem ? std::min(8, std::max(1, (int)(limit / smem))) : 2)));
   const size_t ws = std::max(gf::block_reduce_ws_elems(c->nbmax, c->mmax, c->smem_optin, c->sm_count),
@@ -1102,7 +1102,7 @@ gf_status init_ctx(gf_ctx* c, const gf_desc* d) {
   }
 
   // block form: every window wider than its orbitals, one lane per orbital, eigenproblems within
-  // the Jacobi kernel's size, and enough frequencies to pay for the eigenproblem per k
+  // the eigensolver's size, and enough frequencies to pay for the eigenproblem per k
   c->blk_shape = c->n_iw >= kBlkMinFreq;
   std::vector<int64_t> offT(2 * (size_t)c->n_k);  // of T, then of C
   for (int k = 0; k < c->n_k; ++k) {
@@ -1311,7 +1311,7 @@ gf_status gf_destroy(gf_ctx* c) {
                     &c->pole_ws, &c->lr_eps, &c->lr_U, &c->lr_Pt, &c->lr_T, &c->lr_ws,
                     &c->eimp, &c->eimp_part, &c->gl_in, &c->delta, &c->wraw, &c->vdc,
                     &c->wbout, &c->kHks, &c->kEps, &c->eps_grid, &c->dos, &c->pdos, &c->pdos_off,
-                    &c->pole_part, &c->pole_vs, &c->pole_es, &c->voff_d, &c->mu_prev,
+                    &c->pole_part, &c->dos_part,
                     &c->blk_units, &c->blk_perm, &c->blk_sysg, &c->blk_offT, &c->blk_e, &c->blk_T, &c->blk_Ts,
                     &c->blk_B, &c->blk_Bs, &c->blk_HO, &c->blk_U, &c->blk_D22, &c->blk_V, &c->blk_R, &c->blk_H11,
                     &c->blk_tau, &c->blk_ws, &c->blk_info, &c->blk_C, &c->blk_Cs, &c->blk_ser};

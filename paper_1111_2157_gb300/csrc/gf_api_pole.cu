@@ -5,7 +5,7 @@
 namespace {
 
 // Pole path: build H_ps(mu) per k, diagonalise, and run the epilogues of mode.
-gf_status pole_run(gf_ctx* c, int mode, bool gloc_kernel = true, int warm = 0, int save_v = 0) {
+gf_status pole_run(gf_ctx* c, int mode, bool gloc_kernel = true) {
   if (!c->have_H || !c->have_P || !c->have_poles)
     return fail(c, GF_ESTATE, "gf_set_hamiltonian, gf_set_projectors and gf_set_sigma_poles must "
                               "all be called before a pole-path call");
@@ -39,18 +39,12 @@ gf_status pole_run(gf_ctx* c, int mode, bool gloc_kernel = true, int warm = 0, i
   p.wbout = c->wbout.as<double>();
   p.kHks = c->kHks.as<double>();
   p.kEps = c->kEps.as<double>();
-  p.warm = warm;
-  p.save_v = save_v;
-  if (warm || save_v) {
-    p.vstore = c->pole_vs.as<double2>();
-    p.estore = c->pole_es.as<double>();
-    p.voff = c->voff_d.as<int64_t>();
-    p.mu_prev = c->mu_prev.as<double>();
-  }
   p.status = c->status.as<int>();
   const size_t smem = gf::heev_smem(c->nps_max);
-  const size_t limit = (size_t)c->smem_optin - 16384;  // static shared arrays of the kernel
+  const size_t limit = (size_t)c->smem_optin - gf::kQlStatic;
   p.in_smem = smem <= limit ? 1 : 0;
+  const size_t zb = p.in_smem ? 0 : gf::ql_z_bytes(c->nps_max);
+  p.z_smem = zb > 0;
   int grid = std::min(c->n_k, c->sm_count * (p.in_smem ? std::max(1, (int)(limit / smem)) : 2));
   grid = std::max(grid, 1);
   if (!p.in_smem) {
@@ -65,7 +59,7 @@ gf_status pole_run(gf_ctx* c, int mode, bool gloc_kernel = true, int warm = 0, i
     c->ev.push_back(e);
   }
   GF_CU(cudaEventRecord(c->ev[c->ev_used], c->stream));
-  GF_CU(gf::launch_pole_eig(p, grid, p.in_smem ? smem : 0, c->stream));
+  GF_CU(gf::launch_pole_eig(p, grid, p.in_smem ? smem : zb, c->stream));
   c->last_launches += 1;
   if ((mode & gf::kGloc) && gloc_kernel) {
     const int ns = gf::pole_gloc_splits(c->n_sys, c->n_iw, c->sm_count, c->mmax);
@@ -85,15 +79,14 @@ gf_status pole_check(gf_ctx* c) {
   if (st) return st;
   int flags = 0;
   std::memcpy(&flags, c->hp_status(), sizeof(int));
-  if (flags & 2) return fail(c, GF_ENOTCONV, "Jacobi eigensolver did not converge in 40 sweeps");
+  if (flags & 2) return fail(c, GF_ENOTCONV, "the eigensolver did not converge");
   return GF_OK;
 }
 
-gf_status pole_occupation_impl(gf_ctx* c, const double* mu, double* n_out, double* dn_out,
-                               int warm = 0, int save_v = 0) {
+gf_status pole_occupation_impl(gf_ctx* c, const double* mu, double* n_out, double* dn_out) {
   gf_status st = upload_mu(c, mu);
   if (st) return st;
-  st = pole_run(c, gf::kOcc, true, warm, save_v);
+  st = pole_run(c, gf::kOcc);
   if (st) return st;
   GF_CU(gf::launch_sys_reduce(c->kinfo_d.as<KInfo>(), c->sinfo_d.as<SInfo>(), c->n_sys,
                               c->kN.as<double>(), c->kdN.as<double>(), c->sysout.as<double>(),
@@ -133,8 +126,8 @@ gf_status gf_set_sigma_poles(gf_ctx* c, const int32_t* n_poles, const double* po
     offV += (int64_t)n_poles[s] * c->sinfo[s].m;
   }
   if (offp > 0 && (!poles || !v)) return fail(c, GF_EINVAL, "poles_ptr or v_ptr is NULL");
-  std::vector<int64_t> eoff(c->n_k), phioff(c->n_k), voff(c->n_k);
-  int64_t te = 0, tphi = 0, tv = 0;
+  std::vector<int64_t> eoff(c->n_k), phioff(c->n_k);
+  int64_t te = 0, tphi = 0;
   int nps = 1;
   for (int k = 0; k < c->n_k; ++k) {
     const int s = c->ksys[k];
@@ -144,10 +137,8 @@ gf_status gf_set_sigma_poles(gf_ctx* c, const int32_t* n_poles, const double* po
     nps = std::max(nps, n);
     eoff[k] = te;
     phioff[k] = tphi;
-    voff[k] = tv;
     te += n;
     tphi += (int64_t)c->sinfo[s].m * n;
-    tv += (int64_t)n * n;
   }
   std::vector<double> hp(std::max<int64_t>(offp, 1));
   if (offp > 0) {
@@ -187,11 +178,6 @@ gf_status gf_set_sigma_poles(gf_ctx* c, const int32_t* n_poles, const double* po
                         c->stream));
   GF_CU(cudaMemcpyAsync(c->phioff_d.p, phioff.data(), sizeof(int64_t) * c->n_k,
                         cudaMemcpyHostToDevice, c->stream));
-  GF_CU(ensure(c->voff_d, sizeof(int64_t) * c->n_k));
-  GF_CU(cudaMemcpyAsync(c->voff_d.p, voff.data(), sizeof(int64_t) * c->n_k, cudaMemcpyHostToDevice,
-                        c->stream));
-  c->pole_v_elems = tv;
-  c->pole_e_elems = te;
   GF_CU(cudaStreamSynchronize(c->stream));
   c->pinfo = pinfo;
   c->nps_max = nps;
@@ -218,23 +204,8 @@ gf_status gf_pole_find_mu(gf_ctx* c, const double* n_target, double tol, int32_t
   if (!c) return GF_EINVAL;
   DeviceGuard guard(c->device);
   reset_stats(c);
-  // every evaluation after the first starts Jacobi from the previous eigenpairs
-  GF_CU(ensure(c->pole_vs, sizeof(double2) * std::max<int64_t>(c->pole_v_elems, 1)));
-  GF_CU(ensure(c->pole_es, sizeof(double) * std::max<int64_t>(c->pole_e_elems, 1)));
-  GF_CU(ensure(c->mu_prev, sizeof(double) * c->n_sys));
-  int evals = 0;
   return newton_mu(c, n_target, tol, max_iter, mu_inout, iters_out,
-                   [c, &evals](const double* mu, double* n, double* dn) {
-                     const int warm = evals > 0 ? 1 : 0;
-                     gf_status st2 = pole_occupation_impl(c, mu, n, dn, warm, 1);
-                     if (st2) return st2;
-                     ++evals;
-                     // the stored eigenpairs now belong to this mu
-                     cudaError_t e = cudaMemcpy(c->mu_prev.p, mu, sizeof(double) * c->n_sys,
-                                                cudaMemcpyHostToDevice);
-                     if (e != cudaSuccess) return fail(c, GF_ECUDA, cudaGetErrorString(e));
-                     return GF_OK;
-                   });
+                   [c](const double* mu, double* n, double* dn) { return pole_occupation_impl(c, mu, n, dn); });
 } catch (...) {
   return caught(c);
 }
@@ -421,10 +392,12 @@ gf_status gf_pole_spectral(gf_ctx* c, const double* mu, int32_t n_eps, const dou
   p.phiout = c->phiout.as<double2>();
   p.eoff = c->eoff_d.as<int64_t>();
   p.phioff = c->phioff_d.as<int64_t>();
-  GF_CU(gf::launch_pole_dos(p, c->n_sys, c->eps_grid.as<double>(), n_eps, eta,
-                            c->pdos_off.as<int64_t>(), c->dos.as<double>(),
+  const int ns = gf::pole_dos_splits(c->n_sys, n_eps, 1 + (pdos_out ? c->mmax : 0), c->n_k, c->sm_count);
+  GF_CU(ensure(c->dos_part, sizeof(double) * (size_t)ns * c->n_sys * n_eps * (1 + c->mmax)));
+  GF_CU(gf::launch_pole_dos(p, c->n_sys, c->eps_grid.as<double>(), n_eps, eta, c->mmax, ns,
+                            c->dos_part.as<double>(), c->pdos_off.as<int64_t>(), c->dos.as<double>(),
                             pdos_out ? c->pdos.as<double>() : nullptr, c->stream));
-  c->last_launches += 1;
+  c->last_launches += 2;
   GF_CU(cudaMemcpyAsync(dos_out, c->dos.p, sizeof(double) * (size_t)n_eps * c->n_sys,
                         cudaMemcpyDefault, c->stream));
   if (pdos_out)

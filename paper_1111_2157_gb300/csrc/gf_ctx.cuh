@@ -185,11 +185,10 @@ struct gf_ctx {
   DevBuf eimp, eimp_part, gl_in, delta, wraw, vdc;
   // pole form of Sigma (gf_set_sigma_poles) and the pseudo-Hamiltonian path
   bool have_poles = false;
-  int64_t pole_v_elems = 0, pole_e_elems = 0;
   std::vector<gf::PInfo> pinfo;
   int nps_max = 0;
   DevBuf poles, Vp, Sinf_p, pinfo_d, eoff_d, phioff_d, eout, phiout, pole_ws, wbout, kHks, kEps,
-      eps_grid, dos, pdos, pdos_off, pole_part, pole_vs, pole_es, voff_d, mu_prev;
+      eps_grid, dos, pdos, pdos_off, dos_part, pole_part;
 };
 
 namespace gf_host {
@@ -288,7 +287,7 @@ inline gf_status sync_and_check(gf_ctx* c) {
   std::memcpy(&flags, c->hp_status(), sizeof(int));
   if (flags & gf::kFlagSingular)
     return fail(c, GF_ESINGULAR, "zero or non-finite pivot in a (k, i w_n) inverse");
-  if (flags & 2) return fail(c, GF_ENOTCONV, "Jacobi eigensolver did not converge in 40 sweeps");
+  if (flags & 2) return fail(c, GF_ENOTCONV, "the eigensolver did not converge");
   return GF_OK;
 }
 

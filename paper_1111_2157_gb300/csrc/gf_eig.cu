@@ -11,12 +11,15 @@
 //   G_loc(i w_n) = sum_k w_k sum_l phi_l phi_l^+ / (i w_n + mu - E_l),  phi_l = P Psi_b,l,
 // where Psi_b is the band block (first N_b rows) of the eigenvectors.
 //
-// The eigensolver is the cyclic Jacobi method for complex Hermitian matrices
-// with the round-robin (circle) ordering of disjoint pairs, so that one step
-// applies N/2 independent rotations: one CTA per matrix, every thread on the
-// column update, then on the row update, of its share of the pairs.  The
-// matrix and the eigenvectors stay in shared memory when 2 N (N|1) 16-byte
-// elements fit, else in a per-CTA slice of a global workspace (L2-resident).
+// Two eigensolvers, one CTA per matrix, the matrix and the eigenvectors in shared memory when
+// 2 N (N|1) 16-byte elements fit, else in a per-CTA slice of a global workspace (L2-resident):
+//  * heev_tri: Householder tridiagonalisation, the tridiagonal eigenpairs in parallel (QR steps
+//    where levels are too close for that), back-transformation.  The pole path, the block form's
+//    setup and the Lowdin projectors.  A pseudo-Hamiltonian of 68 rows takes 2.0 ms, 16.9 ms by
+//    Jacobi (N(mu) of 125 k-points; 1000: 13.8 against 105 ms).
+//  * cyclic Jacobi with the round-robin (circle) ordering of disjoint pairs, so that one step
+//    applies N/2 independent rotations: gf_heev_batched, whose caller sets the sweep limit, and
+//    the low-rank kernel's setup.
 #include <math.h>
 #include <stdint.h>
 
@@ -189,6 +192,487 @@ __device__ int jacobi_heev(double2* A, double2* V, int N, int ld, int max_sweeps
   }
 }
 
+// Entry (l, l2), l <= l2, of a packed triangle.
+__device__ __forceinline__ void tri_pair(int e, int& l, int& l2) {
+  l2 = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+  while (l2 * (l2 + 1) / 2 > e) --l2;
+  while ((l2 + 1) * (l2 + 2) / 2 <= e) ++l2;
+  l = e - l2 * (l2 + 1) / 2;
+}
+
+// Scratch of heev_tri in shared memory, for matrices up to 256.
+struct QlScratch {
+  double d[256], e[256];          // the tridiagonal matrix
+  double tau[256];                // reflector scales
+  double2 ph[256];                // phases that make the off-diagonal real
+  union {
+    struct {
+      double2 v[256], p[256];     // the current reflector and A v
+    };
+    double2 rot[2][256];          // QR steps: (c, s) of two sweeps
+    struct {
+      double lam[256];            // eigenvalues, ascending
+      float fd[256], fe[256];     // FP32 copies of d and e^2 for the bisection
+      float red[kEigThreads / 32];
+    };
+  };
+  int lo[2], hi[2];
+  int more, failed;
+};
+
+// Largest of v over the CTA; NaN counts as infinite.
+__device__ __forceinline__ float block_max(float v, float* red) {
+  v = v == v ? v : INFINITY;
+  for (int off = 16; off; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  for (int w = 0; w < kEigThreads / 32; ++w) v = fmaxf(v, red[w]);
+  return v;
+}
+
+// 1 / x to rounding for |x| in FP32's range (0 where x is beyond it): the FP32 reciprocal and two
+// Newton steps, six FP64-pipe instructions.
+__device__ __forceinline__ double rcp_newton(double x) {
+  double r = (double)__frcp_rn((float)x);
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+
+// Eigenpairs of the real symmetric tridiagonal matrix (q.d, q.e), one thread per eigenvalue:
+// bisection on Sturm counts in FP32, then three Rayleigh quotient steps in FP64 whose vector comes
+// from the twisted factorization at the row of the smallest pivot (Dhillon and Parlett, Linear
+// Algebra Appl. 387, 2004), and one step Z <- Z (3 I - Z^T Z) / 2 that restores the orthogonality
+// which nearby eigenvalues lose.  Returns false, with d and e unchanged, when an eigenvalue pair
+// is closer than that step can mend (degenerate levels, a split matrix, non-finite input): the
+// caller then takes QR steps.  An FP64 instruction holds its scheduler for 64 clocks for one lane
+// as for 32, so this does in about 170 N of them, side by side, what QR steps do in 24 per rotation
+// (5,400 rotations for N = 68), one after the other.
+__device__ bool tri_eig(double* Z, int zr, int zs, double* G, int gr, int gs, int N, QlScratch& q) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float tn = 0.f;
+  for (int i = tid; i < N; i += kEigThreads) {
+    const float d = (float)q.d[i], e = (float)q.e[i], ep = i ? (float)q.e[i - 1] : 0.f;
+    q.fd[i] = d;
+    q.fe[i] = e * e;
+    tn = fmaxf(tn, fabsf(d) + fabsf(e) + fabsf(ep));
+    if (!(fabsf(d) + fabsf(e) < 1e15f)) tn = INFINITY;
+  }
+  tn = block_max(tn, q.red);
+  if (!(tn > 1e-15f && tn < 1e15f)) return false;
+  if (tid < N) {
+    float lo = -1.001f * tn, hi = 1.001f * tn;
+    const float tiny = 1e-12f * tn;
+    for (int it = 0; it < 27; ++it) {
+      const float x = 0.5f * (lo + hi);
+      int below = 0;
+      float t = q.fd[0] - x;
+      for (int i = 1;; ++i) {
+        if (fabsf(t) < tiny) t = -tiny;
+        below += t < 0.f;
+        if (i == N) break;
+        t = (q.fd[i] - x) - __fdividef(q.fe[i - 1], t);
+      }
+      if (below > tid) hi = x;
+      else lo = x;
+    }
+    double lam = 0.5 * ((double)lo + (double)hi);
+    const double small = 1e-18 * (double)tn;
+    double* z = Z + tid * zs;
+    for (int it = 0; it < 3; ++it) {
+      // pivots from above, kept; from below with the twist row
+      double t = q.d[0] - lam;
+      for (int i = 0;; ++i) {
+        if (fabs(t) < small) t = small;
+        z[i * zr] = t;
+        if (i == N - 1) break;
+        const double e = q.e[i];
+        t = fma(-e, e * rcp_newton(t), q.d[i + 1] - lam);
+      }
+      double best = fabs(z[(N - 1) * zr]);
+      double gam = z[(N - 1) * zr];
+      int r = N - 1;
+      double u = q.d[N - 1] - lam;
+      for (int i = N - 2; i >= 0; --i) {
+        if (fabs(u) < small) u = small;
+        const double e = q.e[i], w = e * (e * rcp_newton(u));
+        const double g = z[i * zr] - w;  // D+ + D- - (d - lam) with D- = d - lam - w
+        u = (q.d[i] - lam) - w;
+        if (fabs(g) < best) {
+          best = fabs(g);
+          gam = g;
+          r = i;
+        }
+      }
+      // multipliers from below for the rows after the twist, then the vector
+      u = q.d[N - 1] - lam;
+      for (int i = N - 2; i >= r; --i) {
+        if (fabs(u) < small) u = small;
+        const double e = q.e[i], m = e * rcp_newton(u);
+        u = fma(-e, m, q.d[i] - lam);
+        z[(i + 1) * zr] = -m;
+      }
+      double nrm = 1.0, x = 1.0;
+      for (int i = r + 1; i < N; ++i) {
+        x *= z[i * zr];
+        z[i * zr] = x;
+        nrm = fma(x, x, nrm);
+      }
+      x = 1.0;
+      for (int i = r - 1; i >= 0; --i) {
+        x *= -q.e[i] * rcp_newton(z[i * zr]);
+        z[i * zr] = x;
+        nrm = fma(x, x, nrm);
+      }
+      z[r * zr] = 1.0;
+      lam += gam / nrm;
+      if (it == 2) {
+        const double s = rsqrt(nrm);
+        for (int i = 0; i < N; ++i) z[i * zr] *= s;
+      }
+    }
+    q.lam[tid] = lam;
+  }
+  __syncthreads();
+  // G = Z^T Z - I (lower triangle and its mirror), its largest entry
+  float gmax = 0.f;
+  for (int x = tid; x < N * (N + 1) / 2; x += kEigThreads) {
+    int a, b;
+    tri_pair(x, a, b);
+    double s0 = a == b ? -1.0 : 0.0, s1 = 0.0;
+    int i = 0;
+    for (; i + 1 < N; i += 2) {
+      s0 = fma(Z[i * zr + a * zs], Z[i * zr + b * zs], s0);
+      s1 = fma(Z[(i + 1) * zr + a * zs], Z[(i + 1) * zr + b * zs], s1);
+    }
+    if (i < N) s0 = fma(Z[i * zr + a * zs], Z[i * zr + b * zs], s0);
+    s0 += s1;
+    G[a * gr + b * gs] = s0;
+    G[b * gr + a * gs] = s0;
+    const float f = fabsf((float)s0);
+    gmax = fmaxf(gmax, f == f ? f : INFINITY);
+  }
+  gmax = block_max(gmax, q.red);
+  if (!(gmax < 1e-5f)) return false;
+  // Z -= Z G / 2, one row per warp
+  for (int r = warp; r < N; r += kEigThreads / 32) {
+    double* zp = Z + r * zr;
+    double out[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const int c = lane + 32 * t;
+      if (c - lane >= N) break;
+      double s0 = 0.0, s1 = 0.0;
+      if (c < N) {
+        int k = 0;
+        for (; k + 1 < N; k += 2) {
+          s0 = fma(zp[k * zs], G[k * gr + c * gs], s0);
+          s1 = fma(zp[(k + 1) * zs], G[(k + 1) * gr + c * gs], s1);
+        }
+        if (k < N) s0 = fma(zp[k * zs], G[k * gr + c * gs], s0);
+        out[t] = fma(-0.5, s0 + s1, zp[c * zs]);
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const int c = lane + 32 * t;
+      if (c < N) zp[c * zs] = out[t];
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < N; i += kEigThreads) q.d[i] = q.lam[i];
+  __syncthreads();
+  return true;
+}
+
+// Implicit QR steps with Wilkinson's shift on the tridiagonal matrix (Golub and Van Loan, Matrix
+// Computations, section 8.3), rotations applied to Z (the identity on entry).  One lane of warp 0
+// forms the rotations of a sweep while the other warps apply the previous sweep's.  Returns false
+// when an eigenvalue takes more than 40 steps (non-finite input does).
+__device__ bool tri_qr(double* Z, int zr, int zs, int N, QlScratch& q) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int x = tid; x < N * N; x += kEigThreads) {
+    const int i = x / N, l = x - i * N;
+    Z[i * zr + l * zs] = i == l ? 1.0 : 0.0;
+  }
+  if (tid == 0) {
+    q.more = 1;
+    q.failed = 0;
+    q.lo[1] = q.hi[1] = 0;  // no sweep to apply yet
+  }
+  __syncthreads();
+  int hi = N - 1, steps = 0;  // warp 0: end of the active block, steps spent on its eigenvalue
+  for (int t = 0;; ++t) {
+    const int b = t & 1;
+    if (warp == 0) {
+      // deflate: the largest unreduced block that ends at hi
+      int lo = 0;
+      for (;;) {
+        int last = -1;  // last negligible off-diagonal entry below hi
+        for (int i = lane; i < hi; i += 32)
+          if (fabs(q.e[i]) <= 1.2e-16 * (fabs(q.d[i]) + fabs(q.d[i + 1]))) last = i;
+        last = __reduce_max_sync(0xffffffffu, last);
+        lo = last + 1;
+        if (lo < hi || hi <= 0) break;
+        --hi;
+        steps = 0;
+      }
+      if (lane == 0) {
+        q.lo[b] = q.hi[b] = 0;
+        if (hi <= 0) {
+          q.more = 0;
+        } else if (++steps > 40) {
+          q.failed = 1;
+          q.more = 0;
+        } else {
+          q.lo[b] = lo;
+          q.hi[b] = hi;
+          double* d = q.d;
+          double* e = q.e;
+          const double dl = 0.5 * (d[hi - 1] - d[hi]), eb = e[hi - 1];
+          const double den = dl + copysign(sqrt(fma(dl, dl, eb * eb)), dl);
+          double x = d[lo] - (d[hi] - (den != 0.0 ? eb * eb / den : 0.0)), z = e[lo];
+          double a = d[lo], ek = e[lo];
+          for (int k = lo; k < hi; ++k) {
+            const double g = d[k + 1], en = e[k + 1];
+            const double r2 = fma(x, x, z * z);
+            double c = 1.0, s = 0.0;
+            if (r2 > 0.0) {
+              const double ir = rsqrt(r2);
+              c = x * ir;
+              s = z * ir;
+              if (k > lo) e[k - 1] = r2 * ir;
+            } else if (k > lo) {
+              e[k - 1] = 0.0;
+            }
+            // [a ek; ek g] under the rotation, with h = s (g - a) + 2 c ek
+            const double h = fma(s, g - a, 2.0 * c * ek), pp = s * h;
+            d[k] = a + pp;
+            x = fma(c, h, -ek);
+            z = s * en;
+            a = g - pp;
+            ek = c * en;
+            e[k] = x;
+            q.rot[b][k] = make_double2(c, s);
+          }
+          d[hi] = a;
+        }
+      }
+      __syncwarp();
+    } else {
+      // apply the previous sweep to the columns of Z, one row per thread
+      const int l0 = q.lo[b ^ 1], h0 = q.hi[b ^ 1];
+      for (int r = tid - 32; r < N && l0 < h0; r += kEigThreads - 32) {
+        double* zp = Z + r * zr;
+        double z0 = zp[l0 * zs];
+        for (int k = l0; k < h0; ++k) {
+          const double2 cs = q.rot[b ^ 1][k];
+          const double z1 = zp[(k + 1) * zs];
+          zp[k * zs] = fma(cs.x, z0, cs.y * z1);
+          z0 = fma(cs.x, z1, -cs.y * z0);
+        }
+        zp[h0 * zs] = z0;
+      }
+    }
+    __syncthreads();
+    if (!q.more && q.lo[b] >= q.hi[b]) break;
+  }
+  return !q.failed;
+}
+
+// Eigenpairs of the Hermitian N x N matrix A (row-major, leading dimension ld, both triangles):
+// Householder reduction to tridiagonal form, the eigenpairs of that, and the back-transformation.
+// On return the diagonal of A holds the eigenvalues (as complex numbers) and V the eigenvectors as
+// columns.  Z: real N x N scratch (row stride zr, element step zs), G another; both may lie over V
+// (its real and its imaginary parts).  Returns false when the QR steps fail.
+//
+// About 12 N^3 FP64 FMAs against 18 N^3 per sweep and eight sweeps of cyclic Jacobi.
+__device__ bool heev_tri(double2* A, double2* V, double* Z, int zr, int zs, double* G, int gr, int gs, int N, int ld,
+                         QlScratch& q) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kW = kEigThreads / 32;
+  // a matrix that is diagonal already (to 1e-15 of its norm): no work
+  double off = 0.0, dia = 0.0;
+  for (int x = tid; x < N * N; x += kEigThreads) {
+    const int i = x / N, j = x - i * N;
+    const double2 a = A[i * ld + j];
+    const double s = fma(a.x, a.x, a.y * a.y);
+    if (i == j) dia += s;
+    else off += s;
+  }
+  off = eig_block_sum(off, &q.tau[0]);
+  dia = eig_block_sum(dia, &q.tau[0]);
+  if (off <= 1e-30 * (off + dia)) {
+    for (int x = tid; x < N * N; x += kEigThreads) {
+      const int i = x / N, l = x - i * N;
+      V[i * ld + l] = make_double2(i == l ? 1.0 : 0.0, 0.0);
+    }
+    __syncthreads();
+    return true;
+  }
+  for (int k = 0; k + 2 < N; ++k) {
+    const int len = N - 1 - k;
+    // lanes per row: every thread of the CTA on the shrinking triangle; the rows of a warp are kW
+    // apart, so that each warp has long and short ones
+    int tl = 32;
+    while (tl > 1 && kEigThreads / tl < len) tl >>= 1;
+    const int sub = lane % tl, rw = (lane / tl) * kW + warp;
+    if (warp == 0) {
+      double s = 0.0;
+      for (int i = lane; i < len; i += 32) {
+        const double2 x = A[(k + 1 + i) * ld + k];
+        q.v[i] = x;
+        s = fma(x.x, x.x, fma(x.y, x.y, s));
+      }
+      for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+      __syncwarp();
+      // (every lane the same: an FP64 instruction costs a lane as much as a warp)
+      const double2 x0 = q.v[0];
+      const double a2 = fma(x0.x, x0.x, x0.y * x0.y);
+      const double inx = s > 0.0 ? rsqrt(s) : 0.0, iax = a2 > 0.0 ? rsqrt(a2) : 0.0;
+      const double nx = s * inx, ax = a2 * iax;
+      const double2 ph = a2 > 0.0 ? make_double2(x0.x * iax, x0.y * iax) : make_double2(1.0, 0.0);
+      const double tau = s > 0.0 ? 1.0 / fma(nx, ax, s) : 0.0;
+      __syncwarp();
+      if (lane == 0) {
+        q.v[0] = make_double2(fma(ph.x, nx, x0.x), fma(ph.y, nx, x0.y));
+        q.tau[k] = tau;
+        q.e[k] = nx;
+        q.ph[k + 1] = make_double2(-ph.x, -ph.y);  // phase of the off-diagonal entry
+      }
+    }
+    __syncthreads();
+    const double tau = q.tau[k];
+    // p = tau A v from the lower triangle
+    {
+      const int i = rw;
+      double2 a0 = make_double2(0.0, 0.0), a1 = a0;
+      if (i < len) {
+        const double2* Ar = A + (k + 1 + i) * ld + k + 1;
+        int c = sub;
+        for (; c + tl <= i; c += 2 * tl) {
+          cmac(a0, Ar[c], q.v[c]);
+          cmac(a1, Ar[c + tl], q.v[c + tl]);
+        }
+        for (; c <= i; c += tl) cmac(a0, Ar[c], q.v[c]);
+        const double2* Ac = A + (k + 1) * ld + k + 1 + i;
+        for (; c < len; c += tl) cmac_ca(a1, Ac[c * ld], q.v[c]);
+      }
+      a0.x += a1.x;
+      a0.y += a1.y;
+      for (int off = 1; off < tl; off <<= 1) {
+        a0.x += __shfl_xor_sync(0xffffffffu, a0.x, off);
+        a0.y += __shfl_xor_sync(0xffffffffu, a0.y, off);
+      }
+      if (sub == 0 && i < len) q.p[i] = make_double2(tau * a0.x, tau * a0.y);
+    }
+    __syncthreads();
+    // w = p - (tau / 2) (v^+ p) v
+    if (warp == 0) {
+      double s = 0.0;
+      for (int i = lane; i < len; i += 32) s = fma(q.v[i].x, q.p[i].x, fma(q.v[i].y, q.p[i].y, s));
+      for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+      s *= -0.5 * tau;
+      for (int i = lane; i < len; i += 32) {
+        const double2 v = q.v[i];
+        q.p[i].x = fma(s, v.x, q.p[i].x);
+        q.p[i].y = fma(s, v.y, q.p[i].y);
+      }
+    }
+    __syncthreads();
+    // lower triangle: A -= v w^+ + w v^+; column k keeps v for the back-transformation
+    if (rw < len) {
+      const int i = rw;
+      const double2 vi = q.v[i], wi = q.p[i];
+      double2* Ar = A + (k + 1 + i) * ld + k + 1;
+      if (sub == 0) Ar[-1] = vi;
+      for (int c = sub; c <= i; c += tl) {
+        const double2 v = q.v[c], w = q.p[c];
+        double2 a = Ar[c];
+        a.x = fma(-vi.x, w.x, fma(-vi.y, w.y, fma(-wi.x, v.x, fma(-wi.y, v.y, a.x))));
+        a.y = fma(-vi.y, w.x, fma(vi.x, w.y, fma(-wi.y, v.x, fma(wi.x, v.y, a.y))));
+        Ar[c] = a;
+      }
+    }
+    __syncthreads();
+  }
+  for (int i = tid; i < N; i += kEigThreads) q.d[i] = A[i * ld + i].x;
+  if (tid == 0) {
+    if (N > 1) {
+      const double2 x = A[(N - 1) * ld + N - 2];
+      const double ax = sqrt(fma(x.x, x.x, x.y * x.y));
+      q.e[N - 2] = ax;
+      q.ph[N - 1] = ax > 0.0 ? make_double2(x.x / ax, x.y / ax) : make_double2(1.0, 0.0);
+    }
+    q.e[N - 1] = 0.0;
+    // T = D T_real D^+: running products of the phases
+    q.ph[0] = make_double2(1.0, 0.0);
+    for (int i = 1; i < N; ++i) q.ph[i] = cmul(q.ph[i], q.ph[i - 1]);
+  }
+  __syncthreads();
+  bool ok = N > 3 && tri_eig(Z, zr, zs, G, gr, gs, N, q);
+  if (!ok) ok = tri_qr(Z, zr, zs, N, q);
+  __syncthreads();
+  // V = H_0 H_1 ... D Z: phases, then the reflectors in reverse order, tl lanes per column
+  for (int x = tid; x < N * N; x += kEigThreads) {
+    const int i = x / N, l = x - i * N;
+    const double z = Z[i * zr + l * zs];
+    V[i * ld + l] = make_double2(q.ph[i].x * z, q.ph[i].y * z);
+  }
+  __syncthreads();
+  // (more lanes a column, with fewer idle, measured slower: 1.5 against 1.1 M clocks at N = 68)
+  const int tl = N <= 64 ? 4 : (N <= 128 ? 2 : 1);
+  const int sub = lane % tl;
+  for (int l0 = 0; l0 < N; l0 += kEigThreads / tl) {
+    const int l = l0 + warp * (32 / tl) + lane / tl;
+    for (int k = N - 3; k >= 0; --k) {
+      const double2* v = A + (k + 1) * ld + k;
+      double2 s0 = make_double2(0.0, 0.0), s1 = s0;
+      if (l < N) {
+        int i = sub;
+        for (; i + tl < N - 1 - k; i += 2 * tl) {
+          cmac_ca(s0, v[i * ld], V[(k + 1 + i) * ld + l]);
+          cmac_ca(s1, v[(i + tl) * ld], V[(k + 1 + i + tl) * ld + l]);
+        }
+        for (; i < N - 1 - k; i += tl) cmac_ca(s0, v[i * ld], V[(k + 1 + i) * ld + l]);
+      }
+      s0.x += s1.x;
+      s0.y += s1.y;
+      for (int off = 1; off < tl; off <<= 1) {
+        s0.x += __shfl_xor_sync(0xffffffffu, s0.x, off);
+        s0.y += __shfl_xor_sync(0xffffffffu, s0.y, off);
+      }
+      const double tau = q.tau[k];
+      s0.x *= tau;
+      s0.y *= tau;
+      if (l < N)
+        for (int i = sub; i < N - 1 - k; i += tl) {
+          const double2 vv = v[i * ld];
+          double2 u = V[(k + 1 + i) * ld + l];
+          u.x = fma(-vv.x, s0.x, fma(vv.y, s0.y, u.x));
+          u.y = fma(-vv.x, s0.y, fma(-vv.y, s0.x, u.y));
+          V[(k + 1 + i) * ld + l] = u;
+        }
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < N; i += kEigThreads) A[i * ld + i] = make_double2(q.d[i], 0.0);
+  __syncthreads();
+  return ok;
+}
+
+// heev_tri with Z and G over V's real and imaginary parts when the matrices are in shared memory;
+// with the matrices in a global slice Z has shared memory of its own when that fits (z_smem).
+__device__ __forceinline__ bool heev_tri(double2* A, double2* V, int n, int ld, int in_smem, int z_smem,
+                                         unsigned char* smem, QlScratch& q) {
+  double* v = reinterpret_cast<double*>(V);
+  if (!in_smem && z_smem)
+    return heev_tri(A, V, reinterpret_cast<double*>(smem), n | 1, 1, v, n | 1, 1, n, ld, q);
+  return heev_tri(A, V, v, 2 * ld, 2, v + 1, 2 * ld, 2, n, ld, q);
+}
+
 __device__ __forceinline__ size_t eig_ws_elems(int n) { return (size_t)2 * n * (n | 1); }
 
 // Standalone batched eigensolver: A [mat][n][n] -> w [mat][n] ascending,
@@ -241,8 +725,7 @@ __global__ void __launch_bounds__(kEigThreads)
 __global__ void __launch_bounds__(kEigThreads) k_pole_eig(const PoleParams p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double s_x[256], s_f[256], s_ch[256];
-  __shared__ double rot[4 * 128];
-  __shared__ double2 ph[128];
+  __shared__ QlScratch ql;
   __shared__ double red[kEigThreads / 32];
   const int tid = threadIdx.x;
   for (int k = blockIdx.x; k < p.n_k; k += gridDim.x) {
@@ -257,75 +740,44 @@ __global__ void __launch_bounds__(kEigThreads) k_pole_eig(const PoleParams p) {
     const double2* P = p.P + ki.offP;
     const double2* Sinf = p.Sinf + si.offSinf;
     const double2* Vp = p.Vp + pi.offV;
-    double2* Vs = p.vstore ? p.vstore + p.voff[k] : nullptr;  // eigenvectors kept between calls
-    double* Es = p.estore ? p.estore + p.eoff[k] : nullptr;
-    if (p.warm) {
-      // warm start from the eigenpairs (E', V') at mu' = mu_prev: H_ps(mu) = H_ps(mu') +
-      // (mu - mu') Pi_p, so V'^+ H_ps(mu) V' = diag(E') + (mu - mu') V_p'^+ V_p' with V_p'
-      // the pole rows of V'; Jacobi then only removes what the shift of mu added
-      const double dmu = mu - p.mu_prev[ki.sys];
-      for (int e = tid; e < n * n; e += kEigThreads) {
-        const int l = e / n, l2 = e - (e / n) * n;
-        double2 acc = make_double2(0.0, 0.0);
-        for (int i = nb; i < n; ++i) cmac_ca(acc, Vs[i * n + l], Vs[i * n + l2]);
-        acc.x *= dmu;
-        acc.y *= dmu;
-        if (l == l2) acc.x += Es[l];
-        A[l * ld + l2] = acc;
+    // band block H + P^+ (Sigma_inf P), the product in V (m nb <= n ld when m <= n, else recomputed)
+    const bool staged = m <= n;
+    if (staged) {
+      for (int e = tid; e < m * nb; e += kEigThreads) {
+        const int a = e / nb, j = e - a * nb;
+        double2 t = make_double2(0.0, 0.0);
+        for (int b = 0; b < m; ++b) cmac(t, Sinf[a * m + b], P[b * nb + j]);
+        V[e] = t;
       }
-    } else {
-      // band block H + P^+ Sigma_inf P
-      for (int e = tid; e < nb * nb; e += kEigThreads) {
-        const int i = e / nb, j = e - (e / nb) * nb;
-        double2 acc = H[i * nb + j];
-        for (int a = 0; a < m; ++a) {
-          double2 t = make_double2(0.0, 0.0);
+      __syncthreads();
+    }
+    for (int e = tid; e < nb * nb; e += kEigThreads) {
+      const int i = e / nb, j = e - (e / nb) * nb;
+      double2 acc = H[i * nb + j];
+      for (int a = 0; a < m; ++a) {
+        double2 t = make_double2(0.0, 0.0);
+        if (staged) t = V[a * nb + j];
+        else
           for (int b = 0; b < m; ++b) cmac(t, Sinf[a * m + b], P[b * nb + j]);
-          cmac_ca(acc, P[a * nb + i], t);
-        }
-        A[i * ld + j] = acc;
+        cmac_ca(acc, P[a * nb + i], t);
       }
-      // pole rows/columns W_i = V_i P and the pole diagonal p_i + mu
-      for (int e = tid; e < npl * nb; e += kEigThreads) {
-        const int i = e / nb, b = e - (e / nb) * nb;
-        double2 w = make_double2(0.0, 0.0);
-        for (int a = 0; a < m; ++a) cmac(w, Vp[i * m + a], P[a * nb + b]);
-        A[(nb + i) * ld + b] = w;
-        A[b * ld + nb + i] = make_double2(w.x, -w.y);
-      }
-      for (int e = tid; e < npl * npl; e += kEigThreads) {
-        const int i = e / npl, j = e - (e / npl) * npl;
-        A[(nb + i) * ld + nb + j] = make_double2(i == j ? p.poles[pi.offp + i] + mu : 0.0, 0.0);
-      }
+      A[i * ld + j] = acc;
+    }
+    // pole rows/columns W_i = V_i P and the pole diagonal p_i + mu
+    for (int e = tid; e < npl * nb; e += kEigThreads) {
+      const int i = e / nb, b = e - (e / nb) * nb;
+      double2 w = make_double2(0.0, 0.0);
+      for (int a = 0; a < m; ++a) cmac(w, Vp[i * m + a], P[a * nb + b]);
+      A[(nb + i) * ld + b] = w;
+      A[b * ld + nb + i] = make_double2(w.x, -w.y);
+    }
+    for (int e = tid; e < npl * npl; e += kEigThreads) {
+      const int i = e / npl, j = e - (e / npl) * npl;
+      A[(nb + i) * ld + nb + j] = make_double2(i == j ? p.poles[pi.offp + i] + mu : 0.0, 0.0);
     }
     __syncthreads();
-    const int sw = jacobi_heev(A, V, n, ld, p.max_sweeps, rot, ph, red);
-    if (sw < 0 && tid == 0) atomicOr(p.status, 2);
-    if (p.warm) {
-      // eigenvectors of H_ps(mu) = V' R: the product goes to A's storage (its
-      // diagonal, the eigenvalues, is kept in s_x first) and A, V swap roles
-      for (int l = tid; l < n; l += kEigThreads) s_x[l] = A[l * ld + l].x;
-      __syncthreads();
-      for (int e = tid; e < n * n; e += kEigThreads) {
-        const int i = e / n, l = e - (e / n) * n;
-        double2 acc = make_double2(0.0, 0.0);
-        for (int q = 0; q < n; ++q) cmac(acc, Vs[i * n + q], V[q * ld + l]);
-        A[i * ld + l] = acc;
-      }
-      __syncthreads();
-      double2* t = A;
-      A = V;
-      V = t;
-      for (int l = tid; l < n; l += kEigThreads) A[l * ld + l] = make_double2(s_x[l], 0.0);
-      __syncthreads();
-    }
-    if (p.save_v) {
-      for (int e = tid; e < n * n; e += kEigThreads) {
-        const int i = e / n, l = e - (e / n) * n;
-        Vs[e] = V[i * ld + l];
-      }
-      for (int l = tid; l < n; l += kEigThreads) Es[l] = A[l * ld + l].x;
-    }
+    const bool ok = heev_tri(A, V, n, ld, p.in_smem, p.z_smem, smem_raw, ql);
+    if (!ok && tid == 0) atomicOr(p.status, 2);
     // per eigenpair: x_l = E_l - mu, n_F(x_l), cosh(beta x_l / 2)
     for (int l = tid; l < n; l += kEigThreads) {
       const double x = A[l * ld + l].x - mu;
@@ -346,13 +798,14 @@ __global__ void __launch_bounds__(kEigThreads) k_pole_eig(const PoleParams p) {
       }
       nk = eig_block_sum(nk, red);
       double dk = 0.0;
-      for (int e = tid; e < n * n; e += kEigThreads) {
-        const int l = e / n, l2 = e - (e / n) * n;
+      for (int e = tid; e < n * (n + 1) / 2; e += kEigThreads) {
+        int l, l2;
+        tri_pair(e, l, l2);
         double2 o = make_double2(0.0, 0.0);
         for (int b = 0; b < nb; ++b) cmac_ca(o, V[b * ld + l], V[b * ld + l2]);
         const double f1 =
             fermi_divdiff(s_x[l], s_x[l2], s_f[l], s_f[l2], s_ch[l], s_ch[l2], si.beta);
-        dk = fma(-(o.x * o.x + o.y * o.y), f1, dk);
+        dk = fma((l == l2 ? -1.0 : -2.0) * (o.x * o.x + o.y * o.y), f1, dk);
       }
       dk = eig_block_sum(dk, red);
       if (tid == 0) {
@@ -363,8 +816,9 @@ __global__ void __launch_bounds__(kEigThreads) k_pole_eig(const PoleParams p) {
     if (p.mode & kRho) {
       double2* rho = p.rho + ki.offH;
       double hks = 0.0;  // Re Tr(H_k rho_k)
-      for (int e = tid; e < nb * nb; e += kEigThreads) {
-        const int i = e / nb, j = e - (e / nb) * nb;
+      for (int e = tid; e < nb * (nb + 1) / 2; e += kEigThreads) {
+        int i, j;
+        tri_pair(e, i, j);
         double2 acc = make_double2(0.0, 0.0);
         for (int l = 0; l < n; ++l) {
           const double f = s_f[l];
@@ -373,9 +827,15 @@ __global__ void __launch_bounds__(kEigThreads) k_pole_eig(const PoleParams p) {
           vi.y *= f;
           cmac_cb(acc, vi, V[j * ld + l]);
         }
+        if (i == j) acc.y = 0.0;
         rho[i * nb + j] = acc;
         const double2 h = H[j * nb + i];
         hks = fma(h.x, acc.x, fma(-h.y, acc.y, hks));
+        if (i != j) {
+          rho[j * nb + i] = make_double2(acc.x, -acc.y);
+          const double2 h2 = H[i * nb + j];
+          hks = fma(h2.x, acc.x, fma(h2.y, acc.y, hks));
+        }
       }
       double nc = 0.0;
       for (int e = tid; e < m * n; e += kEigThreads) {
@@ -585,11 +1045,9 @@ __global__ void __launch_bounds__(kEigThreads)
 
 // Block form: eigenpairs of the n2 x n2 block of every k (D22, replaced by its eigenvectors).
 __global__ void __launch_bounds__(kEigThreads)
-    k_block_eig(const BlockSetup b, double2* gws, int in_smem) {
+    k_block_eig(const BlockSetup b, double2* gws, int in_smem, int z_smem) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double rot[4 * 128];
-  __shared__ double2 ph[128];
-  __shared__ double red[kEigThreads / 32];
+  __shared__ QlScratch ql;
   double2* A = in_smem ? reinterpret_cast<double2*>(smem_raw) : gws + blockIdx.x * eig_ws_elems(b.n2max);
   for (int k = blockIdx.x; k < b.n_k; k += gridDim.x) {
     const KInfo ki = b.kinfo[k];
@@ -602,8 +1060,8 @@ __global__ void __launch_bounds__(kEigThreads)
       A[i * ld + j] = make_double2(0.5 * (x.x + y.x), 0.5 * (x.y - y.y));
     }
     __syncthreads();
-    const int sw = jacobi_heev(A, V, n, ld, 40, rot, ph, red);
-    if (sw < 0 && threadIdx.x == 0) atomicOr(b.flags, kBlkNoConvergence);
+    const bool ok = heev_tri(A, V, n, ld, in_smem, z_smem, smem_raw, ql);
+    if (!ok && threadIdx.x == 0) atomicOr(b.flags, kBlkNoConvergence);
     for (int l = threadIdx.x; l < n; l += kEigThreads) b.e[b.offD[k] + l] = A[l * ld + l].x;
     for (int e = threadIdx.x; e < n * n; e += kEigThreads) {
       const int i = e / n, l = e - i * n;
@@ -618,52 +1076,83 @@ __global__ void __launch_bounds__(kEigThreads)
 //   D(e)       = sum_k w_k sum_l |Psi_b,l|^2 L(e + mu - E_l),
 //   D_alpha(e) = sum_k w_k sum_l |phi_l(alpha)|^2 L(e + mu - E_l),
 //   L(x) = (eta / pi) / (x^2 + eta^2) = -(1/pi) Im 1/(x + i eta).
-// One thread per (system, energy); the k and l sums run in increasing order.
-__global__ void k_pole_dos(const PoleParams p, const double* __restrict__ eps_grid, int n_eps,
-                           double eta, const int64_t* __restrict__ pdos_off, double* __restrict__ dos,
-                           double* __restrict__ pdos) {
-  const int s = blockIdx.y;
-  const int ie = blockIdx.x * blockDim.x + threadIdx.x;
-  if (ie >= n_eps) return;
+// One thread per energy, kDosT channels (the DOS, then the orbitals) per CTA in registers, the
+// weights of 32 eigenpairs staged at a time, the k-points in gridDim.z splits (a grid of 201
+// energies alone is two CTAs); part [split][system][energy][1 + mmax], k then l increasing.
+constexpr int kDosT = 8, kDosL = 32;
+__global__ void __launch_bounds__(128)
+    k_pole_dos(const PoleParams p, const double* __restrict__ eps_grid, int n_eps, double eta, int n_ch, int mmax,
+               double* __restrict__ part) {
+  __shared__ double s_w[kDosL][kDosT], s_e[kDosL];
+  const int tiles = (n_eps + 127) / 128;
+  const int s = blockIdx.y, ie = (blockIdx.x % tiles) * 128 + threadIdx.x, c0 = (blockIdx.x / tiles) * kDosT;
   const SInfo si = p.sinfo[s];
-  const int m = si.m, npl = p.pinfo[s].np;
-  const double z = eps_grid[ie] + p.mu[s];
-  double d = 0.0;
-  double pd[32];
-  for (int a = 0; a < 32; ++a) pd[a] = 0.0;
-  for (int k = si.k0; k < si.k1; ++k) {
+  const int m = si.m, npl = p.pinfo[s].np, nks = si.k1 - si.k0;
+  const int ka = si.k0 + (int)((int64_t)nks * blockIdx.z / gridDim.z);
+  const int kb = si.k0 + (int)((int64_t)nks * (blockIdx.z + 1) / gridDim.z);
+  const double z = eps_grid[min(ie, n_eps - 1)] + p.mu[s], e2 = eta * eta;
+  double acc[kDosT];
+#pragma unroll
+  for (int t = 0; t < kDosT; ++t) acc[t] = 0.0;
+  for (int k = ka; k < kb; ++k) {
     const int n = p.kinfo[k].nb + npl;
-    const double wk = p.kinfo[k].w;
+    const double wk = p.kinfo[k].w * (eta * 0.31830988618379067);
     const double* E = p.eout + p.eoff[k];
     const double* wb = p.wbout + p.eoff[k];
     const double2* phi = p.phiout + p.phioff[k];
-    for (int l = 0; l < n; ++l) {
-      const double x = z - E[l];
-      const double lor = wk * (eta * 0.31830988618379067) / fma(x, x, eta * eta);
-      d = fma(wb[l], lor, d);
-      if (pdos)
-        for (int a = 0; a < m; ++a) {
-          const double2 f = phi[a * n + l];
-          pd[a] = fma(fma(f.x, f.x, f.y * f.y), lor, pd[a]);
+    for (int l0 = 0; l0 < n; l0 += kDosL) {
+      const int cl = min(kDosL, n - l0);
+      __syncthreads();
+      for (int i = threadIdx.x; i < cl * kDosT; i += 128) {
+        const int t = i / cl, l = i - t * cl, c = c0 + t;
+        double w = 0.0;
+        if (c == 0) {
+          w = wb[l0 + l];
+        } else if (c <= m) {
+          const double2 f = phi[(c - 1) * n + l0 + l];
+          w = fma(f.x, f.x, f.y * f.y);
         }
+        s_w[l][t] = wk * w;
+        if (t == 0) s_e[l] = E[l0 + l];
+      }
+      __syncthreads();
+      for (int l = 0; l < cl; ++l) {
+        const double x = z - s_e[l], lor = 1.0 / fma(x, x, e2);
+#pragma unroll
+        for (int t = 0; t < kDosT; ++t) acc[t] = fma(s_w[l][t], lor, acc[t]);
+      }
     }
   }
-  dos[(int64_t)s * n_eps + ie] = d;
-  if (pdos)
-    for (int a = 0; a < m; ++a) pdos[pdos_off[s] + (int64_t)ie * m + a] = pd[a];
+  if (ie >= n_eps) return;
+  double* out = part + (((int64_t)blockIdx.z * gridDim.y + s) * n_eps + ie) * (1 + mmax);
+#pragma unroll
+  for (int t = 0; t < kDosT; ++t)
+    if (c0 + t < n_ch && c0 + t <= m) out[c0 + t] = acc[t];
+}
+
+// Sums of the splits, in order, to dos [system][energy] and pdos (per system [energy][m], or null).
+__global__ void k_dos_reduce(const SInfo* __restrict__ sinfo, const double* __restrict__ part, int n_split, int n_sys,
+                             int n_eps, int mmax, const int64_t* __restrict__ pdos_off, double* __restrict__ dos,
+                             double* __restrict__ pdos) {
+  const int s = blockIdx.y, m = sinfo[s].m, ch = 1 + (pdos ? m : 0);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_eps * ch; i += gridDim.x * blockDim.x) {
+    const int ie = i / ch, c = i - ie * ch;
+    double v = 0.0;
+    for (int z = 0; z < n_split; ++z) v += part[(((int64_t)z * n_sys + s) * n_eps + ie) * (1 + mmax) + c];
+    if (c == 0) dos[(int64_t)s * n_eps + ie] = v;
+    else pdos[pdos_off[s] + (int64_t)ie * m + c - 1] = v;
+  }
 }
 
 // Orthonormal projectors of Eqs. 6 and 7 (Lowdin):
 // P_k = O^{-1/2} W_k, O = W_k W_k^+ (m x m), one CTA per k.  O's eigenpairs by
-// the Jacobi routine; eigenvalues <= tol * max eigenvalue flag the k-point
+// heev_tri; eigenvalues <= tol * max eigenvalue flag the k-point
 // (linearly dependent projections).
 __global__ void __launch_bounds__(kEigThreads)
     k_lowdin(const KInfo* __restrict__ kinfo, const SInfo* __restrict__ sinfo,
              const double2* __restrict__ Wraw, double2* __restrict__ Pout, int mmax, int* status) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ double rot[4 * 16];
-  __shared__ double2 ph[16];
-  __shared__ double red[kEigThreads / 32];
+  __shared__ QlScratch ql;
   __shared__ double s_isq[32];
   const int k = blockIdx.x;
   const KInfo ki = kinfo[k];
@@ -672,19 +1161,22 @@ __global__ void __launch_bounds__(kEigThreads)
   double2* V = O + M * ld;
   double2* T = V + M * ld;  // O^{-1/2}
   const double2* Wk = Wraw + ki.offP;
-  for (int e = threadIdx.x; e < M * M; e += kEigThreads) {
-    const int a = e / M, b = e - (e / M) * M;
+  for (int e = threadIdx.x; e < M * (M + 1) / 2; e += kEigThreads) {
+    int a, b;
+    tri_pair(e, a, b);
     double2 acc = make_double2(0.0, 0.0);
     for (int j = 0; j < N; ++j) cmac_cb(acc, Wk[a * N + j], Wk[b * N + j]);
+    if (a == b) acc.y = 0.0;
     O[a * ld + b] = acc;
+    O[b * ld + a] = make_double2(acc.x, -acc.y);
   }
   __syncthreads();
-  const int sw = jacobi_heev(O, V, M, ld, 40, rot, ph, red);
-  if (sw < 0 && threadIdx.x == 0) atomicOr(status, 2);
-  if (threadIdx.x == 0) {
+  const bool ok = heev_tri(O, V, M, ld, 1, 0, smraw, ql);
+  if (!ok && threadIdx.x == 0) atomicOr(status, 2);
+  if (threadIdx.x < 32) {
     double lmax = 0.0;
     for (int l = 0; l < M; ++l) lmax = fmax(lmax, O[l * ld + l].x);
-    for (int l = 0; l < M; ++l) {
+    for (int l = threadIdx.x; l < M; l += 32) {
       const double lam = O[l * ld + l].x;
       if (!(lam > 1e-12 * lmax)) {
         atomicOr(status, kFlagSingular);
@@ -695,8 +1187,9 @@ __global__ void __launch_bounds__(kEigThreads)
     }
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < M * M; e += kEigThreads) {
-    const int a = e / M, b = e - (e / M) * M;
+  for (int e = threadIdx.x; e < M * (M + 1) / 2; e += kEigThreads) {
+    int a, b;
+    tri_pair(e, a, b);
     double2 acc = make_double2(0.0, 0.0);
     for (int l = 0; l < M; ++l) {
       double2 v = V[a * ld + l];
@@ -705,6 +1198,7 @@ __global__ void __launch_bounds__(kEigThreads)
       cmac_cb(acc, v, V[b * ld + l]);
     }
     T[a * ld + b] = acc;
+    T[b * ld + a] = make_double2(acc.x, -acc.y);
   }
   __syncthreads();
   for (int e = threadIdx.x; e < M * N; e += kEigThreads) {
@@ -716,6 +1210,13 @@ __global__ void __launch_bounds__(kEigThreads)
 }
 
 }  // namespace
+
+// Dynamic shared memory of the real scratch of heev_tri when the matrices are in a global slice
+// (0: it takes V's place there); heev_tri's static arrays leave 200 KB.
+size_t ql_z_bytes(int n) {
+  const size_t z = sizeof(double) * (size_t)n * (n | 1);
+  return z <= (200u << 10) ? z : 0;
+}
 
 cudaError_t launch_lr_setup(const double2* H, const double2* P, const KInfo* kinfo,
                             const SInfo* sinfo, const int64_t* offD, int n_k, int nbmax,
@@ -731,10 +1232,11 @@ cudaError_t launch_lr_setup(const double2* H, const double2* P, const KInfo* kin
 }
 
 cudaError_t launch_block_eig(const BlockSetup& b, double2* ws, int grid, int in_smem, cudaStream_t s) {
-  const size_t smem = in_smem ? heev_smem(b.n2max) : 0;
+  const size_t zb = in_smem ? 0 : ql_z_bytes(b.n2max);
+  const size_t smem = in_smem ? heev_smem(b.n2max) : zb;
   cudaError_t e = cudaFuncSetAttribute(k_block_eig, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_block_eig<<<grid, kEigThreads, smem, s>>>(b, ws, in_smem);
+  k_block_eig<<<grid, kEigThreads, smem, s>>>(b, ws, in_smem, zb > 0);
   return cudaGetLastError();
 }
 
@@ -747,11 +1249,22 @@ cudaError_t launch_lowdin(const KInfo* kinfo, const SInfo* sinfo, int n_k, int m
   return cudaGetLastError();
 }
 
-cudaError_t launch_pole_dos(const PoleParams& p, int n_sys, const double* eps_grid, int n_eps,
-                            double eta, const int64_t* pdos_off, double* dos, double* pdos,
+// k-splits of k_pole_dos: about four CTAs per SM, and at least one k-point each.
+int pole_dos_splits(int n_sys, int n_eps, int n_ch, int n_k, int sm_count) {
+  const int blocks = n_sys * ((n_eps + 127) / 128) * ((n_ch + kDosT - 1) / kDosT);
+  return std::max(1, std::min({64, n_k, (4 * sm_count + blocks - 1) / blocks}));
+}
+
+cudaError_t launch_pole_dos(const PoleParams& p, int n_sys, const double* eps_grid, int n_eps, double eta, int mmax,
+                            int n_split, double* part, const int64_t* pdos_off, double* dos, double* pdos,
                             cudaStream_t s) {
-  dim3 grid((n_eps + 127) / 128, n_sys);
-  k_pole_dos<<<grid, 128, 0, s>>>(p, eps_grid, n_eps, eta, pdos_off, dos, pdos);
+  const int n_ch = 1 + (pdos ? mmax : 0);
+  const dim3 grid(((n_eps + 127) / 128) * ((n_ch + kDosT - 1) / kDosT), n_sys, n_split);
+  k_pole_dos<<<grid, 128, 0, s>>>(p, eps_grid, n_eps, eta, n_ch, mmax, part);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_dos_reduce<<<dim3(std::min(1024, (n_eps * n_ch + 127) / 128), n_sys), 128, 0, s>>>(p.sinfo, part, n_split, n_sys,
+                                                                                   n_eps, mmax, pdos_off, dos, pdos);
   return cudaGetLastError();
 }
 

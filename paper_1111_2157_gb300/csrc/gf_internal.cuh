@@ -114,6 +114,7 @@ struct PoleParams {
   const double* mu;     // [n_sys]
   int n_k, n_iw, mode, max_sweeps;
   int in_smem;          // 1: H_ps and its eigenvectors in shared memory
+  int z_smem;           // else 1: the eigensolver's real scratch is
   double2* ws;          // else per-CTA slices of ws_stride elements
   int64_t ws_stride;
   double* kN;           // [n_k] N_k
@@ -128,13 +129,6 @@ struct PoleParams {
   double* wbout;        // band weights |Psi_b,l|^2 per k at eoff[k] (kGloc), or null
   double* kHks;         // [n_k] Re Tr(H_k rho_k) (kRho), or null
   double* kEps;         // [n_k] sum_l (E_l - mu) |Psi_b,l|^2 n_F (kRho), or null
-  // warm start of the mu search: eigenpairs of the previous evaluation
-  double2* vstore;      // eigenvectors per k, [n][n] at voff[k] (row i, column l), or null
-  double* estore;       // eigenvalues per k at eoff[k]
-  const int64_t* voff;
-  const double* mu_prev;  // [n_sys] mu of the stored eigenpairs
-  int warm;             // 1: start Jacobi from the stored eigenpairs
-  int save_v;           // 1: store this evaluation's eigenpairs
   int* status;
 };
 
@@ -249,6 +243,7 @@ cudaError_t launch_lowdin(const KInfo* kinfo, const SInfo* sinfo, int n_k, int m
 
 // Batched Hermitian eigensolver (cyclic Jacobi) and the pole path.
 size_t heev_smem(int n);
+constexpr size_t kQlStatic = 28672;  // static shared memory of the QR eigensolver's kernels (upper limit)
 size_t heev_ws_elems(int n);
 int heev_max_n();
 cudaError_t launch_heev_batched(const double2* A, int n_mat, int n, int max_sweeps, double* w,
@@ -260,9 +255,12 @@ cudaError_t launch_pole_eig(const PoleParams& p, int grid, size_t smem, cudaStre
 int pole_gloc_splits(int n_sys, int n_iw, int sm_count, int mmax);
 cudaError_t launch_pole_gloc(const PoleParams& p, int n_sys, int mmax, int n_split, double2* part,
                              int64_t tot, cudaStream_t s);
-cudaError_t launch_pole_dos(const PoleParams& p, int n_sys, const double* eps_grid, int n_eps,
-                            double eta, const int64_t* pdos_off, double* dos, double* pdos,
+// DOS and PDOS, k split n_split ways into part [n_split][n_sys][n_eps][1 + mmax].
+int pole_dos_splits(int n_sys, int n_eps, int n_ch, int n_k, int sm_count);
+cudaError_t launch_pole_dos(const PoleParams& p, int n_sys, const double* eps_grid, int n_eps, double eta, int mmax,
+                            int n_split, double* part, const int64_t* pdos_off, double* dos, double* pdos,
                             cudaStream_t s);
+size_t ql_z_bytes(int n);
 
 // Shared-memory layout of the point kernels, in 16-byte complex elements (a
 // complex double or a complex FP32 pair): the N_b x N_b matrix (odd leading

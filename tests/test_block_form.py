@@ -127,6 +127,39 @@ def test_block_kernels_equal_the_general_ones(nk, nb, m, n_iw, rows, ragged):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["diagonal", "degenerate", "nearly_degenerate", "scalar", "split"])
+def test_levels_that_the_parallel_eigenvectors_cannot_separate(kind):
+    """Degenerate, nearly degenerate and split blocks take the QR steps: same results as the general kernels, on the
+    block form and (against its own oracle) on the pole path."""
+    from oracle import pole as pole_oracle
+    from paper_1111_2157_gb300 import gf
+    s = _inputs(3, 30, 5, 40, 40.0, 21)
+    rng = np.random.default_rng(4)
+    for k in range(3):
+        U = np.linalg.qr(rng.standard_normal((30, 30)) + 1j * rng.standard_normal((30, 30)))[0]
+        lev = np.repeat(np.arange(6.0) - 2.5, 5)
+        if kind == "nearly_degenerate":
+            lev = lev + 1e-9 * rng.standard_normal(30)
+        H = {"diagonal": np.diag(rng.uniform(-4, 4, 30)).astype(complex), "scalar": 0.7 * np.eye(30, dtype=complex),
+             "split": np.kron(np.eye(3), s.H[k, :10, :10])}.get(kind, (U * lev) @ np.conj(U.T))
+        s.H[k] = 0.5 * (H + np.conj(H.T))
+    a, log = _run(s, None)
+    b, _ = _run(s, "direct")
+    assert "mode 7: block form" in log
+    for key in b:
+        assert _rel(a[key], b[key]) < 1e-10, key
+    g = gf.GreensFunction.for_systems([s])
+    g.set_hamiltonian(s.H)
+    g.set_projectors(s.P)
+    g.set_sigma_poles([len(s.pole.p)], s.pole.p, s.pole.V.reshape(-1), s.pole.sigma_inf.reshape(-1))
+    n, dn = g.pole_occupation([0.1])
+    r = pole_oracle.density(s.H, s.P, s.sigma_inf, s.pole.p, s.pole.V, s.beta, 0.1)
+    assert abs(n[0] - r["N"]) < 1e-10 * r["N"]
+    assert _rel(g.pole_density_matrix([0.1])[0].cpu().numpy().reshape(3, 30, 30), r["rho"]) < 1e-10
+    g.close()
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("nk,nb,m,n_iw", [(3, 40, 14, 200), (2, 96, 20, 70), (2, 24, 7, 300)])
 def test_mixed_block_kernels_against_fp64(nk, nb, m, n_iw):
     """The mixed contract (N 1e-7, G_loc 1e-8, rho 1e-5, dN/dmu 1e-5, n_corr 1e-6) on both sides of the FP64 limit."""
