@@ -20,12 +20,14 @@
 
 #include "gf_block.cuh"
 #include "gf_complex.cuh"
+#include "gf_gj64.cuh"
 
 namespace gf {
 
 namespace {
 
 using namespace cx;
+using gj64::crcp_scaled;
 
 constexpr int kSetupThreads = 256;
 
@@ -381,17 +383,6 @@ __device__ __forceinline__ float2 rzero(float2) { return make_float2(0.f, 0.f); 
 __device__ __forceinline__ double rfma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
-// 1 / a with one division: scaled by a power of two near 1 / max(|Re|, |Im|) (bit arithmetic),
-// so that the squared modulus neither overflows nor underflows.
-__device__ __forceinline__ double2 crcp_scaled(double2 a, unsigned long long key) {
-  int ex = 2046 - (int)(key >> 52);
-  ex = ex < 1 ? 1 : ex;
-  const double s = __longlong_as_double((long long)ex << 52);
-  const double x = a.x * s, y = a.y * s;
-  const double q = s / fma(x, x, y * y);
-  return make_double2(x * q, -y * q);
-}
-
 // Coefficients of the Chebyshev series at z (x = (z - c) / r, s = sqrt(x^2 - 1), xi = x - s):
 //   1/(z - e)   = sum_j eps_j xi^j / (r s) T_j,                                eps_0 = 1, eps_j = 2
 //   1/(z - e)^2 = sum_j eps_j xi^j [j/s^2 + x/s^3] / r^2 T_j                    (-d/dz)
@@ -459,11 +450,9 @@ struct LayoutB {
   int yf;   // frequencies of the rho_k columns staged at once
 };
 
-__host__ __device__ inline int block_lanes(int m) { return m <= 8 ? 8 : (m <= 16 ? 16 : 32); }
-
 __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, int low) {
   LayoutB L;
-  L.nf = 32 / block_lanes(mmax);
+  L.nf = 32 / gj64::lanes(mmax);
   const size_t f = L.nf, mm = (size_t)mmax * mmax, r = low ? 8 : 16, W = kBlkWarps;
   const bool needF = (mode & (kOcc | kAdj)) != 0, rho = (mode & kRho) != 0;
   auto al = [](size_t x) { return (x + 15) & ~(size_t)15; };
@@ -515,58 +504,6 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
 
 __device__ __forceinline__ double2 ld_cg(const double2* p) { return __ldg(p); }
 __device__ __forceinline__ float2 ld_cg(const float2* p) { return __ldg(p); }
-
-// S^{-1} in place for the warp's matrices: LW lanes each, Gauss-Jordan in exchange form with
-// partial pivoting and no row interchanges (X[i][c] = A[p_i][q_c], q = p^{-1}).  Every lane
-// group holds a valid matrix, so no lane diverges.
-template <int LW>
-__device__ __forceinline__ void block_invert(double2* A, int M, double2* rc, int* sp, int sl, int* status) {
-  double2* su = rc;
-  double2* sc = rc + M;
-  int* sq = sp + M;
-  bool used = sl >= M;
-  for (int j = 0; j < M; ++j) {
-    unsigned long long best = used ? 0ULL : pivot_key(A[sl * M + j]);
-    int bi = used ? 0x7fffffff : sl;
-    for (int off = LW / 2; off; off >>= 1) {
-      const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, off);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-      if (ob > best || (ob == best && oi < bi)) {
-        best = ob;
-        bi = oi;
-      }
-    }
-    if (sl == 0 && (best == 0ULL || best >= 0x7ff0000000000000ULL)) atomicOr(status, kFlagSingular);
-    const double2 r = crcp_scaled(A[bi * M + j], best);
-    if (sl < M) {
-      const double2 u = A[bi * M + sl], l = A[sl * M + j];
-      su[sl] = (sl == j) ? r : cmul(u, r);
-      sc[sl] = (sl == bi) ? make_double2(-1.0, 0.0) : l;
-    }
-    if (sl == bi) used = true;
-    if (sl == 0) {
-      sp[j] = bi;
-      sq[bi] = j;
-    }
-    __syncwarp();
-    int i = sl / M, c = sl - (sl / M) * M;
-    const int di = LW / M, dc = LW - (LW / M) * M;
-    for (int e = sl; e < M * M; e += LW) {
-      const double2 l = sc[i], u = su[c];
-      double2 v = (i == bi || c == j) ? make_double2(0.0, 0.0) : A[e];
-      v.x = fma(-l.x, u.x, fma(l.y, u.y, v.x));
-      v.y = fma(-l.x, u.y, fma(-l.y, u.x, v.y));
-      A[e] = v;
-      i += di;
-      c += dc;
-      if (c >= M) {
-        c -= M;
-        ++i;
-      }
-    }
-    __syncwarp();
-  }
-}
 
 template <int LW, bool LOW>
 __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
@@ -793,7 +730,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
           if (a != c) Sm[c * M + a] = v;
         }
         __syncwarp();
-        block_invert<LW>(A, M, rcb, sp, sl, p.status);
+        gj64::invert<LW>(A, M, rcb, sp, sl, p.status);
         const int* sq = sp + M;
         const bool mine = mf < nv;
         double2* out = (p.mode & (kGloc | kAdj))
@@ -1283,14 +1220,14 @@ cudaError_t launch_block_finish(const BlockSetup& b, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-int block_batch(int mmax) { return kBlkWarps * (32 / block_lanes(mmax)); }
+int block_batch(int mmax) { return kBlkWarps * (32 / gj64::lanes(mmax)); }
 
 size_t block_smem(int mmax, int n2max, int mode, int low) { return make_layout_b(mmax, n2max, mode, low).bytes; }
 
 cudaError_t launch_point_block(const PointParams& p, const BlockForm& b, const BlockLaunch& l, int low,
                                cudaStream_t s) {
   const size_t smem = block_smem(p.mmax, l.n2max, p.mode, low);
-  switch (block_lanes(p.mmax) + (low ? 1 : 0)) {
+  switch (gj64::lanes(p.mmax) + (low ? 1 : 0)) {
     case 8: return launch_lw<8, false>(p, b, l, smem, s);
     case 9: return launch_lw<8, true>(p, b, l, smem, s);
     case 16: return launch_lw<16, false>(p, b, l, smem, s);

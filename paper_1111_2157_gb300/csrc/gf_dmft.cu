@@ -3,14 +3,15 @@
 //   k_eimp_part, k_eimp_reduce E_imp = sum_k w_k P_k H_k P_k^+ - V_DC I   (Eq. E^imp)
 //   k_hybridization            Delta(i w_n) = (i w_n + mu) I - E_imp - Sigma(i w_n)
 //                                             - G_loc(i w_n)^{-1}          (Eq. dmftloop2)
-//                              one warp per (system, frequency): m x m inverse
-//                              by Gauss-Jordan on [G_loc | I] in shared memory
+//                              one to four frequencies per warp, the m x m inverses
+//                              in shared memory (gf_gj64.cuh)
 // (The orthonormal projectors of Eqs. 6 and 7, k_lowdin, live in gf_eig.cu
-// beside the Jacobi eigensolver they use.)
+// beside the eigensolver they use.)
 #include <math.h>
 #include <stdint.h>
 
 #include "gf_complex.cuh"
+#include "gf_gj64.cuh"
 #include "gf_internal.cuh"
 
 namespace gf {
@@ -48,101 +49,90 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// out[s][e] = sum over the k of system s, in increasing k, of part[k][e] (m_s^2 entries),
-// minus v_dc[s] on the diagonal.
-__global__ void k_eimp_reduce(const SInfo* __restrict__ sinfo, const double2* __restrict__ part,
-                              int mmax, const double* __restrict__ v_dc, double2* __restrict__ out) {
-  const SInfo si = sinfo[blockIdx.x];
-  const int M = si.m;
-  for (int e = threadIdx.x; e < M * M; e += blockDim.x) {
-    double2 acc = make_double2(0.0, 0.0);
-    for (int k = si.k0; k < si.k1; ++k) {
+// out[s][e] = sum over the k of system s of part[k][e] (m_s^2 entries), minus v_dc[s] on the
+// diagonal.  kRedE consecutive entries per CTA and 32 k-strides each, summed in a fixed tree: one
+// CTA per system left a chain of n_k loads per entry (0.25 -> 0.02 ms at 1000 k-points).
+constexpr int kRedE = 8;
+__global__ void __launch_bounds__(32 * kRedE)
+    k_eimp_reduce(const SInfo* __restrict__ sinfo, const double2* __restrict__ part, int mmax,
+                  const double* __restrict__ v_dc, double2* __restrict__ out) {
+  __shared__ double2 s_v[32][kRedE];
+  const SInfo si = sinfo[blockIdx.y];
+  const int M = si.m, t = threadIdx.x % kRedE, r = threadIdx.x / kRedE, e = blockIdx.x * kRedE + t;
+  double2 acc = make_double2(0.0, 0.0);
+  if (e < M * M)
+    for (int k = si.k0 + r; k < si.k1; k += 32) {
       const double2 v = part[(int64_t)k * mmax * mmax + e];
       acc.x += v.x;
       acc.y += v.y;
     }
-    const int a = e / M, b = e - (e / M) * M;
-    if (a == b && v_dc) acc.x -= v_dc[blockIdx.x];
+  s_v[r][t] = acc;
+  for (int h = 16; h; h >>= 1) {
+    __syncthreads();
+    if (r < h) {
+      s_v[r][t].x += s_v[r + h][t].x;
+      s_v[r][t].y += s_v[r + h][t].y;
+    }
+  }
+  if (r == 0 && e < M * M) {
+    acc = s_v[0][t];
+    if (e / M == e % M && v_dc) acc.x -= v_dc[blockIdx.y];
     out[si.offSinf + e] = acc;
   }
 }
 
 constexpr int kHybWarps = 4;
 
-// Delta for one (system, frequency) per warp; lane i owns row i of [G | I].
+// Delta for 32 / LW frequencies of one system per warp.  Bound by the FP64 pipe: in place with
+// LW lanes per matrix the elimination keeps 94 % of the lanes at m = 14, where one row per lane of
+// [G | I] kept 44 % and took twice the columns (0.17 -> 0.04 ms at 1024 frequencies, m = 14).
+template <int LW>
 __global__ void __launch_bounds__(32 * kHybWarps)
-    k_hybridization(const SInfo* __restrict__ sinfo, int n_sys, int n_iw, int mmax,
-                    const double* __restrict__ mu, const double2* __restrict__ eimp,
-                    const double2* __restrict__ Sig, const double2* __restrict__ gloc,
-                    double2* __restrict__ delta, int* status) {
+    k_hybridization(const SInfo* __restrict__ sinfo, int n_iw, int mmax, const double* __restrict__ mu,
+                    const double2* __restrict__ eimp, const double2* __restrict__ Sig,
+                    const double2* __restrict__ gloc, double2* __restrict__ delta, int* status) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int task = blockIdx.x * kHybWarps + warp;
-  if (task >= n_sys * n_iw) return;
-  const int s = task / n_iw, n = task - (task / n_iw) * n_iw;
+  constexpr int F = 32 / LW;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sl = lane % LW, mf = lane / LW;
+  const int n0 = (blockIdx.x * kHybWarps + warp) * F, s = blockIdx.y;
+  if (n0 >= n_iw) return;
   const SInfo si = sinfo[s];
-  const int M = si.m, W = 2 * M;
-  double2* aug = reinterpret_cast<double2*>(smraw) + (size_t)warp * mmax * 2 * mmax;
-  const double2* G = gloc + si.offSig + (int64_t)n * M * M;
-  for (int e = lane; e < M * W; e += 32) {
-    const int i = e / W, c = e - (e / W) * W;
-    aug[e] = c < M ? G[i * M + c] : make_double2(c - M == i ? 1.0 : 0.0, 0.0);
-  }
+  const int M = si.m, MM = M * M, n = min(n0 + mf, n_iw - 1);  // the last warp repeats its last one
+  const size_t wstride = 16 * (size_t)F * (mmax * mmax + 2 * mmax) + 8 * (size_t)F * mmax;
+  unsigned char* wb = smraw + warp * ((wstride + 15) & ~(size_t)15);
+  double2* A = reinterpret_cast<double2*>(wb) + mf * MM;
+  double2* rc = reinterpret_cast<double2*>(wb) + F * mmax * mmax + mf * 2 * M;
+  int* sp = reinterpret_cast<int*>(wb + 16 * (size_t)F * (mmax * mmax + 2 * mmax)) + mf * 2 * M;
+  const int64_t off = si.offSig + (int64_t)n * MM;
+  for (int e = sl; e < MM; e += LW) A[e] = gloc[off + e];
   __syncwarp();
-  bool singular = false;
-  for (int j = 0; j < M; ++j) {
-    unsigned long long best = 0ULL;
-    int bi = 0x7fffffff;
-    for (int i = j + lane; i < M; i += 32) {
-      const unsigned long long key = pivot_key(aug[i * W + j]);
-      if (bi == 0x7fffffff || key > best) { best = key; bi = i; }
-    }
-    for (int off = 16; off; off >>= 1) {
-      const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, off);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-    }
-    if (best == 0ULL || best >= 0x7ff0000000000000ULL) singular = true;
-    if (bi != j)
-      for (int c = lane; c < W; c += 32) {
-        const double2 t = aug[j * W + c];
-        aug[j * W + c] = aug[bi * W + c];
-        aug[bi * W + c] = t;
-      }
-    __syncwarp();
-    const double2 r = crcp(aug[j * W + j]);
-    __syncwarp();
-    for (int c = lane; c < W; c += 32) aug[j * W + c] = c == j ? make_double2(1.0, 0.0) : cmul(aug[j * W + c], r);
-    __syncwarp();
-    for (int i = lane; i < M; i += 32) {
-      if (i == j) continue;
-      const double2 l = aug[i * W + j];
-      for (int c = 0; c < W; ++c) {
-        const double2 u = aug[j * W + c];
-        double2 v = aug[i * W + c];
-        v.x = fma(-l.x, u.x, fma(l.y, u.y, v.x));
-        v.y = fma(-l.x, u.y, fma(-l.y, u.x, v.y));
-        aug[i * W + c] = v;
-      }
-      aug[i * W + j] = make_double2(0.0, 0.0);
-    }
-    __syncwarp();
-  }
-  if (singular && lane == 0) atomicOr(status, kFlagSingular);
+  gj64::invert<LW>(A, M, rc, sp, sl, status);
+  const int* sq = sp + M;
   const double wn = (2.0 * n + 1.0) * 3.14159265358979323846 / si.beta;
-  const double2* Sg = Sig + si.offSig + (int64_t)n * M * M;
-  const double2* E = eimp + si.offSinf;
-  double2* D = delta + si.offSig + (int64_t)n * M * M;
-  for (int e = lane; e < M * M; e += 32) {
-    const int i = e / M, c = e - (e / M) * M;
-    const double2 g = aug[i * W + M + c], sg = Sg[e], ei = E[e];
+  if (n0 + mf >= n_iw) return;
+  for (int e = sl; e < MM; e += LW) {
+    const int i = e / M, c = e - i * M;
+    const double2 g = A[sp[i] * M + sq[c]], sg = Sig[off + e], ei = eimp[si.offSinf + e];
     double2 v = make_double2(-ei.x - sg.x - g.x, -ei.y - sg.y - g.y);
     if (i == c) {
       v.x += mu[s];
       v.y += wn;
     }
-    D[e] = v;
+    delta[off + e] = v;
   }
+}
+
+template <int LW>
+cudaError_t launch_hyb(const SInfo* sinfo, int n_sys, int n_iw, int mmax, const double* mu, const double2* eimp,
+                       const double2* Sig, const double2* gloc, double2* delta, int* status, cudaStream_t s) {
+  constexpr int F = 32 / LW;
+  const size_t w = 16 * (size_t)F * (mmax * mmax + 2 * mmax) + 8 * (size_t)F * mmax;
+  const size_t smem = kHybWarps * ((w + 15) & ~(size_t)15);
+  cudaError_t e = cudaFuncSetAttribute(k_hybridization<LW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_hybridization<LW><<<dim3((n_iw + kHybWarps * F - 1) / (kHybWarps * F), n_sys), 32 * kHybWarps, smem, s>>>(
+      sinfo, n_iw, mmax, mu, eimp, Sig, gloc, delta, status);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -156,22 +146,18 @@ cudaError_t launch_eimp(const KInfo* kinfo, const SInfo* sinfo, int n_k, int n_s
   k_eimp_part<<<n_k, kThreads, smem, s>>>(kinfo, sinfo, H, P, mmax, part);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_eimp_reduce<<<n_sys, kThreads, 0, s>>>(sinfo, part, mmax, v_dc, out);
+  k_eimp_reduce<<<dim3((mmax * mmax + kRedE - 1) / kRedE, n_sys), 32 * kRedE, 0, s>>>(sinfo, part, mmax, v_dc, out);
   return cudaGetLastError();
 }
 
 cudaError_t launch_hybridization(const SInfo* sinfo, int n_sys, int n_iw, int mmax, const double* mu,
                                  const double2* eimp, const double2* Sig, const double2* gloc,
                                  double2* delta, int* status, cudaStream_t s) {
-  const size_t smem = (size_t)kHybWarps * mmax * 2 * mmax * sizeof(double2);
-  cudaError_t e =
-      cudaFuncSetAttribute(k_hybridization, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  const int tasks = n_sys * n_iw;
-  const int grid = (tasks + kHybWarps - 1) / kHybWarps;
-  k_hybridization<<<grid, 32 * kHybWarps, smem, s>>>(sinfo, n_sys, n_iw, mmax, mu, eimp, Sig, gloc,
-                                                      delta, status);
-  return cudaGetLastError();
+  switch (gj64::lanes(mmax)) {
+    case 8: return launch_hyb<8>(sinfo, n_sys, n_iw, mmax, mu, eimp, Sig, gloc, delta, status, s);
+    case 16: return launch_hyb<16>(sinfo, n_sys, n_iw, mmax, mu, eimp, Sig, gloc, delta, status, s);
+    default: return launch_hyb<32>(sinfo, n_sys, n_iw, mmax, mu, eimp, Sig, gloc, delta, status, s);
+  }
 }
 
 }  // namespace gf
