@@ -440,12 +440,13 @@ __device__ __forceinline__ int series_terms(float dx, float w, float r, float bi
 
 // Shared memory of the point kernel in bytes; every array holds the CTA's W F frequencies, warp
 // after warp.  First what is dead once the warps have S^{-1}: F, d^2 / d^3, the pivot row and
-// column, Gbar A^+ (adjoint), and with LOW also S (rho_k then reads the FP32 copy of S^{-1});
-// the columns S^{-1} B D of rho_k are staged over it, yf frequencies at a time.  Then S, the
-// copy, d (and the series coefficients), the pivot tables, the pair list and, with LOW, B.
+// column, Gbar A^+ (adjoint), and with LOW also S and the refinement's residual (rho_k then reads
+// S^{-1} in FP32); the columns S^{-1} B D of rho_k are staged over it, yf frequencies at a time.
+// Then S, with LOW S^{-1} in FP32, d (or the series coefficients), the pivot tables, w_n, the pair
+// list, mu O - H11 by pairs and, with LOW, B.
 struct LayoutB {
-  size_t oS, oF, od2, orc, oM, oY, oG, od, odc, op, oPair, oB, bytes;
-  size_t sS, sF, sd2, src, sG, sd, sdc, sp;  // bytes per warp (sS also of M)
+  size_t oS, oF, od2, orc, oM, oR, oY, oG, od, op, oW, oPair, oHz, oB, bytes;
+  size_t sS, sF, sd2, src, sG, sd, sp;  // bytes per warp (sS also of M, sG of R)
   int nf;   // frequencies per warp
   int yf;   // frequencies of the rho_k columns staged at once
 };
@@ -456,14 +457,12 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   const size_t f = L.nf, mm = (size_t)mmax * mmax, r = low ? 8 : 16, W = kBlkWarps;
   const bool needF = (mode & (kOcc | kAdj)) != 0, rho = (mode & kRho) != 0;
   auto al = [](size_t x) { return (x + 15) & ~(size_t)15; };
-  const size_t jt = n2max < kBlkSeries ? n2max : kBlkSeries;
   L.sS = 16 * f * mm;
   L.sF = needF ? al(r * f * mm) : 0;
   L.sd2 = needF ? al(2 * r * f * n2max) : 0;
-  L.src = 16 * f * 2 * mmax;
+  L.src = (low ? 8 : 16) * f * 2 * mmax;
   L.sG = low ? al(8 * f * mm) : 0;
   L.sd = 16 * f * n2max;
-  L.sdc = rho ? 16 * f * jt : 0;  // rho_k reads d_b also where the sums run over the moments
   L.sp = al(4 * f * 2 * mmax);
   size_t o = 0;
   if (!low) { L.oS = o; o += W * L.sS; }
@@ -473,7 +472,9 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   L.od2 = o; o += W * L.sd2;
   L.orc = o; o += W * L.src;
   L.oM = o; o += (mode & kAdj) ? W * L.sS : 0;
-  const size_t fixed = W * (L.sG + L.sd + L.sdc + L.sp) + al((size_t)mmax * (mmax + 1)) +
+  L.oR = o; o += W * L.sG;
+  const size_t np = (size_t)mmax * (mmax + 1) / 2;
+  const size_t fixed = W * (L.sG + L.sd + L.sp + 8 * f) + al(2 * np) + 16 * np +
                        (low && rho ? 8 * mmax * (((size_t)n2max + 3) & ~(size_t)3) : 0);
   L.yf = 0;
   if (rho) {
@@ -493,10 +494,10 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   }
   L.oG = o; o += W * L.sG;
   L.od = o; o += W * L.sd;
-  L.odc = rho ? o : L.od;
-  o += W * L.sdc;
   L.op = o; o += W * L.sp;
-  L.oPair = o; o += al((size_t)mmax * (mmax + 1));
+  L.oW = o; o = al(o + 8 * W * f);
+  L.oPair = o; o += al(2 * np);
+  L.oHz = o; o += 16 * np;
   L.oB = o; o += low && rho ? 8 * mmax * (((size_t)n2max + 3) & ~(size_t)3) : 0;
   L.bytes = o;
   return L;
@@ -523,7 +524,9 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
   double2* sM = reinterpret_cast<double2*>(smraw + L.oM + wp * L.sS);
   float2* sG = reinterpret_cast<float2*>(smraw + L.oG + wp * L.sG);
   int* sPv = reinterpret_cast<int*>(smraw + L.op + wp * L.sp);
+  double* sW = reinterpret_cast<double*>(smraw + L.oW) + wp * F;
   uchar2* pair = reinterpret_cast<uchar2*>(smraw + L.oPair);
+  double2* hz = reinterpret_cast<double2*>(smraw + L.oHz);
   const int unit = bl.unit0 + blockIdx.x / bl.n_chunks, ch = blockIdx.x % bl.n_chunks;
   const int2 un = bl.units[unit];
   const int n0 = bl.n_begin + ch * bl.chunk_w, n1 = min(bl.n_end, n0 + bl.chunk_w);
@@ -542,13 +545,15 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
     const double cb = (adj && p.nbar) ? p.nbar[ki.sys] * 2.0 / si.beta : 0.0;
     const bool have_gbar = adj && p.gbar != nullptr;
     double2* A = sS + mf * MM;  // this lane group's matrix
-    double2* rcb = reinterpret_cast<double2*>(smraw + L.orc + wp * L.src) + mf * 2 * M;
+    rc_t* rcb = reinterpret_cast<rc_t*>(smraw + L.orc + wp * L.src) + mf * 2 * M;
     int* sp = sPv + mf * 2 * M;
     __syncthreads();
     for (int pr = tid; pr < NP; pr += 32 * W) {
       int a = 0, rem = pr;
       while (rem >= M - a) { rem -= M - a; ++a; }
       pair[pr] = make_uchar2((unsigned char)a, (unsigned char)(a + rem));
+      const double2 h = HO[pr], o = HO[bf.npmax + pr];
+      hz[pr] = make_double2(fma(mu, o.x, -h.x), fma(mu, o.y, -h.y));
     }
     if constexpr (LOW) {
       if (rho) {
@@ -570,7 +575,9 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
         const double2* Tt = T;
         const float2* Tst = nullptr;
         if constexpr (LOW) Tst = bf.Ts + bf.offT[kk];
-        double2* dv = sd;
+        bool series = false;
+        if (lane < F) sW[lane] = (2.0 * min(n + lane, n1 - 1) + 1.0) * pib;
+        __syncwarp();
         {
           const double2 cr = bf.cr[kk];
           const int J = series_terms((float)(mu - cr.x), (float)((2.0 * n + 1.0) * pib), (float)cr.y, 44.8f);
@@ -579,7 +586,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             nt = J;
             Tt = bf.C + bf.offC[kk];
             if constexpr (LOW) Tst = bf.Cs + bf.offC[kk];
-            dv = reinterpret_cast<double2*>(smraw + (rho ? L.odc + wp * L.sdc : L.od + wp * L.sd));
+            series = true;
             const double* tau = bf.tau + (size_t)kBlkSeries * kk;
             int fz = -1;
             SeriesZ z;
@@ -587,7 +594,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             for (int i = lane; i < F * J; i += 32) {
               const int f = i / J, j = i - f * J;
               if (f != fz) {
-                z = series_z(mu - cr.x, (2.0 * min(n + f, n1 - 1) + 1.0) * pib, cr.y, occ || adj);
+                z = series_z(mu - cr.x, sW[f], cr.y, occ || adj);
                 fz = f;
                 if constexpr (LOW) {
                   zf[0] = to_rest(z.c2a, float2{});
@@ -600,7 +607,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
               double2 pw = cpow_int(z.xi, j);
               if (j) pw = make_double2(2.0 * pw.x, 2.0 * pw.y);
               const double2 d = cmul(pw, z.c1);
-              dv[i] = d;
+              sd[i] = d;
               if constexpr (LOW) {
                 if (occ) {
                   const float2 pf = make_float2((float)pw.x, (float)pw.y);
@@ -631,11 +638,10 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             }
           }
         }
-        if (nt == n2 || rho) {
-          const bool sums = nt == n2;
+        auto bands = [&](bool sums) {  // d_b, and with sums its powers and traces
           for (int i = lane; i < F * n2; i += 32) {
             const int f = i / n2, bb = i - f * n2;
-            const double wn = (2.0 * min(n + f, n1 - 1) + 1.0) * pib;
+            const double wn = sW[f];
             const double x = mu - e_k[bb];
             const double s = 1.0 / fma(x, x, wn * wn);
             const double2 d = make_double2(x * s, -wn * s);
@@ -662,7 +668,8 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
               }
             }
           }
-        }
+        };
+        if (!series) bands(true);
         __syncwarp();
         // S and F, pair by pair: with t = B_a conj(B_c), sum t Re d and sum t Im d give both
         // (a, c) and (c, a)
@@ -671,7 +678,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
           const int a = pair[pr].x, c = pair[pr].y;
           const int nn = min(n + f, n1 - 1);
           const double2* t = Tt + pr;
-          const double2* df = dv + f * nt;
+          const double2* df = sd + f * nt;
           double2 xr = make_double2(0.0, 0.0), xi = xr;
           rc_t yr = rzero(rc_t{}), yi = yr;
           if (occ || adj) {
@@ -715,42 +722,75 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
               xi.x = fma(tv.x, d.y, xi.x); xi.y = fma(tv.y, d.y, xi.y);
             }
           }
-          const double2 h = HO[pr], o = HO[bf.npmax + pr];
-          const double wn = (2.0 * nn + 1.0) * pib;
+          const double2 h = hz[pr], o = HO[bf.npmax + pr];
+          const double wn = sW[f];
           const double2* Sg = p.Sig + si.offSig + (int64_t)nn * MM;
           // z o_ac - h_ac - Sigma_ac - g_ac, and (c, a) with conj(o), conj(h)
           const double2 s1 = Sg[a * M + c], s2 = Sg[c * M + a];
           double2 v;
-          v.x = fma(mu, o.x, -wn * o.y) - h.x - s1.x - (xr.x - xi.y);
-          v.y = fma(mu, o.y, wn * o.x) - h.y - s1.y - (xr.y + xi.x);
+          v.x = (fma(-wn, o.y, h.x) - s1.x) - (xr.x - xi.y);
+          v.y = (fma(wn, o.x, h.y) - s1.y) - (xr.y + xi.x);
           double2* Sm = sS + f * MM;
           Sm[a * M + c] = v;
-          v.x = fma(mu, o.x, wn * o.y) - h.x - s2.x - (xr.x + xi.y);
-          v.y = fma(-mu, o.y, wn * o.x) + h.y - s2.y - (xi.x - xr.y);
-          if (a != c) Sm[c * M + a] = v;
+          if (a != c) {
+            v.x = (fma(wn, o.y, h.x) - s2.x) - (xr.x + xi.y);
+            v.y = (fma(wn, o.x, -h.y) - s2.y) - (xi.x - xr.y);
+            Sm[c * M + a] = v;
+          }
         }
         __syncwarp();
-        gj64::invert<LW>(A, M, rcb, sp, sl, p.status);
+        if (series && rho) bands(false);  // rho_k reads d_b (its barrier comes first)
         const int* sq = sp + M;
         const bool mine = mf < nv;
         double2* out = (p.mode & (kGloc | kAdj))
                            ? p.gq + ((int64_t)(unit - p.gb0) * p.n_iw + min(n + mf, n1 - 1)) * p.mmax * p.mmax
                            : nullptr;
         if constexpr (LOW) {
-          // FP32 copy in the orbitals' order: one conversion per entry (it runs on the FP64 pipe)
+          // X0 = S^{-1} in FP32 and one step of refinement, S^{-1} = X0 + X0 R with R = I - S X0
+          // from S in FP32 pairs: 1e-15 of the FP64 inverse at these frequencies, where the FP64
+          // elimination takes 1,500 FP64 instructions a matrix at m = 20.
+          float4* Sp = reinterpret_cast<float4*>(A);
+          float2* X0 = sG + mf * MM;
+          float2* R = reinterpret_cast<float2*>(smraw + L.oR + wp * L.sG) + mf * MM;
           for (int i = sl; i < MM; i += LW) {
-            const int a = i / M, c = i - a * M;
-            const double2 g = A[sp[a] * M + sq[c]];
-            sG[mf * MM + i] = make_float2((float)g.x, (float)g.y);
-            if ((p.mode & kGloc) && mine) gq_put(&out[i], q, make_double2(wk * g.x, wk * g.y));
+            const cf v = from_d2(A[i]);
+            Sp[i] = st4(v);
+            X0[i] = make_float2(v.rh, v.ih);
           }
           __syncwarp();
-        } else if ((p.mode & kGloc) && mine) {
+          gj64::invert<LW>(X0, M, rcb, sp, sl, p.status);
           for (int i = sl; i < MM; i += LW) {
-            const int a = i / M, c = i - a * M;
-            const double2 g = A[sp[a] * M + sq[c]];
-            gq_put(&out[i], q, make_double2(wk * g.x, wk * g.y));
+            const int a = i / M, c = i - a * M, qc = sq[c];
+            cf acc = czero();
+            if (a == c) acc.rh = 1.f;
+            for (int x = 0; x < M; ++x) cacc1(acc, cneg(ld4(Sp[a * M + x])), X0[sp[x] * M + qc]);
+            R[i] = make_float2(__fadd_rn(acc.rh, acc.rl), __fadd_rn(acc.ih, acc.il));
           }
+          __syncwarp();
+          float2* Gn = reinterpret_cast<float2*>(A);  // S^{-1} in the orbitals' order (S is dead)
+          for (int i = sl; i < MM; i += LW) {
+            const int a = i / M, c = i - a * M, pa = sp[a] * M;
+            float2 d = make_float2(0.f, 0.f);
+            for (int x = 0; x < M; ++x) fmac(d, X0[pa + sq[x]], R[x * M + c]);
+            const float2 g = X0[pa + sq[c]];
+            float2 h, l;
+            two_sum(g.x, d.x, h.x, l.x);
+            two_sum(g.y, d.y, h.y, l.y);
+            Gn[i] = h;
+            if ((p.mode & kGloc) && mine)
+              gq_put(&out[i], q, make_double2(wk * ((double)h.x + (double)l.x), wk * ((double)h.y + (double)l.y)));
+          }
+          __syncwarp();
+          for (int i = sl; i < MM; i += LW) X0[i] = Gn[i];
+          __syncwarp();
+        } else {
+          gj64::invert<LW>(A, M, rcb, sp, sl, p.status);
+          if ((p.mode & kGloc) && mine)
+            for (int i = sl; i < MM; i += LW) {
+              const int a = i / M, c = i - a * M;
+              const double2 g = A[sp[a] * M + sq[c]];
+              gq_put(&out[i], q, make_double2(wk * g.x, wk * g.y));
+            }
         }
         if (occ) {
           float low_tr = 0.f, low_g2 = 0.f;  // LOW: this lane's sums over the warp's frequencies

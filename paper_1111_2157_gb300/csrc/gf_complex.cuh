@@ -49,6 +49,14 @@ __device__ __forceinline__ double2 crcp(double2 a) {
   }
 }
 
+// 1 / x to rounding for |x| in FP32's range (0 where x is beyond it): the FP32 reciprocal and two
+// Newton steps, six FP64-pipe instructions.
+__device__ __forceinline__ double rcp_newton(double x) {
+  double r = (double)__frcp_rn((float)x);
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+
 // Pivot key of a complex FP64 number: max(|Re|, |Im|) compared through the IEEE
 // bit pattern, which orders non-negative doubles like their values; no FP64
 // instruction.

@@ -231,14 +231,6 @@ __device__ __forceinline__ float block_max(float v, float* red) {
   return v;
 }
 
-// 1 / x to rounding for |x| in FP32's range (0 where x is beyond it): the FP32 reciprocal and two
-// Newton steps, six FP64-pipe instructions.
-__device__ __forceinline__ double rcp_newton(double x) {
-  double r = (double)__frcp_rn((float)x);
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
-}
-
 // Eigenpairs of the real symmetric tridiagonal matrix (q.d, q.e), one thread per eigenvalue:
 // bisection on Sturm counts in FP32, then three Rayleigh quotient steps in FP64 whose vector comes
 // from the twisted factorization at the row of the smallest pivot (Dhillon and Parlett, Linear

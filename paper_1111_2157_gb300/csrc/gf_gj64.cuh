@@ -13,14 +13,14 @@ using namespace cx;
 // Lanes per matrix for m orbitals (m <= 32).
 __host__ __device__ inline int lanes(int m) { return m <= 8 ? 8 : (m <= 16 ? 16 : 32); }
 
-// 1 / a with one division: scaled by a power of two near 1 / max(|Re|, |Im|) (bit arithmetic),
+// 1 / a with one reciprocal: scaled by a power of two near 1 / max(|Re|, |Im|) (bit arithmetic),
 // so that the squared modulus neither overflows nor underflows.
 __device__ __forceinline__ double2 crcp_scaled(double2 a, unsigned long long key) {
   int ex = 2046 - (int)(key >> 52);
   ex = ex < 1 ? 1 : ex;
   const double s = __longlong_as_double((long long)ex << 52);
   const double x = a.x * s, y = a.y * s;
-  const double q = s / fma(x, x, y * y);
+  const double q = s * rcp_newton(fma(x, x, y * y));  // in [1, 8): within FP32's range
   return make_double2(x * q, -y * q);
 }
 
@@ -64,6 +64,53 @@ __device__ __forceinline__ void invert(double2* A, int M, double2* rc, int* sp, 
       double2 v = (i == bi || c == j) ? make_double2(0.0, 0.0) : A[e];
       v.x = fma(-l.x, u.x, fma(l.y, u.y, v.x));
       v.y = fma(-l.x, u.y, fma(-l.y, u.x, v.y));
+      A[e] = v;
+      i += di;
+      c += dc;
+      if (c >= M) {
+        c -= M;
+        ++i;
+      }
+    }
+    __syncwarp();
+  }
+}
+
+// The same in FP32.
+template <int LW>
+__device__ __forceinline__ void invert(float2* A, int M, float2* rc, int* sp, int sl, int* status) {
+  float2* su = rc;
+  float2* sc = rc + M;
+  int* sq = sp + M;
+  bool used = sl >= M;
+  for (int j = 0; j < M; ++j) {
+    // key with the row in its low bits: the largest wins, ties go to the lowest row
+    unsigned best = used ? 0u : ((pivot_key_s(A[sl * M + j]) & ~31u) | (unsigned)(31 - sl));
+    if constexpr (LW == 32) {
+      best = __reduce_max_sync(0xffffffffu, best);
+    } else {
+#pragma unroll
+      for (int off = LW / 2; off; off >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, off));
+    }
+    const int bi = min(31 - (int)(best & 31u), M - 1);
+    if (sl == 0 && ((best >> 5) == 0u || (best & ~31u) >= 0x7f800000u)) atomicOr(status, kFlagSingular);
+    const float2 r = frcp(A[bi * M + j]);
+    if (sl < M) {
+      const float2 u = A[bi * M + sl], l = A[sl * M + j];
+      su[sl] = (sl == j) ? r : fmul(u, r);
+      sc[sl] = (sl == bi) ? make_float2(-1.f, 0.f) : l;
+    }
+    if (sl == bi) used = true;
+    if (sl == 0) {
+      sp[j] = bi;
+      sq[bi] = j;
+    }
+    __syncwarp();
+    int i = sl / M, c = sl - (sl / M) * M;
+    const int di = LW / M, dc = LW - (LW / M) * M;
+    for (int e = sl; e < M * M; e += LW) {
+      float2 v = (i == bi || c == j) ? make_float2(0.f, 0.f) : A[e];
+      fsub_prod(v, sc[i], su[c]);
       A[e] = v;
       i += di;
       c += dc;
