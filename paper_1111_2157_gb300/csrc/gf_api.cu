@@ -99,12 +99,13 @@ gf_status ensure_block(gf_ctx* c) {
     DevBuf* b;
     size_t bytes;
   } need[] = {{&c->blk_e, 8 * (size_t)c->totNb},    {&c->blk_T, 16 * (size_t)c->blk_totT},
-              {&c->blk_Ts, mixed ? 8 * (size_t)c->blk_totT : 0}, {&c->blk_B, 16 * (size_t)c->totP},
+              {&c->blk_Ts, mixed ? 8 * (size_t)c->blk_totT : 0}, {&c->blk_Tp, mixed ? 16 * (size_t)c->blk_totT : 0}, {&c->blk_B, 16 * (size_t)c->totP},
               {&c->blk_Bs, mixed ? 8 * (size_t)c->totP : 0},     {&c->blk_HO, 32 * npm * c->n_k},
               {&c->blk_U, 16 * (size_t)c->totH},     {&c->blk_D22, 16 * (size_t)c->totH},
               {&c->blk_V, 16 * (size_t)c->totP},     {&c->blk_R, 16 * mm * c->n_k},
               {&c->blk_H11, 16 * mm * c->n_k},       {&c->blk_tau, 8 * (size_t)c->mmax * c->n_k},
               {&c->blk_C, 16 * (size_t)c->blk_totC}, {&c->blk_Cs, mixed ? 8 * (size_t)c->blk_totC : 0},
+              {&c->blk_Cp, mixed ? 16 * (size_t)c->blk_totC : 0},
               {&c->blk_ser, 8 * ((size_t)gf::kBlkSeries + 2) * c->n_k},
               {&c->blk_ws, 16 * ws},                 {&c->blk_info, 8 * ((size_t)c->n_k + 1)}};
   for (auto& n : need) {
@@ -135,12 +136,14 @@ gf_status ensure_block(gf_ctx* c) {
   b.offD = c->offD_d.as<int64_t>();
   b.T = c->blk_T.as<double2>();
   b.Ts = mixed ? c->blk_Ts.as<float2>() : nullptr;
+  b.Tp = c->blk_Tp.as<float4>();
   b.offT = c->blk_offT.as<int64_t>();
   b.Bs = mixed ? c->blk_Bs.as<float2>() : nullptr;
   b.HO = c->blk_HO.as<double2>();
   b.U = c->blk_U.as<double2>();
   b.C = c->blk_C.as<double2>();
   b.Cs = mixed ? c->blk_Cs.as<float2>() : nullptr;
+  b.Cp = c->blk_Cp.as<float4>();
   b.offC = c->blk_offT.as<int64_t>() + c->n_k;
   b.series = c->blk_ser.as<double>();
   b.ws = c->blk_ws.as<double2>();
@@ -531,6 +534,7 @@ gf_status run_block(gf_ctx* c, int mode, gf::PointParams p) {
   b.offD = c->offD_d.as<int64_t>();
   b.T = c->blk_T.as<double2>();
   b.Ts = c->blk_Ts.as<float2>();
+  b.Tp = c->blk_Tp.as<float4>();
   b.offT = c->blk_offT.as<int64_t>();
   b.B = c->blk_B.as<double2>();
   b.Bs = c->blk_Bs.as<float2>();
@@ -538,6 +542,7 @@ gf_status run_block(gf_ctx* c, int mode, gf::PointParams p) {
   b.npmax = c->mmax * (c->mmax + 1) / 2;
   b.C = c->blk_C.as<double2>();
   b.Cs = c->blk_Cs.as<float2>();
+  b.Cp = c->blk_Cp.as<float4>();
   b.offC = c->blk_offT.as<int64_t>() + c->n_k;
   b.tau = c->blk_ser.as<double>();
   b.cr = reinterpret_cast<const double2*>(b.tau + (size_t)gf::kBlkSeries * c->n_k);
@@ -1314,7 +1319,7 @@ gf_status gf_destroy(gf_ctx* c) {
                     &c->pole_part, &c->dos_part,
                     &c->blk_units, &c->blk_perm, &c->blk_sysg, &c->blk_offT, &c->blk_e, &c->blk_T, &c->blk_Ts,
                     &c->blk_B, &c->blk_Bs, &c->blk_HO, &c->blk_U, &c->blk_D22, &c->blk_V, &c->blk_R, &c->blk_H11,
-                    &c->blk_tau, &c->blk_ws, &c->blk_info, &c->blk_C, &c->blk_Cs, &c->blk_ser};
+                    &c->blk_tau, &c->blk_ws, &c->blk_info, &c->blk_C, &c->blk_Cs, &c->blk_ser, &c->blk_Tp, &c->blk_Cp};
   for (DevBuf* b : bufs) release(*b);
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
   if (c->occ_exec) cudaGraphExecDestroy(c->occ_exec);

@@ -266,7 +266,11 @@ __global__ void __launch_bounds__(kSetupThreads) k_block_finish(const BlockSetup
     cmac_cb(t, Bs[a * n2 + l], Bs[c * n2 + l]);
     if (a == c) t.y = 0.0;
     b.T[b.offT[k] + e] = t;
-    if (b.Ts) b.Ts[b.offT[k] + e] = make_float2((float)t.x, (float)t.y);
+    if (b.Ts) {
+      const cf v = from_d2(t);
+      b.Ts[b.offT[k] + e] = make_float2(v.rh, v.ih);
+      b.Tp[b.offT[k] + e] = st4(v);
+    }
   }
   // U = Q diag(R^{-+}, V2): one column per thread, the reflections in reverse order
   double2* U = b.U + ki.offH;
@@ -358,7 +362,11 @@ __global__ void __launch_bounds__(kSetupThreads) k_block_series(const BlockSetup
       v.y = fma(c, t.y, v.y);
     }
     b.C[b.offC[k] + i] = v;
-    if (b.Cs) b.Cs[b.offC[k] + i] = make_float2((float)v.x, (float)v.y);
+    if (b.Cs) {
+      const cf c = from_d2(v);
+      b.Cs[b.offC[k] + i] = make_float2(c.rh, c.ih);
+      b.Cp[b.offC[k] + i] = st4(c);
+    }
   }
 }
 
@@ -374,7 +382,6 @@ struct Rest<true> {
   using c = float2;
   using r = float;
 };
-__device__ __forceinline__ double2 to_rest(double2 v, double2) { return v; }
 __device__ __forceinline__ float2 to_rest(double2 v, float2) { return make_float2((float)v.x, (float)v.y); }
 __device__ __forceinline__ void rmac(double2& a, double2 x, double2 y) { cmac(a, x, y); }
 __device__ __forceinline__ void rmac(float2& a, float2 x, float2 y) { fmac(a, x, y); }
@@ -474,7 +481,7 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   L.oM = o; o += (mode & kAdj) ? W * L.sS : 0;
   L.oR = o; o += W * L.sG;
   const size_t np = (size_t)mmax * (mmax + 1) / 2;
-  const size_t fixed = W * (L.sG + L.sd + L.sp + 8 * f) + al(2 * np) + 16 * np +
+  const size_t fixed = W * (L.sG + L.sd + L.sp + (low ? 16 : 8) * f) + al(2 * np) + (low ? 32 : 16) * np +
                        (low && rho ? 8 * mmax * (((size_t)n2max + 3) & ~(size_t)3) : 0);
   L.yf = 0;
   if (rho) {
@@ -495,9 +502,9 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   L.oG = o; o += W * L.sG;
   L.od = o; o += W * L.sd;
   L.op = o; o += W * L.sp;
-  L.oW = o; o = al(o + 8 * W * f);
+  L.oW = o; o = al(o + (low ? 16 : 8) * W * f);  // w_n (low: and in pairs)
   L.oPair = o; o += al(2 * np);
-  L.oHz = o; o += 16 * np;
+  L.oHz = o; o += (low ? 32 : 16) * np;  // (low: pairs of mu O - H11, then of O)
   L.oB = o; o += low && rho ? 8 * mmax * (((size_t)n2max + 3) & ~(size_t)3) : 0;
   L.bytes = o;
   return L;
@@ -525,6 +532,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
   float2* sG = reinterpret_cast<float2*>(smraw + L.oG + wp * L.sG);
   int* sPv = reinterpret_cast<int*>(smraw + L.op + wp * L.sp);
   double* sW = reinterpret_cast<double*>(smraw + L.oW) + wp * F;
+  float2* sWp = reinterpret_cast<float2*>(smraw + L.oW + 8 * W * F) + wp * F;
   uchar2* pair = reinterpret_cast<uchar2*>(smraw + L.oPair);
   double2* hz = reinterpret_cast<double2*>(smraw + L.oHz);
   const int unit = bl.unit0 + blockIdx.x / bl.n_chunks, ch = blockIdx.x % bl.n_chunks;
@@ -553,7 +561,13 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
       while (rem >= M - a) { rem -= M - a; ++a; }
       pair[pr] = make_uchar2((unsigned char)a, (unsigned char)(a + rem));
       const double2 h = HO[pr], o = HO[bf.npmax + pr];
-      hz[pr] = make_double2(fma(mu, o.x, -h.x), fma(mu, o.y, -h.y));
+      const double2 z0 = make_double2(fma(mu, o.x, -h.x), fma(mu, o.y, -h.y));
+      if constexpr (LOW) {
+        reinterpret_cast<float4*>(hz)[pr] = st4(from_d2(z0));
+        reinterpret_cast<float4*>(hz)[NP + pr] = st4(from_d2(o));
+      } else {
+        hz[pr] = z0;
+      }
     }
     if constexpr (LOW) {
       if (rho) {
@@ -574,18 +588,35 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
         int nt = n2;
         const double2* Tt = T;
         const float2* Tst = nullptr;
-        if constexpr (LOW) Tst = bf.Ts + bf.offT[kk];
+        const float4* Tpt = nullptr;
+        if constexpr (LOW) {
+          Tst = bf.Ts + bf.offT[kk];
+          Tpt = bf.Tp + bf.offT[kk];
+        }
         bool series = false;
-        if (lane < F) sW[lane] = (2.0 * min(n + lane, n1 - 1) + 1.0) * pib;
+        // d (or the series' coefficients) for the sums: in FP32 pairs with LOW
+        auto put_d = [&](int i, double2 d) {
+          if constexpr (LOW) reinterpret_cast<float4*>(sd)[i] = st4(from_d2(d));
+          else sd[i] = d;
+        };
+        if (lane < F) {
+          const double wn = (2.0 * min(n + lane, n1 - 1) + 1.0) * pib;
+          sW[lane] = wn;
+          if constexpr (LOW) split(wn, sWp[lane].x, sWp[lane].y);
+        }
         __syncwarp();
         {
           const double2 cr = bf.cr[kk];
           const int J = series_terms((float)(mu - cr.x), (float)((2.0 * n + 1.0) * pib), (float)cr.y, 44.8f);
-          const int sums = LOW ? 1 : (occ ? 3 : (adj ? 2 : 1));  // FP64 sums
-          if (J <= min(n2, kBlkSeries) && (n2 - J) * NP * F * sums > 1600) {
+          // (LOW: the sums cost a sixth, in FP32 pairs)
+          const int sums = occ ? 3 : (adj ? 2 : 1);
+          if (J <= min(n2, kBlkSeries) && (LOW ? (n2 - J) * NP * F > 5000 : (n2 - J) * NP * F * sums > 1600)) {
             nt = J;
             Tt = bf.C + bf.offC[kk];
-            if constexpr (LOW) Tst = bf.Cs + bf.offC[kk];
+            if constexpr (LOW) {
+              Tst = bf.Cs + bf.offC[kk];
+              Tpt = bf.Cp + bf.offC[kk];
+            }
             series = true;
             const double* tau = bf.tau + (size_t)kBlkSeries * kk;
             int fz = -1;
@@ -607,7 +638,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
               double2 pw = cpow_int(z.xi, j);
               if (j) pw = make_double2(2.0 * pw.x, 2.0 * pw.y);
               const double2 d = cmul(pw, z.c1);
-              sd[i] = d;
+              put_d(i, d);
               if constexpr (LOW) {
                 if (occ) {
                   const float2 pf = make_float2((float)pw.x, (float)pw.y);
@@ -645,8 +676,9 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             const double x = mu - e_k[bb];
             const double s = 1.0 / fma(x, x, wn * wn);
             const double2 d = make_double2(x * s, -wn * s);
-            sd[i] = d;
             if constexpr (LOW) {
+              if (sums) put_d(i, d);
+              else sd[i] = d;
               if (sums && occ) {
                 const float2 df = make_float2((float)d.x, (float)d.y), d2 = fmul(df, df);
                 sd2[i] = d2;
@@ -656,7 +688,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
                   acc_g2 += (double)d2.x;
                 }
               }
-            } else if (sums && (occ || adj)) {
+            } else if (sd[i] = d; sums && (occ || adj)) {
               const double2 d2 = cmul(d, d);
               sd2[i] = d2;
               if (occ) {
@@ -677,69 +709,117 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
           const int f = i / NP, pr = i - f * NP;
           const int a = pair[pr].x, c = pair[pr].y;
           const int nn = min(n + f, n1 - 1);
-          const double2* t = Tt + pr;
-          const double2* df = sd + f * nt;
-          double2 xr = make_double2(0.0, 0.0), xi = xr;
-          rc_t yr = rzero(rc_t{}), yi = yr;
-          if (occ || adj) {
-            const rc_t* d2f = sd2 + f * nt;
-            if constexpr (LOW) {
-              const float2* ts = Tst + pr;
+          if constexpr (LOW) {
+            // S in FP32 pairs, F in FP32
+            const float4* t = Tpt + pr;
+            const float4* df = reinterpret_cast<const float4*>(sd) + f * nt;
+            float xrr[2] = {0.f, 0.f}, xri[2] = {0.f, 0.f}, xir[2] = {0.f, 0.f}, xii[2] = {0.f, 0.f};
+            float2 yr = make_float2(0.f, 0.f), yi = yr;
+            auto add = [&](float4 tv, float4 d) {
+              acc_prod(tv.x, tv.y, d.x, d.y, xrr[0], xrr[1]);
+              acc_prod(tv.z, tv.w, d.x, d.y, xri[0], xri[1]);
+              acc_prod(tv.x, tv.y, d.z, d.w, xir[0], xir[1]);
+              acc_prod(tv.z, tv.w, d.z, d.w, xii[0], xii[1]);
+            };
+            if (occ) {
+              const float2* d2f = sd2 + f * nt;
+#pragma unroll 2
+              for (int bb = 0; bb < nt; ++bb) {
+                const float4 tv = __ldg(t + (size_t)bb * NP);
+                const float2 d2 = d2f[bb];
+                add(tv, df[bb]);
+                yr.x = fmaf(tv.x, d2.x, yr.x); yr.y = fmaf(tv.z, d2.x, yr.y);
+                yi.x = fmaf(tv.x, d2.y, yi.x); yi.y = fmaf(tv.z, d2.y, yi.y);
+              }
+              const float4 o = reinterpret_cast<const float4*>(hz)[NP + pr];
+              float2* Fm = sF + f * MM;
+              Fm[a * M + c] = make_float2(o.x + (yr.x - yi.y), o.z + (yr.y + yi.x));
+              if (a != c) Fm[c * M + a] = make_float2(o.x + (yr.x + yi.y), (yi.x - yr.y) - o.z);
+            } else {
+#pragma unroll 2
+              for (int bb = 0; bb < nt; ++bb) add(__ldg(t + (size_t)bb * NP), df[bb]);
+            }
+            // (a, c): h + i w o - Sigma_ac - g_ac; (c, a): conj(h) + i w conj(o) - Sigma_ca - g_ca
+            const float4 h = reinterpret_cast<const float4*>(hz)[pr], o = reinterpret_cast<const float4*>(hz)[NP + pr];
+            const float2 w = sWp[f];
+            const float4* Sg = p.Sd + si.offSig + (int64_t)nn * MM;
+            float4* Sm = reinterpret_cast<float4*>(sS) + f * MM;
+            auto plus = [](float& sh, float& sl_, float vh, float vl) {  // (sh, sl_) += (vh, vl)
+              float s, e;
+              two_sum(sh, vh, s, e);
+              sh = s;
+              sl_ = __fadd_rn(sl_, __fadd_rn(vl, e));
+            };
+            {
+              const float4 sg = Sg[a * M + c];
+              cf v{h.x, h.y, h.z, h.w};
+              acc_prod(-w.x, -w.y, o.z, o.w, v.rh, v.rl);
+              acc_prod(w.x, w.y, o.x, o.y, v.ih, v.il);
+              plus(v.rh, v.rl, -sg.x, -sg.y);
+              plus(v.ih, v.il, -sg.z, -sg.w);
+              plus(v.rh, v.rl, -xrr[0], -xrr[1]);
+              plus(v.rh, v.rl, xii[0], xii[1]);
+              plus(v.ih, v.il, -xri[0], -xri[1]);
+              plus(v.ih, v.il, -xir[0], -xir[1]);
+              cnorm(v);
+              Sm[a * M + c] = st4(v);
+            }
+            if (a != c) {
+              const float4 sg = Sg[c * M + a];
+              cf v{h.x, h.y, -h.z, -h.w};
+              acc_prod(w.x, w.y, o.z, o.w, v.rh, v.rl);
+              acc_prod(w.x, w.y, o.x, o.y, v.ih, v.il);
+              plus(v.rh, v.rl, -sg.x, -sg.y);
+              plus(v.ih, v.il, -sg.z, -sg.w);
+              plus(v.rh, v.rl, -xrr[0], -xrr[1]);
+              plus(v.rh, v.rl, -xii[0], -xii[1]);
+              plus(v.ih, v.il, xri[0], xri[1]);
+              plus(v.ih, v.il, -xir[0], -xir[1]);
+              cnorm(v);
+              Sm[c * M + a] = st4(v);
+            }
+          } else {
+            const double2* t = Tt + pr;
+            const double2* df = sd + f * nt;
+            double2 xr = make_double2(0.0, 0.0), xi = xr;
+            const double2 o = HO[bf.npmax + pr];
+            if (occ || adj) {
+              double2 yr = make_double2(0.0, 0.0), yi = yr;
+              const double2* d2f = sd2 + f * nt;
 #pragma unroll 4
               for (int bb = 0; bb < nt; ++bb) {
-                const double2 tv = ld_cg(t + (size_t)bb * NP), d = df[bb];
-                const float2 tf = ld_cg(ts + (size_t)bb * NP), d2 = d2f[bb];
+                const double2 tv = __ldg(t + (size_t)bb * NP), d = df[bb], d2 = d2f[bb];
                 xr.x = fma(tv.x, d.x, xr.x); xr.y = fma(tv.y, d.x, xr.y);
                 xi.x = fma(tv.x, d.y, xi.x); xi.y = fma(tv.y, d.y, xi.y);
-                yr.x = rfma(tf.x, d2.x, yr.x); yr.y = rfma(tf.y, d2.x, yr.y);
-                yi.x = rfma(tf.x, d2.y, yi.x); yi.y = rfma(tf.y, d2.y, yi.y);
+                yr.x = fma(tv.x, d2.x, yr.x); yr.y = fma(tv.y, d2.x, yr.y);
+                yi.x = fma(tv.x, d2.y, yi.x); yi.y = fma(tv.y, d2.y, yi.y);
               }
+              double2* Fm = sF + f * MM;
+              Fm[a * M + c] = make_double2(o.x + (yr.x - yi.y), o.y + (yr.y + yi.x));
+              if (a != c) Fm[c * M + a] = make_double2(o.x + (yr.x + yi.y), (yi.x - yr.y) - o.y);
             } else {
 #pragma unroll 4
               for (int bb = 0; bb < nt; ++bb) {
-                const double2 tv = ld_cg(t + (size_t)bb * NP), d = df[bb];
-                const rc_t d2 = d2f[bb];
+                const double2 tv = __ldg(t + (size_t)bb * NP), d = df[bb];
                 xr.x = fma(tv.x, d.x, xr.x); xr.y = fma(tv.y, d.x, xr.y);
                 xi.x = fma(tv.x, d.y, xi.x); xi.y = fma(tv.y, d.y, xi.y);
-                yr.x = rfma(tv.x, d2.x, yr.x); yr.y = rfma(tv.y, d2.x, yr.y);
-                yi.x = rfma(tv.x, d2.y, yi.x); yi.y = rfma(tv.y, d2.y, yi.y);
               }
             }
-            const rc_t o = to_rest(HO[bf.npmax + pr], rc_t{});
-            rc_t* Fm = sF + f * MM;
-            rc_t v;
-            v.x = o.x + (yr.x - yi.y);
-            v.y = o.y + (yr.y + yi.x);
-            Fm[a * M + c] = v;
-            v.x = o.x + (yr.x + yi.y);
-            v.y = (yi.x - yr.y) - o.y;
-            if (a != c) Fm[c * M + a] = v;
-          } else {
-#pragma unroll 4
-            for (int bb = 0; bb < nt; ++bb) {
-              const double2 tv = ld_cg(t + (size_t)bb * NP), d = df[bb];
-              xr.x = fma(tv.x, d.x, xr.x); xr.y = fma(tv.y, d.x, xr.y);
-              xi.x = fma(tv.x, d.y, xi.x); xi.y = fma(tv.y, d.y, xi.y);
-            }
-          }
-          const double2 h = hz[pr], o = HO[bf.npmax + pr];
-          const double wn = sW[f];
-          const double2* Sg = p.Sig + si.offSig + (int64_t)nn * MM;
-          // z o_ac - h_ac - Sigma_ac - g_ac, and (c, a) with conj(o), conj(h)
-          const double2 s1 = Sg[a * M + c], s2 = Sg[c * M + a];
-          double2 v;
-          v.x = (fma(-wn, o.y, h.x) - s1.x) - (xr.x - xi.y);
-          v.y = (fma(wn, o.x, h.y) - s1.y) - (xr.y + xi.x);
-          double2* Sm = sS + f * MM;
-          Sm[a * M + c] = v;
-          if (a != c) {
-            v.x = (fma(wn, o.y, h.x) - s2.x) - (xr.x + xi.y);
-            v.y = (fma(wn, o.x, -h.y) - s2.y) - (xi.x - xr.y);
-            Sm[c * M + a] = v;
+            const double2 h = hz[pr];
+            const double wn = sW[f];
+            const double2* Sg = p.Sig + si.offSig + (int64_t)nn * MM;
+            // (a, c): h + i w o - Sigma_ac - g_ac; (c, a): conj(h) + i w conj(o) - Sigma_ca - g_ca
+            const double2 s1 = Sg[a * M + c], s2 = Sg[c * M + a];
+            double2* Sm = sS + f * MM;
+            Sm[a * M + c] = make_double2((fma(-wn, o.y, h.x) - s1.x) - (xr.x - xi.y),
+                                         (fma(wn, o.x, h.y) - s1.y) - (xr.y + xi.x));
+            if (a != c)
+              Sm[c * M + a] = make_double2((fma(wn, o.y, h.x) - s2.x) - (xr.x + xi.y),
+                                           (fma(wn, o.x, -h.y) - s2.y) - (xi.x - xr.y));
           }
         }
         __syncwarp();
-        if (series && rho) bands(false);  // rho_k reads d_b (its barrier comes first)
+        if (rho && (series || LOW)) bands(false);  // rho_k reads d_b in FP64 (its barrier comes first)
         const int* sq = sp + M;
         const bool mine = mf < nv;
         double2* out = (p.mode & (kGloc | kAdj))
@@ -752,11 +832,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
           float4* Sp = reinterpret_cast<float4*>(A);
           float2* X0 = sG + mf * MM;
           float2* R = reinterpret_cast<float2*>(smraw + L.oR + wp * L.sG) + mf * MM;
-          for (int i = sl; i < MM; i += LW) {
-            const cf v = from_d2(A[i]);
-            Sp[i] = st4(v);
-            X0[i] = make_float2(v.rh, v.ih);
-          }
+          for (int i = sl; i < MM; i += LW) X0[i] = make_float2(Sp[i].x, Sp[i].z);
           __syncwarp();
           gj64::invert<LW>(X0, M, rcb, sp, sl, p.status);
           for (int i = sl; i < MM; i += LW) {

@@ -28,7 +28,8 @@ struct BlockForm {
   const double* e;        // [n2] at offD[k]
   const int64_t* offD;
   const double2* T;       // [n2][np] at offT[k]: B_ab conj(B_cb) over the pairs a <= c, np = m(m+1)/2
-  const float2* Ts;       // its FP32 rounding (GF_PREC_MIXED) or null
+  const float2* Ts;       // its FP32 rounding and FP32 pairs (GF_PREC_MIXED), or null
+  const float4* Tp;
   const int64_t* offT;
   const double2* B;       // [m][n2] at KInfo::offP
   const float2* Bs;
@@ -38,7 +39,8 @@ struct BlockForm {
   // sum_b t_b / (z - e_b)^p = sum_j a_j^(p)(z) C_j, C_j = sum_b t_b T_j(x_b), whose terms fall
   // off like R^-j, R the sum of the half axes of the ellipse with foci c -+ r through z.
   const double2* C;       // [min(n2, kBlkSeries)][np] at offC[k]
-  const float2* Cs;       // its FP32 rounding (GF_PREC_MIXED) or null
+  const float2* Cs;       // its FP32 rounding and FP32 pairs (GF_PREC_MIXED), or null
+  const float4* Cp;
   const int64_t* offC;
   const double* tau;      // [kBlkSeries] per k: sum_b T_j(x_b)
   const double2* cr;      // (c, r) per k
@@ -76,12 +78,14 @@ struct BlockSetup {
   const int64_t* offD;
   double2* T;
   float2* Ts;
+  float4* Tp;
   const int64_t* offT;
   float2* Bs;
   double2* HO;
   double2* U;             // [N_b][N_b] at offH
   double2* C;             // Chebyshev moments, as in BlockForm
   float2* Cs;
+  float4* Cp;
   const int64_t* offC;
   double* series;         // tau, then (c, r) pairs
   double2* ws;            // per-CTA slices of nbmax^2 elements when the matrix exceeds shared memory
