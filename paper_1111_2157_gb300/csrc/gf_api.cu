@@ -512,7 +512,9 @@ gf_status run_block(gf_ctx* c, int mode, gf::PointParams p) {
   const bool kred = (mode & (gf::kGloc | gf::kAdj)) != 0;
   const bool low = c->precision == GF_PREC_MIXED && !c->lowrank && !(mode & gf::kAdj);
   const int nc = low ? c->blk_nc : c->n_iw;
-  const int ch0 = (nc + c->blk_cw - 1) / c->blk_cw;
+  // (the few FP64 frequencies of mixed precision in chunks of one batch: they are latency bound)
+  const int cw0 = low ? gf::block_batch(c->mmax) : c->blk_cw;
+  const int ch0 = (nc + cw0 - 1) / cw0;
   const int ch1 = (c->n_iw - nc + c->blk_cw - 1) / c->blk_cw;
   c->run_chunks = ch0 + ch1;
   p.n_chunks = c->run_chunks;
@@ -548,7 +550,6 @@ gf_status run_block(gf_ctx* c, int mode, gf::PointParams p) {
   b.cr = reinterpret_cast<const double2*>(b.tau + (size_t)gf::kBlkSeries * c->n_k);
   gf::BlockLaunch l{};
   l.n2max = c->blk_n2max;
-  l.chunk_w = c->blk_cw;
   // units: the k-groups in order, then the single k-points by decreasing window
   l.units = c->blk_units.as<int2>() + (kred ? 0 : c->blk_groups);
   l.kperm = c->blk_perm.as<int>() + (kred ? 0 : c->n_k);
@@ -577,11 +578,20 @@ gf_status run_block(gf_ctx* c, int mode, gf::PointParams p) {
       l.n_end = part ? c->n_iw : nc;
       l.chunk0 = part ? ch0 : 0;
       l.n_chunks = part ? ch1 : ch0;
+      l.chunk_w = part ? c->blk_cw : cw0;
       if (l.n_chunks == 0) continue;
-      if (part && mode == gf::kOcc) GF_CU(gf::launch_occ_block32(p, b, l, c->stream));
-      else GF_CU(gf::launch_point_block(p, b, l, part, c->stream));
+      const bool beside = part == 0 && ch1 > 0;
+      if (beside) {
+        GF_CU(cudaEventRecord(c->ev_fork, c->stream));
+        GF_CU(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
+      }
+      const cudaStream_t on = beside ? c->side : c->stream;
+      if (part && mode == gf::kOcc) GF_CU(gf::launch_occ_block32(p, b, l, on));
+      else GF_CU(gf::launch_point_block(p, b, l, part, on));
+      if (beside) GF_CU(cudaEventRecord(c->ev_join, c->side));
       c->last_launches += 1;
     }
+    if (ch0 > 0 && ch1 > 0) GF_CU(cudaStreamWaitEvent(c->stream, c->ev_join, 0));
     if (!c->capturing) {
       GF_CU(cudaEventRecord(c->ev[c->ev_used + 1], c->stream));
       c->ev_used += 2;
@@ -1225,6 +1235,11 @@ gf_status init_ctx(gf_ctx* c, const gf_desc* d) {
         if ((e = cudaMemcpyAsync(u.b->p, u.p, u.bytes, cudaMemcpyHostToDevice, c->stream))) return e;
       }
     }
+    if (c->blk_shape && c->precision == GF_PREC_MIXED && !c->lowrank) {
+      if ((e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking))) return e;
+      if ((e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming))) return e;
+      if ((e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming))) return e;
+    }
     if ((e = cudaMemsetAsync(c->status.p, 0, sizeof(int), c->stream))) return e;
     if (c->use_graph) {
       if ((e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking))) return e;
@@ -1324,6 +1339,9 @@ gf_status gf_destroy(gf_ctx* c) {
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
   if (c->occ_exec) cudaGraphExecDestroy(c->occ_exec);
   if (c->ev_user) cudaEventDestroy(c->ev_user);
+  if (c->ev_fork) cudaEventDestroy(c->ev_fork);
+  if (c->ev_join) cudaEventDestroy(c->ev_join);
+  if (c->side) cudaStreamDestroy(c->side);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->hpin) cudaFreeHost(c->hpin);
   delete c;

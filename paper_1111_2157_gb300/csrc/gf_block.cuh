@@ -47,6 +47,18 @@ struct BlockForm {
 };
 constexpr int kBlkSeries = 40;  // moments kept
 
+// Terms of the series that leave a remainder of e^-bits for every frequency from w on, bits with a
+// margin for the j^2 of the third powers (FP32: only the count depends on it).
+__device__ __forceinline__ int series_terms(float dx, float w, float r, float bits) {
+  const float xr = dx / r, xi = w / r;
+  const float ur = xr * xr - xi * xi - 1.f, ui = 2.f * xr * xi, au = sqrtf(ur * ur + ui * ui);
+  const float p = sqrtf(0.5f * (au + fabsf(ur))), h = p > 0.f ? 0.5f * fabsf(ui) / p : 0.f;
+  const float sr = ur >= 0.f ? p : h, si = ur >= 0.f ? h : p;
+  const float R = sqrtf((fabsf(xr) + sr) * (fabsf(xr) + sr) + (fabsf(xi) + si) * (fabsf(xi) + si));
+  const float lr = logf(R);
+  return lr > 0.02f ? (int)(bits / lr) + 2 : 1 << 20;
+}
+
 // One launch over units (k-points, or k-groups for the k-reductions) x frequency chunks.
 struct BlockLaunch {
   int n_units, unit0;     // units [unit0, unit0 + n_units)

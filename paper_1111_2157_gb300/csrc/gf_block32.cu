@@ -3,7 +3,9 @@
 // window (w_n above a fraction of H's scale; k_point_block takes the others in FP64).
 //
 // A warp takes FW frequencies of one k-point and runs without block barriers:
-//   1. d_b = 1 / (z - e_b) and its powers, one (band, frequency) per lane;
+//   1. d_b = 1 / (z - e_b) and its powers, one (band, frequency) per lane, or the coefficients of
+//      the Chebyshev series where that has fewer terms to 2^-24 (the traces of D stay direct: the
+//      series' real parts carry the rounding of its moduli);
 //   2. band sums of S and F = dS/dz, one orbital pair a <= c per lane and FW frequencies in
 //      registers, so that one load of the pair table feeds 8 FW FMAs;
 //   3. S^{-1} with LW lanes per matrix, one row per lane in registers (Gauss-Jordan in exchange
@@ -28,7 +30,7 @@ __device__ __forceinline__ float2 z2() { return make_float2(0.f, 0.f); }
 // Shared memory (bytes): per CTA x_b = mu - e_b, mu O - H11 and O by pairs and the pair list;
 // per warp d, d^2, d^3 as [band][FW], S and F with rows of NMAX entries, the pivot rows and tables.
 struct Layout32 {
-  size_t oX, oHz, oO, oPair, warp0, wd, wS, wF, wbuf, wp, wstride, bytes;
+  size_t oX, oHz, oO, oPair, warp0, wd, ww, wS, wF, wbuf, wp, wstride, bytes;
 };
 
 __host__ __device__ inline Layout32 make_layout32(int mmax, int n2max, int nmax, int lw, int fw) {
@@ -43,6 +45,7 @@ __host__ __device__ inline Layout32 make_layout32(int mmax, int n2max, int nmax,
   L.warp0 = o;
   size_t g = 0;
   L.wd = g; g = al(g + 24 * (size_t)fw * n2max);
+  L.ww = g; g = al(g + 4 * (size_t)fw);
   L.wS = g; g = al(g + 8 * (size_t)fw * mmax * nmax);
   L.wF = g; g = al(g + 8 * (size_t)fw * mmax * nmax);
   L.wbuf = g; g = al(g + 8 * (size_t)(32 / lw) * nmax);
@@ -74,6 +77,11 @@ __global__ void __launch_bounds__(32 * kBlkWarps, NMAX > 24 ? 2 : 3)
   const int M = si.m, n2 = ki.nb - M, NP = M * (M + 1) / 2;
   const double mu = p.mu[ki.sys], pib = M_PI / si.beta;
   const float2* Ts = bf.Ts + bf.offT[kk];
+  const float2* Cs = bf.Cs + bf.offC[kk];
+  const float cdx = __double2float_rn(mu - bf.cr[kk].x), cr = __double2float_rn(bf.cr[kk].y);
+  // the series where it saves four terms, its own cost
+  const int jmax = min(min(n2, kBlkSeries), n2 - 4);
+  float* sw = reinterpret_cast<float*>(wb + L.ww);
   float2* sd = reinterpret_cast<float2*>(wb + L.wd);
   float2* sd2 = sd + FW * n2;
   float2* sd3 = sd2 + FW * n2;
@@ -99,69 +107,105 @@ __global__ void __launch_bounds__(32 * kBlkWarps, NMAX > 24 ? 2 : 3)
 
   for (int n = n0 + wp * FW; n < n1; n += kBlkWarps * FW) {
     float tr = 0.f, g2 = 0.f;
+    // 22.6 = 24 ln 2 + 6
+    const int J = series_terms(cdx, __double2float_rn((2.0 * n + 1.0) * pib), cr, 22.6f);
+    const bool series = J <= jmax;
+    const int nt = series ? J : n2;
+    const float2* Tt = series ? Cs : Ts;
+    if (lane < FW) sw[lane] = __double2float_rn((2.0 * min(n + lane, n1 - 1) + 1.0) * pib);
+    __syncwarp();
     for (int i = lane; i < FW * n2; i += 32) {
       const int b = i / FW, f = i - b * FW;
-      const float w = __double2float_rn((2.0 * min(n + f, n1 - 1) + 1.0) * pib), x = xs[b];
+      const float w = sw[f], x = xs[b];
       const float q = __frcp_rn(__fmaf_rn(x, x, __fmul_rn(w, w)));
       const float2 d = make_float2(__fmul_rn(x, q), -__fmul_rn(w, q)), d2 = fmul(d, d);
-      sd[i] = d;
-      sd2[i] = d2;
-      sd3[i] = fmul(d2, d);
+      if (!series) {
+        sd[i] = d;
+        sd2[i] = d2;
+        sd3[i] = fmul(d2, d);
+      }
       if (n + f < n1) {
         tr += d.x;
         g2 += d2.x;
       }
     }
+    if (series) {
+      // as series_z of gf_block.cu, with x = (z - c) / r, s = sqrt(x^2 - 1), xi = 1 / (x + s)
+      for (int i = lane; i < FW * J; i += 32) {
+        const int j = i / FW, f = i - j * FW;
+        const float ir = __frcp_rn(cr);
+        const float2 x = make_float2(cdx * ir, sw[f] * ir);
+        const float2 u = make_float2(fmaf(x.x, x.x, -fmaf(x.y, x.y, 1.f)), 2.f * x.x * x.y);
+        const float pr = sqrtf(0.5f * (sqrtf(fmaf(u.x, u.x, u.y * u.y)) + fabsf(u.x))), h = 0.5f * u.y / pr;
+        float2 s = u.x >= 0.f ? make_float2(pr, h) : make_float2(h, pr);
+        if (s.y < 0.f) s = make_float2(-s.x, -s.y);
+        float2 bs = frcp(make_float2(x.x + s.x, x.y + s.y)), pw = make_float2(j ? 2.f : 1.f, 0.f);
+#pragma unroll
+        for (int t = 0; t < 6; ++t) {
+          if ((j >> t) & 1) pw = fmul(pw, bs);
+          bs = fmul(bs, bs);
+        }
+        const float2 is = frcp(s), isr = make_float2(is.x * ir, is.y * ir), t = fmul(x, is);
+        const float fj = (float)j;
+        const float2 d1 = fmul(pw, isr);
+        const float2 c2 = fmul(isr, isr);  // 1 / (s^2 r^2)
+        // [j + t] / (s^2 r^2), then [(j^2 - 1) + 3 j t + 3 t^2] / (2 s^3 r^3), t = x / s
+        const float2 d2 = fmul(fmul(pw, c2), make_float2(fj + t.x, t.y));
+        const float2 t2 = fmul(t, t);
+        const float2 d3 = fmul(fmul(fmul(pw, c2), isr),
+                               make_float2(0.5f * (fmaf(fj, fj, -1.f) + 3.f * fmaf(fj, t.x, t2.x)),
+                                           1.5f * fmaf(fj, t.y, t2.y)));
+        sd[i] = d1;
+        sd2[i] = d2;
+        sd3[i] = d3;
+      }
+    }
     __syncwarp();
     for (int pr = lane; pr < NP; pr += 32) {
       const int a = pair[pr].x, c = pair[pr].y;
-      float2 xr[FW], xi[FW], yr[FW], yi[FW];
+      // packed FMAs: u = sum t.x d and v = sum t.y d, so that xr = (u.x, v.x), xi = (u.y, v.y)
+      float2 u[FW], v[FW], yu[FW], yv[FW];
 #pragma unroll
-      for (int f = 0; f < FW; ++f) xr[f] = xi[f] = yr[f] = yi[f] = z2();
-      const float2* t = Ts + pr;
+      for (int f = 0; f < FW; ++f) u[f] = v[f] = yu[f] = yv[f] = z2();
+      const float2* t = Tt + pr;
 #pragma unroll 4
-      for (int b = 0; b < n2; ++b) {
+      for (int b = 0; b < nt; ++b) {
         const float2 tv = __ldg(t + (size_t)b * NP);
+        const float2 tx = make_float2(tv.x, tv.x), ty = make_float2(tv.y, tv.y);
         const float4* d4 = reinterpret_cast<const float4*>(sd + b * FW);
         const float4* e4 = reinterpret_cast<const float4*>(sd2 + b * FW);
 #pragma unroll
         for (int f = 0; f < FW; f += 2) {
           const float4 d = d4[f / 2], e = e4[f / 2];
-          xr[f].x = __fmaf_rn(tv.x, d.x, xr[f].x);
-          xr[f].y = __fmaf_rn(tv.y, d.x, xr[f].y);
-          xi[f].x = __fmaf_rn(tv.x, d.y, xi[f].x);
-          xi[f].y = __fmaf_rn(tv.y, d.y, xi[f].y);
-          xr[f + 1].x = __fmaf_rn(tv.x, d.z, xr[f + 1].x);
-          xr[f + 1].y = __fmaf_rn(tv.y, d.z, xr[f + 1].y);
-          xi[f + 1].x = __fmaf_rn(tv.x, d.w, xi[f + 1].x);
-          xi[f + 1].y = __fmaf_rn(tv.y, d.w, xi[f + 1].y);
-          yr[f].x = __fmaf_rn(tv.x, e.x, yr[f].x);
-          yr[f].y = __fmaf_rn(tv.y, e.x, yr[f].y);
-          yi[f].x = __fmaf_rn(tv.x, e.y, yi[f].x);
-          yi[f].y = __fmaf_rn(tv.y, e.y, yi[f].y);
-          yr[f + 1].x = __fmaf_rn(tv.x, e.z, yr[f + 1].x);
-          yr[f + 1].y = __fmaf_rn(tv.y, e.z, yr[f + 1].y);
-          yi[f + 1].x = __fmaf_rn(tv.x, e.w, yi[f + 1].x);
-          yi[f + 1].y = __fmaf_rn(tv.y, e.w, yi[f + 1].y);
+          const float2 d0 = make_float2(d.x, d.y), d1 = make_float2(d.z, d.w);
+          const float2 e0 = make_float2(e.x, e.y), e1 = make_float2(e.z, e.w);
+          u[f] = __ffma2_rn(tx, d0, u[f]);
+          v[f] = __ffma2_rn(ty, d0, v[f]);
+          u[f + 1] = __ffma2_rn(tx, d1, u[f + 1]);
+          v[f + 1] = __ffma2_rn(ty, d1, v[f + 1]);
+          yu[f] = __ffma2_rn(tx, e0, yu[f]);
+          yv[f] = __ffma2_rn(ty, e0, yv[f]);
+          yu[f + 1] = __ffma2_rn(tx, e1, yu[f + 1]);
+          yv[f + 1] = __ffma2_rn(ty, e1, yv[f + 1]);
         }
       }
       const float2 h = hz[pr], o = oo[pr];
 #pragma unroll
       for (int f = 0; f < FW; ++f) {
         const int nn = min(n + f, n1 - 1);
-        const float w = __double2float_rn((2.0 * nn + 1.0) * pib);
+        const float w = sw[f];
         const float2* Sg = p.Ss + si.offSig + (int64_t)nn * M * M;
         const float2 s1 = __ldg(Sg + a * M + c), s2 = __ldg(Sg + c * M + a);
         float2* Sm = sS + f * M * NMAX;
         float2* Fm = sF + f * M * NMAX;
         // z o_ac - h_ac - Sigma_ac - g_ac and, with conj(o) and conj(h), (c, a)
-        Sm[a * NMAX + c] = make_float2(__fmaf_rn(-w, o.y, h.x) - s1.x - (xr[f].x - xi[f].y),
-                                       __fmaf_rn(w, o.x, h.y) - s1.y - (xr[f].y + xi[f].x));
-        Fm[a * NMAX + c] = make_float2(o.x + (yr[f].x - yi[f].y), o.y + (yr[f].y + yi[f].x));
+        Sm[a * NMAX + c] = make_float2(__fmaf_rn(-w, o.y, h.x) - s1.x - (u[f].x - v[f].y),
+                                       __fmaf_rn(w, o.x, h.y) - s1.y - (v[f].x + u[f].y));
+        Fm[a * NMAX + c] = make_float2(o.x + (yu[f].x - yv[f].y), o.y + (yv[f].x + yu[f].y));
         if (a != c) {
-          Sm[c * NMAX + a] = make_float2(__fmaf_rn(w, o.y, h.x) - s2.x - (xr[f].x + xi[f].y),
-                                         __fmaf_rn(w, o.x, -h.y) - s2.y - (xi[f].x - xr[f].y));
-          Fm[c * NMAX + a] = make_float2(o.x + (yr[f].x + yi[f].y), (yi[f].x - yr[f].y) - o.y);
+          Sm[c * NMAX + a] = make_float2(__fmaf_rn(w, o.y, h.x) - s2.x - (u[f].x + v[f].y),
+                                         __fmaf_rn(w, o.x, -h.y) - s2.y - (u[f].y - v[f].x));
+          Fm[c * NMAX + a] = make_float2(o.x + (yu[f].x + yv[f].y), (yu[f].y - yv[f].x) - o.y);
         }
       }
     }
@@ -230,26 +274,31 @@ __global__ void __launch_bounds__(32 * kBlkWarps, NMAX > 24 ? 2 : 3)
       // this lane: row i = q_sl of S^{-1}; register x holds the stored column (x + M) mod NMAX,
       // which is column p_c of the inverse.  X = S^{-1} F, row i.
       const int row = sl < M ? sq[sl] : 0;
-      float2 x[NMAX];
+      float2 x[NMAX], xt[NMAX];  // sum g.x F and sum g.y F (packed FMAs)
 #pragma unroll
-      for (int c = 0; c < NMAX; ++c) x[c] = z2();
+      for (int c = 0; c < NMAX; ++c) x[c] = xt[c] = z2();
 #pragma unroll
       for (int y = 0; y < NMAX; ++y) {
         int c = y + M;
         if (c >= NMAX) c -= NMAX;
         if (c < M) {
-          const float2 g = fmul(sc, a[y]);
+          const float2 g = fmul(sc, a[y]), gx = make_float2(g.x, g.x), gy = make_float2(g.y, g.y);
           const int pc = sp[c];
           if (sl < M) Sm[row * NMAX + pc] = g;
           const float4* f4 = reinterpret_cast<const float4*>(Fm + pc * NMAX);
 #pragma unroll
           for (int z = 0; z < NMAX; z += 2) {
             const float4 v = f4[z / 2];
-            fmac(x[z], g, make_float2(v.x, v.y));
-            fmac(x[z + 1], g, make_float2(v.z, v.w));
+            const float2 v0 = make_float2(v.x, v.y), v1 = make_float2(v.z, v.w);
+            x[z] = __ffma2_rn(gx, v0, x[z]);
+            xt[z] = __ffma2_rn(gy, v0, xt[z]);
+            x[z + 1] = __ffma2_rn(gx, v1, x[z + 1]);
+            xt[z + 1] = __ffma2_rn(gy, v1, xt[z + 1]);
           }
         }
       }
+#pragma unroll
+      for (int z = 0; z < NMAX; ++z) x[z] = make_float2(x[z].x - xt[z].y, x[z].y + xt[z].x);
       __syncwarp();  // every lane is done with F
       if (sl < M) {
 #pragma unroll
@@ -271,25 +320,23 @@ __global__ void __launch_bounds__(32 * kBlkWarps, NMAX > 24 ? 2 : 3)
     // 2 Tr(S^{-1} B D^3 B^+)
     for (int pr = lane; pr < NP; pr += 32) {
       const int a = pair[pr].x, c = pair[pr].y;
-      float2 xr[FW], xi[FW];
+      float2 u[FW], v[FW];
 #pragma unroll
-      for (int f = 0; f < FW; ++f) xr[f] = xi[f] = z2();
-      const float2* t = Ts + pr;
+      for (int f = 0; f < FW; ++f) u[f] = v[f] = z2();
+      const float2* t = Tt + pr;
 #pragma unroll 4
-      for (int b = 0; b < n2; ++b) {
+      for (int b = 0; b < nt; ++b) {
         const float2 tv = __ldg(t + (size_t)b * NP);
+        const float2 tx = make_float2(tv.x, tv.x), ty = make_float2(tv.y, tv.y);
         const float4* d4 = reinterpret_cast<const float4*>(sd3 + b * FW);
 #pragma unroll
         for (int f = 0; f < FW; f += 2) {
           const float4 d = d4[f / 2];
-          xr[f].x = __fmaf_rn(tv.x, d.x, xr[f].x);
-          xr[f].y = __fmaf_rn(tv.y, d.x, xr[f].y);
-          xi[f].x = __fmaf_rn(tv.x, d.y, xi[f].x);
-          xi[f].y = __fmaf_rn(tv.y, d.y, xi[f].y);
-          xr[f + 1].x = __fmaf_rn(tv.x, d.z, xr[f + 1].x);
-          xr[f + 1].y = __fmaf_rn(tv.y, d.z, xr[f + 1].y);
-          xi[f + 1].x = __fmaf_rn(tv.x, d.w, xi[f + 1].x);
-          xi[f + 1].y = __fmaf_rn(tv.y, d.w, xi[f + 1].y);
+          const float2 d0 = make_float2(d.x, d.y), d1 = make_float2(d.z, d.w);
+          u[f] = __ffma2_rn(tx, d0, u[f]);
+          v[f] = __ffma2_rn(ty, d0, v[f]);
+          u[f + 1] = __ffma2_rn(tx, d1, u[f + 1]);
+          v[f + 1] = __ffma2_rn(ty, d1, v[f + 1]);
         }
       }
 #pragma unroll
@@ -297,11 +344,11 @@ __global__ void __launch_bounds__(32 * kBlkWarps, NMAX > 24 ? 2 : 3)
         if (n + f >= n1) continue;
         const float2* Sm = sS + f * M * NMAX;
         const float2 g1 = Sm[a * NMAX + c];
-        const float z2x = xr[f].x + xi[f].y, z2y = xi[f].x - xr[f].y;  // (c, a)
+        const float z2x = u[f].x + v[f].y, z2y = u[f].y - v[f].x;  // (c, a)
         float s = __fmaf_rn(g1.x, z2x, -__fmul_rn(g1.y, z2y));
         if (a != c) {
           const float2 gt = Sm[c * NMAX + a];
-          const float z1x = xr[f].x - xi[f].y, z1y = xr[f].y + xi[f].x;  // (a, c)
+          const float z1x = u[f].x - v[f].y, z1y = v[f].x + u[f].y;  // (a, c)
           s = __fmaf_rn(gt.x, z1x, __fmaf_rn(-gt.y, z1y, s));
         }
         g2 = __fmaf_rn(2.f, s, g2);
@@ -340,8 +387,7 @@ struct Shape32 {
 };
 __host__ Shape32 shape32(int m) {
   if (m <= 8) return {8, 8, 4};
-  if (m <= 12) return {12, 16, 4};
-  if (m <= 16) return {16, 16, 4};
+  if (m <= 16) return {(m + 1) & ~1, 16, 4};
   if (m <= 20) return {20, 32, 2};
   if (m <= 24) return {24, 32, 2};
   return {32, 32, 2};
@@ -369,7 +415,9 @@ cudaError_t launch_occ_block32(const PointParams& p, const BlockForm& b, const B
   const size_t smem = block32_smem(p.mmax, l.n2max);
   switch (shape32(p.mmax).nmax) {
     case 8: return launch32<8, 8, 4>(p, b, l, smem, s);
+    case 10: return launch32<10, 16, 4>(p, b, l, smem, s);
     case 12: return launch32<12, 16, 4>(p, b, l, smem, s);
+    case 14: return launch32<14, 16, 4>(p, b, l, smem, s);
     case 16: return launch32<16, 16, 4>(p, b, l, smem, s);
     case 20: return launch32<20, 32, 2>(p, b, l, smem, s);
     case 24: return launch32<24, 32, 2>(p, b, l, smem, s);

@@ -177,6 +177,10 @@ struct gf_ctx {
   int64_t blk_totT = 0, blk_totC = 0;
   int run_chunks = 1;                         // the current call: chunks of its partial sums,
   bool run_on_block = false;                  // and whether it runs on the block form
+  // mixed precision: the FP64 launch of the low frequencies runs beside the FP32 one, on a
+  // stream that forks from the call's and joins it again
+  cudaStream_t side = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int occ_path = 0;                           // path that the captured N(mu) graph holds
   DevBuf blk_units, blk_perm, blk_sysg, blk_offT;  // (blk_offT: offsets of T, then of C)
   DevBuf blk_e, blk_T, blk_Ts, blk_B, blk_Bs, blk_HO, blk_U, blk_D22, blk_V, blk_R, blk_H11, blk_tau,
