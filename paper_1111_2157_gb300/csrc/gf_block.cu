@@ -440,7 +440,7 @@ __device__ __forceinline__ double2 cpow_int(double2 b, int j) {
 // Then S, with LOW S^{-1} in FP32, d (or the series coefficients), the pivot tables, w_n, the pair
 // list, mu O - H11 by pairs and, with LOW, B.
 struct LayoutB {
-  size_t oS, oF, od2, orc, oM, oR, oY, oG, od, op, oW, oPair, oHz, oB, bytes;
+  size_t oS, oF, od2, orc, oM, oR, oY, oG, od, op, oW, oPair, oHz, oX, oB, bytes;
   size_t sS, sF, sd2, src, sG, sd, sp;  // bytes per warp (sS also of M, sG of R)
   int nf;   // frequencies per warp
   int yf;   // frequencies of the rho_k columns staged at once
@@ -467,10 +467,12 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   L.od2 = o; o += W * L.sd2;
   L.orc = o; o += W * L.src;
   L.oM = o; o += (mode & kAdj) ? W * L.sS : 0;
-  L.oR = o; o += W * L.sG;
+  // the refinement's residual: over F, which is read before
+  L.oR = needF ? L.oF : o;
+  if (low && (mode & kGloc) && !needF) o += W * L.sG;
   const size_t np = (size_t)mmax * (mmax + 1) / 2;
   const size_t fixed = W * (L.sG + L.sd + L.sp + (low ? 16 : 8) * f) + al(2 * np) + (low ? 32 : 16) * np +
-                       (low && rho ? 8 * mmax * (((size_t)n2max + 3) & ~(size_t)3) : 0);
+                       (low && rho ? 8 * mmax * (((size_t)n2max + 3) & ~(size_t)3) + al(4 * (size_t)n2max) : 0);
   L.yf = 0;
   if (rho) {
     // as many frequencies as fit over the dead arrays, or as leave three CTAs on an SM, or two:
@@ -493,6 +495,7 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   L.oW = o; o = al(o + (low ? 16 : 8) * W * f);  // w_n (low: and in pairs)
   L.oPair = o; o += al(2 * np);
   L.oHz = o; o += (low ? 32 : 16) * np;  // (low: pairs of mu O - H11, then of O)
+  L.oX = o; o = al(o + (low && rho ? 4 * (size_t)n2max : 0));
   L.oB = o; o += low && rho ? 8 * mmax * (((size_t)n2max + 3) & ~(size_t)3) : 0;
   L.bytes = o;
   return L;
@@ -523,6 +526,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
   float2* sWp = reinterpret_cast<float2*>(smraw + L.oW + 8 * W * F) + wp * F;
   uchar2* pair = reinterpret_cast<uchar2*>(smraw + L.oPair);
   double2* hz = reinterpret_cast<double2*>(smraw + L.oHz);
+  float* xs = reinterpret_cast<float*>(smraw + L.oX);  // x_b = mu - e_b
   const int unit = bl.unit0 + blockIdx.x / bl.n_chunks, ch = blockIdx.x % bl.n_chunks;
   const int2 un = bl.units[unit];
   const int n0 = bl.n_begin + ch * bl.chunk_w, n1 = min(bl.n_end, n0 + bl.chunk_w);
@@ -561,6 +565,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
       if (rho) {
         float2* sB = reinterpret_cast<float2*>(smraw + L.oB);
         const int pt = (n2 + 3) & ~3;
+        for (int i = tid; i < n2; i += 32 * W) xs[i] = __double2float_rn(mu - e_k[i]);
         for (int i = tid; i < M * n2; i += 32 * W) sB[(i / n2) * pt + i % n2] = bf.Bs[ki.offP + i];
       }
     }
@@ -637,7 +642,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
                                                          fmaf(j2, zf[2].y, fmaf(fj, zf[3].y, zf[4].y))));
                   if (f < nv) {
                     acc_tr = fma(tau[j], d.x, acc_tr);
-                    acc_g2 = fma(tau[j], (double)d2.x, acc_g2);
+                    acc_g2 = fma(tau[j], widen(d2.x), acc_g2);
                   }
                 }
               } else if (occ || adj) {
@@ -665,15 +670,14 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             const double s = 1.0 / fma(x, x, wn * wn);
             const double2 d = make_double2(x * s, -wn * s);
             if constexpr (LOW) {
-              if (sums) put_d(i, d);
-              else sd[i] = d;
-              if (sums && occ) {
+              put_d(i, d);
+              if (occ) {
                 const float2 df = make_float2((float)d.x, (float)d.y), d2 = fmul(df, df);
                 sd2[i] = d2;
                 sd2[F * n2 + i] = fmul(d2, df);
                 if (f < nv) {
                   acc_tr += d.x;
-                  acc_g2 += (double)d2.x;
+                  acc_g2 += widen(d2.x);
                 }
               }
             } else if (sd[i] = d; sums && (occ || adj)) {
@@ -807,48 +811,33 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
           }
         }
         __syncwarp();
-        if (rho && (series || LOW)) bands(false);  // rho_k reads d_b in FP64 (its barrier comes first)
+        // rho_k reads d_b (its barrier comes first): in FP32 with LOW
+        if constexpr (LOW) {
+          if (rho)
+            for (int i = lane; i < F * n2; i += 32) {
+              const int f = i / n2;
+              const float x = xs[i - f * n2], w = sWp[f].x, q = __frcp_rn(fmaf(x, x, w * w));
+              reinterpret_cast<float2*>(sd)[i] = make_float2(x * q, -w * q);
+            }
+        } else if (rho && series) {
+          bands(false);
+        }
         const int* sq = sp + M;
         const bool mine = mf < nv;
         double2* out = (p.mode & (kGloc | kAdj))
                            ? p.gq + ((int64_t)(unit - p.gb0) * p.n_iw + min(n + mf, n1 - 1)) * p.mmax * p.mmax
                            : nullptr;
+        const rc_t* inv;  // the warp's inverses, A[p_i][q_c] (LOW: FP32)
         if constexpr (LOW) {
-          // X0 = S^{-1} in FP32 and one step of refinement, S^{-1} = X0 + X0 R with R = I - S X0
-          // from S in FP32 pairs: 1e-15 of the FP64 inverse at these frequencies, where the FP64
-          // elimination takes 1,500 FP64 instructions a matrix at m = 20.
-          float4* Sp = reinterpret_cast<float4*>(A);
+          const float4* Sp = reinterpret_cast<const float4*>(A);
           float2* X0 = sG + mf * MM;
-          float2* R = reinterpret_cast<float2*>(smraw + L.oR + wp * L.sG) + mf * MM;
           for (int i = sl; i < MM; i += LW) X0[i] = make_float2(Sp[i].x, Sp[i].z);
           __syncwarp();
           gj64::invert<LW>(X0, M, rcb, sp, sl, p.status);
-          for (int i = sl; i < MM; i += LW) {
-            const int a = i / M, c = i - a * M, qc = sq[c];
-            cf acc = czero();
-            if (a == c) acc.rh = 1.f;
-            for (int x = 0; x < M; ++x) cacc1(acc, cneg(ld4(Sp[a * M + x])), X0[sp[x] * M + qc]);
-            R[i] = make_float2(__fadd_rn(acc.rh, acc.rl), __fadd_rn(acc.ih, acc.il));
-          }
-          __syncwarp();
-          float2* Gn = reinterpret_cast<float2*>(A);  // S^{-1} in the orbitals' order (S is dead)
-          for (int i = sl; i < MM; i += LW) {
-            const int a = i / M, c = i - a * M, pa = sp[a] * M;
-            float2 d = make_float2(0.f, 0.f);
-            for (int x = 0; x < M; ++x) fmac(d, X0[pa + sq[x]], R[x * M + c]);
-            const float2 g = X0[pa + sq[c]];
-            float2 h, l;
-            two_sum(g.x, d.x, h.x, l.x);
-            two_sum(g.y, d.y, h.y, l.y);
-            Gn[i] = h;
-            if ((p.mode & kGloc) && mine)
-              gq_put(&out[i], q, make_double2(wk * ((double)h.x + (double)l.x), wk * ((double)h.y + (double)l.y)));
-          }
-          __syncwarp();
-          for (int i = sl; i < MM; i += LW) X0[i] = Gn[i];
-          __syncwarp();
+          inv = sG;
         } else {
           gj64::invert<LW>(A, M, rcb, sp, sl, p.status);
+          inv = sS;
           if ((p.mode & kGloc) && mine)
             for (int i = sl; i < MM; i += LW) {
               const int a = i / M, c = i - a * M;
@@ -862,28 +851,17 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             const int f = i / NP, pr = i - f * NP;
             const int a = pair[pr].x, c = pair[pr].y;
             const rc_t* Fm = sF + f * MM;
-            rc_t x1 = rzero(rc_t{}), x2 = x1, g1, g2;
-            if constexpr (LOW) {
-              const float2* Gf = sG + f * MM;
-              for (int j = 0; j < M; ++j) {
-                rmac(x1, Gf[a * M + j], Fm[j * M + c]);
-                rmac(x2, Gf[c * M + j], Fm[j * M + a]);
-              }
-              g1 = Gf[a * M + c];
-              g2 = Gf[c * M + a];
-            } else {
-              const int* pf = sPv + f * 2 * M;
-              const int* qf = pf + M;
-              const double2* Af = sS + f * MM;
-              const int pa = pf[a] * M, pc = pf[c] * M;
-              for (int j = 0; j < M; ++j) {
-                const int fj = pf[j] * M;
-                rmac(x1, Af[pa + j], Fm[fj + c]);
-                if (a != c) rmac(x2, Af[pc + j], Fm[fj + a]);
-              }
-              g1 = Af[pa + qf[c]];
-              g2 = Af[pc + qf[a]];
+            rc_t x1 = rzero(rc_t{}), x2 = x1;
+            const int* pf = sPv + f * 2 * M;
+            const int* qf = pf + M;
+            const rc_t* Af = inv + f * MM;
+            const int pa = pf[a] * M, pc = pf[c] * M;
+            for (int j = 0; j < M; ++j) {
+              const int fj = pf[j] * M;
+              rmac(x1, Af[pa + j], Fm[fj + c]);
+              if (LOW || a != c) rmac(x2, Af[pc + j], Fm[fj + a]);
             }
+            const rc_t g1 = Af[pa + qf[c]], g2 = Af[pc + qf[a]];
             rc_t zr = rzero(rc_t{}), zi = zr;
             const rc_t* d3f = sd2 + F * n2 + f * nt;
             if constexpr (LOW) {
@@ -927,6 +905,45 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             acc_tr += (double)low_tr;
             acc_g2 += (double)low_g2;
           }
+          __syncwarp();
+        }
+        if constexpr (LOW) {
+          // S^{-1} in the orbitals' order for rho_k, and for G_loc one step of refinement,
+          // S^{-1} = X0 + X0 R with R = I - S X0 from S in FP32 pairs: 1e-15 of the FP64 inverse at
+          // these frequencies, where the FP64 elimination takes 1,500 FP64 instructions a matrix
+          // at m = 20.
+          const float4* Sp = reinterpret_cast<const float4*>(A);
+          float2* X0 = sG + mf * MM;
+          float2* R = reinterpret_cast<float2*>(smraw + L.oR + wp * L.sG) + mf * MM;
+          const bool refine = (p.mode & kGloc) != 0;
+          if (refine) {
+            for (int i = sl; i < MM; i += LW) {
+              const int a = i / M, c = i - a * M, qc = sq[c];
+              cf acc = czero();
+              if (a == c) acc.rh = 1.f;
+              for (int x = 0; x < M; ++x) cacc1(acc, cneg(ld4(Sp[a * M + x])), X0[sp[x] * M + qc]);
+              R[i] = make_float2(__fadd_rn(acc.rh, acc.rl), __fadd_rn(acc.ih, acc.il));
+            }
+            __syncwarp();
+          }
+          float2* Gn = reinterpret_cast<float2*>(A);  // (S is dead)
+          for (int i = sl; i < MM; i += LW) {
+            const int a = i / M, c = i - a * M, pa = sp[a] * M;
+            const float2 g = X0[pa + sq[c]];
+            float2 h = g;
+            if (refine) {
+              float2 d = make_float2(0.f, 0.f), l;
+              for (int x = 0; x < M; ++x) fmac(d, X0[pa + sq[x]], R[x * M + c]);
+              two_sum(g.x, d.x, h.x, l.x);
+              two_sum(g.y, d.y, h.y, l.y);
+              if (mine)
+                gq_put(&out[i], q, make_double2(wk * (widen(h.x) + widen(l.x)), wk * (widen(h.y) + widen(l.y))));
+            }
+            Gn[i] = h;
+          }
+          __syncwarp();
+          if (rho)
+            for (int i = sl; i < MM; i += LW) X0[i] = Gn[i];
           __syncwarp();
         }
         if constexpr (!LOW) {
@@ -994,17 +1011,21 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             const int a = i / M, c = i - a * M;
             const double2 o = old(a * nb + c);
             double2 v = make_double2(0.0, 0.0);
-            for (int f = f0; f < f0 + nf; ++f) {
-              double2 g;
-              if constexpr (LOW) {
+            if constexpr (LOW) {
+              float2 g = make_float2(0.f, 0.f);
+              for (int f = f0; f < f0 + nf; ++f) {
                 const float2 gf = reinterpret_cast<const float2*>(smraw + L.oG + (f / F) * L.sG)[(f % F) * MM + i];
-                g = make_double2((double)gf.x, (double)gf.y);
-              } else {
-                const int* pf = piv(f);
-                g = mat(f)[pf[a] * M + pf[M + c]];
+                g.x += gf.x;
+                g.y += gf.y;
               }
-              v.x += g.x;
-              v.y += g.y;
+              v = make_double2(widen(g.x), widen(g.y));
+            } else {
+              for (int f = f0; f < f0 + nf; ++f) {
+                const int* pf = piv(f);
+                const double2 g = mat(f)[pf[a] * M + pf[M + c]];
+                v.x += g.x;
+                v.y += g.y;
+              }
             }
             add(a * nb + c, o, v);
           }
@@ -1016,8 +1037,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             const float2* sB = reinterpret_cast<const float2*>(smraw + L.oB);
             float2* sY = reinterpret_cast<float2*>(smraw + L.oY);  // [yf][M][pt]: S^{-1} B D
             auto dlow = [&](int f, int b) {
-              const double2 d = dof(f)[b];
-              return make_float2((float)d.x, (float)d.y);
+              return reinterpret_cast<const float2*>(smraw + L.od + (f / F) * L.sd)[(f % F) * n2 + b];
             };
             // (1,2) and (2,1): Y = S^{-1} B D, Z = D B^+ S^{-1}; four orbitals and two bands a thread
             const int at4 = (M + 3) / 4, ct = (n2 + 1) / 2;
@@ -1074,8 +1094,8 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
                   if (a0 + u < M) {
-                    add(ar[u] * nb + M + c, o12[u], make_double2(v12[u][v].x, v12[u][v].y));
-                    add((M + c) * nb + ar[u], o21[u], make_double2(v21[u][v].x, v21[u][v].y));
+                    add(ar[u] * nb + M + c, o12[u], make_double2(widen(v12[u][v].x), widen(v12[u][v].y)));
+                    add((M + c) * nb + ar[u], o21[u], make_double2(widen(v21[u][v].x), widen(v21[u][v].y)));
                   }
               }
             }
@@ -1133,14 +1153,14 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
 #pragma unroll
                   for (int w = 0; w < CW; ++w) {
                     if (c0 + w >= n2) break;
-                    double2 s = make_double2(v[u][w].x, v[u][w].y);
+                    float2 s = v[u][w];
                     if (bb == c0 + w)
                       for (int f = f0; f < f0 + nf; ++f) {
-                        const double2 d = dof(f)[bb];
+                        const float2 d = dlow(f, bb);
                         s.x += d.x;
                         s.y += d.y;
                       }
-                    add(at + c0 + w, o[w], s);
+                    add(at + c0 + w, o[w], make_double2(widen(s.x), widen(s.y)));
                   }
                 }
               }

@@ -57,6 +57,16 @@ __device__ __forceinline__ double rcp_newton(double x) {
   return fma(r, fma(-x, r, 1.0), r);
 }
 
+// (double)x by integer arithmetic on the bits: a conversion instruction runs on the FP64 pipe, where
+// it takes a warp as long as an FMA.  Exact; FP32 denormals become 0.
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+  unsigned hi = (u & 0x80000000u) | ((m >> 3) + 0x38000000u);
+  if (m >= 0x7f800000u) hi |= 0x7ff00000u;  // infinity, NaN
+  const bool zero = m < 0x00800000u;
+  return __hiloint2double(zero ? (int)(u & 0x80000000u) : (int)hi, zero ? 0 : (int)(u << 29));
+}
+
 // Pivot key of a complex FP64 number: max(|Re|, |Im|) compared through the IEEE
 // bit pattern, which orders non-negative doubles like their values; no FP64
 // instruction.
