@@ -179,6 +179,13 @@ gf_status ensure_block(gf_ctx* c) {
   return GF_OK;
 }
 
+// Whether the frequencies from blk_nc on run in FP32 and FP32 pairs.  The adjoint's pairs of S, F and
+// Gbar need 5/4 of the FP64 kernel's shared memory: from 30 orbitals on it may stay in FP64.
+bool block_low(const gf_ctx* c, int mode) {
+  return c->precision == GF_PREC_MIXED && !c->lowrank &&
+         (!(mode & gf::kAdj) || gf::block_smem(c->mmax, c->blk_n2max, mode, 1) <= (size_t)c->smem_optin - 1024);
+}
+
 // Whether a call of this mode runs on the block form.  GF_KERNEL=direct keeps the general
 // kernels; with GF_PREC_MIXED every value of GF_KERNEL does, as it names one of them.
 bool use_block(const gf_ctx* c, int mode) {
@@ -191,8 +198,8 @@ bool use_block(const gf_ctx* c, int mode) {
                                     : gf::point_fp64_smem(c->nbmax, c->mmax, mode, 0);
   if (general > limit || (c->lowrank && c->nbmax > gf::heev_max_n())) return false;
   return gf::block_smem(c->mmax, c->blk_n2max, mode, 0) <= limit &&
-         (c->precision != GF_PREC_MIXED || (gf::block_smem(c->mmax, c->blk_n2max, mode, 1) <= limit &&
-                                            gf::block32_smem(c->mmax, c->blk_n2max) <= limit));
+         (!block_low(c, mode) || (gf::block_smem(c->mmax, c->blk_n2max, mode, 1) <= limit &&
+                                  gf::block32_smem(c->mmax, c->blk_n2max) <= limit));
 }
 
 // rho_k partial sums: the low-rank and the block kernels leave them in the basis that makes
@@ -507,10 +514,10 @@ double point_flops_lr(int N, int M, int mode) {
 
 // The point kernels on the block form, for every k (or k-group) and frequency chunk: one
 // launch in FP64, and in mixed precision a second one for the frequencies from blk_nc on,
-// whose traces and rho_k need FP32 only.
+// whose traces and rho_k need FP32 only and whose G_loc and adjoint FP32 pairs.
 gf_status run_block(gf_ctx* c, int mode, gf::PointParams p) {
   const bool kred = (mode & (gf::kGloc | gf::kAdj)) != 0;
-  const bool low = c->precision == GF_PREC_MIXED && !c->lowrank && !(mode & gf::kAdj);
+  const bool low = block_low(c, mode);
   const int nc = low ? c->blk_nc : c->n_iw;
   // (the few FP64 frequencies of mixed precision in chunks of one batch: they are latency bound)
   const int cw0 = low ? gf::block_batch(c->mmax) : c->blk_cw;
@@ -612,7 +619,7 @@ gf_status run_block(gf_ctx* c, int mode, gf::PointParams p) {
   if (c->tuned.find(key) == c->tuned.end()) {
     c->tuned[key] = 0;
     c->tune_log += "mode " + std::to_string(mode) + ": block form, " + std::to_string(nc) + " frequencies in FP64" +
-                   (ch1 ? ", " + std::to_string(c->n_iw - nc) + " in FP32 (traces, rho)" : std::string()) + "; ";
+                   (ch1 ? ", " + std::to_string(c->n_iw - nc) + " in FP32 and FP32 pairs" : std::string()) + "; ";
   }
   return GF_OK;
 }

@@ -441,7 +441,7 @@ __device__ __forceinline__ double2 cpow_int(double2 b, int j) {
 // list, mu O - H11 by pairs and, with LOW, B.
 struct LayoutB {
   size_t oS, oF, od2, orc, oM, oR, oY, oG, od, op, oW, oPair, oHz, oX, oB, bytes;
-  size_t sS, sF, sd2, src, sG, sd, sp;  // bytes per warp (sS also of M, sG of R)
+  size_t sS, sF, sd2, src, sG, sR, sd, sp;  // bytes per warp (sS also of M)
   int nf;   // frequencies per warp
   int yf;   // frequencies of the rho_k columns staged at once
 };
@@ -450,11 +450,12 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   LayoutB L;
   L.nf = 32 / gj64::lanes(mmax);
   const size_t f = L.nf, mm = (size_t)mmax * mmax, r = low ? 8 : 16, W = kBlkWarps;
-  const bool needF = (mode & (kOcc | kAdj)) != 0, rho = (mode & kRho) != 0;
+  const bool adj = (mode & kAdj) != 0, needF = (mode & kOcc) != 0 || adj, rho = (mode & kRho) != 0;
   auto al = [](size_t x) { return (x + 15) & ~(size_t)15; };
   L.sS = 16 * f * mm;
-  L.sF = needF ? al(r * f * mm) : 0;
-  L.sd2 = needF ? al(2 * r * f * n2max) : 0;
+  // (the adjoint's F and d^2 are pairs with LOW)
+  L.sF = needF ? al((adj ? 16 : r) * f * mm) : 0;
+  L.sd2 = needF ? al((low && adj ? 24 : 2 * r) * f * n2max) : 0;
   L.src = (low ? 8 : 16) * f * 2 * mmax;
   L.sG = low ? al(8 * f * mm) : 0;
   L.sd = 16 * f * n2max;
@@ -466,9 +467,10 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   L.oF = o; o += W * L.sF;
   L.od2 = o; o += W * L.sd2;
   L.orc = o; o += W * L.src;
-  L.oM = o; o += (mode & kAdj) ? W * L.sS : 0;
-  // the refinement's residual: over F, which is read before
-  L.oR = needF ? L.oF : o;
+  L.oM = o; o += adj ? W * L.sS : 0;
+  // the refinement's residual: over M or F, of which one is not yet and one no longer in use
+  L.oR = adj ? L.oM : (needF ? L.oF : o);
+  L.sR = adj ? L.sS : L.sG;
   if (low && (mode & kGloc) && !needF) o += W * L.sG;
   const size_t np = (size_t)mmax * (mmax + 1) / 2;
   const size_t fixed = W * (L.sG + L.sd + L.sp + (low ? 16 : 8) * f) + al(2 * np) + (low ? 32 : 16) * np +
@@ -504,7 +506,7 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
 __device__ __forceinline__ double2 ld_cg(const double2* p) { return __ldg(p); }
 __device__ __forceinline__ float2 ld_cg(const float2* p) { return __ldg(p); }
 
-template <int LW, bool LOW>
+template <int LW, bool LOW, bool ADJ>
 __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
     k_point_block(const PointParams p, const BlockForm bf, const BlockLaunch bl) {
   using rc_t = typename Rest<LOW>::c;
@@ -520,6 +522,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
   double2* sd = reinterpret_cast<double2*>(smraw + L.od + wp * L.sd);
   rc_t* sd2 = reinterpret_cast<rc_t*>(smraw + L.od2 + wp * L.sd2);
   double2* sM = reinterpret_cast<double2*>(smraw + L.oM + wp * L.sS);
+  constexpr bool low_adj = LOW && ADJ;  // F and d^2 in pairs
   float2* sG = reinterpret_cast<float2*>(smraw + L.oG + wp * L.sG);
   int* sPv = reinterpret_cast<int*>(smraw + L.op + wp * L.sp);
   double* sW = reinterpret_cast<double*>(smraw + L.oW) + wp * F;
@@ -531,7 +534,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
   const int2 un = bl.units[unit];
   const int n0 = bl.n_begin + ch * bl.chunk_w, n1 = min(bl.n_end, n0 + bl.chunk_w);
   const int chunk = bl.chunk0 + ch;
-  const bool occ = (p.mode & kOcc) != 0, adj = (p.mode & kAdj) != 0, rho = (p.mode & kRho) != 0;
+  const bool occ = (p.mode & kOcc) != 0, adj = ADJ, rho = !ADJ && (p.mode & kRho) != 0;
 
   for (int q = 0; q < un.y; ++q) {
     const int kk = bl.kperm[un.x + q];
@@ -543,8 +546,9 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
     const double2* T = bf.T + bf.offT[kk];
     const double2* HO = bf.HO + (size_t)kk * 2 * bf.npmax;
     const double cb = (adj && p.nbar) ? p.nbar[ki.sys] * 2.0 / si.beta : 0.0;
-    const bool have_gbar = adj && p.gbar != nullptr;
+    const bool have_gbar = adj && (LOW ? (const void*)p.Gbd : (const void*)p.gbar) != nullptr;
     double2* A = sS + mf * MM;  // this lane group's matrix
+    rc_t* sd3 = sd2 + (low_adj ? 2 : 1) * F * n2;
     rc_t* rcb = reinterpret_cast<rc_t*>(smraw + L.orc + wp * L.src) + mf * 2 * M;
     int* sp = sPv + mf * 2 * M;
     __syncthreads();
@@ -633,12 +637,17 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
               const double2 d = cmul(pw, z.c1);
               put_d(i, d);
               if constexpr (LOW) {
+                if (adj) {
+                  const double fj = j;
+                  reinterpret_cast<float4*>(sd2)[i] =
+                      st4(from_d2(cmul(pw, make_double2(fma(fj, z.c2a.x, z.c2b.x), fma(fj, z.c2a.y, z.c2b.y)))));
+                }
                 if (occ) {
                   const float2 pf = make_float2((float)pw.x, (float)pw.y);
                   const float fj = (float)j, j2 = fj * fj - 1.f;
                   const float2 d2 = fmul(pf, make_float2(fmaf(fj, zf[0].x, zf[1].x), fmaf(fj, zf[0].y, zf[1].y)));
-                  sd2[i] = d2;
-                  sd2[F * n2 + i] = fmul(pf, make_float2(fmaf(j2, zf[2].x, fmaf(fj, zf[3].x, zf[4].x)),
+                  if (!adj) sd2[i] = d2;
+                  sd3[i] = fmul(pf, make_float2(fmaf(j2, zf[2].x, fmaf(fj, zf[3].x, zf[4].x)),
                                                          fmaf(j2, zf[2].y, fmaf(fj, zf[3].y, zf[4].y))));
                   if (f < nv) {
                     acc_tr = fma(tau[j], d.x, acc_tr);
@@ -651,7 +660,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
                 sd2[i] = d2;
                 if (occ) {
                   const double j2 = fma(fj, fj, -1.0);
-                  sd2[F * n2 + i] = cmul(pw, make_double2(fma(j2, z.c3a.x, fma(fj, z.c3b.x, z.c3c.x)),
+                  sd3[i] = cmul(pw, make_double2(fma(j2, z.c3a.x, fma(fj, z.c3b.x, z.c3c.x)),
                                                           fma(j2, z.c3a.y, fma(fj, z.c3b.y, z.c3c.y))));
                   if (f < nv) {
                     acc_tr = fma(tau[j], d.x, acc_tr);
@@ -667,14 +676,22 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             const int f = i / n2, bb = i - f * n2;
             const double wn = sW[f];
             const double x = mu - e_k[bb];
-            const double s = 1.0 / fma(x, x, wn * wn);
+            const double xw = fma(x, x, wn * wn);
+            const double s = LOW ? rcp_newton(xw) : 1.0 / xw;
             const double2 d = make_double2(x * s, -wn * s);
             if constexpr (LOW) {
-              put_d(i, d);
+              const cf dp = from_d2(d);
+              reinterpret_cast<float4*>(sd)[i] = st4(dp);
+              if (adj) {
+                cf d2 = czero();
+                cacc(d2, dp, dp);
+                cnorm(d2);
+                reinterpret_cast<float4*>(sd2)[i] = st4(d2);
+              }
               if (occ) {
-                const float2 df = make_float2((float)d.x, (float)d.y), d2 = fmul(df, df);
-                sd2[i] = d2;
-                sd2[F * n2 + i] = fmul(d2, df);
+                const float2 df = make_float2(dp.rh, dp.ih), d2 = fmul(df, df);
+                if (!adj) sd2[i] = d2;
+                sd3[i] = fmul(d2, df);
                 if (f < nv) {
                   acc_tr += d.x;
                   acc_g2 += widen(d2.x);
@@ -684,7 +701,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
               const double2 d2 = cmul(d, d);
               sd2[i] = d2;
               if (occ) {
-                sd2[F * n2 + i] = cmul(d2, d);
+                sd3[i] = cmul(d2, d);
                 if (f < nv) {
                   acc_tr += d.x;
                   acc_g2 += d2.x;
@@ -707,13 +724,49 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             const float4* df = reinterpret_cast<const float4*>(sd) + f * nt;
             float xrr[2] = {0.f, 0.f}, xri[2] = {0.f, 0.f}, xir[2] = {0.f, 0.f}, xii[2] = {0.f, 0.f};
             float2 yr = make_float2(0.f, 0.f), yi = yr;
+            auto plus = [](float& sh, float& sl_, float vh, float vl) {  // (sh, sl_) += (vh, vl)
+              float s, e;
+              two_sum(sh, vh, s, e);
+              sh = s;
+              sl_ = __fadd_rn(sl_, __fadd_rn(vl, e));
+            };
             auto add = [&](float4 tv, float4 d) {
               acc_prod(tv.x, tv.y, d.x, d.y, xrr[0], xrr[1]);
               acc_prod(tv.z, tv.w, d.x, d.y, xri[0], xri[1]);
               acc_prod(tv.x, tv.y, d.z, d.w, xir[0], xir[1]);
               acc_prod(tv.z, tv.w, d.z, d.w, xii[0], xii[1]);
             };
-            if (occ) {
+            if (adj) {
+              const float4* d2f = reinterpret_cast<const float4*>(sd2) + f * nt;
+              cf v1 = czero(), v2 = czero();  // sum t Re d^2 and sum t Im d^2
+#pragma unroll 2
+              for (int bb = 0; bb < nt; ++bb) {
+                const float4 tv = __ldg(t + (size_t)bb * NP), d2 = d2f[bb];
+                add(tv, df[bb]);
+                acc_prod(tv.x, tv.y, d2.x, d2.y, v1.rh, v1.rl);
+                acc_prod(tv.z, tv.w, d2.x, d2.y, v1.ih, v1.il);
+                acc_prod(tv.x, tv.y, d2.z, d2.w, v2.rh, v2.rl);
+                acc_prod(tv.z, tv.w, d2.z, d2.w, v2.ih, v2.il);
+              }
+              const float4 o = reinterpret_cast<const float4*>(hz)[NP + pr];
+              float4* Fm = reinterpret_cast<float4*>(sF) + f * MM;
+              cf g{o.x, o.y, o.z, o.w};
+              plus(g.rh, g.rl, v1.rh, v1.rl);
+              plus(g.rh, g.rl, -v2.ih, -v2.il);
+              plus(g.ih, g.il, v1.ih, v1.il);
+              plus(g.ih, g.il, v2.rh, v2.rl);
+              cnorm(g);
+              Fm[a * M + c] = st4(g);
+              if (a != c) {
+                cf h{o.x, o.y, -o.z, -o.w};
+                plus(h.rh, h.rl, v1.rh, v1.rl);
+                plus(h.rh, h.rl, v2.ih, v2.il);
+                plus(h.ih, h.il, -v1.ih, -v1.il);
+                plus(h.ih, h.il, v2.rh, v2.rl);
+                cnorm(h);
+                Fm[c * M + a] = st4(h);
+              }
+            } else if (occ) {
               const float2* d2f = sd2 + f * nt;
 #pragma unroll 2
               for (int bb = 0; bb < nt; ++bb) {
@@ -736,12 +789,6 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             const float2 w = sWp[f];
             const float4* Sg = p.Sd + si.offSig + (int64_t)nn * MM;
             float4* Sm = reinterpret_cast<float4*>(sS) + f * MM;
-            auto plus = [](float& sh, float& sl_, float vh, float vl) {  // (sh, sl_) += (vh, vl)
-              float s, e;
-              two_sum(sh, vh, s, e);
-              sh = s;
-              sl_ = __fadd_rn(sl_, __fadd_rn(vl, e));
-            };
             {
               const float4 sg = Sg[a * M + c];
               cf v{h.x, h.y, h.z, h.w};
@@ -846,7 +893,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             }
         }
         if (occ) {
-          float low_tr = 0.f, low_g2 = 0.f;  // LOW: this lane's sums over the warp's frequencies
+          float low_tr = 0.f, low_g2 = 0.f, low_xx = 0.f;  // LOW: this lane's sums over the warp's frequencies
           for (int i = lane; i < F * NP; i += 32) {
             const int f = i / NP, pr = i - f * NP;
             const int a = pair[pr].x, c = pair[pr].y;
@@ -858,12 +905,19 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             const int pa = pf[a] * M, pc = pf[c] * M;
             for (int j = 0; j < M; ++j) {
               const int fj = pf[j] * M;
-              rmac(x1, Af[pa + j], Fm[fj + c]);
-              if (LOW || a != c) rmac(x2, Af[pc + j], Fm[fj + a]);
+              if (low_adj) {
+                const float4* Fp = reinterpret_cast<const float4*>(sF) + f * MM;
+                const float4 u = Fp[fj + c], v = Fp[fj + a];
+                rmac(x1, Af[pa + j], rc_t{u.x, u.z});
+                rmac(x2, Af[pc + j], rc_t{v.x, v.z});
+              } else {
+                rmac(x1, Af[pa + j], Fm[fj + c]);
+                if (LOW || a != c) rmac(x2, Af[pc + j], Fm[fj + a]);
+              }
             }
             const rc_t g1 = Af[pa + qf[c]], g2 = Af[pc + qf[a]];
             rc_t zr = rzero(rc_t{}), zi = zr;
-            const rc_t* d3f = sd2 + F * n2 + f * nt;
+            const rc_t* d3f = sd3 + f * nt;
             if constexpr (LOW) {
               const float2* ts = Tst + pr;
 #pragma unroll 4
@@ -894,6 +948,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
               if constexpr (LOW) {
                 if (a == c) low_tr += x1.x;
                 low_g2 += s;
+                low_xx += xx;
               } else {
                 if (a == c) acc_tr += x1.x;
                 acc_g2 += s;
@@ -904,18 +959,19 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
           if constexpr (LOW) {
             acc_tr += (double)low_tr;
             acc_g2 += (double)low_g2;
+            if (have_gbar) acc_mu += cb * wk * (double)low_xx;
           }
           __syncwarp();
         }
         if constexpr (LOW) {
-          // S^{-1} in the orbitals' order for rho_k, and for G_loc one step of refinement,
-          // S^{-1} = X0 + X0 R with R = I - S X0 from S in FP32 pairs: 1e-15 of the FP64 inverse at
+          // S^{-1} in the orbitals' order for rho_k, and for G_loc and the adjoint one step of
+          // refinement, S^{-1} = X0 + X0 R with R = I - S X0 from S in FP32 pairs: 1e-15 of the FP64 inverse at
           // these frequencies, where the FP64 elimination takes 1,500 FP64 instructions a matrix
           // at m = 20.
           const float4* Sp = reinterpret_cast<const float4*>(A);
           float2* X0 = sG + mf * MM;
-          float2* R = reinterpret_cast<float2*>(smraw + L.oR + wp * L.sG) + mf * MM;
-          const bool refine = (p.mode & kGloc) != 0;
+          float2* R = reinterpret_cast<float2*>(smraw + L.oR + wp * L.sR) + mf * MM;
+          const bool refine = (p.mode & (kGloc | kAdj)) != 0;
           if (refine) {
             for (int i = sl; i < MM; i += LW) {
               const int a = i / M, c = i - a * M, qc = sq[c];
@@ -936,40 +992,90 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
               for (int x = 0; x < M; ++x) fmac(d, X0[pa + sq[x]], R[x * M + c]);
               two_sum(g.x, d.x, h.x, l.x);
               two_sum(g.y, d.y, h.y, l.y);
-              if (mine)
+              if (adj) reinterpret_cast<float4*>(A)[i] = make_float4(h.x, l.x, h.y, l.y);
+              else if (mine)
                 gq_put(&out[i], q, make_double2(wk * (widen(h.x) + widen(l.x)), wk * (widen(h.y) + widen(l.y))));
             }
-            Gn[i] = h;
+            if (!adj) Gn[i] = h;
           }
           __syncwarp();
           if (rho)
             for (int i = sl; i < MM; i += LW) X0[i] = Gn[i];
           __syncwarp();
         }
-        if constexpr (!LOW) {
-          if (adj) {
-            // Sigma_bar = A^+ Ghat A^+ with Ghat = Gbar + c F^+ (c = n_bar 2 / beta), A = S^{-1}:
-            // Mt = Ghat A^+, then A^+ Mt; Re<Gbar, A F A> = Re Tr(F^+ Sigma_bar) - c Re Tr (A F)^2
-            double2* Mt = sM + mf * MM;
-            double2* Fm = reinterpret_cast<double2*>(sF) + mf * MM;
-            const double2* Gb = have_gbar ? p.gbar + si.offSig + (int64_t)min(n + mf, n1 - 1) * MM : nullptr;
+        if (adj) {
+          // Sigma_bar = A^+ Ghat A^+ with Ghat = Gbar + c F^+ (c = n_bar 2 / beta), A = S^{-1}: Ghat,
+          // then Ghat A^+ over it (whole rows, so that a row is read before it is written), then
+          // A^+ (Ghat A^+); Re<Gbar, A F A> = Re Tr(F^+ Sigma_bar) - c Re Tr (A F)^2.  With LOW the
+          // matrices and products are FP32 pairs (1e-13 of the FP64 kernel, which is bound by the FP64
+          // pipe: 256 k-points x 1024 frequencies of 40 bands, 14 orbitals 44 ms, in pairs 15 ms).
+          const int rows = LW / M, ra = sl / M, rb = sl - ra * M;  // (rows >= 1: m <= LW)
+          const int64_t gb0 = si.offSig + (int64_t)min(n + mf, n1 - 1) * MM;
+          if constexpr (LOW) {
+            float4* Gh = reinterpret_cast<float4*>(sM) + mf * MM;
+            const float4* Fm = reinterpret_cast<const float4*>(sF) + mf * MM;
+            const float4* Ap = reinterpret_cast<const float4*>(A);
+            float ch, cl;
+            split(cb, ch, cl);
             for (int i = sl; i < MM; i += LW) {
               const int a = i / M, c = i - a * M;
-              double2 acc = make_double2(0.0, 0.0);
-              const int pc = sp[c] * M;
-              for (int x = 0; x < M; ++x) {
-                // Ghat[a][x'] conj(A[c][x']) with x' = p_x, A[c][p_x] at column q_{p_x} = x
-                const int xx = sp[x];
-                const double2 fv = Fm[xx * M + a];
-                double2 g = make_double2(cb * fv.x, -cb * fv.y);
+              const float4 fv = Fm[c * M + a];
+              cf g = have_gbar ? ld4(__ldg(p.Gbd + gb0 + i)) : czero();
+              acc_prod(ch, cl, fv.x, fv.y, g.rh, g.rl);
+              acc_prod(-ch, -cl, fv.z, fv.w, g.ih, g.il);
+              cnorm(g);
+              Gh[i] = st4(g);
+            }
+            __syncwarp();
+            for (int a0 = 0; a0 < M; a0 += rows) {
+              const int a = a0 + ra;
+              const bool in = ra < rows && a < M;
+              cf acc = czero();
+              if (in)
+                for (int x = 0; x < M; ++x) cacc_cb(acc, ld4(Gh[a * M + x]), ld4(Ap[rb * M + x]));
+              cnorm(acc);
+              __syncwarp();
+              if (in) Gh[a * M + rb] = st4(acc);
+            }
+            __syncwarp();
+            for (int i = sl; i < MM; i += LW) {
+              const int a = i / M, c = i - a * M;
+              cf acc = czero();
+              for (int x = 0; x < M; ++x) cacc_ca(acc, ld4(Ap[x * M + a]), ld4(Gh[x * M + c]));
+              if (mine) {
+                const double2 v = make_double2(widen(acc.rh) + widen(acc.rl), widen(acc.ih) + widen(acc.il));
+                gq_put(&out[i], q, make_double2(wk * v.x, wk * v.y));
                 if (have_gbar) {
-                  const double2 gb = Gb[a * M + xx];
-                  g.x += gb.x;
-                  g.y += gb.y;
+                  const float4 fv = Fm[i];
+                  acc_mu -= wk * fma(widen(fv.x) + widen(fv.y), v.x, (widen(fv.z) + widen(fv.w)) * v.y);
                 }
-                cmac_cb(acc, g, A[pc + x]);
               }
-              Mt[i] = acc;
+            }
+          } else {
+            double2* Gh = sM + mf * MM;
+            const double2* Fm = reinterpret_cast<const double2*>(sF) + mf * MM;
+            for (int i = sl; i < MM; i += LW) {
+              const int a = i / M, c = i - a * M;
+              const double2 fv = Fm[c * M + a];
+              double2 g = make_double2(cb * fv.x, -cb * fv.y);
+              if (have_gbar) {
+                const double2 gb = __ldg(p.gbar + gb0 + i);
+                g.x += gb.x;
+                g.y += gb.y;
+              }
+              Gh[i] = g;
+            }
+            __syncwarp();
+            for (int a0 = 0; a0 < M; a0 += rows) {
+              const int a = a0 + ra;
+              const bool in = ra < rows && a < M;
+              double2 acc = make_double2(0.0, 0.0);
+              if (in) {
+                const int pc = sp[rb] * M;  // A[c][p_x] at column x of row p_c
+                for (int x = 0; x < M; ++x) cmac_cb(acc, Gh[a * M + sp[x]], A[pc + x]);
+              }
+              __syncwarp();
+              if (in) Gh[a * M + rb] = acc;
             }
             __syncwarp();
             for (int i = sl; i < MM; i += LW) {
@@ -977,7 +1083,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
               double2 acc = make_double2(0.0, 0.0);
               const int qa = sq[a];
               // conj(A[x][a]) Mt[x][c], A[x][a] at row p_x, column q_a
-              for (int x = 0; x < M; ++x) cmac_ca(acc, A[sp[x] * M + qa], Mt[x * M + c]);
+              for (int x = 0; x < M; ++x) cmac_ca(acc, A[sp[x] * M + qa], Gh[x * M + c]);
               if (mine) {
                 gq_put(&out[i], q, make_double2(wk * acc.x, wk * acc.y));
                 if (have_gbar) {
@@ -1304,15 +1410,21 @@ int reduce_grid(int nbmax, int mmax, int n_k, int smem_optin, int sm_count) {
   return std::max(1, std::min(n_k, sm_count * std::min(per_sm, 8)));
 }
 
-template <int LW, bool LOW>
-cudaError_t launch_lw(const PointParams& p, const BlockForm& b, const BlockLaunch& l, size_t smem, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(k_point_block<LW, LOW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <int LW, bool LOW, bool ADJ>
+cudaError_t launch_lw_adj(const PointParams& p, const BlockForm& b, const BlockLaunch& l, size_t smem, cudaStream_t s) {
+  cudaError_t e =
+      cudaFuncSetAttribute(k_point_block<LW, LOW, ADJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_point_block<LW, LOW>, cudaFuncAttributePreferredSharedMemoryCarveout,
+  e = cudaFuncSetAttribute(k_point_block<LW, LOW, ADJ>, cudaFuncAttributePreferredSharedMemoryCarveout,
                            (int)cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
-  k_point_block<LW, LOW><<<l.n_units * l.n_chunks, 32 * kBlkWarps, smem, s>>>(p, b, l);
+  k_point_block<LW, LOW, ADJ><<<l.n_units * l.n_chunks, 32 * kBlkWarps, smem, s>>>(p, b, l);
   return cudaGetLastError();
+}
+
+template <int LW, bool LOW>
+cudaError_t launch_lw(const PointParams& p, const BlockForm& b, const BlockLaunch& l, size_t smem, cudaStream_t s) {
+  return p.mode & kAdj ? launch_lw_adj<LW, LOW, true>(p, b, l, smem, s) : launch_lw_adj<LW, LOW, false>(p, b, l, smem, s);
 }
 
 }  // namespace

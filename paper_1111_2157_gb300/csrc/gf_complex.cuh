@@ -57,16 +57,6 @@ __device__ __forceinline__ double rcp_newton(double x) {
   return fma(r, fma(-x, r, 1.0), r);
 }
 
-// (double)x by integer arithmetic on the bits: a conversion instruction runs on the FP64 pipe, where
-// it takes a warp as long as an FMA.  Exact; FP32 denormals become 0.
-__device__ __forceinline__ double widen(float x) {
-  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
-  unsigned hi = (u & 0x80000000u) | ((m >> 3) + 0x38000000u);
-  if (m >= 0x7f800000u) hi |= 0x7ff00000u;  // infinity, NaN
-  const bool zero = m < 0x00800000u;
-  return __hiloint2double(zero ? (int)(u & 0x80000000u) : (int)hi, zero ? 0 : (int)(u << 29));
-}
-
 // Pivot key of a complex FP64 number: max(|Re|, |Im|) compared through the IEEE
 // bit pattern, which orders non-negative doubles like their values; no FP64
 // instruction.
@@ -78,6 +68,16 @@ __device__ __forceinline__ unsigned long long pivot_key(double2 a) {
 }
 
 // ------------------------------------------------------------------ FP32 pairs
+// (double)x by integer arithmetic on the bits: a conversion instruction runs on the FP64 pipe, where
+// it takes a warp as long as an FMA.  Exact; FP32 denormals become 0.
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+  unsigned hi = (u & 0x80000000u) | ((m >> 3) + 0x38000000u);
+  if (m >= 0x7f800000u) hi |= 0x7ff00000u;  // infinity, NaN
+  const bool zero = m < 0x00800000u;
+  return __hiloint2double(zero ? (int)(u & 0x80000000u) : (int)hi, zero ? 0 : (int)(u << 29));
+}
+
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);
   const float bb = __fsub_rn(s, a);
@@ -118,7 +118,7 @@ __device__ __forceinline__ void renorm_fast(float& h, float& l) {
 }
 __device__ __forceinline__ void split(double x, float& h, float& l) {
   h = __double2float_rn(x);
-  l = __double2float_rn(x - (double)h);
+  l = __double2float_rn(x - widen(h));
 }
 
 struct cf {

@@ -160,13 +160,13 @@ def test_levels_that_the_parallel_eigenvectors_cannot_separate(kind):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("nk,nb,m,n_iw", [(3, 40, 14, 200), (2, 96, 20, 70), (2, 24, 7, 300)])
+@pytest.mark.parametrize("nk,nb,m,n_iw", [(3, 40, 14, 200), (2, 96, 20, 70), (2, 24, 7, 300), (2, 48, 32, 40)])
 def test_mixed_block_kernels_against_fp64(nk, nb, m, n_iw):
     """The mixed contract (N 1e-7, G_loc 1e-8, rho 1e-5, dN/dmu 1e-5, n_corr 1e-6) on both sides of the FP64 limit."""
     s = _inputs(nk, nb, m, n_iw, 100.0, nb)
     a, log = _run(s, None, precision="mixed")
     b, _ = _run(s, "direct")
-    assert "in FP32 (traces, rho)" in log
+    assert "in FP32 and FP32 pairs" in log
     tol = {"N": 1e-7, "occ": 1e-7, "gloc": 1e-8, "loc": 1e-8, "rho": 1e-5, "dm": 1e-5, "dN_dmu": 1e-5, "docc": 1e-5,
            "n_corr": 1e-6, "dm_nc": 1e-6}
     for key in b:
