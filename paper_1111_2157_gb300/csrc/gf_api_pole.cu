@@ -62,11 +62,9 @@ gf_status pole_run(gf_ctx* c, int mode, bool gloc_kernel = true) {
   GF_CU(gf::launch_pole_eig(p, grid, p.in_smem ? smem : zb, c->stream));
   c->last_launches += 1;
   if ((mode & gf::kGloc) && gloc_kernel) {
-    const int ns = gf::pole_gloc_splits(c->n_sys, c->n_iw, c->sm_count, c->mmax);
-    GF_CU(ensure(c->pole_part, sizeof(double2) * (size_t)ns * c->totSig));
-    GF_CU(gf::launch_pole_gloc(p, c->n_sys, c->mmax, ns, c->pole_part.as<double2>(), c->totSig,
-                               c->stream));
-    c->last_launches += 2;
+    GF_CU(ensure(c->pole_part, sizeof(double2) * gf::pole_gloc_ws_elems(c->n_sys, c->n_iw, c->mmax, c->sm_count)));
+    GF_CU(gf::launch_pole_gloc(p, c->n_sys, c->mmax, c->nps_max, c->sm_count, c->pole_part.as<double2>(), c->stream));
+    c->last_launches += 4;
   }
   GF_CU(cudaEventRecord(c->ev[c->ev_used + 1], c->stream));
   c->ev_used += 2;

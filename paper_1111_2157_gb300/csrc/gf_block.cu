@@ -21,6 +21,7 @@
 #include "gf_block.cuh"
 #include "gf_complex.cuh"
 #include "gf_gj64.cuh"
+#include "gf_series.cuh"
 
 namespace gf {
 
@@ -28,6 +29,9 @@ namespace {
 
 using namespace cx;
 using gj64::crcp_scaled;
+using series::cpow_int;
+using series::series_z;
+using series::SeriesZ;
 
 constexpr int kSetupThreads = 256;
 
@@ -390,49 +394,6 @@ __device__ __forceinline__ float2 rzero(float2) { return make_float2(0.f, 0.f); 
 __device__ __forceinline__ double rfma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
-// Coefficients of the Chebyshev series at z (x = (z - c) / r, s = sqrt(x^2 - 1), xi = x - s):
-//   1/(z - e)   = sum_j eps_j xi^j / (r s) T_j,                                eps_0 = 1, eps_j = 2
-//   1/(z - e)^2 = sum_j eps_j xi^j [j/s^2 + x/s^3] / r^2 T_j                    (-d/dz)
-//   1/(z - e)^3 = sum_j eps_j xi^j [(j^2 - 1)/s^3 + 3 j x/s^4 + 3 x^2/s^5] / (2 r^3) T_j
-// The j-independent factors of one frequency:
-struct SeriesZ {
-  double2 xi, c1, c2a, c2b, c3a, c3b, c3c;  // c1; c2a j + c2b; c3a (j^2 - 1) + c3b j + c3c
-};
-__device__ __forceinline__ SeriesZ series_z(double dx, double w, double r, bool powers) {
-  SeriesZ q;
-  const double ir = 1.0 / r;
-  const double2 x = make_double2(dx * ir, w * ir);
-  // s = sqrt(x^2 - 1) with Im s > 0: from |u| and the larger component first
-  const double2 u = make_double2(fma(x.x, x.x, -fma(x.y, x.y, 1.0)), 2.0 * x.x * x.y);
-  const double au = sqrt(fma(u.x, u.x, u.y * u.y));
-  const double p = sqrt(0.5 * (au + fabs(u.x)));
-  const double h = 0.5 * u.y / p;
-  double2 s = u.x >= 0.0 ? make_double2(p, h) : make_double2(h, p);
-  if (s.y < 0.0 || (s.y == 0.0 && x.x < 0.0)) s = make_double2(-s.x, -s.y);
-  q.xi = crcp_scaled(make_double2(x.x + s.x, x.y + s.y), pivot_key(make_double2(x.x + s.x, x.y + s.y)));
-  const double2 is = crcp_scaled(s, pivot_key(s));
-  q.c1 = make_double2(is.x * ir, is.y * ir);
-  if (powers) {
-    q.c2a = cmul(q.c1, make_double2(is.x * ir, is.y * ir));                  // 1 / (s^2 r^2)
-    const double2 t = cmul(x, is);                                           // x / s
-    q.c2b = cmul(q.c2a, t);                                                  // x / (s^3 r^2)
-    const double g = 0.5 * ir;
-    const double2 is2 = make_double2(is.x * g, is.y * g);
-    q.c3a = cmul(q.c2a, is2);                                                // 1 / (2 s^3 r^3)
-    q.c3b = cmul(q.c2b, make_double2(3.0 * is2.x, 3.0 * is2.y));             // 3 x / (2 s^4 r^3)
-    q.c3c = cmul(q.c3b, t);                                                  // 3 x^2 / (2 s^5 r^3)
-  }
-  return q;
-}
-__device__ __forceinline__ double2 cpow_int(double2 b, int j) {
-  double2 v = make_double2(1.0, 0.0);
-#pragma unroll
-  for (int t = 0; t < 6; ++t) {  // j < 64
-    if ((j >> t) & 1) v = cmul(v, b);
-    b = cmul(b, b);
-  }
-  return v;
-}
 // Shared memory of the point kernel in bytes; every array holds the CTA's W F frequencies, warp
 // after warp.  First what is dead once the warps have S^{-1}: F, d^2 / d^3, the pivot row and
 // column, Gbar A^+ (adjoint), and with LOW also S and the refinement's residual (rho_k then reads
@@ -632,7 +593,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
                   zf[4] = to_rest(z.c3c, float2{});
                 }
               }
-              double2 pw = cpow_int(z.xi, j);
+              double2 pw = cpow_int<6>(z.xi, j);
               if (j) pw = make_double2(2.0 * pw.x, 2.0 * pw.y);
               const double2 d = cmul(pw, z.c1);
               put_d(i, d);

@@ -28,6 +28,7 @@
 #include "gf_block.cuh"
 #include "gf_complex.cuh"
 #include "gf_internal.cuh"
+#include "gf_series.cuh"
 
 namespace gf {
 
@@ -880,116 +881,248 @@ __global__ void __launch_bounds__(kEigThreads) k_pole_eig(const PoleParams p) {
   }
 }
 
-// G_loc(i w_n) = sum_k w_k sum_l phi_l phi_l^+ / (i w_n + mu - E_l) for one
-// system and F consecutive frequencies per CTA.  With t = phi_a conj(phi_b)
-// and g = w_k / (i w + mu - E) = gr + i gi: G_ab = Xr + i Xi and
-// G_ba = conj(Xr) + i conj(Xi) with Xr = sum t gr, Xi = sum t gi, so each
-// thread sums QP pairs a <= b.  phi and E are staged in shared memory kCh
-// eigenpairs at a time; the sums run over k, then l, in increasing order.
+// G_loc(i w_n) = sum_k w_k sum_l t_l / (i w_n + mu - E_l), t = phi_a conj(phi_b), of one system.
+// Frequencies below nd are summed as they stand: with g = w_k / (i w + mu - E) = gr + i gi,
+// G_ab = Xr + i Xi and G_ba = conj(Xr) + i conj(Xi) with Xr = sum t gr, Xi = sum t gi.  From nd
+// on 1 / (z - E) is a Chebyshev series in E over the interval of the levels, whose moments
+// sum_k w_k sum_l t_l T_j(x_l), j < J, serve all of them: a moment costs half a frequency's sum.
+// A tile is F frequencies or 2 F moments of all pairs a <= b, QP pairs per thread; a CTA sums one
+// tile over a share of the system's levels (the tiles times their splits fill the chip), phi and
+// the factors staged in shared memory kCh levels at a time, in increasing order.
+// J is the multiple of 2 F with the fewest tiles: the frequencies whose series of J terms leaves
+// less than e^-37 are those with J asinh(w / r) >= 37, r half the width of the interval (a
+// frequency's ellipse of convergence is smallest above the middle of the interval).
+// Bound: the FP64 pipe.  125 k-points of 68 levels, 14 orbitals, 512 frequencies: 1.1 ms, 6.2 ms by
+// sums alone.
 constexpr int kCh = 32;
+constexpr int kGlocTerms = 256;  // moments kept at most
 
+struct GlocPlan {
+  double c, r;         // middle and half width of the levels' interval
+  int nd, J, tiles;    // frequencies summed directly, moments, tiles of both
+};
+
+__global__ void __launch_bounds__(kEigThreads) k_pole_span(const PoleParams p, int F, GlocPlan* plan) {
+  __shared__ double s_lo[kEigThreads], s_hi[kEigThreads];
+  const SInfo si = p.sinfo[blockIdx.x];
+  const int tid = threadIdx.x;
+  const int64_t e0 = p.eoff[si.k0], e1 = p.eoff[si.k1 - 1] + p.kinfo[si.k1 - 1].nb + p.pinfo[blockIdx.x].np;
+  double lo = INFINITY, hi = -INFINITY;
+  for (int64_t e = e0 + tid; e < e1; e += kEigThreads) {
+    const double v = p.eout[e];
+    lo = fmin(lo, v);
+    hi = fmax(hi, v);
+  }
+  s_lo[tid] = lo;
+  s_hi[tid] = hi;
+  __syncthreads();
+  for (int w = kEigThreads / 2; w; w >>= 1) {
+    if (tid < w) {
+      s_lo[tid] = fmin(s_lo[tid], s_lo[tid + w]);
+      s_hi[tid] = fmax(s_hi[tid], s_hi[tid + w]);
+    }
+    __syncthreads();
+  }
+  if (tid >= 32) return;
+  lo = s_lo[0];
+  hi = s_hi[0];
+  const double r = fmax(0.5 * (hi - lo) * (1.0 + 1e-12), 1e-6);
+  // one candidate J per lane, J = 0 (every frequency as it stands) in lane 0
+  int best = (p.n_iw + F - 1) / F, nd = p.n_iw, J = 0;
+  for (int j = 2 * F * (tid + 1); j <= kGlocTerms; j += 2 * F * 32) {
+    const double n = ceil(0.5 * (r * sinh(37.0 / j) * si.beta / M_PI - 1.0));
+    if (!(n < (double)p.n_iw)) continue;  // (also an interval that is not finite)
+    const int d = (int)fmax(n, 0.0), t = (d + F - 1) / F + j / (2 * F);
+    if (t < best) {
+      best = t;
+      nd = d;
+      J = j;
+    }
+  }
+  for (int off = 16; off; off >>= 1) {
+    const int ot = __shfl_xor_sync(0xffffffffu, best, off), on = __shfl_xor_sync(0xffffffffu, nd, off);
+    const int oj = __shfl_xor_sync(0xffffffffu, J, off);
+    if (ot < best || (ot == best && oj < J)) {
+      best = ot;
+      nd = on;
+      J = oj;
+    }
+  }
+  if (tid == 0) plan[blockIdx.x] = GlocPlan{0.5 * (hi + lo), r, nd, J, best};
+}
+
+// Sums of one (tile, split): part[blockIdx.x 2 F + slot][pair], slot 2 f of Xr and
+// 2 f + 1 of Xi, or the moment of the tile.
 template <int QP, int F>
 __global__ void __launch_bounds__(kEigThreads)
-    k_pole_gloc(const PoleParams p, int blocks_per_sys, int n_split, double2* part, int64_t tot) {
+    k_pole_gloc(const PoleParams p, const GlocPlan* plan, int per_sys, int nps_max, int npairs_max, double2* part) {
   __shared__ double2 s_phi[32 * kCh];  // m <= 32
-  __shared__ double2 s_g[F * kCh];
-  const int s = blockIdx.x / blocks_per_sys;
-  const int f0 = (blockIdx.x - s * blocks_per_sys) * F;
-  const int split = blockIdx.y;
+  __shared__ double2 s_g[F * kCh];     // w_k / (i w + mu - E), or w_k T_j: [2 F][kCh]
+  __shared__ double s_th[kCh];
+  const int s = blockIdx.x / per_sys, item = blockIdx.x % per_sys;
+  const GlocPlan pl = plan[s];
+  const int splits = max(1, per_sys / pl.tiles);
+  if (item >= pl.tiles * splits) return;
+  const int tile = item % pl.tiles, split = item / pl.tiles;
+  const int td = (pl.nd + F - 1) / F;
+  const bool mom = tile >= td;
+  const int f0 = tile * F, j0 = (tile - td) * 2 * F;
   const SInfo si = p.sinfo[s];
-  // k-points [ka, kb) of this split of the system
-  const int nks = si.k1 - si.k0;
-  const int ka = si.k0 + (int)((int64_t)nks * split / n_split);
-  const int kb = si.k0 + (int)((int64_t)nks * (split + 1) / n_split);
-  const int m = si.m;
+  const int m = si.m, np = p.pinfo[s].np;
   const int npairs = m * (m + 1) / 2;
-  const double mu = p.mu[s];
-  const int tid = threadIdx.x;
+  const double mu = p.mu[s], ir = 1.0 / pl.r;
+  const int tid = threadIdx.x, nt = blockDim.x;
   int pa[QP], pb[QP];
 #pragma unroll
   for (int q = 0; q < QP; ++q) {
-    int rem = tid + q * kEigThreads, a = 0;
+    int rem = tid + q * nt, a = 0;
     if (rem >= npairs) rem = 0;
     while (rem >= m - a) { rem -= m - a; ++a; }
     pa[q] = a;
     pb[q] = a + rem;
   }
-  double2 xr[QP][F], xi[QP][F];
+  double2 x[QP][2 * F];
 #pragma unroll
   for (int q = 0; q < QP; ++q)
 #pragma unroll
-    for (int f = 0; f < F; ++f) {
-      xr[q][f] = make_double2(0.0, 0.0);
-      xi[q][f] = make_double2(0.0, 0.0);
-    }
-  for (int k = ka; k < kb; ++k) {
-    const int n = p.kinfo[k].nb + p.pinfo[s].np;
+    for (int f = 0; f < 2 * F; ++f) x[q][f] = make_double2(0.0, 0.0);
+  // chunks of levels, nch per k-point, [ca, cb) of this split
+  const int nch = (nps_max + kCh - 1) / kCh;
+  const int64_t tot = (int64_t)(si.k1 - si.k0) * nch;
+  const int64_t ca = tot * split / splits, cb = tot * (split + 1) / splits;
+  for (int64_t ch = ca; ch < cb; ++ch) {
+    const int k = si.k0 + (int)(ch / nch), i = (int)(ch % nch);
+    const int n = p.kinfo[k].nb + np;
+    const int l0 = n * i / nch, cl = n * (i + 1) / nch - l0;
     const double wk = p.kinfo[k].w;
-    const double* E = p.eout + p.eoff[k];
-    const double2* phi = p.phiout + p.phioff[k];
-    for (int l0 = 0; l0 < n; l0 += kCh) {
-      const int cl = min(kCh, n - l0);
-      __syncthreads();
-      for (int e = tid; e < m * cl; e += kEigThreads) {
-        const int a = e / cl, l = e - (e / cl) * cl;
-        s_phi[a * kCh + l] = phi[a * n + l0 + l];
+    const double* E = p.eout + p.eoff[k] + l0;
+    const double2* phi = p.phiout + p.phioff[k] + l0;
+    __syncthreads();
+    for (int e = tid; e < m * cl; e += nt) {
+      const int a = e / cl, l = e - (e / cl) * cl;
+      s_phi[a * kCh + l] = phi[a * n + l];
+    }
+    if (mom) {
+      if (tid < cl) {
+        const double t = (E[tid] - pl.c) * ir;
+        s_th[tid] = acos(t > 1.0 ? 1.0 : (t < -1.0 ? -1.0 : t));
       }
-      for (int e = tid; e < F * cl; e += kEigThreads) {
+      __syncthreads();
+      double* T = reinterpret_cast<double*>(s_g);
+      for (int e = tid; e < 2 * F * cl; e += nt) {
+        const int j = e / cl, l = e - (e / cl) * cl;
+        T[j * kCh + l] = wk * cos((j0 + j) * s_th[l]);
+      }
+    } else {
+      for (int e = tid; e < F * cl; e += nt) {
         const int f = e / cl, l = e - (e / cl) * cl;
-        const int nn = f0 + f;
-        const double wn = (2.0 * nn + 1.0) * 3.14159265358979323846 / si.beta;
+        const double wn = (2.0 * (f0 + f) + 1.0) * 3.14159265358979323846 / si.beta;
         // w_k / (mu - E + i w) = w_k (x - i w) / (x^2 + w^2), x = mu - E
-        const double x = mu - E[l0 + l];
-        const double d = wk / fma(x, x, wn * wn);
-        s_g[f * kCh + l] = make_double2(x * d, -wn * d);
+        const double xe = mu - E[l];
+        const double d = wk / fma(xe, xe, wn * wn);
+        s_g[f * kCh + l] = make_double2(xe * d, -wn * d);
       }
-      __syncthreads();
+    }
+    __syncthreads();
 #pragma unroll
-      for (int q = 0; q < QP; ++q) {
-        if (tid + q * kEigThreads >= npairs) continue;
-        const int a = pa[q], b = pb[q];
-        for (int l = 0; l < cl; ++l) {
-          double2 t = make_double2(0.0, 0.0);
-          cmac_cb(t, s_phi[a * kCh + l], s_phi[b * kCh + l]);
+    for (int q = 0; q < QP; ++q) {
+      if (tid + q * nt >= npairs) continue;
+      const int a = pa[q], b = pb[q];
+      const double* T = reinterpret_cast<const double*>(s_g);
+      for (int l = 0; l < cl; ++l) {
+        double2 t = make_double2(0.0, 0.0);
+        cmac_cb(t, s_phi[a * kCh + l], s_phi[b * kCh + l]);
+        if (mom) {
+#pragma unroll
+          for (int j = 0; j < 2 * F; ++j) {
+            const double g = T[j * kCh + l];
+            x[q][j].x = fma(t.x, g, x[q][j].x);
+            x[q][j].y = fma(t.y, g, x[q][j].y);
+          }
+        } else {
 #pragma unroll
           for (int f = 0; f < F; ++f) {
             const double2 g = s_g[f * kCh + l];
-            xr[q][f].x = fma(t.x, g.x, xr[q][f].x);
-            xr[q][f].y = fma(t.y, g.x, xr[q][f].y);
-            xi[q][f].x = fma(t.x, g.y, xi[q][f].x);
-            xi[q][f].y = fma(t.y, g.y, xi[q][f].y);
+            x[q][2 * f].x = fma(t.x, g.x, x[q][2 * f].x);
+            x[q][2 * f].y = fma(t.y, g.x, x[q][2 * f].y);
+            x[q][2 * f + 1].x = fma(t.x, g.y, x[q][2 * f + 1].x);
+            x[q][2 * f + 1].y = fma(t.y, g.y, x[q][2 * f + 1].y);
           }
         }
       }
     }
   }
+  double2* out = part + (int64_t)blockIdx.x * 2 * F * npairs_max;
 #pragma unroll
   for (int q = 0; q < QP; ++q) {
-    if (tid + q * kEigThreads >= npairs) continue;
-    const int a = pa[q], b = pb[q];
+    const int pr = tid + q * nt;
+    if (pr >= npairs) continue;
 #pragma unroll
-    for (int f = 0; f < F; ++f) {
-      const int nn = f0 + f;
-      if (nn >= p.n_iw) continue;
-      double2* out = part + (int64_t)split * tot + si.offSig + (int64_t)nn * m * m;
-      out[a * m + b] = make_double2(xr[q][f].x - xi[q][f].y, xr[q][f].y + xi[q][f].x);
-      out[b * m + a] = make_double2(xr[q][f].x + xi[q][f].y, xi[q][f].x - xr[q][f].y);
-    }
+    for (int f = 0; f < 2 * F; ++f) out[f * npairs_max + pr] = x[q][f];
   }
 }
 
-// gloc[e] = sum over the splits, in order, of part[split][e].
-__global__ void k_split_reduce(const double2* __restrict__ part, int n_split, int64_t tot,
-                               double2* __restrict__ out) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    double2 acc = part[e];
-    for (int sp = 1; sp < n_split; ++sp) {
-      const double2 v = part[(int64_t)sp * tot + e];
-      acc.x += v.x;
-      acc.y += v.y;
+// part of the first split = sum over the splits, in order.
+__global__ void k_gloc_splits(const GlocPlan* __restrict__ plan, int blocks_per_sys, int per_sys, int64_t per_tile,
+                              double2* part) {
+  const int s = blockIdx.x / blocks_per_sys, blk = blockIdx.x % blocks_per_sys;
+  const GlocPlan pl = plan[s];
+  const int splits = max(1, per_sys / pl.tiles);
+  double2* v = part + (int64_t)s * per_sys * per_tile;
+  const int64_t tot = pl.tiles * per_tile;
+  for (int64_t e = blk * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)blocks_per_sys * blockDim.x) {
+    double2 acc = v[e];
+    for (int sp = 1; sp < splits; ++sp) {
+      const double2 u = v[sp * tot + e];
+      acc.x += u.x;
+      acc.y += u.y;
     }
-    out[e] = acc;
+    v[e] = acc;
+  }
+}
+
+// G_loc of one frequency and system from the sums: Xr and Xi as they stand, or
+// Xr + i Xi = sum_j c_j M_j with complex c_j and M_ba = conj(M_ab).
+__global__ void __launch_bounds__(128) k_gloc_write(const PoleParams p, const GlocPlan* __restrict__ plan, int per_sys,
+                                                    int F, int npairs_max, const double2* __restrict__ part) {
+  __shared__ double2 s_c[kGlocTerms];
+  const int s = blockIdx.x / p.n_iw, n = blockIdx.x % p.n_iw, tid = threadIdx.x;
+  const GlocPlan pl = plan[s];
+  const SInfo si = p.sinfo[s];
+  const int m = si.m, td = (pl.nd + F - 1) / F;
+  const double2* v = part + (int64_t)s * per_sys * 2 * F * npairs_max;
+  if (n >= pl.nd) {
+    const double wn = (2.0 * n + 1.0) * 3.14159265358979323846 / si.beta;
+    const series::SeriesZ z = series::series_z(p.mu[s] - pl.c, wn, pl.r, false);
+    for (int j = tid; j < pl.J; j += 128) {
+      const double2 c = cmul(series::cpow_int<8>(z.xi, j), z.c1);
+      s_c[j] = j ? make_double2(2.0 * c.x, 2.0 * c.y) : c;
+    }
+  }
+  __syncthreads();
+  double2* out = p.gloc + si.offSig + (int64_t)n * m * m;
+  for (int pr = tid; pr < m * (m + 1) / 2; pr += 128) {
+    int b = pr, a = 0;
+    while (b >= m - a) { b -= m - a; ++a; }
+    b += a;
+    double2 xr = make_double2(0.0, 0.0), xi = xr;  // sums of t with the real and imaginary parts
+    if (n < pl.nd) {
+      const double2* u = v + ((int64_t)(n / F) * 2 * F + 2 * (n % F)) * npairs_max + pr;
+      xr = u[0];
+      xi = u[npairs_max];
+    } else {
+      const double2* u = v + (int64_t)td * 2 * F * npairs_max + pr;
+#pragma unroll 4
+      for (int j = 0; j < pl.J; ++j) {
+        const double2 t = u[(int64_t)j * npairs_max], c = s_c[j];
+        xr.x = fma(t.x, c.x, xr.x);
+        xr.y = fma(t.y, c.x, xr.y);
+        xi.x = fma(t.x, c.y, xi.x);
+        xi.y = fma(t.y, c.y, xi.y);
+      }
+    }
+    out[a * m + b] = make_double2(xr.x - xi.y, xr.y + xi.x);
+    out[b * m + a] = make_double2(xr.x + xi.y, xi.x - xr.y);
   }
 }
 
@@ -1283,27 +1416,40 @@ cudaError_t launch_pole_eig(const PoleParams& p, int grid, size_t smem, cudaStre
   return cudaGetLastError();
 }
 
-// frequencies per CTA of k_pole_gloc: 8 with one pair per thread, else 4
-int pole_gloc_f(int mmax) { return mmax * (mmax + 1) / 2 <= kEigThreads ? 8 : 4; }
+namespace {
+// pairs per thread and frequencies per tile of k_pole_gloc (32 sums per thread, 48 with three pairs)
+int gloc_qp(int mmax) { return (mmax * (mmax + 1) / 2 + kEigThreads - 1) / kEigThreads; }  // 1..3 for m <= 32
+int gloc_f(int mmax) { return gloc_qp(mmax) == 1 ? 8 : 4; }
+// (tile, split) pairs per system: four CTAs per SM, but at least every frequency's tile
+int gloc_per_sys(int n_sys, int n_iw, int mmax, int sm_count) {
+  const int F = gloc_f(mmax);
+  return std::max((n_iw + F - 1) / F, (4 * sm_count + n_sys - 1) / n_sys);
+}
+size_t gloc_plan_elems(int n_sys) { return (sizeof(GlocPlan) * n_sys + sizeof(double2) - 1) / sizeof(double2); }
+}  // namespace
 
-int pole_gloc_splits(int n_sys, int n_iw, int sm_count, int mmax) {
-  const int F = pole_gloc_f(mmax);
-  const int blocks = n_sys * ((n_iw + F - 1) / F);
-  return std::max(1, std::min(64, (2 * sm_count + blocks - 1) / blocks));
+size_t pole_gloc_ws_elems(int n_sys, int n_iw, int mmax, int sm_count) {
+  return gloc_plan_elems(n_sys) +
+         (size_t)n_sys * gloc_per_sys(n_sys, n_iw, mmax, sm_count) * gloc_f(mmax) * mmax * (mmax + 1);
 }
 
-cudaError_t launch_pole_gloc(const PoleParams& p, int n_sys, int mmax, int n_split, double2* part,
-                             int64_t tot, cudaStream_t s) {
-  const int F = pole_gloc_f(mmax);
-  const int bps = (p.n_iw + F - 1) / F;
-  const dim3 grid(n_sys * bps, n_split);
-  const int qp = (mmax * (mmax + 1) / 2 + kEigThreads - 1) / kEigThreads;  // 1..3 for m <= 32
-  if (qp <= 1) k_pole_gloc<1, 8><<<grid, kEigThreads, 0, s>>>(p, bps, n_split, part, tot);
-  else if (qp <= 2) k_pole_gloc<2, 4><<<grid, kEigThreads, 0, s>>>(p, bps, n_split, part, tot);
-  else k_pole_gloc<3, 4><<<grid, kEigThreads, 0, s>>>(p, bps, n_split, part, tot);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_split_reduce<<<std::min<int64_t>(4096, (tot + 255) / 256), 256, 0, s>>>(part, n_split, tot, p.gloc);
+cudaError_t launch_pole_gloc(const PoleParams& p, int n_sys, int mmax, int nps_max, int sm_count, double2* ws,
+                             cudaStream_t s) {
+  const int F = gloc_f(mmax), qp = gloc_qp(mmax), npairs = mmax * (mmax + 1) / 2;
+  const int per_sys = gloc_per_sys(n_sys, p.n_iw, mmax, sm_count);
+  const int threads = ((npairs + qp - 1) / qp + 31) / 32 * 32;
+  GlocPlan* plan = reinterpret_cast<GlocPlan*>(ws);
+  double2* part = ws + gloc_plan_elems(n_sys);
+  k_pole_span<<<n_sys, kEigThreads, 0, s>>>(p, F, plan);
+  const int grid = per_sys * n_sys;
+  if (qp == 1) k_pole_gloc<1, 8><<<grid, threads, 0, s>>>(p, plan, per_sys, nps_max, npairs, part);
+  else if (qp == 2) k_pole_gloc<2, 4><<<grid, threads, 0, s>>>(p, plan, per_sys, nps_max, npairs, part);
+  else k_pole_gloc<3, 4><<<grid, threads, 0, s>>>(p, plan, per_sys, nps_max, npairs, part);
+  const int64_t per_tile = (int64_t)2 * F * npairs;
+  const int64_t most = per_tile * ((p.n_iw + F - 1) / F);
+  const int bps = (int)std::min<int64_t>(std::max(1, 4096 / n_sys), (most + 127) / 128);
+  k_gloc_splits<<<bps * n_sys, 128, 0, s>>>(plan, bps, per_sys, per_tile, part);
+  k_gloc_write<<<p.n_iw * n_sys, 128, 0, s>>>(p, plan, per_sys, F, npairs, part);
   return cudaGetLastError();
 }
 

@@ -250,11 +250,10 @@ cudaError_t launch_heev_batched(const double2* A, int n_mat, int n, int max_swee
                                 double2* V, double2* gws, int grid, int in_smem, int* status,
                                 cudaStream_t s);
 cudaError_t launch_pole_eig(const PoleParams& p, int grid, size_t smem, cudaStream_t s);
-// G_loc from the eigenpairs, k split n_split ways into part [n_split][tot] and
-// summed in split order into p.gloc.
-int pole_gloc_splits(int n_sys, int n_iw, int sm_count, int mmax);
-cudaError_t launch_pole_gloc(const PoleParams& p, int n_sys, int mmax, int n_split, double2* part,
-                             int64_t tot, cudaStream_t s);
+// G_loc from the eigenpairs into p.gloc; ws holds pole_gloc_ws_elems elements.
+size_t pole_gloc_ws_elems(int n_sys, int n_iw, int mmax, int sm_count);
+cudaError_t launch_pole_gloc(const PoleParams& p, int n_sys, int mmax, int nps_max, int sm_count, double2* ws,
+                             cudaStream_t s);
 // DOS and PDOS, k split n_split ways into part [n_split][n_sys][n_eps][1 + mmax].
 int pole_dos_splits(int n_sys, int n_eps, int n_ch, int n_k, int sm_count);
 cudaError_t launch_pole_dos(const PoleParams& p, int n_sys, const double* eps_grid, int n_eps, double eta, int mmax,

@@ -174,6 +174,31 @@ def test_mixed_block_kernels_against_fp64(nk, nb, m, n_iw):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("nk,nb,m,n_iw,beta,ragged", [
+    (1, 3, 1, 5, 4.0, False),        # one pair, fewer frequencies than a tile
+    (3, 9, 3, 200, 5.0, False),      # most frequencies by the series
+    (7, 40, 14, 512, 100.0, True),   # both, windows that differ from k to k
+    (2, 30, 23, 130, 20.0, False),   # two pairs per thread
+    (2, 36, 32, 65, 20.0, False),    # three
+    (2, 20, 5, 24, 400.0, False),    # every frequency as it stands
+])
+def test_pole_local_by_moments_equals_the_resolvent(nk, nb, m, n_iw, beta, ragged):
+    """G_loc of the pole path, sums and Chebyshev moments, against the inverse at every frequency."""
+    from oracle import pole as pole_oracle
+    from paper_1111_2157_gb300 import gf
+    s = _inputs(nk, nb, m, n_iw, beta, 7 * nb + m, "orthonormal", ragged)
+    g = gf.GreensFunction.for_systems([s])
+    g.set_hamiltonian(s.H)
+    g.set_projectors(s.P)
+    g.set_sigma_poles([len(s.pole.p)], s.pole.p, s.pole.V.reshape(-1), s.pole.sigma_inf.reshape(-1))
+    for mu in (0.1, -30.0):  # inside and outside the levels
+        ref = pole_oracle.local(s.H, s.P, s.sigma_inf, s.pole.p, s.pole.V, s.beta, mu, s.n_iw).reshape(n_iw, -1)
+        gl = g.pole_local([mu]).cpu().numpy().reshape(n_iw, -1)
+        assert np.max(np.abs(gl - ref) / np.max(np.abs(ref), axis=1, keepdims=True)) < 1e-11
+    g.close()
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("what", ["non_hermitian", "rank_deficient", "few_frequencies"])
 def test_inputs_outside_the_rule_keep_the_general_kernels(what):
     s = _inputs(3, 20, 6, 8 if what == "few_frequencies" else 40, 40.0, 9)
