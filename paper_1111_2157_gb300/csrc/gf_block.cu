@@ -638,7 +638,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             const double wn = sW[f];
             const double x = mu - e_k[bb];
             const double xw = fma(x, x, wn * wn);
-            const double s = LOW ? rcp_newton(xw) : 1.0 / xw;
+            const double s = rcp_newton(xw);
             const double2 d = make_double2(x * s, -wn * s);
             if constexpr (LOW) {
               const cf dp = from_d2(d);

@@ -49,10 +49,11 @@ __device__ __forceinline__ double2 crcp(double2 a) {
   }
 }
 
-// 1 / x to rounding for |x| in FP32's range (0 where x is beyond it): the FP32 reciprocal and two
-// Newton steps, six FP64-pipe instructions.
+// 1 / x to rounding for normal x and 1 / x: the 20-bit seed of rcp.approx.ftz.f64, which the FP64 pipe
+// does not take part in, and two Newton steps, four FP64-pipe instructions.
 __device__ __forceinline__ double rcp_newton(double x) {
-  double r = (double)__frcp_rn((float)x);
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
   r = fma(r, fma(-x, r, 1.0), r);
   return fma(r, fma(-x, r, 1.0), r);
 }

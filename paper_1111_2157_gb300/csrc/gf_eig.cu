@@ -272,52 +272,53 @@ __device__ bool tri_eig(double* Z, int zr, int zs, double* G, int gr, int gs, in
     double lam = 0.5 * ((double)lo + (double)hi);
     const double small = 1e-18 * (double)tn;
     double* z = Z + tid * zs;
+    double* g = G + tid * gs;
+    const long long small_bits = __double_as_longlong(small), mask = 0x7fffffffffffffffLL;
     for (int it = 0; it < 3; ++it) {
-      // pivots from above, kept; from below with the twist row
-      double t = q.d[0] - lam;
-      for (int i = 0;; ++i) {
-        if (fabs(t) < small) t = small;
-        z[i * zr] = t;
-        if (i == N - 1) break;
-        const double e = q.e[i];
-        t = fma(-e, e * rcp_newton(t), q.d[i + 1] - lam);
+      // multipliers from above, l_i = e_i / t_i, and from below, m_i = e_i / u_{i+1}, side by side
+      double t = q.d[0] - lam, u = q.d[N - 1] - lam;
+      for (int i = 0; i + 1 < N; ++i) {
+        const int j = N - 2 - i;
+        if ((__double_as_longlong(t) & mask) < small_bits) t = small;
+        if ((__double_as_longlong(u) & mask) < small_bits) u = small;
+        const double l = q.e[i] * rcp_newton(t), m = q.e[j] * rcp_newton(u);
+        z[i * zr] = l;
+        g[j * gr] = m;
+        t = fma(-q.e[i], l, q.d[i + 1] - lam);
+        u = fma(-q.e[j], m, q.d[j] - lam);
       }
-      double best = fabs(z[(N - 1) * zr]);
-      double gam = z[(N - 1) * zr];
+      // the twist: the row of the smallest gamma_i = t_i - e_i m_i
+      double gam = t, el = 0.0;
       int r = N - 1;
-      double u = q.d[N - 1] - lam;
-      for (int i = N - 2; i >= 0; --i) {
-        if (fabs(u) < small) u = small;
-        const double e = q.e[i], w = e * (e * rcp_newton(u));
-        const double g = z[i * zr] - w;  // D+ + D- - (d - lam) with D- = d - lam - w
-        u = (q.d[i] - lam) - w;
-        if (fabs(g) < best) {
-          best = fabs(g);
-          gam = g;
+      long long best = __double_as_longlong(t) & mask;
+      for (int i = 0; i + 1 < N; ++i) {
+        const double v = fma(-q.e[i], g[i * gr], (q.d[i] - lam) - el);
+        el = q.e[i] * z[i * zr];
+        const long long key = __double_as_longlong(v) & mask;
+        if (key < best) {
+          best = key;
+          gam = v;
           r = i;
         }
       }
-      // multipliers from below for the rows after the twist, then the vector
-      u = q.d[N - 1] - lam;
-      for (int i = N - 2; i >= r; --i) {
-        if (fabs(u) < small) u = small;
-        const double e = q.e[i], m = e * rcp_newton(u);
-        u = fma(-e, m, q.d[i] - lam);
-        z[(i + 1) * zr] = -m;
-      }
-      double nrm = 1.0, x = 1.0;
-      for (int i = r + 1; i < N; ++i) {
-        x *= z[i * zr];
-        z[i * zr] = x;
-        nrm = fma(x, x, nrm);
-      }
-      x = 1.0;
-      for (int i = r - 1; i >= 0; --i) {
-        x *= -q.e[i] * rcp_newton(z[i * zr]);
-        z[i * zr] = x;
-        nrm = fma(x, x, nrm);
-      }
+      // the vector, from the twist in both directions
+      double n0 = 1.0, n1 = 0.0, x = 1.0, y = 1.0;
       z[r * zr] = 1.0;
+      for (int s = 1; s < N; ++s) {
+        const int iu = r - s, id = r + s;
+        if (iu < 0 && id >= N) break;
+        if (iu >= 0) {
+          x *= -z[iu * zr];
+          z[iu * zr] = x;
+          n0 = fma(x, x, n0);
+        }
+        if (id < N) {
+          y *= -g[(id - 1) * gr];
+          z[id * zr] = y;
+          n1 = fma(y, y, n1);
+        }
+      }
+      const double nrm = n0 + n1;
       lam += gam / nrm;
       if (it == 2) {
         const double s = rsqrt(nrm);
@@ -506,11 +507,9 @@ __device__ bool heev_tri(double2* A, double2* V, double* Z, int zr, int zs, doub
   }
   for (int k = 0; k + 2 < N; ++k) {
     const int len = N - 1 - k;
-    // lanes per row: every thread of the CTA on the shrinking triangle; the rows of a warp are kW
-    // apart, so that each warp has long and short ones
-    int tl = 32;
-    while (tl > 1 && kEigThreads / tl < len) tl >>= 1;
-    const int sub = lane % tl, rw = (lane / tl) * kW + warp;
+    // tl lanes per row, consecutive rows per warp: as many lanes as the rows leave
+    const int rpw = (len + kW - 1) / kW, tl = 32 / rpw;
+    const int sub = lane % tl, rw = lane / tl < rpw ? warp * rpw + lane / tl : len;
     if (warp == 0) {
       double s = 0.0;
       for (int i = lane; i < len; i += 32) {
@@ -555,8 +554,11 @@ __device__ bool heev_tri(double2* A, double2* V, double* Z, int zr, int zs, doub
       a0.x += a1.x;
       a0.y += a1.y;
       for (int off = 1; off < tl; off <<= 1) {
-        a0.x += __shfl_xor_sync(0xffffffffu, a0.x, off);
-        a0.y += __shfl_xor_sync(0xffffffffu, a0.y, off);
+        const double bx = __shfl_down_sync(0xffffffffu, a0.x, off), by = __shfl_down_sync(0xffffffffu, a0.y, off);
+        if (sub + off < tl) {
+          a0.x += bx;
+          a0.y += by;
+        }
       }
       if (sub == 0 && i < len) q.p[i] = make_double2(tau * a0.x, tau * a0.y);
     }
@@ -574,18 +576,31 @@ __device__ bool heev_tri(double2* A, double2* V, double* Z, int zr, int zs, doub
       }
     }
     __syncthreads();
-    // lower triangle: A -= v w^+ + w v^+; column k keeps v for the back-transformation
-    if (rw < len) {
-      const int i = rw;
-      const double2 vi = q.v[i], wi = q.p[i];
-      double2* Ar = A + (k + 1 + i) * ld + k + 1;
-      if (sub == 0) Ar[-1] = vi;
-      for (int c = sub; c <= i; c += tl) {
-        const double2 v = q.v[c], w = q.p[c];
-        double2 a = Ar[c];
-        a.x = fma(-vi.x, w.x, fma(-vi.y, w.y, fma(-wi.x, v.x, fma(-wi.y, v.y, a.x))));
-        a.y = fma(-vi.y, w.x, fma(vi.x, w.y, fma(-wi.y, v.x, fma(wi.x, v.y, a.y))));
-        Ar[c] = a;
+    // lower triangle: A -= v w^+ + w v^+, rows i and len - 1 - i together, so that all lanes have
+    // len + 1 entries; column k keeps v for the back-transformation
+    {
+      const int half = (len + 1) / 2, ppw = (half + kW - 1) / kW, tp = 32 / ppw;
+      const int i = warp * ppw + lane / tp, i2 = len - 1 - i, sp = lane % tp;
+      if (lane / tp < ppw && i < half) {
+        const double2 va = q.v[i], wa = q.p[i], vb = q.v[i2], wb = q.p[i2];
+        double2* Ar = A + (k + 1 + i) * ld + k + 1;
+        double2* Br = A + (k + 1 + i2) * ld + k + 1;
+        if (sp == 0) {
+          Ar[-1] = va;
+          Br[-1] = vb;
+        }
+        const int end = i == i2 ? i + 1 : len + 1;
+        for (int x = sp; x < end; x += tp) {
+          const bool first = x <= i;
+          const int c = first ? x : x - i - 1;
+          const double2 vi = first ? va : vb, wi = first ? wa : wb;
+          double2* at = (first ? Ar : Br) + c;
+          const double2 v = q.v[c], w = q.p[c];
+          double2 a = *at;
+          a.x = fma(-vi.x, w.x, fma(-vi.y, w.y, fma(-wi.x, v.x, fma(-wi.y, v.y, a.x))));
+          a.y = fma(-vi.y, w.x, fma(vi.x, w.y, fma(-wi.y, v.x, fma(wi.x, v.y, a.y))));
+          *at = a;
+        }
       }
     }
     __syncthreads();
@@ -614,41 +629,43 @@ __device__ bool heev_tri(double2* A, double2* V, double* Z, int zr, int zs, doub
     V[i * ld + l] = make_double2(q.ph[i].x * z, q.ph[i].y * z);
   }
   __syncthreads();
-  // (more lanes a column, with fewer idle, measured slower: 1.5 against 1.1 M clocks at N = 68)
-  const int tl = N <= 64 ? 4 : (N <= 128 ? 2 : 1);
-  const int sub = lane % tl;
-  for (int l0 = 0; l0 < N; l0 += kEigThreads / tl) {
-    const int l = l0 + warp * (32 / tl) + lane / tl;
-    for (int k = N - 3; k >= 0; --k) {
-      const double2* v = A + (k + 1) * ld + k;
-      double2 s0 = make_double2(0.0, 0.0), s1 = s0;
-      if (l < N) {
-        int i = sub;
-        for (; i + tl < N - 1 - k; i += 2 * tl) {
-          cmac_ca(s0, v[i * ld], V[(k + 1 + i) * ld + l]);
-          cmac_ca(s1, v[(i + tl) * ld], V[(k + 1 + i + tl) * ld + l]);
-        }
-        for (; i < N - 1 - k; i += tl) cmac_ca(s0, v[i * ld], V[(k + 1 + i) * ld + l]);
+  const int cpw = (N + kW - 1) / kW, tl = 32 / cpw;  // consecutive columns per warp (N <= 256)
+  const int sub = lane % tl, base = lane - sub;
+  const int l = warp * cpw + lane / tl;
+  const bool on = lane / tl < cpw && l < N;
+  for (int k = N - 3; k >= 0; --k) {
+    const double2* v = A + (k + 1) * ld + k;
+    const int len = N - 1 - k;
+    double2 s0 = make_double2(0.0, 0.0), s1 = s0;
+    if (on) {
+      int i = sub;
+      for (; i + tl < len; i += 2 * tl) {
+        cmac_ca(s0, v[i * ld], V[(k + 1 + i) * ld + l]);
+        cmac_ca(s1, v[(i + tl) * ld], V[(k + 1 + i + tl) * ld + l]);
       }
-      s0.x += s1.x;
-      s0.y += s1.y;
-      for (int off = 1; off < tl; off <<= 1) {
-        s0.x += __shfl_xor_sync(0xffffffffu, s0.x, off);
-        s0.y += __shfl_xor_sync(0xffffffffu, s0.y, off);
-      }
-      const double tau = q.tau[k];
-      s0.x *= tau;
-      s0.y *= tau;
-      if (l < N)
-        for (int i = sub; i < N - 1 - k; i += tl) {
-          const double2 vv = v[i * ld];
-          double2 u = V[(k + 1 + i) * ld + l];
-          u.x = fma(-vv.x, s0.x, fma(vv.y, s0.y, u.x));
-          u.y = fma(-vv.x, s0.y, fma(-vv.y, s0.x, u.y));
-          V[(k + 1 + i) * ld + l] = u;
-        }
-      __syncwarp();
+      for (; i < len; i += tl) cmac_ca(s0, v[i * ld], V[(k + 1 + i) * ld + l]);
     }
+    s0.x += s1.x;
+    s0.y += s1.y;
+    for (int off = 1; off < tl; off <<= 1) {
+      const double bx = __shfl_down_sync(0xffffffffu, s0.x, off), by = __shfl_down_sync(0xffffffffu, s0.y, off);
+      if (sub + off < tl) {
+        s0.x += bx;
+        s0.y += by;
+      }
+    }
+    const double tau = q.tau[k];
+    s0.x = tau * __shfl_sync(0xffffffffu, s0.x, base);
+    s0.y = tau * __shfl_sync(0xffffffffu, s0.y, base);
+    if (on)
+      for (int i = sub; i < len; i += tl) {
+        const double2 vv = v[i * ld];
+        double2 u = V[(k + 1 + i) * ld + l];
+        u.x = fma(-vv.x, s0.x, fma(vv.y, s0.y, u.x));
+        u.y = fma(-vv.x, s0.y, fma(-vv.y, s0.x, u.y));
+        V[(k + 1 + i) * ld + l] = u;
+      }
+    __syncwarp();
   }
   __syncthreads();
   for (int i = tid; i < N; i += kEigThreads) A[i * ld + i] = make_double2(q.d[i], 0.0);

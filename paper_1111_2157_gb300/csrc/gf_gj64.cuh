@@ -20,7 +20,7 @@ __device__ __forceinline__ double2 crcp_scaled(double2 a, unsigned long long key
   ex = ex < 1 ? 1 : ex;
   const double s = __longlong_as_double((long long)ex << 52);
   const double x = a.x * s, y = a.y * s;
-  const double q = s * rcp_newton(fma(x, x, y * y));  // in [1, 8): within FP32's range
+  const double q = s * rcp_newton(fma(x, x, y * y));  // of [1, 8)
   return make_double2(x * q, -y * q);
 }
 
