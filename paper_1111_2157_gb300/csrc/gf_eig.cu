@@ -481,9 +481,13 @@ __device__ bool tri_qr(double* Z, int zr, int zs, int N, QlScratch& q) {
 // columns.  Z: real N x N scratch (row stride zr, element step zs), G another; both may lie over V
 // (its real and its imaginary parts).  Returns false when the QR steps fail.
 //
+// With nr >= 0 only the rows [r0, r0 + nr) of the eigenvectors are wanted (2 nr <= N): they are left
+// in the first nr rows of A, the eigenvalues in q.d, and V is scratch.  The reflectors are then
+// applied to those rows of the identity, and the result to Z: 6 nr N^2 FMAs instead of 4 N^3.
+//
 // About 12 N^3 FP64 FMAs against 18 N^3 per sweep and eight sweeps of cyclic Jacobi.
 __device__ bool heev_tri(double2* A, double2* V, double* Z, int zr, int zs, double* G, int gr, int gs, int N, int ld,
-                         QlScratch& q) {
+                         QlScratch& q, int r0 = 0, int nr = -1) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int kW = kEigThreads / 32;
   // a matrix that is diagonal already (to 1e-15 of its norm): no work
@@ -498,7 +502,13 @@ __device__ bool heev_tri(double2* A, double2* V, double* Z, int zr, int zs, doub
   off = eig_block_sum(off, &q.tau[0]);
   dia = eig_block_sum(dia, &q.tau[0]);
   if (off <= 1e-30 * (off + dia)) {
-    for (int x = tid; x < N * N; x += kEigThreads) {
+    for (int i = tid; i < N; i += kEigThreads) q.d[i] = A[i * ld + i].x;
+    __syncthreads();
+    for (int x = tid; x < nr * N; x += kEigThreads) {
+      const int r = x / N, l = x - r * N;
+      A[r * ld + l] = make_double2(r0 + r == l ? 1.0 : 0.0, 0.0);
+    }
+    for (int x = tid; x < N * N && nr < 0; x += kEigThreads) {
       const int i = x / N, l = x - i * N;
       V[i * ld + l] = make_double2(i == l ? 1.0 : 0.0, 0.0);
     }
@@ -622,6 +632,82 @@ __device__ bool heev_tri(double2* A, double2* V, double* Z, int zr, int zs, doub
   bool ok = N > 3 && tri_eig(Z, zr, zs, G, gr, gs, N, q);
   if (!ok) ok = tri_qr(Z, zr, zs, N, q);
   __syncthreads();
+  if (nr >= 0) {
+    // L = (rows of the identity) H_0 H_1 ..., its parts in the first 2 nr rows of G, tl lanes per row
+    for (int x = tid; x < nr * N; x += kEigThreads) {
+      const int r = x / N, c = x - r * N;
+      G[r * gr + c * gs] = r0 + r == c ? 1.0 : 0.0;
+      G[(nr + r) * gr + c * gs] = 0.0;
+    }
+    __syncthreads();
+    const int rpw = max(1, (nr + kW - 1) / kW), tl = 32 / rpw;
+    const int sub = lane % tl, base = lane - sub, r = warp * rpw + lane / tl;
+    const bool on = lane / tl < rpw && r < nr;
+    double* Lr = G + (on ? r : 0) * gr;
+    double* Li = Lr + nr * gr;
+    for (int k = 0; k + 2 < N; ++k) {
+      const double2* v = A + (k + 1) * ld + k;
+      const int len = N - 1 - k;
+      double2 s0 = make_double2(0.0, 0.0), s1 = s0;
+      if (on) {
+        int i = sub;
+        for (; i + tl < len; i += 2 * tl) {
+          cmac(s0, make_double2(Lr[(k + 1 + i) * gs], Li[(k + 1 + i) * gs]), v[i * ld]);
+          cmac(s1, make_double2(Lr[(k + 1 + i + tl) * gs], Li[(k + 1 + i + tl) * gs]), v[(i + tl) * ld]);
+        }
+        for (; i < len; i += tl) cmac(s0, make_double2(Lr[(k + 1 + i) * gs], Li[(k + 1 + i) * gs]), v[i * ld]);
+      }
+      s0.x += s1.x;
+      s0.y += s1.y;
+      for (int off = 1; off < tl; off <<= 1) {
+        const double bx = __shfl_down_sync(0xffffffffu, s0.x, off), by = __shfl_down_sync(0xffffffffu, s0.y, off);
+        if (sub + off < tl) {
+          s0.x += bx;
+          s0.y += by;
+        }
+      }
+      const double tau = q.tau[k];
+      s0.x = tau * __shfl_sync(0xffffffffu, s0.x, base);
+      s0.y = tau * __shfl_sync(0xffffffffu, s0.y, base);
+      if (on)
+        for (int i = sub; i < len; i += tl) {  // L -= s v^+
+          const double2 vv = v[i * ld];
+          double* lr = Lr + (k + 1 + i) * gs;
+          double* li = Li + (k + 1 + i) * gs;
+          *lr = fma(-s0.x, vv.x, fma(-s0.y, vv.y, *lr));
+          *li = fma(-s0.y, vv.x, fma(s0.x, vv.y, *li));
+        }
+      __syncwarp();
+    }
+    if (on)
+      for (int c = sub; c < N; c += tl) {
+        const double2 x = cmul(make_double2(Lr[c * gs], Li[c * gs]), q.ph[c]);
+        Lr[c * gs] = x.x;
+        Li[c * gs] = x.y;
+      }
+    __syncthreads();
+    for (int x = tid; x < nr * N; x += kEigThreads) {
+      const int a = x / N, l = x - a * N;
+      const double *ar = G + a * gr, *ai = ar + nr * gr;
+      double2 s0 = make_double2(0.0, 0.0), s1 = s0;
+      int c = 0;
+      for (; c + 1 < N; c += 2) {
+        const double z0 = Z[c * zr + l * zs], z1 = Z[(c + 1) * zr + l * zs];
+        s0.x = fma(ar[c * gs], z0, s0.x);
+        s0.y = fma(ai[c * gs], z0, s0.y);
+        s1.x = fma(ar[(c + 1) * gs], z1, s1.x);
+        s1.y = fma(ai[(c + 1) * gs], z1, s1.y);
+      }
+      if (c < N) {
+        const double z0 = Z[c * zr + l * zs];
+        s0.x = fma(ar[c * gs], z0, s0.x);
+        s0.y = fma(ai[c * gs], z0, s0.y);
+      }
+      A[a * ld + l] = make_double2(s0.x + s1.x, s0.y + s1.y);
+    }
+    __syncthreads();
+    return ok;
+  }
   // V = H_0 H_1 ... D Z: phases, then the reflectors in reverse order, tl lanes per column
   for (int x = tid; x < N * N; x += kEigThreads) {
     const int i = x / N, l = x - i * N;
@@ -676,11 +762,11 @@ __device__ bool heev_tri(double2* A, double2* V, double* Z, int zr, int zs, doub
 // heev_tri with Z and G over V's real and imaginary parts when the matrices are in shared memory;
 // with the matrices in a global slice Z has shared memory of its own when that fits (z_smem).
 __device__ __forceinline__ bool heev_tri(double2* A, double2* V, int n, int ld, int in_smem, int z_smem,
-                                         unsigned char* smem, QlScratch& q) {
+                                         unsigned char* smem, QlScratch& q, int r0 = 0, int nr = -1) {
   double* v = reinterpret_cast<double*>(V);
   if (!in_smem && z_smem)
-    return heev_tri(A, V, reinterpret_cast<double*>(smem), n | 1, 1, v, n | 1, 1, n, ld, q);
-  return heev_tri(A, V, v, 2 * ld, 2, v + 1, 2 * ld, 2, n, ld, q);
+    return heev_tri(A, V, reinterpret_cast<double*>(smem), n | 1, 1, v, n | 1, 1, n, ld, q, r0, nr);
+  return heev_tri(A, V, v, 2 * ld, 2, v + 1, 2 * ld, 2, n, ld, q, r0, nr);
 }
 
 __device__ __forceinline__ size_t eig_ws_elems(int n) { return (size_t)2 * n * (n | 1); }
@@ -786,33 +872,38 @@ __global__ void __launch_bounds__(kEigThreads) k_pole_eig(const PoleParams p) {
       A[(nb + i) * ld + nb + j] = make_double2(i == j ? p.poles[pi.offp + i] + mu : 0.0, 0.0);
     }
     __syncthreads();
-    const bool ok = heev_tri(A, V, n, ld, p.in_smem, p.z_smem, smem_raw, ql);
+    // N(mu) needs Psi_b^+ Psi_b = 1 - Psi_p^+ Psi_p only: the pole rows, where they are the fewer
+    // (125 k-points of 40 bands and 28 poles 1.42 ms, all rows 1.64 ms)
+    const bool few = p.mode == kOcc && npl <= nb;
+    const bool ok = heev_tri(A, V, n, ld, p.in_smem, p.z_smem, smem_raw, ql, nb, few ? npl : -1);
     if (!ok && tid == 0) atomicOr(p.status, 2);
     // per eigenpair: x_l = E_l - mu, n_F(x_l), cosh(beta x_l / 2)
     for (int l = tid; l < n; l += kEigThreads) {
-      const double x = A[l * ld + l].x - mu;
+      const double x = (few ? ql.d[l] : A[l * ld + l].x) - mu;
       s_x[l] = x;
       s_f[l] = fermi(x, si.beta);
       s_ch[l] = cosh(0.5 * si.beta * x);
     }
     __syncthreads();
     if (p.mode & kOcc) {
+      const double2* W = few ? A : V;
+      const int nw = few ? npl : nb;
       double nk = 0.0;
       for (int l = tid; l < n; l += kEigThreads) {
         double wb = 0.0;
-        for (int b = 0; b < nb; ++b) {
-          const double2 v = V[b * ld + l];
+        for (int b = 0; b < nw; ++b) {
+          const double2 v = W[b * ld + l];
           wb = fma(v.x, v.x, fma(v.y, v.y, wb));
         }
-        nk = fma(wb, s_f[l], nk);
+        nk = fma(few ? 1.0 - wb : wb, s_f[l], nk);
       }
       nk = eig_block_sum(nk, red);
       double dk = 0.0;
       for (int e = tid; e < n * (n + 1) / 2; e += kEigThreads) {
         int l, l2;
         tri_pair(e, l, l2);
-        double2 o = make_double2(0.0, 0.0);
-        for (int b = 0; b < nb; ++b) cmac_ca(o, V[b * ld + l], V[b * ld + l2]);
+        double2 o = make_double2(few && l == l2 ? -1.0 : 0.0, 0.0);  // (its modulus is wanted)
+        for (int b = 0; b < nw; ++b) cmac_ca(o, W[b * ld + l], W[b * ld + l2]);
         const double f1 =
             fermi_divdiff(s_x[l], s_x[l2], s_f[l], s_f[l2], s_ch[l], s_ch[l2], si.beta);
         dk = fma((l == l2 ? -1.0 : -2.0) * (o.x * o.x + o.y * o.y), f1, dk);
