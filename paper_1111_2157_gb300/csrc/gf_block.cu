@@ -403,6 +403,7 @@ __device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf
 struct LayoutB {
   size_t oS, oF, od2, orc, oM, oR, oY, oG, od, op, oW, oPair, oHz, oX, oB, bytes;
   size_t sS, sF, sd2, src, sG, sR, sd, sp;  // bytes per warp (sS also of M)
+  size_t fG;  // bytes of S^{-1} in FP32 per frequency
   int nf;   // frequencies per warp
   int yf;   // frequencies of the rho_k columns staged at once
 };
@@ -418,7 +419,9 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   L.sF = needF ? al((adj ? 16 : r) * f * mm) : 0;
   L.sd2 = needF ? al((low && adj ? 24 : 2 * r) * f * n2max) : 0;
   L.src = (low ? 8 : 16) * f * 2 * mmax;
-  L.sG = low ? al(8 * f * mm) : 0;
+  const size_t kp = (mmax + 1) / 2, pb = ((size_t)n2max + 3) & ~(size_t)3;
+  L.fG = low ? (rho ? 16 * kp * mmax : 8 * mm) : 0;  // (rho_k reads it by pairs of rows)
+  L.sG = al(f * L.fG);
   L.sd = 16 * f * n2max;
   L.sp = al(4 * f * 2 * mmax);
   size_t o = 0;
@@ -435,12 +438,12 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   if (low && (mode & kGloc) && !needF) o += W * L.sG;
   const size_t np = (size_t)mmax * (mmax + 1) / 2;
   const size_t fixed = W * (L.sG + L.sd + L.sp + (low ? 16 : 8) * f) + al(2 * np) + (low ? 32 : 16) * np +
-                       (low && rho ? 8 * mmax * (((size_t)n2max + 3) & ~(size_t)3) + al(4 * (size_t)n2max) : 0);
+                       (low && rho ? 16 * kp * pb + al(4 * (size_t)n2max) : 0);
   L.yf = 0;
   if (rho) {
     // as many frequencies as fit over the dead arrays, or as leave three CTAs on an SM, or two:
     // the chunk's sum is read and written once per stage
-    const size_t one = mmax * (low ? 8 * (((size_t)n2max + 3) & ~(size_t)3) : 16 * (size_t)n2max);
+    const size_t one = 16 * (low ? kp : mmax) * (size_t)n2max;
     const size_t all = f * W;
     size_t room = o - L.oY;
     for (size_t lim = 74u << 10; lim <= (112u << 10); lim += 38u << 10)
@@ -459,7 +462,7 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   L.oPair = o; o += al(2 * np);
   L.oHz = o; o += (low ? 32 : 16) * np;  // (low: pairs of mu O - H11, then of O)
   L.oX = o; o = al(o + (low && rho ? 4 * (size_t)n2max : 0));
-  L.oB = o; o += low && rho ? 8 * mmax * (((size_t)n2max + 3) & ~(size_t)3) : 0;
+  L.oB = o; o += low && rho ? 16 * kp * pb : 0;
   L.bytes = o;
   return L;
 }
@@ -528,10 +531,17 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
     }
     if constexpr (LOW) {
       if (rho) {
-        float2* sB = reinterpret_cast<float2*>(smraw + L.oB);
-        const int pt = (n2 + 3) & ~3;
+        // B by pairs of rows, {Re, Re, Im, Im}; 0 beyond M and n2
+        float4* sB = reinterpret_cast<float4*>(smraw + L.oB);
+        const int pb = (n2 + 3) & ~3;
+        const float2* Bk = bf.Bs + ki.offP;
         for (int i = tid; i < n2; i += 32 * W) xs[i] = __double2float_rn(mu - e_k[i]);
-        for (int i = tid; i < M * n2; i += 32 * W) sB[(i / n2) * pt + i % n2] = bf.Bs[ki.offP + i];
+        for (int i = tid; i < (M + 1) / 2 * pb; i += 32 * W) {
+          const int x = i / pb * 2, b = i % pb;
+          const float2 zero = make_float2(0.f, 0.f);
+          const float2 u = b < n2 ? Bk[x * n2 + b] : zero, v = b < n2 && x + 1 < M ? Bk[(x + 1) * n2 + b] : zero;
+          sB[i] = make_float4(u.x, v.x, u.y, v.y);
+        }
       }
     }
     __syncthreads();
@@ -838,7 +848,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
         const rc_t* inv;  // the warp's inverses, A[p_i][q_c] (LOW: FP32)
         if constexpr (LOW) {
           const float4* Sp = reinterpret_cast<const float4*>(A);
-          float2* X0 = sG + mf * MM;
+          float2* X0 = sG + mf * (L.fG / sizeof(float2));
           for (int i = sl; i < MM; i += LW) X0[i] = make_float2(Sp[i].x, Sp[i].z);
           __syncwarp();
           gj64::invert<LW>(X0, M, rcb, sp, sl, p.status);
@@ -862,7 +872,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             rc_t x1 = rzero(rc_t{}), x2 = x1;
             const int* pf = sPv + f * 2 * M;
             const int* qf = pf + M;
-            const rc_t* Af = inv + f * MM;
+            const rc_t* Af = inv + f * (LOW ? (int)(L.fG / sizeof(float2)) : MM);
             const int pa = pf[a] * M, pc = pf[c] * M;
             for (int j = 0; j < M; ++j) {
               const int fj = pf[j] * M;
@@ -930,7 +940,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
           // these frequencies, where the FP64 elimination takes 1,500 FP64 instructions a matrix
           // at m = 20.
           const float4* Sp = reinterpret_cast<const float4*>(A);
-          float2* X0 = sG + mf * MM;
+          float2* X0 = sG + mf * (L.fG / sizeof(float2));
           float2* R = reinterpret_cast<float2*>(smraw + L.oR + wp * L.sR) + mf * MM;
           const bool refine = (p.mode & (kGloc | kAdj)) != 0;
           if (refine) {
@@ -960,8 +970,12 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
             if (!adj) Gn[i] = h;
           }
           __syncwarp();
-          if (rho)
-            for (int i = sl; i < MM; i += LW) X0[i] = Gn[i];
+          if (rho)  // by pairs of rows, {Re, Re, Im, Im}
+            for (int i = sl; i < (M + 1) / 2 * M; i += LW) {
+              const int a = i / M * 2, c = i - a / 2 * M;
+              const float2 u = Gn[a * M + c], v = a + 1 < M ? Gn[(a + 1) * M + c] : make_float2(0.f, 0.f);
+              reinterpret_cast<float4*>(X0)[i] = make_float4(u.x, v.x, u.y, v.y);
+            }
           __syncwarp();
         }
         if (adj) {
@@ -1073,170 +1087,171 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
           // them, so that the L2 latency passes under the arithmetic
           auto old = [&](int at) { return put ? make_double2(0.0, 0.0) : Sk[at]; };
           auto add = [&](int at, double2 o, double2 v) { Sk[at] = make_double2(o.x + v.x, o.y + v.y); };
-          // (1,1) block
-          for (int i = tid; i < MM; i += 32 * W) {
-            const int a = i / M, c = i - a * M;
-            const double2 o = old(a * nb + c);
-            double2 v = make_double2(0.0, 0.0);
-            if constexpr (LOW) {
-              float2 g = make_float2(0.f, 0.f);
-              for (int f = f0; f < f0 + nf; ++f) {
-                const float2 gf = reinterpret_cast<const float2*>(smraw + L.oG + (f / F) * L.sG)[(f % F) * MM + i];
-                g.x += gf.x;
-                g.y += gf.y;
+          if constexpr (LOW) {
+            // FP32 products, summed over the nf frequencies in FP32 and added to the chunk's FP64 sum
+            // once (each FP64 add or conversion takes the SM 16 clocks).  Rows 1 of G_k are [A, Y],
+            // Y = A B D, rows 2 are D B^+ [A, Y] + D: orbitals lie in pairs of rows, {Re, Re, Im, Im},
+            // so that the packed FMAs take two terms of the contraction over them, and columns of a
+            // thread lie a third of the matrix apart, so that a warp's loads are consecutive.
+            const int KP = (M + 1) / 2, CT = M + n2, pb = (n2 + 3) & ~3;
+            const float4* sB = reinterpret_cast<const float4*>(smraw + L.oB);
+            const float4* sA = reinterpret_cast<const float4*>(smraw + L.oG);  // [frequency][KP][M]
+            const int fA = (int)(L.fG / sizeof(float4));
+            float4* sY = reinterpret_cast<float4*>(smraw + L.oY);  // [yf][KP][n2]
+            auto dlow = [&](int f, int b) {
+              return reinterpret_cast<const float2*>(smraw + L.od + (f / F) * L.sd)[(f % F) * n2 + b];
+            };
+            // Y: four pairs of orbitals of one band a thread
+            const int at = (KP + 3) / 4;
+            for (int i = tid; i < nf * at * n2; i += 32 * W) {
+              const int r = i / n2, c = i - r * n2, f = r / at, p0 = (r - f * at) * 4;
+              const float4* ga[4];
+#pragma unroll
+              for (int u = 0; u < 4; ++u) ga[u] = sA + (size_t)(f0 + f) * fA + min(p0 + u, KP - 1) * M;
+              float2 re[4], im[4];
+#pragma unroll
+              for (int u = 0; u < 4; ++u) re[u] = im[u] = make_float2(0.f, 0.f);
+              auto mac = [&](int x, float br, float bi) {
+                const float2 r2 = make_float2(br, br), i2 = make_float2(bi, bi), n2i = make_float2(-bi, -bi);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  const float4 g = ga[u][x];
+                  const float2 gr = make_float2(g.x, g.y), gi = make_float2(g.z, g.w);
+                  re[u] = __ffma2_rn(gr, r2, re[u]);
+                  im[u] = __ffma2_rn(gr, i2, im[u]);
+                  re[u] = __ffma2_rn(gi, n2i, re[u]);
+                  im[u] = __ffma2_rn(gi, r2, im[u]);
+                }
+              };
+              int x = 0;
+              for (; x + 1 < M; x += 2) {
+                const float4 b = sB[(x >> 1) * pb + c];
+                mac(x, b.x, b.z);
+                mac(x + 1, b.y, b.w);
               }
-              v = make_double2(widen(g.x), widen(g.y));
-            } else {
+              if (x < M) {
+                const float4 b = sB[(x >> 1) * pb + c];
+                mac(x, b.x, b.z);
+              }
+              const float2 d = dlow(f0 + f, c);
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+                if (p0 + u < KP)
+                  sY[(size_t)(f * KP + p0 + u) * n2 + c] =
+                      make_float4(fmaf(re[u].x, d.x, -im[u].x * d.y), fmaf(re[u].y, d.x, -im[u].y * d.y),
+                                  fmaf(re[u].x, d.y, im[u].x * d.x), fmaf(re[u].y, d.y, im[u].y * d.x));
+            }
+            __syncthreads();
+            // (1,1) and (1,2): the sum over the frequencies
+            for (int i = tid; i < KP * CT; i += 32 * W) {
+              const int pr = i / CT, c = i - pr * CT, a = 2 * pr;
+              const bool two = a + 1 < M;
+              const double2 o0 = old(a * nb + c), o1 = two ? old((a + 1) * nb + c) : make_double2(0.0, 0.0);
+              const float4* v = c < M ? sA + (size_t)f0 * fA + pr * M + c : sY + pr * n2 + (c - M);
+              const int fs = c < M ? fA : KP * n2;
+              float4 t = v[0];
+              for (int f = 1; f < nf; ++f) {
+                const float4 w = v[(size_t)f * fs];
+                t = make_float4(t.x + w.x, t.y + w.y, t.z + w.z, t.w + w.w);
+              }
+              add(a * nb + c, o0, make_double2(widen(t.x), widen(t.z)));
+              if (two) add((a + 1) * nb + c, o1, make_double2(widen(t.y), widen(t.w)));
+            }
+            // (2,1) and (2,2) in tiles of four rows and CW columns
+            constexpr int CW = 3;
+            const int ctl = (CT + CW - 1) / CW, ntl = pb / 4 * ctl;
+            for (int i = tid; i < ntl; i += 32 * W) {
+              const int b0 = (i / ctl) * 4, c0 = i - (i / ctl) * ctl;
+              const float4* src[CW];
+              int ks[CW], fs[CW];  // steps of a pair of orbitals and of a frequency
+#pragma unroll
+              for (int w = 0; w < CW; ++w) {
+                const int c = min(c0 + w * ctl, CT - 1);
+                src[w] = c < M ? sA + (size_t)f0 * fA + c : sY + (c - M);
+                ks[w] = c < M ? M : n2;
+                fs[w] = c < M ? fA : KP * n2;
+              }
+              float2 v[4][CW];
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int w = 0; w < CW; ++w) v[u][w] = make_float2(0.f, 0.f);
+              for (int f = 0; f < nf; ++f) {
+                float2 re[4][CW], im[4][CW];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                  for (int w = 0; w < CW; ++w) re[u][w] = im[u][w] = make_float2(0.f, 0.f);
+                for (int k = 0; k < KP; ++k) {
+                  float2 yr[CW], yi[CW];
+#pragma unroll
+                  for (int w = 0; w < CW; ++w) {
+                    const float4 y = src[w][(size_t)f * fs[w] + k * ks[w]];
+                    yr[w] = make_float2(y.x, y.y);
+                    yi[w] = make_float2(y.z, y.w);
+                  }
+#pragma unroll
+                  for (int u = 0; u < 4; ++u) {
+                    const float4 b = sB[k * pb + b0 + u];
+                    const float2 br = make_float2(b.x, b.y), bi = make_float2(b.z, b.w);
+                    const float2 nbi = make_float2(-b.z, -b.w);
+#pragma unroll
+                    for (int w = 0; w < CW; ++w) {  // conj(b) y
+                      re[u][w] = __ffma2_rn(br, yr[w], re[u][w]);
+                      im[u][w] = __ffma2_rn(br, yi[w], im[u][w]);
+                      re[u][w] = __ffma2_rn(bi, yi[w], re[u][w]);
+                      im[u][w] = __ffma2_rn(nbi, yr[w], im[u][w]);
+                    }
+                  }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  const float2 d = dlow(f0 + f, min(b0 + u, n2 - 1));
+#pragma unroll
+                  for (int w = 0; w < CW; ++w)
+                    fmac(v[u][w], make_float2(re[u][w].x + re[u][w].y, im[u][w].x + im[u][w].y), d);
+                }
+              }
+              double2 o[4][CW];  // (all loads before the first store)
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int w = 0; w < CW; ++w)
+                  o[u][w] = old((M + min(b0 + u, n2 - 1)) * nb + min(c0 + w * ctl, CT - 1));
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const int bb = b0 + u;
+                if (bb >= n2) break;
+#pragma unroll
+                for (int w = 0; w < CW; ++w) {
+                  const int c = c0 + w * ctl;
+                  if (c >= CT) break;
+                  float2 t = v[u][w];
+                  if (M + bb == c)
+                    for (int f = f0; f < f0 + nf; ++f) {
+                      const float2 d = dlow(f, bb);
+                      t.x += d.x;
+                      t.y += d.y;
+                    }
+                  add((M + bb) * nb + c, o[u][w], make_double2(widen(t.x), widen(t.y)));
+                }
+              }
+            }
+            __syncthreads();
+          } else {
+            // (1,1) block
+            for (int i = tid; i < MM; i += 32 * W) {
+              const int a = i / M, c = i - a * M;
+              const double2 o = old(a * nb + c);
+              double2 v = make_double2(0.0, 0.0);
               for (int f = f0; f < f0 + nf; ++f) {
                 const int* pf = piv(f);
                 const double2 g = mat(f)[pf[a] * M + pf[M + c]];
                 v.x += g.x;
                 v.y += g.y;
               }
+              add(a * nb + c, o, v);
             }
-            add(a * nb + c, o, v);
-          }
-          if constexpr (LOW) {
-            // FP32 products in register tiles, summed over the nf frequencies in FP32 and added
-            // to the chunk's FP64 sum once (each FP64 add or conversion takes the SM 16 clocks)
-            auto matf = [&](int f) { return reinterpret_cast<const float2*>(smraw + L.oG + (f / F) * L.sG) + (f % F) * MM; };
-            const int pt = (n2 + 3) & ~3;
-            const float2* sB = reinterpret_cast<const float2*>(smraw + L.oB);
-            float2* sY = reinterpret_cast<float2*>(smraw + L.oY);  // [yf][M][pt]: S^{-1} B D
-            auto dlow = [&](int f, int b) {
-              return reinterpret_cast<const float2*>(smraw + L.od + (f / F) * L.sd)[(f % F) * n2 + b];
-            };
-            // (1,2) and (2,1): Y = S^{-1} B D, Z = D B^+ S^{-1}; four orbitals and two bands a thread
-            const int at4 = (M + 3) / 4, ct = (n2 + 1) / 2;
-            for (int i = tid; i < at4 * ct; i += 32 * W) {
-              const int a0 = (i / ct) * 4, c0 = i - (i / ct) * ct, c1 = min(c0 + ct, n2 - 1);
-              int ar[4];
-#pragma unroll
-              for (int u = 0; u < 4; ++u) ar[u] = min(a0 + u, M - 1);
-              float2 v12[4][2], v21[4][2];
-#pragma unroll
-              for (int u = 0; u < 4; ++u) v12[u][0] = v12[u][1] = v21[u][0] = v21[u][1] = make_float2(0.f, 0.f);
-              for (int f = 0; f < nf; ++f) {
-                const float2* Gf = matf(f0 + f);
-                float2 y[4][2], z[4][2];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) y[u][0] = y[u][1] = z[u][0] = z[u][1] = make_float2(0.f, 0.f);
-                for (int x = 0; x < M; ++x) {
-                  const float2 b0 = sB[x * pt + c0], b1 = sB[x * pt + c1];
-#pragma unroll
-                  for (int u = 0; u < 4; ++u) {
-                    const float2 g = Gf[ar[u] * M + x], h = Gf[x * M + ar[u]];
-                    fmac(y[u][0], g, b0);
-                    fmac(y[u][1], g, b1);
-                    fmac_ca(z[u][0], b0, h);
-                    fmac_ca(z[u][1], b1, h);
-                  }
-                }
-                const float2 d0 = dlow(f0 + f, c0), d1 = dlow(f0 + f, c1);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                  y[u][0] = fmul(y[u][0], d0);
-                  y[u][1] = fmul(y[u][1], d1);
-                  fmac(v21[u][0], z[u][0], d0);
-                  fmac(v21[u][1], z[u][1], d1);
-                  v12[u][0].x += y[u][0].x; v12[u][0].y += y[u][0].y;
-                  v12[u][1].x += y[u][1].x; v12[u][1].y += y[u][1].y;
-                  if (a0 + u < M) {
-                    float2* Yr = sY + (size_t)(f * M + a0 + u) * pt;
-                    Yr[c0] = y[u][0];
-                    if (c0 + ct < n2) Yr[c1] = y[u][1];
-                  }
-                }
-              }
-#pragma unroll
-              for (int v = 0; v < 2; ++v) {
-                const int c = v ? c1 : c0;
-                if (v && c0 + ct >= n2) break;
-                double2 o12[4], o21[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                  o12[u] = old(ar[u] * nb + M + c);
-                  o21[u] = old((M + c) * nb + ar[u]);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                  if (a0 + u < M) {
-                    add(ar[u] * nb + M + c, o12[u], make_double2(widen(v12[u][v].x), widen(v12[u][v].y)));
-                    add((M + c) * nb + ar[u], o21[u], make_double2(widen(v21[u][v].x), widen(v21[u][v].y)));
-                  }
-              }
-            }
-            __syncthreads();
-            // (2,2): D + D (B^+ Y) in tiles of four rows and CW columns
-            auto tiles = [&](auto cw) {
-              constexpr int CW = decltype(cw)::value;
-              const int ctl = (n2 + CW - 1) / CW, ntl = ((n2 + 3) / 4) * ctl;
-              for (int i = tid; i < ntl; i += 32 * W) {
-                const int b0 = (i / ctl) * 4, c0 = (i - (i / ctl) * ctl) * CW;
-                float2 v[4][CW];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-#pragma unroll
-                  for (int w = 0; w < CW; ++w) v[u][w] = make_float2(0.f, 0.f);
-                for (int f = 0; f < nf; ++f) {
-                  float2 t[4][CW];
-#pragma unroll
-                  for (int u = 0; u < 4; ++u)
-#pragma unroll
-                    for (int w = 0; w < CW; ++w) t[u][w] = make_float2(0.f, 0.f);
-#pragma unroll 2
-                  for (int a = 0; a < M; ++a) {
-                    const float4* bp = reinterpret_cast<const float4*>(sB + a * pt + b0);
-                    const float4* yp = reinterpret_cast<const float4*>(sY + (size_t)(f * M + a) * pt + c0);
-                    const float4 b01 = bp[0], b23 = bp[1];
-                    const float2 b[4] = {{b01.x, b01.y}, {b01.z, b01.w}, {b23.x, b23.y}, {b23.z, b23.w}};
-                    float2 y[CW];
-#pragma unroll
-                    for (int w = 0; w < CW; w += 2) {
-                      const float4 q4 = yp[w / 2];
-                      y[w] = make_float2(q4.x, q4.y);
-                      y[w + 1] = make_float2(q4.z, q4.w);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-#pragma unroll
-                      for (int w = 0; w < CW; ++w) fmac_ca(t[u][w], b[u], y[w]);
-                  }
-#pragma unroll
-                  for (int u = 0; u < 4; ++u) {
-                    const float2 d = dlow(f0 + f, min(b0 + u, n2 - 1));
-#pragma unroll
-                    for (int w = 0; w < CW; ++w) fmac(v[u][w], t[u][w], d);
-                  }
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                  const int bb = b0 + u;
-                  if (bb >= n2) break;
-                  const int at = (M + bb) * nb + M;
-                  double2 o[CW];
-#pragma unroll
-                  for (int w = 0; w < CW; ++w) o[w] = old(at + min(c0 + w, n2 - 1));
-#pragma unroll
-                  for (int w = 0; w < CW; ++w) {
-                    if (c0 + w >= n2) break;
-                    float2 s = v[u][w];
-                    if (bb == c0 + w)
-                      for (int f = f0; f < f0 + nf; ++f) {
-                        const float2 d = dlow(f, bb);
-                        s.x += d.x;
-                        s.y += d.y;
-                      }
-                    add(at + c0 + w, o[w], make_double2(widen(s.x), widen(s.y)));
-                  }
-                }
-              }
-            };
-            // the wide tile only where it still gives every thread one
-            if (n2 > 40) tiles(std::integral_constant<int, 4>{});
-            else tiles(std::integral_constant<int, 2>{});
-            __syncthreads();
-          } else {
             const double2* Bk = bf.B + ki.offP;
             double2* sY = reinterpret_cast<double2*>(smraw + L.oY);
             // (1,2) and (2,1): Y = S^{-1} B D, Z = D B^+ S^{-1}
