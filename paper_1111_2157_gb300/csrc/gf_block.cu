@@ -401,8 +401,8 @@ __device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf
 // Then S, with LOW S^{-1} in FP32, d (or the series coefficients), the pivot tables, w_n, the pair
 // list, mu O - H11 by pairs and, with LOW, B.
 struct LayoutB {
-  size_t oS, oF, od2, orc, oM, oR, oY, oG, od, op, oW, oPair, oHz, oX, oB, bytes;
-  size_t sS, sF, sd2, src, sG, sR, sd, sp;  // bytes per warp (sS also of M)
+  size_t oS, oF, od2, orc, oM, oY, oG, od, op, oW, oPair, oHz, oX, oB, bytes;
+  size_t sS, sF, sd2, src, sG, sd, sp;  // bytes per warp (sS also of M)
   size_t fG;  // bytes of S^{-1} in FP32 per frequency
   int nf;   // frequencies per warp
   int yf;   // frequencies of the rho_k columns staged at once
@@ -432,10 +432,6 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   L.od2 = o; o += W * L.sd2;
   L.orc = o; o += W * L.src;
   L.oM = o; o += adj ? W * L.sS : 0;
-  // the refinement's residual: over M or F, of which one is not yet and one no longer in use
-  L.oR = adj ? L.oM : (needF ? L.oF : o);
-  L.sR = adj ? L.sS : L.sG;
-  if (low && (mode & kGloc) && !needF) o += W * L.sG;
   const size_t np = (size_t)mmax * (mmax + 1) / 2;
   const size_t fixed = W * (L.sG + L.sd + L.sp + (low ? 16 : 8) * f) + al(2 * np) + (low ? 32 : 16) * np +
                        (low && rho ? 16 * kp * pb + al(4 * (size_t)n2max) : 0);
@@ -470,8 +466,14 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
 __device__ __forceinline__ double2 ld_cg(const double2* p) { return __ldg(p); }
 __device__ __forceinline__ float2 ld_cg(const float2* p) { return __ldg(p); }
 
-template <int LW, bool LOW, bool ADJ>
-__global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
+// What an instance of the kernel holds beside S^{-1}: the traces, and rho_k or the adjoint.  G_loc
+// alone in FP32 pairs runs in 128 registers and less shared memory, four CTAs on an SM: 5.4 ms
+// instead of 6.2 (256 k-points x 1024 frequencies, 40 bands, 14 orbitals); with the traces the
+// shared memory leaves three, and fewer registers cost 9 %.
+enum { kGlocOnly, kPlain, kWithRho, kWithAdj };
+
+template <int LW, bool LOW, int PART>
+__global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 || PART == kGlocOnly ? 4 : 3)
     k_point_block(const PointParams p, const BlockForm bf, const BlockLaunch bl) {
   using rc_t = typename Rest<LOW>::c;
   using rr_t = typename Rest<LOW>::r;
@@ -486,7 +488,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
   double2* sd = reinterpret_cast<double2*>(smraw + L.od + wp * L.sd);
   rc_t* sd2 = reinterpret_cast<rc_t*>(smraw + L.od2 + wp * L.sd2);
   double2* sM = reinterpret_cast<double2*>(smraw + L.oM + wp * L.sS);
-  constexpr bool low_adj = LOW && ADJ;  // F and d^2 in pairs
+  constexpr bool low_adj = LOW && PART == kWithAdj;  // F and d^2 in pairs
   float2* sG = reinterpret_cast<float2*>(smraw + L.oG + wp * L.sG);
   int* sPv = reinterpret_cast<int*>(smraw + L.op + wp * L.sp);
   double* sW = reinterpret_cast<double*>(smraw + L.oW) + wp * F;
@@ -498,7 +500,8 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
   const int2 un = bl.units[unit];
   const int n0 = bl.n_begin + ch * bl.chunk_w, n1 = min(bl.n_end, n0 + bl.chunk_w);
   const int chunk = bl.chunk0 + ch;
-  const bool occ = (p.mode & kOcc) != 0, adj = ADJ, rho = !ADJ && (p.mode & kRho) != 0;
+  const bool occ = PART != kGlocOnly && (p.mode & kOcc) != 0;
+  constexpr bool adj = PART == kWithAdj, rho = PART == kWithRho;
 
   for (int q = 0; q < un.y; ++q) {
     const int kk = bl.kperm[un.x + q];
@@ -941,19 +944,25 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
           // at m = 20.
           const float4* Sp = reinterpret_cast<const float4*>(A);
           float2* X0 = sG + mf * (L.fG / sizeof(float2));
-          float2* R = reinterpret_cast<float2*>(smraw + L.oR + wp * L.sR) + mf * MM;
+          float2* R = reinterpret_cast<float2*>(A);  // over the rows of S that are done with
           const bool refine = (p.mode & (kGloc | kAdj)) != 0;
           if (refine) {
-            for (int i = sl; i < MM; i += LW) {
-              const int a = i / M, c = i - a * M, qc = sq[c];
+            // (LW entries of R take as many bytes as LW / 2 of S, and a round finishes more than that)
+            for (int i0 = 0; i0 < MM; i0 += LW) {
+              const int i = i0 + sl, a = i / M, c = i - a * M;
               cf acc = czero();
-              if (a == c) acc.rh = 1.f;
-              for (int x = 0; x < M; ++x) cacc1(acc, cneg(ld4(Sp[a * M + x])), X0[sp[x] * M + qc]);
-              R[i] = make_float2(__fadd_rn(acc.rh, acc.rl), __fadd_rn(acc.ih, acc.il));
+              if (i < MM) {
+                const int qc = sq[c];
+                if (a == c) acc.rh = 1.f;
+                for (int x = 0; x < M; ++x) cacc1(acc, cneg(ld4(Sp[a * M + x])), X0[sp[x] * M + qc]);
+              }
+              __syncwarp();
+              if (i < MM) R[i] = make_float2(__fadd_rn(acc.rh, acc.rl), __fadd_rn(acc.ih, acc.il));
             }
             __syncwarp();
           }
-          float2* Gn = reinterpret_cast<float2*>(A);  // (S is dead)
+          float2* Gn = R + MM;
+          float4* Ap = reinterpret_cast<float4*>(sM) + mf * MM;  // (adjoint)
           for (int i = sl; i < MM; i += LW) {
             const int a = i / M, c = i - a * M, pa = sp[a] * M;
             const float2 g = X0[pa + sq[c]];
@@ -963,7 +972,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
               for (int x = 0; x < M; ++x) fmac(d, X0[pa + sq[x]], R[x * M + c]);
               two_sum(g.x, d.x, h.x, l.x);
               two_sum(g.y, d.y, h.y, l.y);
-              if (adj) reinterpret_cast<float4*>(A)[i] = make_float4(h.x, l.x, h.y, l.y);
+              if (adj) Ap[i] = make_float4(h.x, l.x, h.y, l.y);
               else if (mine)
                 gq_put(&out[i], q, make_double2(wk * (widen(h.x) + widen(l.x)), wk * (widen(h.y) + widen(l.y))));
             }
@@ -987,9 +996,9 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 ? 4 : 3)
           const int rows = LW / M, ra = sl / M, rb = sl - ra * M;  // (rows >= 1: m <= LW)
           const int64_t gb0 = si.offSig + (int64_t)min(n + mf, n1 - 1) * MM;
           if constexpr (LOW) {
-            float4* Gh = reinterpret_cast<float4*>(sM) + mf * MM;
+            float4* Gh = reinterpret_cast<float4*>(A);  // (S is dead)
             const float4* Fm = reinterpret_cast<const float4*>(sF) + mf * MM;
-            const float4* Ap = reinterpret_cast<const float4*>(A);
+            const float4* Ap = reinterpret_cast<const float4*>(sM) + mf * MM;
             float ch, cl;
             split(cb, ch, cl);
             for (int i = sl; i < MM; i += LW) {
@@ -1386,21 +1395,24 @@ int reduce_grid(int nbmax, int mmax, int n_k, int smem_optin, int sm_count) {
   return std::max(1, std::min(n_k, sm_count * std::min(per_sm, 8)));
 }
 
-template <int LW, bool LOW, bool ADJ>
-cudaError_t launch_lw_adj(const PointParams& p, const BlockForm& b, const BlockLaunch& l, size_t smem, cudaStream_t s) {
+template <int LW, bool LOW, int PART>
+cudaError_t launch_part(const PointParams& p, const BlockForm& b, const BlockLaunch& l, size_t smem, cudaStream_t s) {
   cudaError_t e =
-      cudaFuncSetAttribute(k_point_block<LW, LOW, ADJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(k_point_block<LW, LOW, PART>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_point_block<LW, LOW, ADJ>, cudaFuncAttributePreferredSharedMemoryCarveout,
+  e = cudaFuncSetAttribute(k_point_block<LW, LOW, PART>, cudaFuncAttributePreferredSharedMemoryCarveout,
                            (int)cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
-  k_point_block<LW, LOW, ADJ><<<l.n_units * l.n_chunks, 32 * kBlkWarps, smem, s>>>(p, b, l);
+  k_point_block<LW, LOW, PART><<<l.n_units * l.n_chunks, 32 * kBlkWarps, smem, s>>>(p, b, l);
   return cudaGetLastError();
 }
 
 template <int LW, bool LOW>
 cudaError_t launch_lw(const PointParams& p, const BlockForm& b, const BlockLaunch& l, size_t smem, cudaStream_t s) {
-  return p.mode & kAdj ? launch_lw_adj<LW, LOW, true>(p, b, l, smem, s) : launch_lw_adj<LW, LOW, false>(p, b, l, smem, s);
+  if (p.mode & kAdj) return launch_part<LW, LOW, kWithAdj>(p, b, l, smem, s);
+  if (p.mode & kRho) return launch_part<LW, LOW, kWithRho>(p, b, l, smem, s);
+  if (LOW && !(p.mode & kOcc)) return launch_part<LW, LOW, LOW ? kGlocOnly : kPlain>(p, b, l, smem, s);
+  return launch_part<LW, LOW, kPlain>(p, b, l, smem, s);
 }
 
 }  // namespace
