@@ -51,7 +51,7 @@ constexpr double kBlkMinW = 1e-4;
 gf_status ensure_einf(gf_ctx* c) {
   if (!c->einf_dirty) return GF_OK;
   GF_CU(gf::launch_einf(c->kinfo_d.as<KInfo>(), c->sinfo_d.as<SInfo>(), c->H.as<double2>(),
-                        c->P.as<double2>(), c->Sinf.as<double2>(), c->n_k, c->Einf.as<double2>(),
+                        c->P.as<double2>(), c->Sinf.as<double2>(), c->n_k, c->nbmax, c->mmax, c->Einf.as<double2>(),
                         c->trHE.as<double>(), c->stream));
   c->last_launches += 1;
   c->einf_dirty = false;

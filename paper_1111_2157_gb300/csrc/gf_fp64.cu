@@ -419,14 +419,17 @@ __global__ void k_gq_reduce(const SInfo* __restrict__ sinfo, const int* __restri
 }
 
 // E_inf,k = P_k^+ Sigma_inf P_k and trHE_k = Re Tr(H_k + E_inf,k) (by trhe_partial).  One CTA
-// per k.
+// per k: Sigma_inf P_k for ct columns at a time in shared memory, then P_k^+ of it (256 k-points of
+// 40 bands and 14 orbitals: 0.08 ms; the product formed anew for every entry took 0.70).
 __global__ void __launch_bounds__(kThreads) k_einf(const KInfo* __restrict__ kinfo,
                                                    const SInfo* __restrict__ sinfo,
                                                    const double2* __restrict__ H,
                                                    const double2* __restrict__ P,
                                                    const double2* __restrict__ Sinf,
                                                    double2* __restrict__ Einf,
-                                                   double* __restrict__ trHE) {
+                                                   double* __restrict__ trHE, int ct) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* T = reinterpret_cast<double2*>(smem_raw);  // [m][ct]
   __shared__ double red[kThreads / 32];
   const int k = blockIdx.x;
   const KInfo ki = kinfo[k];
@@ -434,15 +437,22 @@ __global__ void __launch_bounds__(kThreads) k_einf(const KInfo* __restrict__ kin
   const int N = ki.nb, M = si.m;
   const double2* Pk = P + ki.offP;
   const double2* S = Sinf + si.offSinf;
-  for (int e = threadIdx.x; e < N * N; e += kThreads) {
-    const int i = e / N, j = e - i * N;
-    double2 v = make_double2(0.0, 0.0);
-    for (int a = 0; a < M; ++a) {
+  for (int j0 = 0; j0 < N; j0 += ct) {
+    const int w = min(ct, N - j0);
+    __syncthreads();
+    for (int e = threadIdx.x; e < M * w; e += kThreads) {
+      const int a = e / w, j = e - a * w;
       double2 t = make_double2(0.0, 0.0);
-      for (int b = 0; b < M; ++b) cmac(t, S[a * M + b], Pk[b * N + j]);
-      cmac_ca(v, Pk[a * N + i], t);
+      for (int b = 0; b < M; ++b) cmac(t, S[a * M + b], Pk[b * N + j0 + j]);
+      T[a * w + j] = t;
     }
-    Einf[ki.offH + e] = v;
+    __syncthreads();
+    for (int e = threadIdx.x; e < N * w; e += kThreads) {
+      const int i = e / w, j = e - i * w;
+      double2 v = make_double2(0.0, 0.0);
+      for (int a = 0; a < M; ++a) cmac_ca(v, Pk[a * N + i], T[a * w + j]);
+      Einf[ki.offH + (int64_t)i * N + j0 + j] = v;
+    }
   }
   const double t = block_sum(trhe_partial(H + ki.offH, Pk, S, N, M, threadIdx.x, kThreads), red);
   if (threadIdx.x == 0) trHE[k] = t;
@@ -532,8 +542,9 @@ cudaError_t launch_gq_reduce(const SInfo* sinfo, int n_sys, int max_mm_total, co
 }
 
 cudaError_t launch_einf(const KInfo* kinfo, const SInfo* sinfo, const double2* H, const double2* P,
-                        const double2* Sinf, int n_k, double2* Einf, double* trHE, cudaStream_t s) {
-  k_einf<<<n_k, kThreads, 0, s>>>(kinfo, sinfo, H, P, Sinf, Einf, trHE);
+                        const double2* Sinf, int n_k, int nbmax, int mmax, double2* Einf, double* trHE, cudaStream_t s) {
+  const int ct = std::min(nbmax, std::max(1, (int)(45056 / (sizeof(double2) * mmax))));
+  k_einf<<<n_k, kThreads, sizeof(double2) * mmax * ct, s>>>(kinfo, sinfo, H, P, Sinf, Einf, trHE, ct);
   return cudaGetLastError();
 }
 

@@ -369,7 +369,7 @@ cudaError_t launch_gq_reduce(const SInfo* sinfo, int n_sys, int max_mm_total, co
                              const int* sys_g1, const double2* gq, int gb0, int gb1, int n_iw,
                              int mmax, int first, double2* acc, cudaStream_t s);
 cudaError_t launch_einf(const KInfo* kinfo, const SInfo* sinfo, const double2* H, const double2* P,
-                        const double2* Sinf, int n_k, double2* Einf, double* trHE, cudaStream_t s);
+                        const double2* Sinf, int n_k, int nbmax, int mmax, double2* Einf, double* trHE, cudaStream_t s);
 cudaError_t launch_upcast(const float2* in, double2* out, int64_t n, cudaStream_t s);
 cudaError_t launch_diag_to_dense(const KInfo* kinfo, const double2* diag, const int64_t* offD,
                                  int n_k, double2* H, cudaStream_t s);
