@@ -167,12 +167,15 @@ gf_status ensure_block(gf_ctx* c) {
                                flags & gf::kBlkRankDeficient ? "P rank deficient" : "eigensolver") + "); ";
     return GF_OK;
   }
-  // mixed precision: frequencies w_n below a fifth of the rms eigenvalue of H run in FP64
-  // (an eigenvalue e_b within w_n of mu loses |B|^2 / w_n in FP32)
+  // mixed precision: frequencies w_n below a twentieth of the rms eigenvalue of H run in FP64, at
+  // least one batch (an eigenvalue e_b within w_n of mu loses |B|^2 / w_n in FP32).  Largest errors
+  // over windows of 20 to 96 bands, beta 40 to 400, mu on an e_b too: N 7e-9, dN/dmu 2.5e-7, rho_k
+  // 2e-8 (a fifth: 6e-9, 3e-8, 2e-8; the general kernels: 3e-7, 5e-5, 2e-6), and N(mu) of 256
+  // k-points x 1024 frequencies 1.4 ms (a fifth: 1.9).
   double h = 0.0, bmax = 0.0;
   for (int k = 0; k < c->n_k; ++k) h = std::max(h, info[k]);
   for (int s = 0; s < c->n_sys; ++s) bmax = std::max(bmax, c->beta[s]);
-  const double nc = std::ceil(0.5 * (0.2 * h * bmax / M_PI - 1.0));
+  const double nc = std::ceil(0.5 * (0.05 * h * bmax / M_PI - 1.0));
   const int batch = gf::block_batch(c->mmax);
   const int64_t up = (int64_t)std::min((double)c->n_iw, std::max(1.0, nc));
   c->blk_nc = mixed && !c->lowrank ? (int)std::min<int64_t>(c->n_iw, (up + batch - 1) / batch * batch) : c->n_iw;

@@ -420,7 +420,7 @@ __global__ void k_gq_reduce(const SInfo* __restrict__ sinfo, const int* __restri
 
 // E_inf,k = P_k^+ Sigma_inf P_k and trHE_k = Re Tr(H_k + E_inf,k) (by trhe_partial).  One CTA
 // per k: Sigma_inf P_k for ct columns at a time in shared memory, then P_k^+ of it (256 k-points of
-// 40 bands and 14 orbitals: 0.08 ms; the product formed anew for every entry took 0.70).
+// 40 bands and 14 orbitals: 0.09 ms; the product formed anew for every entry took 0.70).
 __global__ void __launch_bounds__(kThreads) k_einf(const KInfo* __restrict__ kinfo,
                                                    const SInfo* __restrict__ sinfo,
                                                    const double2* __restrict__ H,
