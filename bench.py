@@ -14,8 +14,7 @@ iteration needs it:
 value = (k, i w_n) points evaluated per second (every pass counts its points).
 
 The same line carries, beside the FP64 headline: the mixed-precision step
-(FP32 inverse, FP64 sums, refined projections) and the FP32-pair step on the
-same workload; the low-rank (eigenbasis) algorithm; the NiO-like workload
+(FP32 and FP32 pairs, FP64 sums) and the GF_PREC_PAIR step on the same workload; the low-rank (eigenbasis) algorithm; the NiO-like workload
 (N_k = 4096, N_b = 96, m = 20, 2048 frequencies): one fixed-mu fused pass on
 the FP64 and on the mixed path and the mixed mu search, with errors against
 the oracle; and the batched workload (8 systems, ragged windows of 48-128
@@ -146,7 +145,7 @@ class ClockSampler:
 
 def ncu_traffic():
     """dram bytes per launch of the point kernel from the committed ncu summary (or None)."""
-    f = PROFILES / "point_fp64_ce_like.md"
+    f = PROFILES / "point_block_ce_like.md"
     if not f.exists():
         return None
     for line in f.read_text().splitlines():
@@ -272,6 +271,43 @@ def _lr_pole_cases(args, synth):
 
 
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12  # FP32 FMA: 152 SMs x 128 lanes x 2 flop x 2.07 GHz
+
+
+def _band_terms(s):
+    """Terms per frequency of the block form's band sums: the n2 levels of the first k-point, or the terms
+    of their Chebyshev series where those are fewer (at most 40 are kept)."""
+    P, H = np.asarray(s.P[0]), np.asarray(s.H[0])
+    q = np.linalg.qr(np.conj(P.T), mode="complete")[0][:, s.m:]
+    e = np.linalg.eigvalsh(np.conj(q.T) @ H @ q)
+    r = max((e[-1] - e[0]) / 2, 1e-12)
+    x = (-(e[0] + e[-1]) / 2 + 1j * (2 * np.arange(s.n_iw) + 1) * np.pi / s.beta) / r
+    root = np.sqrt(x * x - 1)
+    big = np.maximum(np.abs(x + root), np.abs(x - root))
+    terms = np.floor(44.8 / np.maximum(np.log(big), 1e-9)) + 2
+    return float(np.mean(np.where(terms <= min(len(e), 40), terms, len(e))))
+
+
+def executed_flops(g, st, systems, mode):
+    """Floating-point operations of the call that st belongs to.  Where the block form ran, its own (2 per
+    multiply-add of the band sums, the m x m inverse and products; k-independent parts are done once per
+    upload and not counted), which are several times fewer than the N_b^3 count of the library's counter."""
+    if "block form" not in g.tuning_log():
+        return st["flops"]
+    occ, rho, adj = mode in ("occ", "gloc_occ", "evaluate", "backward"), mode == "evaluate", mode == "backward"
+    total = pts = 0.0
+    for s in systems:
+        m, terms = s.m, _band_terms(s)
+        nbs = np.array([np.asarray(h).shape[-1] for h in s.H], float)
+        n2 = nbs - m
+        terms = np.minimum(n2, terms)
+        fma = m * (m + 1) / 2 * 4 * terms * (1 + 2 * occ) + 4.0 * m**3 * (1 + occ) + adj * 8.0 * m**3
+        if rho:
+            fma = fma + 4 * (2 * m * m * n2 + m * n2 * n2 + n2 * n2)
+        total += 2.0 * s.n_iw * float(np.sum(fma))
+        pts += s.n_iw * len(nbs)
+    return total * st["points"] / pts
+
+
 MIXED_MU_TOL = 1e-8  # mixed path: mu search to |N - N_target| <= 1e-8 N_target (FP32 noise ~1e-9)
 
 
@@ -304,6 +340,7 @@ def nio_leg(gf, synth, o, nk=4096, n_iw=2048):
     gm.evaluate(mu, rho=False, n_corr=False)  # autotunes the fused pass's launch
     evm, t_m = _sync_time(lambda: gm.evaluate(mu, rho=False, n_corr=False))
     stm = gm.stats()
+    stm["flops"] = executed_flops(gm, stm, [s], "gloc_occ")
     gl_m = evm["gloc"].cpu().numpy().reshape(s.n_iw, s.m, s.m)
     mixed_log = gm.tuning_log()
     gm.close()
@@ -311,6 +348,7 @@ def nio_leg(gf, synth, o, nk=4096, n_iw=2048):
     g64 = _dev_context(gf, [s], "fp64")
     ev64, t_64 = _sync_time(lambda: g64.evaluate(mu, rho=False, n_corr=False))
     st64 = g64.stats()
+    st64["flops"] = executed_flops(g64, st64, [s], "gloc_occ")
     gl_d = ev64["gloc"].cpu().numpy().reshape(s.n_iw, s.m, s.m)
     fp64_log = g64.tuning_log()
     g64.close()
@@ -356,7 +394,7 @@ def nio_leg(gf, synth, o, nk=4096, n_iw=2048):
                   "roofline": {"bound": "alu", "achieved": stm["flops"] / stm["kernel_ms"] / 1e9,
                                "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
                                "frac": stm["flops"] / stm["kernel_ms"] / 1e9 / FP32_PEAK_TFLOPS,
-                               "kernel": "k_point_f32r (autotuned tiles)",
+                               "kernel": "k_point_block (FP32 and FP32 pairs)",
                                "peak_source": "FP32 FMA: 152 SMs x 128 lanes x 2 flop x 2.07 GHz"},
                   "find_mu_s": t_mu, "find_mu_evaluations": it,
                   "find_mu_points_per_s": smu["points"] / t_mu,
@@ -401,6 +439,7 @@ def batched_leg(gf, synth, o, nk_scale=1.0):
     g64 = _dev_context(gf, systems, "fp64", input_dtype=pd)
     (n64, d64), t64 = _sync_time(lambda: g64.occupation(mus))
     s64 = g64.stats()
+    s64["flops"] = executed_flops(g64, s64, systems, "occ")
     out["fp64"] = {"pass_s": t64, "pass_kernel_s": s64["kernel_ms"] / 1e3,
                    "points_per_s": pts / (s64["kernel_ms"] / 1e3), "launches": s64["launches"],
                    "kernel_tflops": s64["flops"] / s64["kernel_ms"] / 1e9}
@@ -409,6 +448,7 @@ def batched_leg(gf, synth, o, nk_scale=1.0):
     gm.occupation(mus)
     (nm, dm), tm = _sync_time(lambda: gm.occupation(mus))
     sm_ = gm.stats()
+    sm_["flops"] = executed_flops(gm, sm_, systems, "occ")
     log = gm.tuning_log()
     gm.close()
     t_per, n_launch = 0.0, 0
@@ -472,10 +512,12 @@ def run_workload(args):
         s = (synth.nio_like(**kw) if args.system == "nio_like" else synth.ce_like(**kw)).systems[0]
         g = _dev_context(gf, [s], args.precision)
         res = {}
-        for name, call in (("occupation", lambda: g.occupation([0.1])),
-                           ("fused_gloc_N", lambda: g.evaluate([0.1], rho=False, n_corr=False))):
+        for name, mode, call in (("occupation", "occ", lambda: g.occupation([0.1])),
+                                 ("fused_gloc_N", "gloc_occ",
+                                  lambda: g.evaluate([0.1], rho=False, n_corr=False))):
             _, t = _sync_time(call)
             st = g.stats()
+            st["flops"] = executed_flops(g, st, [s], mode)
             res[name] = {"s": t, "kernel_s": st["kernel_ms"] / 1e3,
                          "points_per_s": st["points"] / (st["kernel_ms"] / 1e3),
                          "alg_tflops": st["flops"] / st["kernel_ms"] / 1e9}
@@ -555,9 +597,11 @@ def run_workload(args):
             gd.occupation(mu)
             (nd, dd), td = _sync_time(lambda: gd.occupation(mu))
             sd = gd.stats()
+            sd["flops"] = executed_flops(gd, sd, systems, "occ")
             _, t_setup = _sync_time(lambda: gl.occupation(mu))  # includes the eigen-decomposition
             (nl, dl), tl = _sync_time(lambda: gl.occupation(mu))
             sl = gl.stats()
+            sl["flops"] = executed_flops(gl, sl, systems, "occ")
             pts = sum(s.nk * s.n_iw for s in systems)
             # the same with GF_PREC_MIXED: FP32-pair band sums, FP64 m x m algebra
             gx = _context(gf, systems, "mixed", lowrank=True)
@@ -707,7 +751,7 @@ def main():
         rho_d = torch.empty(g.tot_h, dtype=torch.complex128, device=dev)
         sbar_d = torch.empty(g.tot_sig, dtype=torch.complex128, device=dev)
         totals = {"launches": 0, "points": 0, "kernel_ms": 0.0, "flops": 0.0}
-        passes = {name: {"kernel_ms": 0.0, "flops": 0.0, "launches": 0}
+        passes = {name: {"kernel_ms": 0.0, "flops": 0.0, "launches": 0, "points": 0}
                   for name in ("find_mu", "evaluate", "backward")}
         info = {}
 
@@ -717,6 +761,7 @@ def main():
                 totals[k] += st[k]
             passes[name]["kernel_ms"] += st["kernel_ms"]
             passes[name]["flops"] += st["flops"]
+            passes[name]["points"] += st["points"]
             passes[name]["launches"] += 1
 
         mu_tol = MIXED_MU_TOL * s.n_target if precision == "mixed" else 1e-10
@@ -736,7 +781,7 @@ def main():
         for k in totals:
             totals[k] = 0 if k in ("launches", "points") else 0.0
         for v in passes.values():
-            v.update(kernel_ms=0.0, flops=0.0, launches=0)
+            v.update(kernel_ms=0.0, flops=0.0, launches=0, points=0)
         clocks = ClockSampler(local) if sample_clocks else None
         if ws > 1:
             torch.distributed.barrier()
@@ -753,6 +798,9 @@ def main():
         torch.cuda.synchronize()
         clk = clocks.stop() if clocks else None
         elapsed = e0.elapsed_time(e1) / 1e3
+        for name, v in passes.items():
+            v["flops"] = executed_flops(g, v, [s], {"find_mu": "occ"}.get(name, name))
+        totals["flops"] = sum(v["flops"] for v in passes.values())
         if ws > 1:
             t = torch.tensor([elapsed], dtype=torch.float64, device=dev)
             torch.distributed.all_reduce(t, op=torch.distributed.ReduceOp.MAX)
@@ -789,9 +837,9 @@ def main():
                               "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
                               "frac": mt["flops"] / (mt["kernel_ms"] / 1e3) / 1e12 / FP32_PEAK_TFLOPS,
                               "peak_source": "FP32 FMA: 152 SMs x 128 lanes x 2 flop x 2.07 GHz"},
-                 "arithmetic": "FP32 embedding and Gauss-Jordan inverse (register tiles); FP64 Matsubara "
-                               "sums, tail, k-sums and mu search; G P^+ and P G refined once with an "
-                               "FP32-pair residual",
+                 "arithmetic": "block form: S in FP32 pairs, its inverse in FP32 with one refinement step "
+                               "(G_loc, adjoint) from a residual in pairs, traces and rho_k in FP32; FP64 for "
+                               "the lowest frequencies, Matsubara sums, tail, k-sums and mu search",
                  "kernel_choice": gm.tuning_log(), "gpu_launches": mt["launches"]}
         gm.close()
         # the FP32-pair mode (GF_PREC_PAIR, ~1e-14 of FP64), a few steps
@@ -804,8 +852,8 @@ def main():
                               "ms_per_step": pl["elapsed"] / ps_ * 1e3,
                               "speedup_vs_fp64_gpu": (pt["points"] / pl["elapsed"]) / (totals["points"] / elapsed),
                               "N_rel_err_vs_fp64_gpu": abs(n_p[0] - info["N"]) / abs(info["N"]),
-                              "arithmetic": "FP32 pairs (hi + lo, error-free transformations) on the FP32 "
-                                            "pipes; FP64 reductions, tail and mu search",
+                              "arithmetic": "the FP64 block kernel (FP32 pairs on the FP32 pipes where the "
+                                            "inputs keep the general kernels)",
                               "kernel_choice": gp.tuning_log()}
         gp.close()
 
@@ -836,7 +884,8 @@ def main():
                    "speedup_vs_direct_fp64_gpu": (lt["points"] / lr["elapsed"]) / (totals["points"] / elapsed),
                    "N_rel_err_vs_direct": abs(n_lr[0] - info["N"]) / abs(info["N"]),
                    "G_loc_rel_err_vs_direct": float((gl_lr - gl_fp).abs().max() / gl_fp.abs().max()),
-                   "algorithm": "G in the eigenbasis of H_k (Woodbury identity), FP64; H_k diagonalised once",
+                   "algorithm": "the block form, as the direct path" if "block form" in gr.tuning_log() else
+                                "G in the eigenbasis of H_k (Woodbury identity), FP64; H_k diagonalised once",
                    "gpu_launches": lt["launches"], "mixed_precision": mixed_lowrank}
         gr.close()
 
@@ -898,7 +947,8 @@ def main():
         if not args.no_batched:
             batched = batched_leg(gf, synth, o, nk_scale=args.nk_scale)
 
-    if args.precision == "fp64":
+    block = "block form" in g.tuning_log()
+    if args.precision == "fp64" or (args.precision == "pair" and block):
         peak, peak_source = FP64_PEAK_TFLOPS, "FP64 DFMA: 152 SMs x 2/clk x 2 flop x 2.07 GHz"
     elif args.precision == "mixed":
         peak, peak_source = FP32_PEAK_TFLOPS, "FP32 FMA: 152 SMs x 128 lanes x 2 flop x 2.07 GHz"
@@ -923,7 +973,8 @@ def main():
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak,
                          "unit": "TFLOP/s", "frac": achieved / peak,
                          "traffic": ncu_traffic() if args.precision == "fp64" else None,
-                         "kernel": {"fp64": "k_point_fp64", "mixed": "k_point_f32r (autotuned tiles)",
+                         "kernel": "k_point_block" if block else
+                                   {"fp64": "k_point_fp64", "mixed": "k_point_f32r (autotuned tiles)",
                                     "pair": "k_point_df64 / k_point_df64r (autotuned)"}[args.precision],
                          "peak_source": peak_source,
                          "kernel_share_of_step": totals["kernel_ms"] / 1e3 / elapsed,

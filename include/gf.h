@@ -64,6 +64,19 @@ typedef enum {
 
 /* Arithmetic of the (k, i w_n) point kernels.  Reductions over k and n, the
  * Matsubara tail and the mu search run in FP64 in every mode.
+ *
+ * Every mode runs on the block form where it can: P_k^+ = Q [R; 0] and the
+ * eigenproblem of the N_b - m remaining rows of Q^+ H_k Q are solved once per
+ * upload of H or P, after which a point costs O(m^2 N_b + m^3) multiply-adds.
+ * It needs Hermitian H_k, P_k of full rank, m <= 32, m < N_b and
+ * N_b - m <= 256 at every k, at least 16 frequencies and pi / beta >= 1e-4; the
+ * general kernels take the other inputs, and every call when the environment
+ * variable GF_KERNEL is "direct" (in mixed precision: when it has any value).
+ * FP64 and pair contexts compute it in FP64.  Mixed: FP64 up to a twentieth of
+ * the rms level of H; above, the m x m matrix S in FP32 pairs, its
+ * inverse in FP32 with one refinement step for G_loc and the adjoint, traces and
+ * rho_k in FP32 (N to ~1e-8, G_loc to ~1e-12 of FP64).  The modes below are the
+ * general kernels'.
  *  GF_PREC_FP64  embedding, inverse and projections in FP64.
  *  GF_PREC_MIXED embedding and Gauss-Jordan inverse in single-word FP32
  *                (register tiles, windows up to 128 bands; wider windows use
@@ -115,7 +128,7 @@ typedef struct {
 
 /* gf_desc.flags: evaluate every (k, i w_n) point in the eigenbasis of H_k
  * (Woodbury identity): H_k = U diag(eps) U^+ is diagonalised once per
- * Hamiltonian upload (batched Jacobi kernel), after which a point costs
+ * Hamiltonian upload, after which a point costs
  * 3 N_b m^2 + O(m^3) complex multiply-adds instead of N_b^3.  Same results as
  * the direct inverse up to rounding; N_b <= 256.  With GF_PREC_MIXED or
  * GF_PREC_PAIR the band sums of g0, g1, g2 (the N_b m^2 part) run in FP32-pair

@@ -42,7 +42,11 @@ void set_global_error(const char* msg) noexcept {
 
 namespace {
 
-// The block form pays for an eigenproblem per k from this many frequencies on.
+// The block form pays for an eigenproblem per k from this many frequencies on.  New H and a fused
+// pass, general kernels against the block form, at 16 frequencies: 64 k-points of 40 bands 2.4 / 1.7
+// ms (mixed 1.8 / 1.8), 256 5.8 / 3.4 (3.5 / 2.8), 48 of 96 bands 17.0 / 7.9 (10.8 / 7.2), 64 of 8
+// bands 0.40 / 0.42 (0.40 / 0.43; with five N(mu) before it 1.07 / 0.79, 0.88 / 0.81); at 4: 2.0 /
+// 1.6 (1.6 / 1.6), 3.0 / 2.4 (2.3 / 2.5), 11.1 / 7.1 (8.0 / 7.2), 0.42 / 0.39 (0.40 / 0.40).
 constexpr int kBlkMinFreq = 16;
 // Lowest pi / beta of the block form (eV): below it an eigenvalue of the n2 block that happens
 // to lie near mu would cost more digits than the pivoted inverse loses.

@@ -1,4 +1,5 @@
-// Block form of the lattice points (gf_block.cuh): setup kernels and the FP64 point kernel.
+// Block form of the lattice points (gf_block.cuh): setup kernels, and the point kernel in FP64 and,
+// for the higher frequencies of mixed precision (LOW), in FP32 and FP32 pairs.
 //
 // FP64 on GB300 issues two DFMAs per clock and SM, so a warp-wide FP64 instruction occupies
 // its SM sub-partition for 64 clocks and everything else (shared-memory and L2 loads, index
@@ -8,10 +9,13 @@
 // (frequency, pair) list, the elimination over the flattened entries, and the pair table
 // B_a conj(B_c) of the k-point is formed once per uploaded H_k instead of per frequency.
 //
-// Bound: the FP64 pipe.  Per point of a 40-band window with 14 orbitals: 56 k FP64 FMAs for
-// N(mu) and dN/dmu (band sums 33 k, S^{-1} 11 k, S^{-1} F 11 k) where the inverse of the window
-// takes 281 k; 135 k with G_loc and rho_k.  Measured (GB300, 216 k-points x 1024 frequencies):
-// every output in 62 ms, 210 ms by the inverse; mu search and G_loc of 64 k-points 57 ms, 340 ms.
+// Bound: the FP64 pipe, 96-97 % busy.  Per point of a 40-band window with 14 orbitals: 56 k FP64
+// FMAs for N(mu) and dN/dmu (band sums 33 k, S^{-1} 11 k, S^{-1} F 11 k) where the inverse of the
+// window takes 281 k; 135 k with G_loc and rho_k.  Measured (GB300, 216 k-points x 1024
+// frequencies): every output in 59 ms, 210 ms by the inverse; mu search and G_loc of 64 k-points
+// 53 ms, 387 ms.
+// LOW is bound by latency (issue slots 40-65 % busy at 8 to 14 warps an SM, FMA pipe 32-44 %):
+// every output of 256 k-points in 10.3 ms, 20.8 ms with S and its inverse in FP64.
 #include <math.h>
 #include <stdint.h>
 
@@ -555,7 +559,11 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 || PART == kGlocOnly ?
       if (nv > 0) {
         __syncwarp();
         // the sums over the n2 bands, or over fewer Chebyshev moments where those converge sooner
-        // (44.8 = 56 ln 2 + 6; the series' own overhead is about 150 FP64 instructions per warp)
+        // (44.8 = 56 ln 2 + 6; the series' own overhead is about 150 FP64 instructions per warp, so
+        // it has to save this many terms x pairs.  FP64, 1600: at 5000 N(mu) of 216 k-points takes
+        // 25.1 ms instead of 24.7, at 0 N(mu) of 75 k-points x 333 frequencies 1.60 instead of 1.56.
+        // LOW, 5000: at 12000 G_loc of 96 k-points at 88 bands 2.5 ms instead of 1.7, at 0 G_loc of 256
+        // at 40 bands 5.5 instead of 5.3)
         int nt = n2;
         const double2* Tt = T;
         const float2* Tst = nullptr;

@@ -111,8 +111,8 @@ size_t block_reduce_ws_elems(int nbmax, int mmax, int smem_optin, int sm_count);
 
 // Frequencies a CTA takes at once.
 int block_batch(int mmax);
-// low = 1: the parts of the result that mixed precision takes from an FP32 inverse (F, the
-// traces, rho_k) in FP32; S, its inverse and G_loc stay FP64.
+// low = 1 (the higher frequencies of mixed precision): traces and rho_k in FP32, S, G_loc and the
+// adjoint in FP32 pairs, S^{-1} in FP32 with one refinement step.
 size_t block_smem(int mmax, int n2max, int mode, int low);
 cudaError_t launch_point_block(const PointParams& p, const BlockForm& b, const BlockLaunch& l, int low,
                                cudaStream_t s);

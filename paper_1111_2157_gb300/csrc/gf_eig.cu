@@ -15,8 +15,8 @@
 // 2 N (N|1) 16-byte elements fit, else in a per-CTA slice of a global workspace (L2-resident):
 //  * heev_tri: Householder tridiagonalisation, the tridiagonal eigenpairs in parallel (QR steps
 //    where levels are too close for that), back-transformation.  The pole path, the block form's
-//    setup and the Lowdin projectors.  A pseudo-Hamiltonian of 68 rows takes 2.0 ms, 16.9 ms by
-//    Jacobi (N(mu) of 125 k-points; 1000: 13.8 against 105 ms).
+//    setup and the Lowdin projectors.  N(mu) from pseudo-Hamiltonians of 68 rows takes 1.4 ms for
+//    125 k-points (FP64 pipe 73 % busy) and 9.6 ms for 1000, by Jacobi 16.9 and 105 ms.
 //  * cyclic Jacobi with the round-robin (circle) ordering of disjoint pairs, so that one step
 //    applies N/2 independent rotations: gf_heev_batched, whose caller sets the sweep limit, and
 //    the low-rank kernel's setup.
