@@ -401,9 +401,9 @@ __device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf
 // Shared memory of the point kernel in bytes; every array holds the CTA's W F frequencies, warp
 // after warp.  First what is dead once the warps have S^{-1}: F, d^2 / d^3, the pivot row and
 // column, Gbar A^+ (adjoint), and with LOW also S and the refinement's residual (rho_k then reads
-// S^{-1} in FP32); the columns S^{-1} B D of rho_k are staged over it, yf frequencies at a time.
-// Then S, with LOW S^{-1} in FP32, d (or the series coefficients), the pivot tables, w_n, the pair
-// list, mu O - H11 by pairs and, with LOW, B.
+// S^{-1} in FP32); with LOW B, and the columns S^{-1} B D of rho_k are staged over it, yf frequencies
+// at a time.  Then S, with LOW S^{-1} in FP32, d (or the series coefficients), the pivot tables, w_n,
+// the pair list and mu O - H11 by pairs.
 struct LayoutB {
   size_t oS, oF, od2, orc, oM, oY, oG, od, op, oW, oPair, oHz, oX, oB, bytes;
   size_t sS, sF, sd2, src, sG, sd, sp;  // bytes per warp (sS also of M)
@@ -438,15 +438,18 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   L.oM = o; o += adj ? W * L.sS : 0;
   const size_t np = (size_t)mmax * (mmax + 1) / 2;
   const size_t fixed = W * (L.sG + L.sd + L.sp + (low ? 16 : 8) * f) + al(2 * np) + (low ? 32 : 16) * np +
-                       (low && rho ? 16 * kp * pb + al(4 * (size_t)n2max) : 0);
+                       (low && rho ? al(4 * (size_t)n2max) : 0);
+  const size_t sB = low && rho ? 16 * kp * pb : 0;
+  L.oB = L.oY;
+  L.oY += sB;
   L.yf = 0;
   if (rho) {
     // as many frequencies as fit over the dead arrays, or as leave three CTAs on an SM, or two:
     // the chunk's sum is read and written once per stage
     const size_t one = 16 * (low ? kp : mmax) * (size_t)n2max;
     const size_t all = f * W;
-    size_t room = o - L.oY;
-    for (size_t lim = 74u << 10; lim <= (112u << 10); lim += 38u << 10)
+    size_t room = o > L.oY ? o - L.oY : 0;
+    for (size_t lim = (75u << 10) - 128; lim < (113u << 10); lim += 38u << 10)  // (and 128 B of static arrays)
       if (room < all * one && L.oY + fixed + (room > one ? room : one) <= lim) {
         room = lim - L.oY - fixed;
         break;
@@ -462,7 +465,6 @@ __host__ __device__ inline LayoutB make_layout_b(int mmax, int n2max, int mode, 
   L.oPair = o; o += al(2 * np);
   L.oHz = o; o += (low ? 32 : 16) * np;  // (low: pairs of mu O - H11, then of O)
   L.oX = o; o = al(o + (low && rho ? 4 * (size_t)n2max : 0));
-  L.oB = o; o += low && rho ? 16 * kp * pb : 0;
   L.bytes = o;
   return L;
 }
@@ -538,17 +540,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 || PART == kGlocOnly ?
     }
     if constexpr (LOW) {
       if (rho) {
-        // B by pairs of rows, {Re, Re, Im, Im}; 0 beyond M and n2
-        float4* sB = reinterpret_cast<float4*>(smraw + L.oB);
-        const int pb = (n2 + 3) & ~3;
-        const float2* Bk = bf.Bs + ki.offP;
         for (int i = tid; i < n2; i += 32 * W) xs[i] = __double2float_rn(mu - e_k[i]);
-        for (int i = tid; i < (M + 1) / 2 * pb; i += 32 * W) {
-          const int x = i / pb * 2, b = i % pb;
-          const float2 zero = make_float2(0.f, 0.f);
-          const float2 u = b < n2 ? Bk[x * n2 + b] : zero, v = b < n2 && x + 1 < M ? Bk[(x + 1) * n2 + b] : zero;
-          sB[i] = make_float4(u.x, v.x, u.y, v.y);
-        }
       }
     }
     __syncthreads();
@@ -1097,6 +1089,23 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 || PART == kGlocOnly ?
         auto dof = [&](int f) { return reinterpret_cast<const double2*>(smraw + L.od + (f / F) * L.sd) + (f % F) * n2; };
         const bool first = (base == n0);
         __syncthreads();
+        if constexpr (LOW) {
+          // B by pairs of rows, {Re, Re, Im, Im}, 0 beyond M and n2: over the dead arrays like Y, anew
+          // for each batch (12 KB from L2 for 4 frequencies at 76 levels and 20 orbitals), since the
+          // room it would hold costs the third CTA on an SM: 14.1 -> 12.7 ms for every output of 48
+          // k-points x 2048 frequencies at 96 bands
+          float4* sB = reinterpret_cast<float4*>(smraw + L.oB);
+          const int pb = (n2 + 3) & ~3;
+          const float2* Bk = bf.Bs + ki.offP;
+          for (int i = tid; i < (M + 1) / 2 * pb; i += 32 * W) {
+            const int x = i / pb * 2, b = i % pb;
+            const float2 zero = make_float2(0.f, 0.f);
+            const float2 u = b < n2 ? __ldg(Bk + x * n2 + b) : zero;
+            const float2 v = b < n2 && x + 1 < M ? __ldg(Bk + (x + 1) * n2 + b) : zero;
+            sB[i] = make_float4(u.x, v.x, u.y, v.y);
+          }
+          __syncthreads();
+        }
         for (int f0 = 0; f0 < tot; f0 += L.yf) {
           const int nf = min(L.yf, tot - f0);
           const bool put = first && f0 == 0;
