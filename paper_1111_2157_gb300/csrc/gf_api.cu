@@ -1150,17 +1150,20 @@ gf_status init_ctx(gf_ctx* c, const gf_desc* d) {
   std::vector<int2> units;
   std::vector<int> perm(2 * (size_t)c->n_k), bsysg;
   if (c->blk_shape) {
-    // chunks: whole batches of a CTA, about eight CTAs per resident one; k-groups: about six.
-    // (the FP32 N(mu) kernel's batch is a multiple of the FP64 one's)
+    // chunks: whole batches of a CTA, about 16 CTAs per resident one; k-groups: about 12 (the FP32
+    // N(mu) kernel's batch is a multiple of the FP64 one's).  Half as many leave a longer last wave:
+    // G_loc of 256 k-points of 40 bands in mixed precision 5.3 instead of 5.1 ms, every output of 48
+    // of 96 bands 12.7 instead of 12.2, N(mu) of 32 of 64 bands in FP64 4.5 instead of 4.2; twice as
+    // many gain nothing, and 32 cost N(mu) of 96 of 88 bands in mixed precision 0.76 instead of 0.48.
     const double res = 3.0 * c->sm_count, pts = (double)c->n_k * c->n_iw;
-    double batch = gf::block_batch(c->mmax), w = std::ceil(pts / (8.0 * res) / batch) * batch;
+    double batch = gf::block_batch(c->mmax), w = std::ceil(pts / (16.0 * res) / batch) * batch;
     if (c->precision == GF_PREC_MIXED && w > batch) {
       batch = gf::block32_batch(c->mmax);
       w = std::ceil(w / batch) * batch;
     }
     c->blk_cw = (int)std::min(std::max(batch, w), std::ceil((double)c->n_iw / batch) * batch);
     const int nch = (c->n_iw + c->blk_cw - 1) / c->blk_cw;
-    c->blk_kg = (int)std::max(1.0, std::min((double)gf::kMaxKGroup, std::floor((double)c->n_k * nch / (6.0 * res))));
+    c->blk_kg = (int)std::max(1.0, std::min((double)gf::kMaxKGroup, std::floor((double)c->n_k * nch / (12.0 * res))));
     c->blk_sys_g0.assign(c->n_sys, 0);
     c->blk_sys_g1.assign(c->n_sys, 0);
     for (int s = 0; s < c->n_sys; ++s) {
