@@ -13,14 +13,22 @@ using namespace cx;
 // Lanes per matrix for m orbitals (m <= 32).
 __host__ __device__ inline int lanes(int m) { return m <= 8 ? 8 : (m <= 16 ? 16 : 32); }
 
-// 1 / a with one reciprocal: scaled by a power of two near 1 / max(|Re|, |Im|) (bit arithmetic),
-// so that the squared modulus neither overflows nor underflows.
+// x 2^k by integer arithmetic on the exponent (a product would hold the FP64 pipe); results below the
+// normal range become 0, infinity and NaN stay.
+__device__ __forceinline__ double scale2(double x, int k) {
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff, n = e + k;
+  if (e == 0x7ff) return x;
+  if (e == 0 || n <= 0) return __hiloint2double(hi & (int)0x80000000, 0);
+  if (n >= 0x7ff) return __hiloint2double((hi & (int)0x80000000) | 0x7ff00000, 0);
+  return __hiloint2double(hi + k * 0x100000, __double2loint(x));
+}
+
+// 1 / a with one reciprocal: scaled by a power of two near 1 / max(|Re|, |Im|), so that the squared
+// modulus, of [1, 8), neither overflows nor underflows.
 __device__ __forceinline__ double2 crcp_scaled(double2 a, unsigned long long key) {
-  int ex = 2046 - (int)(key >> 52);
-  ex = ex < 1 ? 1 : ex;
-  const double s = __longlong_as_double((long long)ex << 52);
-  const double x = a.x * s, y = a.y * s;
-  const double q = s * rcp_newton(fma(x, x, y * y));  // of [1, 8)
+  const int k = 1023 - max((int)(key >> 52), 1);
+  const double x = scale2(a.x, k), y = scale2(a.y, k);
+  const double q = scale2(rcp_newton(fma(x, x, y * y)), k);
   return make_double2(x * q, -y * q);
 }
 
