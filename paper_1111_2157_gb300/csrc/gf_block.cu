@@ -12,10 +12,10 @@
 // Bound: the FP64 pipe, 96-97 % busy.  Per point of a 40-band window with 14 orbitals: 56 k FP64
 // FMAs for N(mu) and dN/dmu (band sums 33 k, S^{-1} 11 k, S^{-1} F 11 k) where the inverse of the
 // window takes 281 k; 135 k with G_loc and rho_k.  Measured (GB300, 216 k-points x 1024
-// frequencies): every output in 59 ms, 210 ms by the inverse; mu search and G_loc of 64 k-points
-// 53 ms, 387 ms.
-// LOW is bound by latency (issue slots 40-65 % busy at 8 to 14 warps an SM, FMA pipe 32-44 %):
-// every output of 256 k-points in 10.3 ms, 20.8 ms with S and its inverse in FP64.
+// frequencies): every output in 58.7 ms, 210 ms by the inverse; mu search and G_loc of 64 k-points
+// 50 ms, 340 ms.
+// LOW is bound by latency (issue slots 50-65 % busy at 11 to 14 warps an SM, FMA pipe 37-44 %):
+// every output of 256 k-points in 10.2 ms, 20.8 ms with S and its inverse in FP64.
 #include <math.h>
 #include <stdint.h>
 
