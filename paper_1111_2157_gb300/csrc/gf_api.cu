@@ -827,12 +827,13 @@ gf_status occupation_impl(gf_ctx* c, const double* mu, double* n_out, double* dn
   gf_status st = check_ready(c);
   if (st) return st;
   if (c->use_graph) {
-    // a new H or P can change the path (or the FP64 frequencies of mixed precision): the
-    // captured graph then goes, and the next call runs normally (scratch, autotuner)
+    // A new H or P can change the path (or the FP64 frequencies of mixed precision), and another
+    // call on such inputs can have moved the partial sums or the matrix slices whose addresses the
+    // graph holds: the graph then goes, and the next call runs normally (scratch, autotuner).
     st = ensure_block(c);
     if (st) return st;
     const int path = use_block(c, gf::kOcc) ? 1 + c->blk_nc : 0;
-    if (c->occ_path != path) {
+    if (c->occ_path != path || c->occ_moves != c->occ_part.moves + c->a_scratch.moves) {
       if (c->occ_exec) GF_CU(cudaGraphExecDestroy(c->occ_exec));
       c->occ_exec = nullptr;
       c->occ_calls = 0;
@@ -846,6 +847,7 @@ gf_status occupation_impl(gf_ctx* c, const double* mu, double* n_out, double* dn
     for (int s2 = 0; s2 < c->n_sys; ++s2) c->hp_mu()[s2] = mu[s2];
     st = enqueue_occupation(c);
     if (st) return st;
+    c->occ_moves = c->occ_part.moves + c->a_scratch.moves;
     return finish_occupation(c, c->stream, n_out, dn_out);
   }
   // graph mode: E_inf and the low-rank eigenbasis outside the graph (inputs may

@@ -28,6 +28,7 @@ namespace gf_host {
 struct DevBuf {
   void* p = nullptr;
   size_t bytes = 0;
+  unsigned moves = 0;  // times the memory was given back: what still holds its address is stale
   template <class T>
   T* as() const { return static_cast<T*>(p); }
 };
@@ -35,7 +36,10 @@ struct DevBuf {
 inline cudaError_t ensure(DevBuf& b, size_t bytes) {
   if (bytes == 0) bytes = 16;
   if (b.bytes >= bytes) return cudaSuccess;
-  if (b.p) cudaFree(b.p);
+  if (b.p) {
+    cudaFree(b.p);
+    ++b.moves;
+  }
   b.p = nullptr;
   b.bytes = 0;
   cudaError_t e = cudaMalloc(&b.p, bytes);
@@ -44,7 +48,10 @@ inline cudaError_t ensure(DevBuf& b, size_t bytes) {
 }
 
 inline void release(DevBuf& b) {
-  if (b.p) cudaFree(b.p);
+  if (b.p) {
+    cudaFree(b.p);
+    ++b.moves;
+  }
   b.p = nullptr;
   b.bytes = 0;
 }
@@ -181,7 +188,8 @@ struct gf_ctx {
   // stream that forks from the call's and joins it again
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  int occ_path = 0;                           // path that the captured N(mu) graph holds
+  int occ_path = 0;                           // path that the captured N(mu) graph holds,
+  unsigned occ_moves = 0;                     // and the moves of the scratch that other calls can grow
   DevBuf blk_units, blk_perm, blk_sysg, blk_offT;  // (blk_offT: offsets of T, then of C)
   DevBuf blk_e, blk_T, blk_Ts, blk_B, blk_Bs, blk_HO, blk_U, blk_D22, blk_V, blk_R, blk_H11, blk_tau,
       blk_ws, blk_info, blk_C, blk_Cs, blk_ser, blk_Tp, blk_Cp;

@@ -1,0 +1,45 @@
+"""Which inputs the block form takes, what it computes for those near its limits, and what the inputs outside it
+get: results of the general kernels (GF_KERNEL=direct), of the CPU oracle, or of a fresh context."""
+import numpy as np
+import pytest
+
+from paper_1111_2157_gb300 import gf, synth
+from tests.test_block_form import _inputs, _rel
+
+
+def _context(s, **kw):
+    g = gf.GreensFunction.for_systems([s], **kw)
+    g.set_hamiltonian(s.H)
+    g.set_projectors(s.P)
+    g.set_sigma(s.sigma, s.sigma_inf)
+    return g
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("call", ["evaluate", "backward"])
+@pytest.mark.parametrize("precision,other,size", [("fp64", "not_hermitian", (4, 20, 6, 64)),
+                                                  ("mixed", "larger_norm", (150, 6, 2, 1024))])
+def test_a_captured_graph_does_not_outlive_the_scratch_it_writes(precision, other, size, call):
+    """N(mu) captured for one H, another H on another path (or with more FP64 frequencies) in a call that is not an
+    N(mu) call and needs more partial sums, then the first H again: the replay must not use the scratch given back."""
+    s = _inputs(*size, 40.0, 3)
+    H2 = s.H.copy()
+    if other == "not_hermitian":
+        H2[0, 1, 3] += 1e-5
+    else:
+        H2 *= 40.0
+    g = _context(s, precision=precision)
+    ref = g.occupation([0.2])
+    g.close()
+    g = _context(s, precision=precision, graph=True)
+    for _ in range(2):
+        for _ in range(3):
+            n, dn = g.occupation([0.2])
+            assert n[0] == ref[0][0] and dn[0] == ref[1][0]
+        g.set_hamiltonian(H2)
+        if call == "evaluate":
+            g.evaluate([0.2])
+        else:
+            g.backward([0.2], n_bar=[1.0])
+        g.set_hamiltonian(s.H)
+    g.close()
