@@ -157,7 +157,7 @@ gf_status ensure_block(gf_ctx* c) {
   GF_CU(gf::launch_block_reduce(b, c->smem_optin, c->sm_count, c->stream));
   GF_CU(gf::launch_block_eig(b, c->blk_ws.as<double2>(), grid, in_smem, c->stream));
   GF_CU(gf::launch_block_finish(b, c->stream));
-  c->last_launches += 4;
+  c->last_launches += 5;
   std::vector<double> info((size_t)c->n_k + 1);
   GF_CU(cudaMemcpyAsync(info.data(), c->blk_info.p, 8 * info.size(), cudaMemcpyDeviceToHost, c->stream));
   GF_CU(cudaStreamSynchronize(c->stream));
@@ -193,10 +193,10 @@ bool block_low(const gf_ctx* c, int mode) {
          (!(mode & gf::kAdj) || gf::block_smem(c->mmax, c->blk_n2max, mode, 1) <= (size_t)c->smem_optin - 1024);
 }
 
-// Whether a call of this mode runs on the block form.  GF_KERNEL=direct keeps the general
-// kernels; with GF_PREC_MIXED every value of GF_KERNEL does, as it names one of them.
-bool use_block(const gf_ctx* c, int mode) {
-  if (!c->blk_shape || !c->blk_ok) return false;
+// Whether a call of this mode runs on the block form if H and P allow it.  GF_KERNEL=direct keeps
+// the general kernels; with GF_PREC_MIXED every value of GF_KERNEL does, as it names one of them.
+bool block_wanted(const gf_ctx* c, int mode) {
+  if (!c->blk_shape) return false;
   const char* only = std::getenv("GF_KERNEL");
   if (only && (std::strcmp(only, "direct") == 0 || (c->precision == GF_PREC_MIXED && !c->lowrank))) return false;
   // sizes that the general kernels refuse stay refused
@@ -207,6 +207,15 @@ bool use_block(const gf_ctx* c, int mode) {
   return gf::block_smem(c->mmax, c->blk_n2max, mode, 0) <= limit &&
          (!block_low(c, mode) || (gf::block_smem(c->mmax, c->blk_n2max, mode, 1) <= limit &&
                                   gf::block32_smem(c->mmax, c->blk_n2max) <= limit));
+}
+
+// Whether it does: the set-up runs only for calls that could use it.
+gf_status use_block(gf_ctx* c, int mode, bool* block) {
+  *block = false;
+  if (!block_wanted(c, mode)) return GF_OK;
+  gf_status st = ensure_block(c);
+  *block = c->blk_shape && c->blk_ok;
+  return st;
 }
 
 // rho_k partial sums: the low-rank and the block kernels leave them in the basis that makes
@@ -640,9 +649,10 @@ gf_status run_points(gf_ctx* c, int mode) {
   st = ensure_einf(c);
   if (st) return st;
   GF_CU(cudaMemsetAsync(c->status.p, 0, sizeof(int), c->stream));
-  st = ensure_block(c);
+  bool block = false;
+  st = use_block(c, mode, &block);
   if (st) return st;
-  const bool block = c->run_on_block = use_block(c, mode);
+  c->run_on_block = block;
   if (!block) {
     st = ensure_lr(c);
     if (st) return st;
@@ -826,13 +836,14 @@ gf_status occupation_impl(gf_ctx* c, const double* mu, double* n_out, double* dn
     if (!std::isfinite(mu[s2])) return fail(c, GF_EINVAL, "mu is not finite");
   gf_status st = check_ready(c);
   if (st) return st;
+  bool block = false;  // (graph)
   if (c->use_graph) {
     // A new H or P can change the path (or the FP64 frequencies of mixed precision), and another
     // call on such inputs can have moved the partial sums or the matrix slices whose addresses the
     // graph holds: the graph then goes, and the next call runs normally (scratch, autotuner).
-    st = ensure_block(c);
+    st = use_block(c, gf::kOcc, &block);
     if (st) return st;
-    const int path = use_block(c, gf::kOcc) ? 1 + c->blk_nc : 0;
+    const int path = block ? 1 + c->blk_nc : 0;
     if (c->occ_path != path || c->occ_moves != c->occ_part.moves + c->a_scratch.moves) {
       if (c->occ_exec) GF_CU(cudaGraphExecDestroy(c->occ_exec));
       c->occ_exec = nullptr;
@@ -855,7 +866,7 @@ gf_status occupation_impl(gf_ctx* c, const double* mu, double* n_out, double* dn
   GF_CU(cudaStreamSynchronize(c->stream));
   st = ensure_einf(c);
   if (st) return st;
-  if (c->lowrank && c->lr_dirty && !use_block(c, gf::kOcc)) {
+  if (c->lowrank && c->lr_dirty && !block) {
     GF_CU(cudaMemsetAsync(c->status.p, 0, sizeof(int), c->stream));
     st = ensure_lr(c);
     if (st) return st;

@@ -55,81 +55,124 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// P_k^+ = Q [R; 0] by Householder reflections H_j = I - tau v v^+ (real tau, so H_j is
-// Hermitian and unitary; the phases stay in R), then Q^+ H_k Q by one rank-2 update per
-// reflection.  One CTA per k-point (grid-stride).
-__global__ void __launch_bounds__(kSetupThreads) k_block_reduce(const BlockSetup b, int in_smem) {
+// Whether H_k and P_k allow the block form, and P_k^+ = Q [R; 0] by Householder reflections H_j = I -
+// tau v v^+ (real tau, so H_j is Hermitian and unitary; the phases stay in R).  One CTA per k-point,
+// ahead of the other kernels, which return at once when any k-point set a flag: the first mixed N(mu) (16
+// frequencies) after a refused upload of 256 k-points of 40 bands takes 0.65 ms, 1.81 with the whole set-up.
+__global__ void __launch_bounds__(kSetupThreads) k_block_check(const BlockSetup b) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double red[kSetupThreads / 32];
   double2* X = reinterpret_cast<double2*>(smraw);      // [m][N]: columns of P^+, then the vectors v_j
   double2* R = X + (size_t)b.mmax * b.nbmax;           // [m][m]
-  double2* pv = R + (size_t)b.mmax * b.mmax;           // [N]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kWarps = kSetupThreads / 32;
+  const int k = blockIdx.x;
+  const KInfo ki = b.kinfo[k];
+  const int N = ki.nb, M = b.sinfo[ki.sys].m;
+  const double2* H = b.H + ki.offH;
+  const double2* P = b.P + ki.offP;
+  // the norm of H_k and its distance from a Hermitian matrix
+  double nrm = 0.0, anti = 0.0, big = 0.0;
+  for (int e = tid; e < N * N; e += kSetupThreads) {
+    const int i = e / N, j = e - i * N;
+    const double2 h = H[e], t = H[j * N + i];
+    nrm += h.x * h.x + h.y * h.y;
+    anti = fmax(anti, fmax(fabs(h.x - t.x), fabs(h.y + t.y)));
+    big = fmax(big, fmax(fabs(h.x), fabs(h.y)));
+  }
+  nrm = setup_sum(nrm, red);
+  for (int off = 16; off; off >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, off));
+  __syncthreads();
+  if (lane == 0) red[warp] = big;
+  __syncthreads();
+  big = red[0];
+  for (int w = 1; w < kWarps; ++w) big = fmax(big, red[w]);
+  if (tid == 0) b.hnorm[k] = sqrt(nrm / N);
+  // (NaN and infinity fail the comparison and take the general path)
+  if (__syncthreads_or(!(anti <= 8.9e-16 * big) || !isfinite(nrm))) {
+    if (tid == 0) atomicOr(b.flags, kBlkNonHermitian);
+    return;
+  }
+  for (int e = tid; e < M * N; e += kSetupThreads) {
+    const double2 p = P[e];
+    X[e] = make_double2(p.x, -p.y);
+  }
+  __syncthreads();
+  for (int j = 0; j < M; ++j) {
+    double2* x = X + j * N;
+    double s = 0.0;
+    for (int i = j + tid; i < N; i += kSetupThreads) s += x[i].x * x[i].x + x[i].y * x[i].y;
+    s = setup_sum(s, red);
+    const double nx = sqrt(s);
+    const double2 x0 = x[j];
+    const double ax = sqrt(x0.x * x0.x + x0.y * x0.y);
+    const double2 ph = ax > 0.0 ? make_double2(x0.x / ax, x0.y / ax) : make_double2(1.0, 0.0);
+    const double tau = nx > 0.0 ? 1.0 / (nx * (nx + ax)) : 0.0;
+    __syncthreads();
+    if (tid == 0) {
+      x[j] = make_double2(x0.x + ph.x * nx, x0.y + ph.y * nx);
+      R[j * M + j] = make_double2(-ph.x * nx, -ph.y * nx);
+      b.tau[(size_t)k * b.mmax + j] = tau;
+    }
+    __syncthreads();
+    // the later columns: x_c -= tau v (v^+ x_c)
+    for (int c = j + 1 + warp; c < M; c += kWarps) {
+      double2* y = X + c * N;
+      double2 d = make_double2(0.0, 0.0);
+      for (int i = j + lane; i < N; i += 32) cmac_ca(d, x[i], y[i]);
+      d.x = tau * warp_sum(d.x);
+      d.y = tau * warp_sum(d.y);
+      for (int i = j + lane; i < N; i += 32) {
+        const double2 v = x[i];
+        y[i].x -= fma(v.x, d.x, -v.y * d.y);
+        y[i].y -= fma(v.x, d.y, v.y * d.x);
+      }
+      __syncwarp();
+      if (lane == 0) R[j * M + c] = y[j];
+    }
+    __syncthreads();
+  }
+  // rank of P: the triangular factor must be safely invertible
+  if (tid == 0) {
+    double lo = INFINITY, hi = 0.0;
+    for (int j = 0; j < M; ++j) {
+      const double d = fmax(fabs(R[j * M + j].x), fabs(R[j * M + j].y));
+      lo = fmin(lo, d);
+      for (int c = j; c < M; ++c) hi = fmax(hi, fmax(fabs(R[j * M + c].x), fabs(R[j * M + c].y)));
+      if (!(d > 0.0)) lo = 0.0;
+    }
+    if (!(lo > 1e-3 * hi) || !isfinite(hi)) atomicOr(b.flags, kBlkRankDeficient);
+  }
+  for (int e = tid; e < M * N; e += kSetupThreads) {
+    const int j = e / N, i = e - j * N;
+    b.V[ki.offP + e] = i < j ? make_double2(0.0, 0.0) : X[e];
+  }
+  for (int e = tid; e < M * M; e += kSetupThreads) {
+    const int i = e / M, c = e - i * M;
+    b.R[(size_t)k * b.mmax * b.mmax + e] = c >= i ? R[e] : make_double2(0.0, 0.0);
+  }
+}
+
+// Q^+ H_k Q by one rank-2 update per reflection.  One CTA per k-point (grid-stride).
+__global__ void __launch_bounds__(kSetupThreads) k_block_reduce(const BlockSetup b, int in_smem) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ double red[kSetupThreads / 32];
+  if (*b.flags) return;
+  double2* X = reinterpret_cast<double2*>(smraw);      // [m][N]: the vectors v_j
+  double2* pv = X + (size_t)b.mmax * b.nbmax;          // [N]
   double2* A = in_smem ? pv + b.nbmax : b.ws + (size_t)blockIdx.x * b.nbmax * b.nbmax;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int kWarps = kSetupThreads / 32;
   for (int k = blockIdx.x; k < b.n_k; k += gridDim.x) {
     const KInfo ki = b.kinfo[k];
     const int N = ki.nb, M = b.sinfo[ki.sys].m, n2 = N - M;
-    const double2* H = b.H + ki.offH;
-    const double2* P = b.P + ki.offP;
     __syncthreads();
-    // H_k, its norm and its distance from a Hermitian matrix
-    double nrm = 0.0, anti = 0.0, big = 0.0;
-    for (int e = tid; e < N * N; e += kSetupThreads) {
-      const int i = e / N, j = e - i * N;
-      const double2 h = H[e], t = H[j * N + i];
-      A[e] = h;
-      nrm += h.x * h.x + h.y * h.y;
-      anti = fmax(anti, fmax(fabs(h.x - t.x), fabs(h.y + t.y)));
-      big = fmax(big, fmax(fabs(h.x), fabs(h.y)));
-    }
-    nrm = setup_sum(nrm, red);
-    for (int off = 16; off; off >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, off));
-    __syncthreads();
-    if (lane == 0) red[warp] = big;
-    __syncthreads();
-    big = red[0];
-    for (int w = 1; w < kWarps; ++w) big = fmax(big, red[w]);
-    // (NaN and infinity fail the comparison and take the general path)
-    if (!(anti <= 8.9e-16 * big) || !isfinite(nrm)) atomicOr(b.flags, kBlkNonHermitian);
-    if (tid == 0) b.hnorm[k] = sqrt(nrm / N);
-    for (int e = tid; e < M * N; e += kSetupThreads) {
-      const double2 p = P[e];
-      X[e] = make_double2(p.x, -p.y);
-    }
+    for (int e = tid; e < N * N; e += kSetupThreads) A[e] = b.H[ki.offH + e];
+    for (int e = tid; e < M * N; e += kSetupThreads) X[e] = b.V[ki.offP + e];
     __syncthreads();
     for (int j = 0; j < M; ++j) {
-      double2* x = X + j * N;
-      double s = 0.0;
-      for (int i = j + tid; i < N; i += kSetupThreads) s += x[i].x * x[i].x + x[i].y * x[i].y;
-      s = setup_sum(s, red);
-      const double nx = sqrt(s);
-      const double2 x0 = x[j];
-      const double ax = sqrt(x0.x * x0.x + x0.y * x0.y);
-      const double2 ph = ax > 0.0 ? make_double2(x0.x / ax, x0.y / ax) : make_double2(1.0, 0.0);
-      const double tau = nx > 0.0 ? 1.0 / (nx * (nx + ax)) : 0.0;
-      __syncthreads();
-      if (tid == 0) {
-        x[j] = make_double2(x0.x + ph.x * nx, x0.y + ph.y * nx);
-        R[j * M + j] = make_double2(-ph.x * nx, -ph.y * nx);
-        b.tau[(size_t)k * b.mmax + j] = tau;
-      }
-      __syncthreads();
-      // the later columns: x_c -= tau v (v^+ x_c)
-      for (int c = j + 1 + warp; c < M; c += kWarps) {
-        double2* y = X + c * N;
-        double2 d = make_double2(0.0, 0.0);
-        for (int i = j + lane; i < N; i += 32) cmac_ca(d, x[i], y[i]);
-        d.x = tau * warp_sum(d.x);
-        d.y = tau * warp_sum(d.y);
-        for (int i = j + lane; i < N; i += 32) {
-          const double2 v = x[i];
-          y[i].x -= fma(v.x, d.x, -v.y * d.y);
-          y[i].y -= fma(v.x, d.y, v.y * d.x);
-        }
-        __syncwarp();
-        if (lane == 0) R[j * M + c] = y[j];
-      }
+      const double2* x = X + j * N;
+      const double tau = b.tau[(size_t)k * b.mmax + j];
       // A <- H_j A H_j: p = tau A v, w = p - (tau / 2) (v^+ p) v, A -= v w^+ + w v^+
       for (int i = warp; i < N; i += kWarps) {
         double2 d = make_double2(0.0, 0.0);
@@ -165,24 +208,8 @@ __global__ void __launch_bounds__(kSetupThreads) k_block_reduce(const BlockSetup
       }
       __syncthreads();
     }
-    // rank of P: the triangular factor must be safely invertible
-    if (tid == 0) {
-      double lo = INFINITY, hi = 0.0;
-      for (int j = 0; j < M; ++j) {
-        const double d = fmax(fabs(R[j * M + j].x), fabs(R[j * M + j].y));
-        lo = fmin(lo, d);
-        for (int c = j; c < M; ++c) hi = fmax(hi, fmax(fabs(R[j * M + c].x), fabs(R[j * M + c].y)));
-        if (!(d > 0.0)) lo = 0.0;
-      }
-      if (!(lo > 1e-3 * hi) || !isfinite(hi)) atomicOr(b.flags, kBlkRankDeficient);
-    }
-    for (int e = tid; e < M * N; e += kSetupThreads) {
-      const int j = e / N, i = e - j * N;
-      b.V[ki.offP + e] = i < j ? make_double2(0.0, 0.0) : X[e];
-    }
     for (int e = tid; e < M * M; e += kSetupThreads) {
       const int i = e / M, c = e - i * M;
-      b.R[(size_t)k * b.mmax * b.mmax + e] = c >= i ? R[e] : make_double2(0.0, 0.0);
       b.H11[(size_t)k * b.mmax * b.mmax + e] = A[i * N + c];
     }
     for (int e = tid; e < M * n2; e += kSetupThreads) {
@@ -199,6 +226,7 @@ __global__ void __launch_bounds__(kSetupThreads) k_block_reduce(const BlockSetup
 // B, H11, O, the pair table and U of one k-point per CTA (gf_block.cuh).
 __global__ void __launch_bounds__(kSetupThreads) k_block_finish(const BlockSetup b) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  if (*b.flags) return;
   const int k = blockIdx.x;
   const KInfo ki = b.kinfo[k];
   const int N = ki.nb, M = b.sinfo[ki.sys].m, n2 = N - M, np = M * (M + 1) / 2;
@@ -319,6 +347,7 @@ __global__ void __launch_bounds__(kSetupThreads) k_block_series(const BlockSetup
   extern __shared__ __align__(16) unsigned char smraw[];
   double* Tj = reinterpret_cast<double*>(smraw);  // [jt][n2]
   __shared__ double s_cr[2];
+  if (*b.flags) return;
   const int k = blockIdx.x;
   const KInfo ki = b.kinfo[k];
   const int M = b.sinfo[ki.sys].m, n2 = ki.nb - M, np = M * (M + 1) / 2, jt = min(n2, kBlkSeries);
@@ -1400,8 +1429,7 @@ __global__ void __launch_bounds__(kSetupThreads)
 }
 
 size_t reduce_smem(int nbmax, int mmax, bool matrix) {
-  return sizeof(double2) * ((size_t)mmax * nbmax + (size_t)mmax * mmax + nbmax +
-                            (matrix ? (size_t)nbmax * nbmax : 0));
+  return sizeof(double2) * ((size_t)mmax * nbmax + nbmax + (matrix ? (size_t)nbmax * nbmax : 0));
 }
 bool reduce_in_smem(int nbmax, int mmax, int smem_optin) {
   return reduce_smem(nbmax, mmax, true) <= (size_t)smem_optin - 1024;
@@ -1440,9 +1468,14 @@ size_t block_reduce_ws_elems(int nbmax, int mmax, int smem_optin, int sm_count) 
 }
 
 cudaError_t launch_block_reduce(const BlockSetup& b, int smem_optin, int sm_count, cudaStream_t s) {
+  const size_t chk = sizeof(double2) * ((size_t)b.mmax * b.nbmax + (size_t)b.mmax * b.mmax);
+  cudaError_t e = cudaFuncSetAttribute(k_block_check, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chk);
+  if (e != cudaSuccess) return e;
+  k_block_check<<<b.n_k, kSetupThreads, chk, s>>>(b);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const bool in = reduce_in_smem(b.nbmax, b.mmax, smem_optin);
   const size_t smem = reduce_smem(b.nbmax, b.mmax, in);
-  cudaError_t e = cudaFuncSetAttribute(k_block_reduce, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = cudaFuncSetAttribute(k_block_reduce, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   k_block_reduce<<<reduce_grid(b.nbmax, b.mmax, b.n_k, smem_optin, sm_count), kSetupThreads, smem, s>>>(b, in ? 1 : 0);
   return cudaGetLastError();

@@ -70,7 +70,7 @@ struct BlockLaunch {
   int n2max;
 };
 
-// Setup over the k-points: reduction (QR, Q^+ H Q), eigenpairs of the n2 block, and the
+// Setup over the k-points: check and QR, Q^+ H Q, eigenpairs of the n2 block, and the
 // tables above.  flags (device int): kBlkNonHermitian, kBlkRankDeficient,
 // kBlkNoConvergence; hnorm (device, n_k): ||H_k||_F / sqrt(N_b).
 constexpr int kBlkNonHermitian = 1, kBlkRankDeficient = 2, kBlkNoConvergence = 4;
@@ -104,7 +104,7 @@ struct BlockSetup {
   int* flags;
   double* hnorm;
 };
-cudaError_t launch_block_reduce(const BlockSetup& b, int smem_optin, int sm_count, cudaStream_t s);
+cudaError_t launch_block_reduce(const BlockSetup& b, int smem_optin, int sm_count, cudaStream_t s);  // (two kernels)
 cudaError_t launch_block_eig(const BlockSetup& b, double2* ws, int grid, int in_smem, cudaStream_t s);
 cudaError_t launch_block_finish(const BlockSetup& b, cudaStream_t s);  // (two kernels)
 size_t block_reduce_ws_elems(int nbmax, int mmax, int smem_optin, int sm_count);

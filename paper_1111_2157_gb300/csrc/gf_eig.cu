@@ -1281,6 +1281,7 @@ __global__ void __launch_bounds__(kEigThreads)
     k_block_eig(const BlockSetup b, double2* gws, int in_smem, int z_smem) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ QlScratch ql;
+  if (*b.flags & ~kBlkNoConvergence) return;  // (other CTAs set that bit meanwhile)
   double2* A = in_smem ? reinterpret_cast<double2*>(smem_raw) : gws + blockIdx.x * eig_ws_elems(b.n2max);
   for (int k = blockIdx.x; k < b.n_k; k += gridDim.x) {
     const KInfo ki = b.kinfo[k];

@@ -43,3 +43,36 @@ def test_a_captured_graph_does_not_outlive_the_scratch_it_writes(precision, othe
             g.backward([0.2], n_bar=[1.0])
         g.set_hamiltonian(s.H)
     g.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("why", ["not_hermitian", "kernel_named"])
+def test_a_call_on_the_general_kernels_does_not_pay_for_the_set_up(why, monkeypatch):
+    """N(mu) right after an upload against N(mu) repeated: the whole set-up of these windows (8 ms) would double the
+    first, the check of H and P is 0.1 ms of it.  (Bound: a third of the pass, and 0.5 ms for what follows an
+    upload.)"""
+    import time
+    rng = synth.rng_for(1)
+    nk, nb, m, n_iw = 152, 128, 14, 40
+    pole = synth.sigma_two_pole(rng, m, 4.0)
+    s = synth.System(synth.hamiltonian_dense(rng, nk, nb, -8.0, 8.0, 0.3), synth.projectors(rng, nk, nb, m), pole,
+                     pole.sample(40.0, n_iw), 40.0, nb / 2.0)
+    if why == "kernel_named":
+        monkeypatch.setenv("GF_KERNEL", "f32r")
+    else:
+        s.H[-1, 0, 1] += 1e-3
+    g = _context(s, precision="mixed")
+
+    def seconds():
+        t = time.perf_counter()
+        g.occupation([0.1])
+        return time.perf_counter() - t
+
+    seconds()  # (autotuner)
+    first, again = [], []
+    for _ in range(5):
+        g.set_hamiltonian(s.H)
+        first.append(seconds())
+        again.append(seconds())
+    g.close()
+    assert min(first) < 1.33 * min(again) + 5e-4
