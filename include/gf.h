@@ -68,7 +68,9 @@ typedef enum {
  * Every mode runs on the block form where it can: P_k^+ = Q [R; 0] and the
  * eigenproblem of the N_b - m remaining rows of Q^+ H_k Q are solved once per
  * upload of H or P, after which a point costs O(m^2 N_b + m^3) multiply-adds.
- * It needs Hermitian H_k, P_k of full rank, m <= 32, m < N_b and
+ * It needs Hermitian H_k (to 4 rounding errors of its largest entry), P_k P_k^+
+ * with a condition number of at most about 100 (mixed: 32) and entries of P_k
+ * within 1e-60 to 1e60 (mixed: 1e-6 to 1e6), m <= 32, m < N_b and
  * N_b - m <= 256 at every k, at least 16 frequencies and pi / beta >= 1e-4; the
  * general kernels take the other inputs, and every call when the environment
  * variable GF_KERNEL is "direct" (in mixed precision: when it has any value).

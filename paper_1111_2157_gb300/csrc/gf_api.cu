@@ -51,6 +51,14 @@ constexpr int kBlkMinFreq = 16;
 // Lowest pi / beta of the block form (eV): below it an eigenvalue of the n2 block that happens
 // to lie near mu would cost more digits than the pivoted inverse loses.
 constexpr double kBlkMinW = 1e-4;
+// Largest condition number of O = (P P^+)^{-1}, as k_block_check estimates it.  Mixed, at 40 to 46: N
+// to 5e-9, dN/dmu 7e-8, rho_k 2e-8, G_loc 9e-13, each no further from FP64 than the general kernels (7e-9,
+// 4e-6, 2e-7, 6e-12); at 66 to 96 G_loc 2.6e-12 and N 1.1e-8, at 350 1.7e-11 and 1.7e-8, at 2300 2e-9 and 2e-7.
+// FP64 against the general kernel: up to 100 dN/dmu 4e-12 and G_loc 2e-13, at 860 2e-10 and 1e-12.  (Windows of 24 to
+// 96 bands, 5 to 30 orbitals, beta 40 to 400, one small singular value of P or a geometric row of them.)
+constexpr double kBlkCondMixed = 32.0, kBlkCondFp64 = 100.0;
+// ... and of |R|^2, |R^{-1}|^2 (the scale of P), from which O and B B^+ stay far inside the number range.
+constexpr double kBlkRangeMixed = 1e12, kBlkRangeFp64 = 1e120;
 
 gf_status ensure_einf(gf_ctx* c) {
   if (!c->einf_dirty) return GF_OK;
@@ -106,7 +114,7 @@ gf_status ensure_block(gf_ctx* c) {
               {&c->blk_Ts, mixed ? 8 * (size_t)c->blk_totT : 0}, {&c->blk_Tp, mixed ? 16 * (size_t)c->blk_totT : 0}, {&c->blk_B, 16 * (size_t)c->totP},
               {&c->blk_Bs, mixed ? 8 * (size_t)c->totP : 0},     {&c->blk_HO, 32 * npm * c->n_k},
               {&c->blk_U, 16 * (size_t)c->totH},     {&c->blk_D22, 16 * (size_t)c->totH},
-              {&c->blk_V, 16 * (size_t)c->totP},     {&c->blk_R, 16 * mm * c->n_k},
+              {&c->blk_V, 16 * (size_t)c->totP},     {&c->blk_Ri, 16 * mm * c->n_k},
               {&c->blk_H11, 16 * mm * c->n_k},       {&c->blk_tau, 8 * (size_t)c->mmax * c->n_k},
               {&c->blk_C, 16 * (size_t)c->blk_totC}, {&c->blk_Cs, mixed ? 8 * (size_t)c->blk_totC : 0},
               {&c->blk_Cp, mixed ? 16 * (size_t)c->blk_totC : 0},
@@ -130,9 +138,11 @@ gf_status ensure_block(gf_ctx* c) {
   b.mmax = c->mmax;
   b.n2max = c->blk_n2max;
   b.npmax = (int)npm;
+  b.cond = mixed && !c->lowrank ? kBlkCondMixed : kBlkCondFp64;
+  b.range = mixed && !c->lowrank ? kBlkRangeMixed : kBlkRangeFp64;
   b.D22 = c->blk_D22.as<double2>();
   b.V = c->blk_V.as<double2>();
-  b.R = c->blk_R.as<double2>();
+  b.Ri = c->blk_Ri.as<double2>();
   b.tau = c->blk_tau.as<double>();
   b.H11 = c->blk_H11.as<double2>();
   b.B = c->blk_B.as<double2>();
@@ -168,7 +178,7 @@ gf_status ensure_block(gf_ctx* c) {
   if (flags) {
     c->tune_log += "block form: general kernels (" +
                    std::string(flags & gf::kBlkNonHermitian ? "H not Hermitian" :
-                               flags & gf::kBlkRankDeficient ? "P rank deficient" : "eigensolver") + "); ";
+                               flags & gf::kBlkIllConditioned ? "P ill-conditioned" : "eigensolver") + "); ";
     return GF_OK;
   }
   // mixed precision: frequencies w_n below a twentieth of the rms eigenvalue of H run in FP64, at
@@ -1363,7 +1373,7 @@ gf_status gf_destroy(gf_ctx* c) {
                     &c->wbout, &c->kHks, &c->kEps, &c->eps_grid, &c->dos, &c->pdos, &c->pdos_off,
                     &c->pole_part, &c->dos_part,
                     &c->blk_units, &c->blk_perm, &c->blk_sysg, &c->blk_offT, &c->blk_e, &c->blk_T, &c->blk_Ts,
-                    &c->blk_B, &c->blk_Bs, &c->blk_HO, &c->blk_U, &c->blk_D22, &c->blk_V, &c->blk_R, &c->blk_H11,
+                    &c->blk_B, &c->blk_Bs, &c->blk_HO, &c->blk_U, &c->blk_D22, &c->blk_V, &c->blk_Ri, &c->blk_H11,
                     &c->blk_tau, &c->blk_ws, &c->blk_info, &c->blk_C, &c->blk_Cs, &c->blk_ser, &c->blk_Tp, &c->blk_Cp};
   for (DevBuf* b : bufs) release(*b);
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);

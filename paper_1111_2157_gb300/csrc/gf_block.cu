@@ -132,25 +132,39 @@ __global__ void __launch_bounds__(kSetupThreads) k_block_check(const BlockSetup 
     }
     __syncthreads();
   }
-  // rank of P: the triangular factor must be safely invertible
-  if (tid == 0) {
-    double lo = INFINITY, hi = 0.0;
-    for (int j = 0; j < M; ++j) {
-      const double d = fmax(fabs(R[j * M + j].x), fabs(R[j * M + j].y));
-      lo = fmin(lo, d);
-      for (int c = j; c < M; ++c) hi = fmax(hi, fmax(fabs(R[j * M + c].x), fabs(R[j * M + c].y)));
-      if (!(d > 0.0)) lo = 0.0;
-    }
-    if (!(lo > 1e-3 * hi) || !isfinite(hi)) atomicOr(b.flags, kBlkRankDeficient);
-  }
   for (int e = tid; e < M * N; e += kSetupThreads) {
     const int j = e / N, i = e - j * N;
     b.V[ki.offP + e] = i < j ? make_double2(0.0, 0.0) : X[e];
   }
-  for (int e = tid; e < M * M; e += kSetupThreads) {
-    const int i = e / M, c = e - i * M;
-    b.R[(size_t)k * b.mmax * b.mmax + e] = c >= i ? R[e] : make_double2(0.0, 0.0);
+  __syncthreads();
+  // R^{-1} over X (M < N), column c by back substitution, and the conditioning of P: B, H11 and O carry
+  // R^{-1}, so the errors of the form grow with the condition number of O = (P P^+)^{-1}, which
+  // |R|^2 |R^{-1}|^2 / m - (m - 1) estimates (Frobenius norms; 1 for orthonormal rows, exact for one
+  // small singular value beside equal ones).
+  double r2 = 0.0, ri2 = 0.0;
+  for (int c = tid; c < M; c += kSetupThreads) {
+    for (int i = M - 1; i >= 0; --i) {
+      double2 s = make_double2(i == c ? 1.0 : 0.0, 0.0), x = make_double2(0.0, 0.0);
+      if (i <= c) {
+        for (int j = i + 1; j <= c; ++j) {
+          const double2 r = R[i * M + j], y = X[j * M + c];
+          s.x -= fma(r.x, y.x, -r.y * y.y);
+          s.y -= fma(r.x, y.y, r.y * y.x);
+        }
+        const double2 r = R[i * M + c];
+        x = cmul(s, crcp(R[i * M + i]));
+        r2 = fma(r.x, r.x, fma(r.y, r.y, r2));
+        ri2 = fma(x.x, x.x, fma(x.y, x.y, ri2));
+      }
+      X[i * M + c] = x;
+    }
   }
+  r2 = setup_sum(r2, red);
+  ri2 = setup_sum(ri2, red);
+  // (rows that are zero, infinite or NaN fail the comparisons)
+  if (tid == 0 && !(r2 * ri2 <= M * (b.cond + (M - 1)) && r2 < b.range && ri2 < b.range))
+    atomicOr(b.flags, kBlkIllConditioned);
+  for (int e = tid; e < M * M; e += kSetupThreads) b.Ri[(size_t)k * b.mmax * b.mmax + e] = X[e];
 }
 
 // Q^+ H_k Q by one rank-2 update per reflection.  One CTA per k-point (grid-stride).
@@ -234,24 +248,8 @@ __global__ void __launch_bounds__(kSetupThreads) k_block_finish(const BlockSetup
   double2* Ri = reinterpret_cast<double2*>(smraw);        // R^{-1}
   double2* W = Ri + (size_t)b.mmax * b.mmax;              // m x m
   double2* Bs = W + (size_t)b.mmax * b.mmax;              // m x n2: H12 V, then B
-  const double2* R = b.R + (size_t)k * b.mmax * b.mmax;
   const double2* V2 = b.D22 + ki.offH;
-  // column c of R^{-1} by back substitution
-  for (int c = tid; c < M; c += kSetupThreads) {
-    for (int i = M - 1; i >= 0; --i) {
-      if (i > c) {
-        Ri[i * M + c] = make_double2(0.0, 0.0);
-        continue;
-      }
-      double2 s = make_double2(i == c ? 1.0 : 0.0, 0.0);
-      for (int j = i + 1; j <= c; ++j) {
-        const double2 r = R[i * M + j], x = Ri[j * M + c];
-        s.x -= fma(r.x, x.x, -r.y * x.y);
-        s.y -= fma(r.x, x.y, r.y * x.x);
-      }
-      Ri[i * M + c] = cmul(s, crcp(R[i * M + i]));
-    }
-  }
+  for (int e = tid; e < M * M; e += kSetupThreads) Ri[e] = b.Ri[(size_t)k * b.mmax * b.mmax + e];
   for (int e = tid; e < M * n2; e += kSetupThreads) {
     const int a = e / n2, c = e - a * n2;
     double2 s = make_double2(0.0, 0.0);

@@ -71,18 +71,19 @@ struct BlockLaunch {
 };
 
 // Setup over the k-points: check and QR, Q^+ H Q, eigenpairs of the n2 block, and the
-// tables above.  flags (device int): kBlkNonHermitian, kBlkRankDeficient,
+// tables above.  flags (device int): kBlkNonHermitian, kBlkIllConditioned,
 // kBlkNoConvergence; hnorm (device, n_k): ||H_k||_F / sqrt(N_b).
-constexpr int kBlkNonHermitian = 1, kBlkRankDeficient = 2, kBlkNoConvergence = 4;
+constexpr int kBlkNonHermitian = 1, kBlkIllConditioned = 2, kBlkNoConvergence = 4;
 struct BlockSetup {
   const double2* H;
   const double2* P;
   const KInfo* kinfo;
   const SInfo* sinfo;
   int n_k, nbmax, mmax, n2max, npmax;
+  double cond, range;     // largest condition number of O, and of |R|^2 and |R^{-1}|^2
   double2* D22;           // [n2][n2] at offH: the n2 block, then its eigenvectors
   double2* V;             // [m][N_b] at offP: Householder vectors (row j: vector j)
-  double2* R;             // [m][m] at k * mmax^2
+  double2* Ri;            // [m][m] at k * mmax^2: R^{-1}
   double* tau;            // [m] at k * mmax
   double2* H11;           // [m][m] at k * mmax^2
   double2* B;             // [m][n2] at offP: Q1^+ H Q2, then B

@@ -191,7 +191,7 @@ struct gf_ctx {
   int occ_path = 0;                           // path that the captured N(mu) graph holds,
   unsigned occ_moves = 0;                     // and the moves of the scratch that other calls can grow
   DevBuf blk_units, blk_perm, blk_sysg, blk_offT;  // (blk_offT: offsets of T, then of C)
-  DevBuf blk_e, blk_T, blk_Ts, blk_B, blk_Bs, blk_HO, blk_U, blk_D22, blk_V, blk_R, blk_H11, blk_tau,
+  DevBuf blk_e, blk_T, blk_Ts, blk_B, blk_Bs, blk_HO, blk_U, blk_D22, blk_V, blk_Ri, blk_H11, blk_tau,
       blk_ws, blk_info, blk_C, blk_Cs, blk_ser, blk_Tp, blk_Cp;
   // DMFT step and projector construction
   DevBuf eimp, eimp_part, gl_in, delta, wraw, vdc;

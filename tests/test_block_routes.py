@@ -3,8 +3,9 @@ get: results of the general kernels (GF_KERNEL=direct), of the CPU oracle, or of
 import numpy as np
 import pytest
 
+import oracle
 from paper_1111_2157_gb300 import gf, synth
-from tests.test_block_form import _inputs, _rel
+from tests.test_block_form import _inputs, _rel, _run
 
 
 def _context(s, **kw):
@@ -76,3 +77,50 @@ def test_a_call_on_the_general_kernels_does_not_pay_for_the_set_up(why, monkeypa
         again.append(seconds())
     g.close()
     assert min(first) < 1.33 * min(again) + 5e-4
+
+
+def _near_dependent(s, delta, seed):
+    """P of every k with singular values 1 but for one delta."""
+    rng = np.random.default_rng(seed)
+    nk, m, nb = s.P.shape
+
+    def unitary(n, k):
+        return np.linalg.qr(rng.standard_normal((n, k)) + 1j * rng.standard_normal((n, k)))[0]
+
+    for k in range(nk):
+        s.P[k] = (unitary(m, m) * np.r_[np.ones(m - 1), delta]) @ np.conj(unitary(nb, m).T)
+    return s
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision,delta,on_block", [
+    ("fp64", 0.11, True), ("fp64", 0.09, False), ("fp64", 0.002, False), ("fp64", 0.0, False),
+    ("mixed", 0.2, True), ("mixed", 0.16, False), ("mixed", 0.01, False), ("mixed", 0.002, False)])
+def test_projectors_with_nearly_dependent_rows(precision, delta, on_block):
+    """delta^-2 is the condition number of (P P^+)^{-1}: the limits are 32 in mixed precision and 100 in FP64.  The
+    bounds are the contracts (mixed: of the G_loc, N, rho and dN/dmu tests; FP64 1e-10)."""
+    s = _near_dependent(_inputs(3, 40, 14, 64, 100.0, 31), delta, 7)
+    a, log = _run(s, None, precision=precision)
+    b, _ = _run(s, "direct")
+    assert ("mode 7: block form" in log) == on_block
+    assert on_block or "P ill-conditioned" in log
+    tol = {"N": 1e-7, "occ": 1e-7, "gloc": 1e-8, "loc": 1e-8, "rho": 1e-5, "dm": 1e-5, "dN_dmu": 1e-5, "docc": 1e-5,
+           "n_corr": 1e-6, "dm_nc": 1e-6}
+    for key in b:
+        bound = tol.get(key, 1e-5 if key.startswith("mb") else 1e-8) if precision == "mixed" else 1e-10
+        assert _rel(a[key], b[key]) < bound, key
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision,scale", [("mixed", 1e-20), ("mixed", 1e-7), ("fp64", 1e-70)])
+def test_projectors_of_a_scale_that_the_block_form_cannot_hold(precision, scale):
+    """(P P^+)^{-1} of such rows leaves the number range of S: N and rho_k are those of H_k alone."""
+    s = _inputs(2, 20, 6, 48, 40.0, 5)
+    s.P *= scale
+    g = _context(s, precision=precision)
+    r = g.evaluate([0.1])
+    assert "block form, " not in g.tuning_log()
+    g.close()
+    ref = oracle.get().density(s.H, s.P, s.sigma, s.sigma_inf, s.beta, 0.1)
+    assert abs(r["N"][0] - ref["N"]) < (1e-7 if precision == "mixed" else 1e-10) * ref["N"]
+    assert _rel(r["rho"].cpu().numpy(), ref["rho"].reshape(-1)) < (1e-5 if precision == "mixed" else 1e-10)
