@@ -37,7 +37,8 @@ namespace {
 using namespace cx;
 
 constexpr int kEigThreads = 256;
-
+// tri_eig: largest entry of Z^T Z - I, and largest residual |T z - lambda z| of the norm (others 3e-16)
+constexpr float kTriOrth = 3e-8f, kTriRes = 3e-15f;
 
 __device__ __forceinline__ double eig_block_sum(double v, double* red) {
   // Deterministic: fixed xor tree inside each warp, then warp 0 over the warps.
@@ -238,8 +239,11 @@ __device__ __forceinline__ float block_max(float v, float* red) {
 // Algebra Appl. 387, 2004), and one step Z <- Z (3 I - Z^T Z) / 2 that restores the orthogonality
 // which nearby eigenvalues lose.  Returns false, with d and e unchanged, when an eigenvalue pair
 // is closer than that step can mend (degenerate levels, a split matrix, non-finite input): the
-// caller then takes QR steps.  An FP64 instruction holds its scheduler for 64 clocks for one lane
-// as for 32, so this does in about 170 N of them, side by side, what QR steps do in 24 per rotation
+// caller then takes QR steps.  The step leaves Z^T Z = I - (3/4) G^2, 7e-16 at the largest G taken, and
+// a pair that three quotient steps did not separate keeps a residual; without the residual's limit and
+// with G up to 1e-5, levels 1e-6 of the norm apart (two or five, of 26 and 68) came out with
+// |T Z - Z L| 4e-12 and |Z^T Z - I| 9e-11.  An FP64 instruction holds its scheduler for 64 clocks for one
+// lane as for 32, so this does in about 170 N of them, side by side, what QR steps do in 24 per rotation
 // (5,400 rotations for N = 68), one after the other.
 __device__ bool tri_eig(double* Z, int zr, int zs, double* G, int gr, int gs, int N, QlScratch& q) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -253,6 +257,7 @@ __device__ bool tri_eig(double* Z, int zr, int zs, double* G, int gr, int gs, in
   }
   tn = block_max(tn, q.red);
   if (!(tn > 1e-15f && tn < 1e15f)) return false;
+  float gmax = 0.f;
   if (tid < N) {
     float lo = -1.001f * tn, hi = 1.001f * tn;
     const float tiny = 1e-12f * tn;
@@ -322,6 +327,7 @@ __device__ bool tri_eig(double* Z, int zr, int zs, double* G, int gr, int gs, in
       lam += gam / nrm;
       if (it == 2) {
         const double s = rsqrt(nrm);
+        gmax = (kTriOrth / kTriRes) * (float)(fabs(gam) * s) / tn;
         for (int i = 0; i < N; ++i) z[i * zr] *= s;
       }
     }
@@ -329,7 +335,7 @@ __device__ bool tri_eig(double* Z, int zr, int zs, double* G, int gr, int gs, in
   }
   __syncthreads();
   // G = Z^T Z - I (lower triangle and its mirror), its largest entry
-  float gmax = 0.f;
+  gmax = gmax == gmax ? gmax : INFINITY;
   for (int x = tid; x < N * (N + 1) / 2; x += kEigThreads) {
     int a, b;
     tri_pair(x, a, b);
@@ -347,7 +353,7 @@ __device__ bool tri_eig(double* Z, int zr, int zs, double* G, int gr, int gs, in
     gmax = fmaxf(gmax, f == f ? f : INFINITY);
   }
   gmax = block_max(gmax, q.red);
-  if (!(gmax < 1e-5f)) return false;
+  if (!(gmax < kTriOrth)) return false;
   // Z -= Z G / 2, one row per warp
   for (int r = warp; r < N; r += kEigThreads / 32) {
     double* zp = Z + r * zr;

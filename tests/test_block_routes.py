@@ -124,3 +124,46 @@ def test_projectors_of_a_scale_that_the_block_form_cannot_hold(precision, scale)
     ref = oracle.get().density(s.H, s.P, s.sigma, s.sigma_inf, s.beta, 0.1)
     assert abs(r["N"][0] - ref["N"]) < (1e-7 if precision == "mixed" else 1e-10) * ref["N"]
     assert _rel(r["rho"].cpu().numpy(), ref["rho"].reshape(-1)) < (1e-5 if precision == "mixed" else 1e-10)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("split", [3e-5, 3e-6, 1e-6, 3e-7, 1e-7, 1e-9, 1e-11])
+@pytest.mark.parametrize("nb,m,p", [(31, 5, 2), (60, 6, 5)])
+def test_levels_that_nearly_coincide(nb, m, p, split):
+    """Clusters of p levels, split of the norm apart, in the block that the set-up makes diagonal, and as eigenvalues
+    of the pseudo-Hamiltonian: unitary eigenvectors to rounding.  (Bound: cond(A) ~ |H| / w_0 = 1e2 roundings, 1e2
+    of their sums; vectors orthogonal to 1e-11 fail it.)"""
+    from oracle import pole as pole_oracle
+    s = _inputs(4, nb, m, 48, 40.0, 17)
+    rng = np.random.default_rng(int(1e12 * split) + nb)
+    n2 = nb - m
+    for k in range(4):
+        lev = np.linspace(-8.0, 8.0, n2) + 0.1 * rng.standard_normal(n2)
+        hidden = np.zeros(n2, bool)
+        for c in range(1, n2 - p, n2 // 3):
+            lev[c:c + p] = lev[c] + 8.0 * split * np.arange(p) * (1.0 + 0.3 * rng.random(p))
+            hidden[c:c + p] = k >= 2  # (k 0 and 1: coupled to the orbitals; 2 and 3: not, so levels of the whole H)
+        B = 0.3 * (rng.standard_normal((m, n2)) + 1j * rng.standard_normal((m, n2)))
+        B[:, hidden] = 0.0
+        U = np.linalg.qr(rng.standard_normal((n2, n2)) + 1j * rng.standard_normal((n2, n2)))[0]
+        H = s.H[k].copy()
+        H[m:, m:] = (U * lev) @ np.conj(U.T)
+        H[:m, m:] = B @ np.conj(U.T)
+        H[m:, :m] = np.conj(H[:m, m:].T)
+        s.H[k] = 0.5 * (H + np.conj(H.T))
+        s.P[k] = np.eye(m, nb)
+    a, log = _run(s, None)
+    b, _ = _run(s, "direct")
+    assert "mode 7: block form" in log
+    for key in ("N", "rho", "n_corr", "gloc"):
+        assert _rel(a[key], b[key]) < 1e-12, key
+    g = gf.GreensFunction.for_systems([s])
+    g.set_hamiltonian(s.H)
+    g.set_projectors(s.P)
+    g.set_sigma_poles([len(s.pole.p)], s.pole.p, s.pole.V.reshape(-1), s.pole.sigma_inf.reshape(-1))
+    n, _ = g.pole_occupation([0.1])
+    rho, _ = g.pole_density_matrix([0.1])
+    g.close()
+    ref = pole_oracle.density(s.H, s.P, s.sigma_inf, s.pole.p, s.pole.V, s.beta, 0.1)
+    assert abs(n[0] - ref["N"]) < 1e-12 * ref["N"]
+    assert _rel(rho.cpu().numpy(), np.asarray(ref["rho"]).reshape(-1)) < 1e-12
