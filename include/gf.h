@@ -63,7 +63,9 @@ typedef enum {
 } gf_status;
 
 /* Arithmetic of the (k, i w_n) point kernels.  Reductions over k and n, the
- * Matsubara tail and the mu search run in FP64 in every mode.
+ * Matsubara tail and the mu search run in FP64 in every mode (mixed, on the
+ * block form: rho_k and the traces over a batch of up to 16 frequencies in FP32
+ * pairs, 48 bits, and FP64 over the batches).
  *
  * Every mode runs on the block form where it can: P_k^+ = Q [R; 0] and the
  * eigenproblem of the N_b - m remaining rows of Q^+ H_k Q are solved once per

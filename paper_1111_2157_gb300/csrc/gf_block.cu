@@ -502,11 +502,14 @@ __device__ __forceinline__ float2 ld_cg(const float2* p) { return __ldg(p); }
 // What an instance of the kernel holds beside S^{-1}: the traces, and rho_k or the adjoint.  G_loc
 // alone in FP32 pairs runs in 128 registers and less shared memory, four CTAs on an SM: 5.4 ms
 // instead of 6.2 (256 k-points x 1024 frequencies, 40 bands, 14 orbitals); with the traces the
-// shared memory leaves three, and fewer registers cost 9 %.
+// shared memory leaves three, and fewer registers cost 9 %.  Eight lanes a matrix run in 128 registers but
+// for rho_k in FP32, whose pairs spill there: 64 k-points x 1024 frequencies, 96 bands, 7 orbitals 3.8 ms, 3.4
+// in 168.
 enum { kGlocOnly, kPlain, kWithRho, kWithAdj };
 
 template <int LW, bool LOW, int PART>
-__global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 || PART == kGlocOnly ? 4 : 3)
+__global__ void __launch_bounds__(32 * kBlkWarps,
+                                  PART == kGlocOnly || (LW == 8 && !(LOW && PART == kWithRho)) ? 4 : 3)
     k_point_block(const PointParams p, const BlockForm bf, const BlockLaunch bl) {
   using rc_t = typename Rest<LOW>::c;
   using rr_t = typename Rest<LOW>::r;
@@ -894,7 +897,8 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 || PART == kGlocOnly ?
             }
         }
         if (occ) {
-          float low_tr = 0.f, low_g2 = 0.f, low_xx = 0.f;  // LOW: this lane's sums over the warp's frequencies
+          // LOW: this lane's sums of (Tr X, Tr G^2) and Tr X^2 over the warp's frequencies, in pairs
+          float2 low_h = make_float2(0.f, 0.f), low_l = low_h, low_xh = low_h, low_xl = low_h;
           for (int i = lane; i < F * NP; i += 32) {
             const int f = i / NP, pr = i - f * NP;
             const int a = pair[pr].x, c = pair[pr].y;
@@ -947,9 +951,8 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 || PART == kGlocOnly ?
               if (a != c) s = rfma(g2.x, z1x, rfma(-g2.y, z1y, s));
               s = rfma(rr_t(2), s, xx);
               if constexpr (LOW) {
-                if (a == c) low_tr += x1.x;
-                low_g2 += s;
-                low_xx += xx;
+                pair2_add(low_h, low_l, make_float2(a == c ? x1.x : 0.f, s));
+                if (have_gbar) pair2_add(low_xh, low_xl, make_float2(xx, 0.f));
               } else {
                 if (a == c) acc_tr += x1.x;
                 acc_g2 += s;
@@ -958,9 +961,9 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 || PART == kGlocOnly ?
             }
           }
           if constexpr (LOW) {
-            acc_tr += (double)low_tr;
-            acc_g2 += (double)low_g2;
-            if (have_gbar) acc_mu += cb * wk * (double)low_xx;
+            acc_tr += widen(low_h.x) + widen(low_l.x);
+            acc_g2 += widen(low_h.y) + widen(low_l.y);
+            if (have_gbar) acc_mu += cb * wk * (widen(low_xh.x) + widen(low_xl.x));
           }
           __syncwarp();
         }
@@ -1141,8 +1144,8 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 || PART == kGlocOnly ?
           auto old = [&](int at) { return put ? make_double2(0.0, 0.0) : Sk[at]; };
           auto add = [&](int at, double2 o, double2 v) { Sk[at] = make_double2(o.x + v.x, o.y + v.y); };
           if constexpr (LOW) {
-            // FP32 products, summed over the nf frequencies in FP32 and added to the chunk's FP64 sum
-            // once (each FP64 add or conversion takes the SM 16 clocks).  Rows 1 of G_k are [A, Y],
+            // FP32 products, summed over the nf frequencies in pairs (in FP32 the sums would be off by 1e-8 and
+            // 7 % faster) and added to the chunk's FP64 sum once (each FP64 add takes the SM 16 clocks).  Rows 1 of G_k are [A, Y],
             // Y = A B D, rows 2 are D B^+ [A, Y] + D: orbitals lie in pairs of rows, {Re, Re, Im, Im},
             // so that the packed FMAs take two terms of the contraction over them, and columns of a
             // thread lie a third of the matrix apart, so that a warp's loads are consecutive.
@@ -1202,13 +1205,15 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 || PART == kGlocOnly ?
               const double2 o0 = old(a * nb + c), o1 = two ? old((a + 1) * nb + c) : make_double2(0.0, 0.0);
               const float4* v = c < M ? sA + (size_t)f0 * fA + pr * M + c : sY + pr * n2 + (c - M);
               const int fs = c < M ? fA : KP * n2;
-              float4 t = v[0];
+              float2 re = make_float2(v[0].x, v[0].y), im = make_float2(v[0].z, v[0].w);
+              float2 rl = make_float2(0.f, 0.f), il = rl;
               for (int f = 1; f < nf; ++f) {
                 const float4 w = v[(size_t)f * fs];
-                t = make_float4(t.x + w.x, t.y + w.y, t.z + w.z, t.w + w.w);
+                pair2_add(re, rl, make_float2(w.x, w.y));
+                pair2_add(im, il, make_float2(w.z, w.w));
               }
-              add(a * nb + c, o0, make_double2(widen(t.x), widen(t.z)));
-              if (two) add((a + 1) * nb + c, o1, make_double2(widen(t.y), widen(t.w)));
+              add(a * nb + c, o0, make_double2(widen(re.x) + widen(rl.x), widen(im.x) + widen(il.x)));
+              if (two) add((a + 1) * nb + c, o1, make_double2(widen(re.y) + widen(rl.y), widen(im.y) + widen(il.y)));
             }
             // (2,1) and (2,2) in tiles of four rows and CW columns
             constexpr int CW = 3;
@@ -1224,11 +1229,11 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 || PART == kGlocOnly ?
                 ks[w] = c < M ? M : n2;
                 fs[w] = c < M ? fA : KP * n2;
               }
-              float2 v[4][CW];
+              float2 v[4][CW], vl[4][CW];
 #pragma unroll
               for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int w = 0; w < CW; ++w) v[u][w] = make_float2(0.f, 0.f);
+                for (int w = 0; w < CW; ++w) v[u][w] = vl[u][w] = make_float2(0.f, 0.f);
               for (int f = 0; f < nf; ++f) {
                 float2 re[4][CW], im[4][CW];
 #pragma unroll
@@ -1262,7 +1267,8 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 || PART == kGlocOnly ?
                   const float2 d = dlow(f0 + f, min(b0 + u, n2 - 1));
 #pragma unroll
                   for (int w = 0; w < CW; ++w)
-                    fmac(v[u][w], make_float2(re[u][w].x + re[u][w].y, im[u][w].x + im[u][w].y), d);
+                    pair2_add(v[u][w], vl[u][w],
+                              fmul(make_float2(re[u][w].x + re[u][w].y, im[u][w].x + im[u][w].y), d));
                 }
               }
               double2 o[4][CW];  // (all loads before the first store)
@@ -1279,14 +1285,10 @@ __global__ void __launch_bounds__(32 * kBlkWarps, LW == 8 || PART == kGlocOnly ?
                 for (int w = 0; w < CW; ++w) {
                   const int c = c0 + w * ctl;
                   if (c >= CT) break;
-                  float2 t = v[u][w];
+                  float2 t = v[u][w], tl = vl[u][w];
                   if (M + bb == c)
-                    for (int f = f0; f < f0 + nf; ++f) {
-                      const float2 d = dlow(f, bb);
-                      t.x += d.x;
-                      t.y += d.y;
-                    }
-                  add((M + bb) * nb + c, o[u][w], make_double2(widen(t.x), widen(t.y)));
+                    for (int f = f0; f < f0 + nf; ++f) pair2_add(t, tl, dlow(f, bb));
+                  add((M + bb) * nb + c, o[u][w], make_double2(widen(t.x) + widen(tl.x), widen(t.y) + widen(tl.y)));
                 }
               }
             }

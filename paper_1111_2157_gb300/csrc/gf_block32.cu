@@ -12,7 +12,7 @@
 //      form, rows rotated one column per pivot, lazy row scales, as warp_invert of
 //      gf_warp_gj.cuh), then X = S^{-1} F row by row from the same registers;
 //   4. Tr X, Tr X^2, and 2 Tr(S^{-1} B D^3 B^+) from a second sweep over the pair table.
-// The sums over frequencies are FP64.
+// The sums over frequencies are FP32 pairs within a warp's batch of FW, FP64 over the batches.
 //
 // Bound by latency: issue slots 46 % and FMA pipe 32 % busy at 11 warps an SM.  N(mu) of 256
 // k-points x 1024 frequencies at 40 bands, 14 orbitals: 1.4 ms with the FP64 frequencies beside it;
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, NMAX > 24 ? 2 : 3)
   double acc_tr = 0.0, acc_g2 = 0.0;
 
   for (int n = n0 + wp * FW; n < n1; n += kBlkWarps * FW) {
-    float tr = 0.f, g2 = 0.f;
+    float2 th = z2(), tl = th;  // this lane's sums of (Tr G, Tr G^2) over the warp's frequencies, in pairs
     // 22.6 = 24 ln 2 + 6
     const int J = series_terms(cdx, __double2float_rn((2.0 * n + 1.0) * pib), cr, 22.6f);
     const bool series = J <= jmax;
@@ -129,8 +129,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps, NMAX > 24 ? 2 : 3)
         sd3[i] = fmul(d2, d);
       }
       if (n + f < n1) {
-        tr += d.x;
-        g2 += d2.x;
+        pair2_add(th, tl, make_float2(d.x, d2.x));
       }
     }
     if (series) {
@@ -311,13 +310,14 @@ __global__ void __launch_bounds__(32 * kBlkWarps, NMAX > 24 ? 2 : 3)
       }
       __syncwarp();
       if (valid && sl < M) {
-        tr += Fm[row * NMAX + row].x;
+        float g2 = 0.f;
 #pragma unroll
         for (int z = 0; z < NMAX; ++z)
           if (z < M) {
             const float2 y = Fm[z * NMAX + row];
             g2 = __fmaf_rn(x[z].x, y.x, __fmaf_rn(-x[z].y, y.y, g2));
           }
+        pair2_add(th, tl, make_float2(Fm[row * NMAX + row].x, g2));
       }
       __syncwarp();
     }
@@ -355,12 +355,12 @@ __global__ void __launch_bounds__(32 * kBlkWarps, NMAX > 24 ? 2 : 3)
           const float z1x = u[f].x - v[f].y, z1y = v[f].x + u[f].y;  // (a, c)
           s = __fmaf_rn(gt.x, z1x, __fmaf_rn(-gt.y, z1y, s));
         }
-        g2 = __fmaf_rn(2.f, s, g2);
+        pair2_add(th, tl, make_float2(0.f, 2.f * s));
       }
     }
     __syncwarp();  // d, S and F are rewritten by the next batch
-    acc_tr += (double)tr;
-    acc_g2 += (double)g2;
+    acc_tr += widen(th.x) + widen(tl.x);
+    acc_g2 += widen(th.y) + widen(tl.y);
   }
   // deterministic: xor tree in each warp, then the warps in order
   for (int off = 16; off; off >>= 1) {

@@ -84,6 +84,13 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   const float bb = __fsub_rn(s, a);
   e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
+// (h, l) += v per component, packed: two_sum, its errors summed in l.
+__device__ __forceinline__ void pair2_add(float2& h, float2& l, float2 v) {
+  const float2 m1 = make_float2(-1.f, -1.f), s = __fadd2_rn(h, v), bb = __ffma2_rn(h, m1, s);
+  const float2 e = __fadd2_rn(__ffma2_rn(__ffma2_rn(bb, m1, s), m1, h), __ffma2_rn(bb, m1, v));
+  h = s;
+  l = __fadd2_rn(l, e);
+}
 // (sh, sl) += (ah + al)(bh + bl): exact head product, first-order cross terms,
 // head sum by two_sum; (sh, sl) is left unnormalised.
 __device__ __forceinline__ void acc_prod(float ah, float al, float bh, float bl, float& sh, float& sl) {

@@ -167,3 +167,30 @@ def test_levels_that_nearly_coincide(nb, m, p, split):
     ref = pole_oracle.density(s.H, s.P, s.sigma_inf, s.pole.p, s.pole.V, s.beta, 0.1)
     assert abs(n[0] - ref["N"]) < 1e-12 * ref["N"]
     assert _rel(rho.cpu().numpy(), np.asarray(ref["rho"]).reshape(-1)) < 1e-12
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nb,m,n_iw", [(13, 5, 300), (40, 14, 200), (60, 20, 130), (9, 1, 257)])
+def test_mixed_frequency_sums_keep_more_bits_than_their_terms(nb, m, n_iw):
+    """Levels that do not couple to the orbitals: rho_k there is the sum over the frequencies of 1 / (i w + mu - e),
+    FP32 numbers above the FP64 limit.  Against the FP64 sum of the same FP32 numbers (bound: 1e2 roundings of FP64
+    times beta; FP32 sums of a batch are off by 1e-9)."""
+    beta, rng = 1.0, np.random.default_rng(nb)
+    s = _inputs(2, nb, m, n_iw, beta, 1)
+    e = rng.choice([-1.0, 1.0], (2, nb)) * rng.integers(40 * 64, 80 * 64, (2, nb)) / 64.0
+    s.H[:] = e[:, :, None] * np.eye(nb)
+    s.P[:] = np.eye(m, nb)
+    g = _context(s, precision="mixed")
+    rho = g.density_matrix([0.0])[0].cpu().numpy().reshape(2, nb, nb)
+    log = g.tuning_log()
+    g.close()
+    n64 = int(log.split("block form, ")[1].split()[0])
+    assert "in FP32 and FP32 pairs" in log and n64 < n_iw
+    w = (2.0 * np.arange(n_iw) + 1.0) * np.pi / beta
+    x, w32 = (-e[:, m:]).astype(np.float32)[:, :, None], w.astype(np.float32)
+    q = np.float32(1.0) / (x.astype(np.float64) ** 2 + (w32 * w32).astype(np.float64)).astype(np.float32)
+    d = np.where(np.arange(n_iw) < n64, -e[:, m:, None] / (e[:, m:, None] ** 2 + w * w), (x * q).astype(np.float64))
+    tail = 2.0 / beta * np.sum((1.0 / (w * w))[::-1]) - beta / 4.0
+    ref = 2.0 / beta * d.sum(2) + tail * e[:, m:] + 0.5
+    got = np.diagonal(rho, axis1=1, axis2=2)[:, m:]
+    assert np.max(np.abs(got - ref)) < 2e-14
