@@ -48,6 +48,8 @@ namespace {
 // bands 0.40 / 0.42 (0.40 / 0.43; with five N(mu) before it 1.07 / 0.79, 0.88 / 0.81); at 4: 2.0 /
 // 1.6 (1.6 / 1.6), 3.0 / 2.4 (2.3 / 2.5), 11.1 / 7.1 (8.0 / 7.2), 0.42 / 0.39 (0.40 / 0.40).
 constexpr int kBlkMinFreq = 16;
+// CTAs of a launch per SM, which set the widths of the frequency chunks.
+constexpr double kBlkItems = 48.0;
 // Lowest pi / beta of the block form (eV): below it an eigenvalue of the n2 block that happens
 // to lie near mu would cost more digits than the pivoted inverse loses.
 constexpr double kBlkMinW = 1e-4;
@@ -545,8 +547,11 @@ gf_status run_block(gf_ctx* c, int mode, gf::PointParams p) {
   const bool kred = (mode & (gf::kGloc | gf::kAdj)) != 0;
   const bool low = block_low(c, mode);
   const int nc = low ? c->blk_nc : c->n_iw;
-  // (the few FP64 frequencies of mixed precision in chunks of one batch: they are latency bound)
-  const int cw0 = low ? gf::block_batch(c->mmax) : c->blk_cw;
+  // (the FP64 frequencies of mixed precision, mostly few, in chunks of one batch: they are latency bound.
+  // Their number grows with beta, and each chunk of rho_k holds as much as H: then wider, as blk_cw)
+  const int batch = gf::block_batch(c->mmax);
+  const double items = std::ceil((double)c->n_k * ((nc + batch - 1) / batch) / (kBlkItems * c->sm_count));
+  const int cw0 = low ? batch * (int)std::max(1.0, items) : c->blk_cw;
   const int ch0 = (nc + cw0 - 1) / cw0;
   const int ch1 = (c->n_iw - nc + c->blk_cw - 1) / c->blk_cw;
   c->run_chunks = ch0 + ch1;
@@ -1173,20 +1178,20 @@ gf_status init_ctx(gf_ctx* c, const gf_desc* d) {
   std::vector<int2> units;
   std::vector<int> perm(2 * (size_t)c->n_k), bsysg;
   if (c->blk_shape) {
-    // chunks: whole batches of a CTA, about 16 CTAs per resident one; k-groups: about 12 (the FP32
+    // chunks: whole batches of a CTA, about 16 CTAs per resident one (three an SM); k-groups: about 12 (the FP32
     // N(mu) kernel's batch is a multiple of the FP64 one's).  Half as many leave a longer last wave:
     // G_loc of 256 k-points of 40 bands in mixed precision 5.3 instead of 5.1 ms, every output of 48
     // of 96 bands 12.7 instead of 12.2, N(mu) of 32 of 64 bands in FP64 4.5 instead of 4.2; twice as
     // many gain nothing, and 32 cost N(mu) of 96 of 88 bands in mixed precision 0.76 instead of 0.48.
-    const double res = 3.0 * c->sm_count, pts = (double)c->n_k * c->n_iw;
-    double batch = gf::block_batch(c->mmax), w = std::ceil(pts / (16.0 * res) / batch) * batch;
+    const double pts = (double)c->n_k * c->n_iw;
+    double batch = gf::block_batch(c->mmax), w = std::ceil(pts / (kBlkItems * c->sm_count) / batch) * batch;
     if (c->precision == GF_PREC_MIXED && w > batch) {
       batch = gf::block32_batch(c->mmax);
       w = std::ceil(w / batch) * batch;
     }
     c->blk_cw = (int)std::min(std::max(batch, w), std::ceil((double)c->n_iw / batch) * batch);
     const int nch = (c->n_iw + c->blk_cw - 1) / c->blk_cw;
-    c->blk_kg = (int)std::max(1.0, std::min((double)gf::kMaxKGroup, std::floor((double)c->n_k * nch / (12.0 * res))));
+    c->blk_kg = (int)std::max(1.0, std::min((double)gf::kMaxKGroup, std::floor((double)c->n_k * nch / (36.0 * c->sm_count))));
     c->blk_sys_g0.assign(c->n_sys, 0);
     c->blk_sys_g1.assign(c->n_sys, 0);
     for (int s = 0; s < c->n_sys; ++s) {

@@ -194,3 +194,33 @@ def test_mixed_frequency_sums_keep_more_bits_than_their_terms(nb, m, n_iw):
     ref = 2.0 / beta * d.sum(2) + tail * e[:, m:] + 0.5
     got = np.diagonal(rho, axis1=1, axis2=2)[:, m:]
     assert np.max(np.abs(got - ref)) < 2e-14
+
+
+@pytest.mark.gpu
+def test_low_temperature_does_not_multiply_the_scratch_of_rho(monkeypatch):
+    """Mixed precision at beta = 1e4, where 400 frequencies run in FP64, over many k-points: device memory of rho_k no
+    more than the general kernels take, but for the tables of the set-up (U, the n2 blocks, the pairs of B with their
+    moments in three widths, the rotation: 12 times H for these windows)."""
+    import torch
+    nk, nb, m, n_iw, beta = 6000, 12, 3, 512, 1e4
+    rng = synth.rng_for(2)
+    pole = synth.sigma_two_pole(rng, m, 4.0)
+    s = synth.System(synth.hamiltonian_dense(rng, nk, nb, -8.0, 8.0, 0.3), synth.projectors(rng, nk, nb, m), pole,
+                     pole.sample(beta, n_iw), beta, nb / 2.0)
+
+    def taken():
+        g = _context(s, precision="mixed")
+        out = torch.zeros(nk * nb * nb, dtype=torch.complex128, device="cuda")
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        g.density_matrix([0.1], out=out)
+        used = free - torch.cuda.mem_get_info()[0]
+        log = g.tuning_log()
+        g.close()
+        return used, log
+
+    block, log = taken()
+    assert int(log.split("block form, ")[1].split()[0]) >= 400
+    monkeypatch.setenv("GF_KERNEL", "f32r")
+    general, _ = taken()
+    assert block < general + 12 * 16 * nk * nb * nb
