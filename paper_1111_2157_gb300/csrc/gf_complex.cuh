@@ -49,13 +49,17 @@ __device__ __forceinline__ double2 crcp(double2 a) {
   }
 }
 
-// 1 / x to rounding for normal x and 1 / x: the 20-bit seed of rcp.approx.ftz.f64, which the FP64 pipe
-// does not take part in, and two Newton steps, four FP64-pipe instructions.
+// 1 / x within one unit in the last place where x and 1 / x are normal: the 20-bit seed of
+// rcp.approx.ftz.f64, which the FP64 pipe does not take part in, and two steps of Newton's iteration r <- r
+// + r (1 - x r), four FP64-pipe instructions.  The seed itself where it is 0 or infinite (x infinite or above
+// 2^1022, zero or denormal), which the steps would turn into NaN: band denominators (mu - e)^2 + w^2 overflow
+// for |mu| above 1e154 (their w is at least 1e-4); pivots are scaled to [1, 8), the eigensolver's kept off 0.
 __device__ __forceinline__ double rcp_newton(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
+  const unsigned e = ((unsigned)__double2hiint(r) >> 20) & 0x7ffu;
+  const double q = fma(r, fma(-x, r, 1.0), r), v = fma(q, fma(-x, q, 1.0), q);
+  return e - 1u < 0x7feu ? v : r;
 }
 
 // Pivot key of a complex FP64 number: max(|Re|, |Im|) compared through the IEEE

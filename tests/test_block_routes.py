@@ -224,3 +224,16 @@ def test_low_temperature_does_not_multiply_the_scratch_of_rho(monkeypatch):
     monkeypatch.setenv("GF_KERNEL", "f32r")
     general, _ = taken()
     assert block < general + 12 * 16 * nk * nb * nb
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision,mu", [("fp64", 1e170), ("fp64", -1e155), ("fp64", 1e100)])
+def test_a_chemical_potential_whose_square_overflows(precision, mu):
+    """1 / (i w + mu - e) of every level is below the sums' last place: N and dN/dmu are the tail's, as on the general
+    kernels."""
+    s = _inputs(2, 40, 14, 64, 40.0, 8)
+    a, log = _run(s, None, precision=precision, mu=mu)
+    b, _ = _run(s, "direct", mu=mu)
+    assert "mode 7: block form" in log
+    for key in ("N", "occ", "dN_dmu", "docc", "rho", "n_corr"):
+        assert _rel(a[key], b[key]) < (1e-10 if precision == "fp64" else 1e-6), key
