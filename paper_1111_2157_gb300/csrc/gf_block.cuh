@@ -51,6 +51,7 @@ constexpr int kBlkSeries = 40;  // moments kept
 // margin for the j^2 of the third powers (FP32: only the count depends on it).
 __device__ __forceinline__ int series_terms(float dx, float w, float r, float bits) {
   const float xr = dx / r, xi = w / r;
+  if (!(fabsf(xr) < 1e9f && xi < 1e9f)) return 1 << 20;  // (x^4 leaves the FP32 range)
   const float ur = xr * xr - xi * xi - 1.f, ui = 2.f * xr * xi, au = sqrtf(ur * ur + ui * ui);
   const float p = sqrtf(0.5f * (au + fabsf(ur))), h = p > 0.f ? 0.5f * fabsf(ui) / p : 0.f;
   const float sr = ur >= 0.f ? p : h, si = ur >= 0.f ? h : p;

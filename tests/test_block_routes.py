@@ -227,7 +227,8 @@ def test_low_temperature_does_not_multiply_the_scratch_of_rho(monkeypatch):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("precision,mu", [("fp64", 1e170), ("fp64", -1e155), ("fp64", 1e100)])
+@pytest.mark.parametrize("precision,mu", [("fp64", 1e170), ("fp64", -1e155), ("fp64", 1e100), ("mixed", 1e30),
+                                          ("mixed", -1e18)])
 def test_a_chemical_potential_whose_square_overflows(precision, mu):
     """1 / (i w + mu - e) of every level is below the sums' last place: N and dN/dmu are the tail's, as on the general
     kernels."""
