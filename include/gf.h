@@ -73,9 +73,10 @@ typedef enum {
  * It needs Hermitian H_k (to 4 rounding errors of its largest entry), P_k P_k^+
  * with a condition number of at most about 100 (mixed: 32) and entries of P_k
  * within 1e-60 to 1e60 (mixed: 1e-6 to 1e6), m <= 32, m < N_b and
- * N_b - m <= 256 at every k, at least 16 frequencies and pi / beta >= 1e-4; the
- * general kernels take the other inputs, and every call when the environment
- * variable GF_KERNEL is "direct" (in mixed precision: when it has any value).
+ * N_b - m <= 256 at every k, at least 16 frequencies (mixed: 40) and
+ * pi / beta >= 1e-4; the general kernels take the other inputs, and every call
+ * when the environment variable GF_KERNEL is "direct" (in mixed precision: when
+ * it has any value).
  * FP64 and pair contexts compute it in FP64.  Mixed: FP64 up to a twentieth of
  * the rms level of H; above, the m x m matrix S in FP32 pairs, its
  * inverse in FP32 with one refinement step for G_loc and the adjoint, traces and

@@ -42,12 +42,13 @@ void set_global_error(const char* msg) noexcept {
 
 namespace {
 
-// The block form pays for an eigenproblem per k from this many frequencies on.  New H and a fused
-// pass, general kernels against the block form, at 16 frequencies: 64 k-points of 40 bands 2.4 / 1.7
-// ms (mixed 1.8 / 1.8), 256 5.8 / 3.4 (3.5 / 2.8), 48 of 96 bands 17.0 / 7.9 (10.8 / 7.2), 64 of 8
-// bands 0.40 / 0.42 (0.40 / 0.43; with five N(mu) before it 1.07 / 0.79, 0.88 / 0.81); at 4: 2.0 /
-// 1.6 (1.6 / 1.6), 3.0 / 2.4 (2.3 / 2.5), 11.1 / 7.1 (8.0 / 7.2), 0.42 / 0.39 (0.40 / 0.40).
-constexpr int kBlkMinFreq = 16;
+// The block form pays for an eigenproblem per k from this many frequencies on.  New H, four N(mu) and
+// G_loc, general kernels / block form, FP64 at 16 frequencies: 64 k-points of 8 bands 0.76 / 0.57 ms, 256 of
+// 40 17.5 / 4.4, 64 of 96 52 / 7.7, 4 of 40 4.0 / 2.1 (one N(mu) alone 0.22 / 0.25, 3.6 / 2.1, 10.6 / 5.4,
+// 0.95 / 1.27).  Mixed at 16: 0.54 / 0.59, 2.9 / 3.2, 5.5 / 6.8, 1.2 / 2.2; at 40: 0.60 / 0.60, 5.0 / 3.3, 12.6
+// / 7.0, 1.2 / 2.2 (one N(mu) alone 0.19 / 0.26, 0.87 / 1.88, 2.3 / 5.2, 0.41 / 1.29, equal from about 150, but
+// for 4 k-points, which pay 0.9 ms on every new H and gain 0.2 on every later N(mu)).
+constexpr int kBlkMinFreq = 16, kBlkMinFreqMixed = 40;
 // CTAs of a launch per SM, which set the widths of the frequency chunks.
 constexpr double kBlkItems = 48.0;
 // Lowest pi / beta of the block form (eV): below it an eigenvalue of the n2 block that happens
@@ -1160,7 +1161,7 @@ gf_status init_ctx(gf_ctx* c, const gf_desc* d) {
 
   // block form: every window wider than its orbitals, one lane per orbital, eigenproblems within
   // the eigensolver's size, and enough frequencies to pay for the eigenproblem per k
-  c->blk_shape = c->n_iw >= kBlkMinFreq;
+  c->blk_shape = c->n_iw >= (c->precision == GF_PREC_MIXED && !c->lowrank ? kBlkMinFreqMixed : kBlkMinFreq);
   std::vector<int64_t> offT(2 * (size_t)c->n_k);  // of T, then of C
   for (int k = 0; k < c->n_k; ++k) {
     const int m = c->msys[c->ksys[k]], n2 = c->nb[k] - m;

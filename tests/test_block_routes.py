@@ -238,3 +238,18 @@ def test_a_chemical_potential_whose_square_overflows(precision, mu):
     assert "mode 7: block form" in log
     for key in ("N", "occ", "dN_dmu", "docc", "rho", "n_corr"):
         assert _rel(a[key], b[key]) < (1e-10 if precision == "fp64" else 1e-6), key
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision,lowrank,n_iw,on_block", [
+    ("fp64", False, 15, False), ("fp64", False, 16, True), ("mixed", False, 39, False), ("mixed", False, 40, True),
+    ("mixed", True, 16, True)])
+def test_few_frequencies_do_not_pay_for_the_set_up(precision, lowrank, n_iw, on_block):
+    """The first number of frequencies on the block form of each precision, and N on both sides of it."""
+    s = _inputs(2, 24, 7, n_iw, 20.0, 4)
+    g = _context(s, precision=precision, lowrank=lowrank)
+    n, _ = g.occupation([0.1])
+    assert ("block form, " in g.tuning_log()) == on_block
+    g.close()
+    ref = oracle.get().density(s.H, s.P, s.sigma, s.sigma_inf, s.beta, 0.1, want_rho=False)
+    assert abs(n[0] - ref["N"]) < (1e-7 if precision == "mixed" else 1e-10) * ref["N"]
