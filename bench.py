@@ -291,7 +291,7 @@ def executed_flops(g, st, systems, mode):
     """Floating-point operations of the call that st belongs to.  Where the block form ran, its own (2 per
     multiply-add of the band sums, the m x m inverse and products; k-independent parts are done once per
     upload and not counted), which are several times fewer than the N_b^3 count of the library's counter."""
-    if "block form" not in g.tuning_log():
+    if "block form, " not in g.tuning_log():
         return st["flops"]
     occ, rho, adj = mode in ("occ", "gloc_occ", "evaluate", "backward"), mode == "evaluate", mode == "backward"
     total = pts = 0.0
@@ -884,7 +884,7 @@ def main():
                    "speedup_vs_direct_fp64_gpu": (lt["points"] / lr["elapsed"]) / (totals["points"] / elapsed),
                    "N_rel_err_vs_direct": abs(n_lr[0] - info["N"]) / abs(info["N"]),
                    "G_loc_rel_err_vs_direct": float((gl_lr - gl_fp).abs().max() / gl_fp.abs().max()),
-                   "algorithm": "the block form, as the direct path" if "block form" in gr.tuning_log() else
+                   "algorithm": "the block form, as the direct path" if "block form, " in gr.tuning_log() else
                                 "G in the eigenbasis of H_k (Woodbury identity), FP64; H_k diagonalised once",
                    "gpu_launches": lt["launches"], "mixed_precision": mixed_lowrank}
         gr.close()
@@ -947,7 +947,7 @@ def main():
         if not args.no_batched:
             batched = batched_leg(gf, synth, o, nk_scale=args.nk_scale)
 
-    block = "block form" in g.tuning_log()
+    block = "block form, " in g.tuning_log()
     if args.precision == "fp64" or (args.precision == "pair" and block):
         peak, peak_source = FP64_PEAK_TFLOPS, "FP64 DFMA: 152 SMs x 2/clk x 2 flop x 2.07 GHz"
     elif args.precision == "mixed":

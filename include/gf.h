@@ -380,7 +380,9 @@ const char *gf_tuning_log(const gf_ctx *ctx);
  * point-kernel launches in milliseconds (CUDA events recorded on the context's
  * stream around each launch), and their algorithmic floating-point operations
  * (8 per complex multiply-add: N_b^3 for the inverse, m^2 N_b + m N_b^2 for the
- * embedding, plus the epilogue's projections and traces). */
+ * embedding, plus the epilogue's projections and traces; with GF_FLAG_LOWRANK
+ * those of its form).  On the block form the count is the same, of work that it
+ * does not do. */
 gf_status gf_last_stats(const gf_ctx *ctx, int64_t *kernel_launches, int64_t *points,
                         double *point_kernel_ms, double *point_flops);
 

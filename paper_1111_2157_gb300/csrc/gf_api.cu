@@ -178,10 +178,11 @@ gf_status ensure_block(gf_ctx* c) {
   int flags = 0;
   std::memcpy(&flags, &info[c->n_k], sizeof(int));
   c->blk_ok = flags == 0;
-  if (flags) {
-    c->tune_log += "block form: general kernels (" +
-                   std::string(flags & gf::kBlkNonHermitian ? "H not Hermitian" :
-                               flags & gf::kBlkIllConditioned ? "P ill-conditioned" : "eigensolver") + "); ";
+  if (flags) {  // (said once: uploads can follow one another for the life of the context)
+    const std::string why = "block form: general kernels (" +
+                            std::string(flags & gf::kBlkNonHermitian ? "H not Hermitian" :
+                                        flags & gf::kBlkIllConditioned ? "P ill-conditioned" : "eigensolver") + "); ";
+    if (c->tune_log.find(why) == std::string::npos) c->tune_log += why;
     return GF_OK;
   }
   // mixed precision: frequencies w_n below a twentieth of the rms eigenvalue of H run in FP64, at

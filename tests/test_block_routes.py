@@ -253,3 +253,18 @@ def test_few_frequencies_do_not_pay_for_the_set_up(precision, lowrank, n_iw, on_
     g.close()
     ref = oracle.get().density(s.H, s.P, s.sigma, s.sigma_inf, s.beta, 0.1, want_rho=False)
     assert abs(n[0] - ref["N"]) < (1e-7 if precision == "mixed" else 1e-10) * ref["N"]
+
+
+@pytest.mark.gpu
+def test_the_log_does_not_grow_with_the_uploads():
+    s = _inputs(2, 12, 4, 24, 20.0, 4)
+    s.H[0, 0, 1] += 1e-3
+    g = _context(s)
+    g.occupation([0.1])
+    log = g.tuning_log()
+    assert log.count("H not Hermitian") == 1
+    for _ in range(3):
+        g.set_hamiltonian(s.H)
+        g.occupation([0.1])
+    assert g.tuning_log() == log
+    g.close()
