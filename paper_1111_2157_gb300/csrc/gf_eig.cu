@@ -839,7 +839,8 @@ __global__ void __launch_bounds__(kEigThreads) k_pole_eig(const PoleParams p) {
   __shared__ QlScratch ql;
   __shared__ double red[kEigThreads / 32];
   const int tid = threadIdx.x;
-  for (int k = blockIdx.x; k < p.n_k; k += gridDim.x) {
+  bool all = false;  // a second pass over k with every row of the eigenvectors
+  for (int k = blockIdx.x; k < p.n_k;) {
     const KInfo ki = p.kinfo[k];
     const SInfo si = p.sinfo[ki.sys];
     const PInfo pi = p.pinfo[ki.sys];
@@ -888,8 +889,9 @@ __global__ void __launch_bounds__(kEigThreads) k_pole_eig(const PoleParams p) {
     }
     __syncthreads();
     // N(mu) needs Psi_b^+ Psi_b = 1 - Psi_p^+ Psi_p only: the pole rows, where they are the fewer
-    // (125 k-points of 40 bands and 28 poles 1.42 ms, all rows 1.64 ms)
-    const bool few = p.mode == kOcc && npl <= nb;
+    // (125 k-points of 40 bands and 28 poles 1.42 ms, all rows 1.64 ms), unless the difference loses
+    // digits: N_k far below the number of occupied pole levels (at N_k = 5e-5 of it 5e-12, all rows 2e-14)
+    const bool few = p.mode == kOcc && npl <= nb && !all;
     const bool ok = heev_tri(A, V, n, ld, p.in_smem, p.z_smem, smem_raw, ql, nb, few ? npl : -1);
     if (!ok && tid == 0) atomicOr(p.status, 2);
     // per eigenpair: x_l = E_l - mu, n_F(x_l), cosh(beta x_l / 2)
@@ -913,6 +915,10 @@ __global__ void __launch_bounds__(kEigThreads) k_pole_eig(const PoleParams p) {
         nk = fma(few ? 1.0 - wb : wb, s_f[l], nk);
       }
       nk = eig_block_sum(nk, red);
+      if (few && !(nk >= 0.0625 * npl)) {
+        all = true;
+        continue;
+      }
       double dk = 0.0;
       for (int e = tid; e < n * (n + 1) / 2; e += kEigThreads) {
         int l, l2;
@@ -1001,6 +1007,8 @@ __global__ void __launch_bounds__(kEigThreads) k_pole_eig(const PoleParams p) {
       }
     }
     __syncthreads();
+    all = false;
+    k += gridDim.x;
   }
 }
 

@@ -52,3 +52,24 @@ def test_few_distinct_levels(kind, n, m):
         assert "mode 7: block form" in log
         for key in ("N", "rho", "gloc", "n_corr"):
             assert _rel(a[key], b[key]) < 1e-12, key
+
+
+@pytest.mark.parametrize("n,m,offset", [(12, 3, 100.0), (31, 5, 1000.0), (70, 6, 1e4), (31, 5, 8.0), (20, 12, 100.0)])
+def test_few_electrons(n, m, offset):
+    """Bands far above mu, where N is the bands' small share of the occupied pole levels: relative to N, not to the
+    number of poles.  (Bound: the eigenvectors' 1e-15, over amplitudes of U / offset, on two k-points that differ.)"""
+    rng = np.random.default_rng(n)
+    H = np.array([synth.hamiltonian_dense(synth.rng_for(n), 1, n, -2.0, 2.0, 0.3)[0] + x * np.eye(n)
+                  for x in (offset, 0.0)])
+    P = np.array([np.linalg.qr(rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n)))[0][:m] for _ in range(2)])
+    pole = synth.sigma_two_pole(synth.rng_for(3), m, 3.0)
+    for ks in ([0], [0, 1]):
+        g = gf.GreensFunction([n] * len(ks), [m], 24, [40.0])
+        g.set_hamiltonian(H[ks].reshape(-1))
+        g.set_projectors(P[ks].reshape(-1))
+        g.set_sigma_poles([len(pole.p)], pole.p, pole.V.reshape(-1), pole.sigma_inf.reshape(-1))
+        num, dn = g.pole_occupation([0.1])
+        g.close()
+        ref = pole_oracle.density(H[ks], P[ks], pole.sigma_inf, pole.p, pole.V, 40.0, 0.1)
+        assert abs(num[0] - ref["N"]) < 1e-15 * (10.0 + offset) * 10.0 * ref["N"]
+        assert abs(dn[0] - ref["dN_dmu"]) < 1e-10 * abs(ref["dN_dmu"])
