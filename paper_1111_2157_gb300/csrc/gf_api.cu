@@ -97,6 +97,17 @@ gf_status ensure_lr(gf_ctx* c) {
   return GF_OK;
 }
 
+// No device memory for the block form's tables or for its scratch beside them: the general kernels from now on.
+void drop_block(gf_ctx* c, const char* what) {
+  cudaGetLastError();
+  for (DevBuf* b : {&c->blk_e, &c->blk_T, &c->blk_Ts, &c->blk_Tp, &c->blk_B, &c->blk_Bs, &c->blk_HO, &c->blk_U,
+                    &c->blk_D22, &c->blk_V, &c->blk_Ri, &c->blk_H11, &c->blk_tau, &c->blk_C, &c->blk_Cs, &c->blk_Cp,
+                    &c->blk_ser, &c->blk_ws, &c->blk_info})
+    release(*b);
+  c->blk_shape = c->blk_ok = false;
+  c->tune_log += std::string("block form: general kernels (") + what + " does not fit in device memory); ";
+}
+
 // Block form (gf_block.cuh) of the uploaded H and P, once per upload.  blk_ok is false when an
 // H_k is not Hermitian to rounding, a P_k has (nearly) dependent rows, an eigenproblem does not
 // converge or the tables do not fit: every call then takes the general kernels.
@@ -125,10 +136,7 @@ gf_status ensure_block(gf_ctx* c) {
               {&c->blk_ws, 16 * ws},                 {&c->blk_info, 8 * ((size_t)c->n_k + 1)}};
   for (auto& n : need) {
     if (ensure(*n.b, n.bytes) == cudaSuccess) continue;
-    cudaGetLastError();
-    for (auto& r : need) release(*r.b);
-    c->blk_shape = false;  // no room for the tables: the general kernels from now on
-    c->tune_log += "block form: tables do not fit in device memory; ";
+    drop_block(c, "a table");
     return GF_OK;
   }
   gf::BlockSetup b{};
@@ -566,6 +574,8 @@ gf_status run_block(gf_ctx* c, int mode, gf::PointParams p) {
     p.rho_chunk_stride = c->totH;
     GF_CU(ensure(c->rho_part, sizeof(double2) * (size_t)c->totH * c->run_chunks));
     p.rho_part = c->rho_part.as<double2>();
+    GF_CU(ensure(c->lr_T, sizeof(double2) * c->totH));  // (what follows the kernels: no room shows here)
+    GF_CU(ensure(c->rho_out, sizeof(double2) * c->totH));
   }
   if (mode & gf::kAdj) {
     GF_CU(ensure(c->mubar_part, sizeof(double) * (size_t)c->n_k * c->run_chunks));
@@ -705,7 +715,17 @@ gf_status run_points(gf_ctx* c, int mode) {
     p.Gbd = (df64 && c->have_gbar_for_call) ? c->Gbd.as<float4>() : nullptr;
     p.nbar = c->nbar.as<double>();
   }
-  if (block) return run_block(c, mode, p);
+  if (block) {
+    st = run_block(c, mode, p);
+    if (st != GF_ENOMEM || c->capturing) return st;
+    GF_CU(cudaStreamSynchronize(c->stream));
+    drop_block(c, "the scratch");
+    c->run_on_block = false;
+    c->run_chunks = c->n_chunks;
+    c->err.clear();
+    st = ensure_lr(c);
+    if (st) return st;
+  }
   if (mode & gf::kOcc) {
     GF_CU(ensure(c->occ_part, sizeof(double) * 2 * (size_t)c->n_k * c->n_chunks));
     p.occ_part = c->occ_part.as<double>();

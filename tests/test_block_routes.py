@@ -268,3 +268,49 @@ def test_the_log_does_not_grow_with_the_uploads():
         g.occupation([0.1])
     assert g.tuning_log() == log
     g.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_scratch_that_does_not_fit_beside_the_tables(precision):
+    """Device memory for the block form's tables but not for its scratch beside them, and enough for the general
+    kernels: the call runs on those."""
+    import torch
+    nk, nb, m, n_iw = 2000, 40, 24, 64
+    rng = synth.rng_for(2)
+    pole = synth.sigma_two_pole(rng, m, 4.0)
+    s = synth.System(synth.hamiltonian_dense(rng, nk, nb, -8.0, 8.0, 0.3), synth.projectors(rng, nk, nb, m), pole,
+                     pole.sample(40.0, n_iw), 40.0, nb / 2.0)
+    out = torch.zeros(nk * nb * nb, dtype=torch.complex128, device="cuda")
+    torch.cuda.empty_cache()
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    def taken(kernel):
+        with pytest.MonkeyPatch.context() as mp:
+            if kernel:
+                mp.setenv("GF_KERNEL", kernel)
+            g = _context(s, precision=precision)
+            before = free()
+            g.density_matrix([0.1], out=out)
+            used = before - free()
+            log = g.tuning_log()
+            g.close()
+        return used, log, out.clone()
+
+    block, log, ref = taken(None)
+    general, _, _ = taken("direct" if precision == "fp64" else "f32r")
+    assert "block form, " in log and general < block - (64 << 20)
+    g = _context(s, precision=precision)
+    hold = torch.empty(free() - block + (24 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        g.density_matrix([0.1], out=out)
+        log = g.tuning_log()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert "does not fit in device memory" in log and "mode 2: block form" not in log
+    assert _rel(out.cpu().numpy(), ref.cpu().numpy()) < (1e-10 if precision == "fp64" else 1e-5)
+    g.close()
