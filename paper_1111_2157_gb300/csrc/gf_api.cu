@@ -54,11 +54,11 @@ constexpr double kBlkItems = 48.0;
 // Lowest pi / beta of the block form (eV): below it an eigenvalue of the n2 block that happens
 // to lie near mu would cost more digits than the pivoted inverse loses.
 constexpr double kBlkMinW = 1e-4;
-// Largest condition number of O = (P P^+)^{-1}, as k_block_check estimates it.  Mixed, at 40 to 46: N
-// to 5e-9, dN/dmu 7e-8, rho_k 2e-8, G_loc 9e-13, each no further from FP64 than the general kernels (7e-9,
-// 4e-6, 2e-7, 6e-12); at 66 to 96 G_loc 2.6e-12 and N 1.1e-8, at 350 1.7e-11 and 1.7e-8, at 2300 2e-9 and 2e-7.
-// FP64 against the general kernel: up to 100 dN/dmu 4e-12 and G_loc 2e-13, at 860 2e-10 and 1e-12.  (Windows of 24 to
-// 96 bands, 5 to 30 orbitals, beta 40 to 400, one small singular value of P or a geometric row of them.)
+// Largest condition number of O = (P P^+)^{-1}, as k_block_check estimates it.  Mixed, at 40 to 46: N to
+// 5e-9, dN/dmu 7e-8, rho_k 2e-8, G_loc 9e-13, each no further from FP64 than the general kernels (7e-9, 4e-6,
+// 2e-7, 6e-12); at 66 to 96 G_loc 2.6e-12 and N 1.1e-8, at 350 1.7e-11 and 1.7e-8, at 2300 2e-9 and 2e-7.
+// FP64 against the general kernel: up to 100 dN/dmu 4e-12 and G_loc 2e-13, at 860 2e-10 and 1e-12.  (Windows
+// of 24 to 96 bands, 5 to 30 orbitals, beta 40 to 400, one small singular value of P or a geometric row.)
 constexpr double kBlkCondMixed = 32.0, kBlkCondFp64 = 100.0;
 // ... and of |R|^2, |R^{-1}|^2 (the scale of P), from which O and B B^+ stay far inside the number range.
 constexpr double kBlkRangeMixed = 1e12, kBlkRangeFp64 = 1e120;

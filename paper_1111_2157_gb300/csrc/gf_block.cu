@@ -15,7 +15,7 @@
 // frequencies): every output in 58.7 ms, 210 ms by the inverse; mu search and G_loc of 64 k-points
 // 50 ms, 340 ms.
 // LOW is bound by latency (issue slots 50-65 % busy at 11 to 14 warps an SM, FMA pipe 37-44 %):
-// every output of 256 k-points in 10.2 ms, 20.8 ms with S and its inverse in FP64.
+// every output of 256 k-points in 9.7 ms, 20.8 ms with S and its inverse in FP64.
 #include <math.h>
 #include <stdint.h>
 
@@ -1123,7 +1123,7 @@ __global__ void __launch_bounds__(32 * kBlkWarps,
           // B by pairs of rows, {Re, Re, Im, Im}, 0 beyond M and n2: over the dead arrays like Y, anew
           // for each batch (12 KB from L2 for 4 frequencies at 76 levels and 20 orbitals), since the
           // room it would hold costs the third CTA on an SM: 14.1 -> 12.7 ms for every output of 48
-          // k-points x 2048 frequencies at 96 bands
+          // k-points x 2048 frequencies at 96 bands (13.2 with the frequency sums in pairs)
           float4* sB = reinterpret_cast<float4*>(smraw + L.oB);
           const int pb = (n2 + 3) & ~3;
           const float2* Bk = bf.Bs + ki.offP;
@@ -1145,10 +1145,11 @@ __global__ void __launch_bounds__(32 * kBlkWarps,
           auto add = [&](int at, double2 o, double2 v) { Sk[at] = make_double2(o.x + v.x, o.y + v.y); };
           if constexpr (LOW) {
             // FP32 products, summed over the nf frequencies in pairs (in FP32 the sums would be off by 1e-8 and
-            // 7 % faster) and added to the chunk's FP64 sum once (each FP64 add takes the SM 16 clocks).  Rows 1 of G_k are [A, Y],
-            // Y = A B D, rows 2 are D B^+ [A, Y] + D: orbitals lie in pairs of rows, {Re, Re, Im, Im},
-            // so that the packed FMAs take two terms of the contraction over them, and columns of a
-            // thread lie a third of the matrix apart, so that a warp's loads are consecutive.
+            // the pass 7 % faster) and added to the chunk's FP64 sum once (each FP64 add takes the SM 16
+            // clocks).  Rows 1 of G_k are [A, Y], Y = A B D, rows 2 are D B^+ [A, Y] + D: orbitals lie in
+            // pairs of rows, {Re, Re, Im, Im}, so that the packed FMAs take two terms of the contraction over
+            // them, and columns of a thread lie a third of the matrix apart, so that a warp's loads are
+            // consecutive.
             const int KP = (M + 1) / 2, CT = M + n2, pb = (n2 + 3) & ~3;
             const float4* sB = reinterpret_cast<const float4*>(smraw + L.oB);
             const float4* sA = reinterpret_cast<const float4*>(smraw + L.oG);  // [frequency][KP][M]

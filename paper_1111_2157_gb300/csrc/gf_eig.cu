@@ -416,7 +416,8 @@ __device__ bool tri_qr(double* Z, int zr, int zs, int N, QlScratch& q) {
   int hi = N - 1, steps = 0;  // warp 0: end of the active block, steps spent on its eigenvalue
   double tiny = 0.0;          // and the rounding of the norm
   if (warp == 0) {
-    for (int i = lane; i < N; i += 32) tiny = fmax(tiny, fabs(q.d[i]) + fabs(q.e[i]) + (i ? fabs(q.e[i - 1]) : 0.0));
+    for (int i = lane; i < N; i += 32)
+      tiny = fmax(tiny, fabs(q.d[i]) + fabs(q.e[i]) + (i ? fabs(q.e[i - 1]) : 0.0));
     for (int off = 16; off; off >>= 1) tiny = fmax(tiny, __shfl_xor_sync(0xffffffffu, tiny, off));
     tiny *= 1.2e-16;
   }
